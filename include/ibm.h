@@ -298,7 +298,7 @@ ibm_status ibm_body3d_create(const double *verts, int nverts, const int32_t *tri
                              ibm_body3d **out);
 
 /* Classify the lattice, tag it, build the lists and the closest features
- * (five kernels, asynchronous on the body's stream).  Device buffers are
+ * (seven kernels, asynchronous on the body's stream).  Device buffers are
  * (re)allocated when the lattice size changes; the lists hold the nodes
  * within three nodes of the bounding box.  IBM_EINVAL for an empty or
  * oversized lattice. */

@@ -25,8 +25,7 @@ extern "C" ibm_status ibm__noalloc_fail(ibm_status s, const char *msg);
 
 namespace {
 
-constexpr int B3 = 256;        // threads per block of the per-node kernels
-constexpr int CBLK = 1024;     // nodes per block of the list compaction
+constexpr int B3 = 256;        // threads per block
 constexpr uint8_t T_FLUID = IBM_TAG_FLUID, T_SOLID = IBM_TAG_SOLID, T_IB = IBM_TAG_IB, T_G1 = IBM_TAG_G1;
 
 struct Lattice {
@@ -34,50 +33,112 @@ struct Lattice {
   double lo[3], d[3];
 };
 
+// exact per-face data of the closest-feature search: vertices, the entries of the barycentric normal equations and
+// the squared edge lengths (the operations of evaluating them at every node, done once on the host)
+struct FaceExact {
+  double V[3][3];
+  double a11, a12, a22, det;
+  double ee[3];
+};
+
+constexpr int CL = 32;    // faces per cluster (Morton order of the centroids): one face per lane
+constexpr int FPLANES = 6;
+
 struct Mesh {
-  int nv, ntri;
+  int nv, ntri, ncl;
   const double *v;    // [nv][3]
   const int *tri;     // [ntri][3]
   const double *fn;   // [ntri][3] unit face normals
   const double *vn;   // [nv][3] unit angle-weighted vertex pseudo-normals
   const int *enb;     // [ntri][3] the face across edge k (vertices k, k+1), -1 if none
-  const float4 *fbox; // [ntri][2] per face: box corners (lo, hi), widened by the cull margin (culling only)
-  const float4 *fsph; // [ntri] per face: bounding-sphere centre and radius, widened by the cull margin
+  const FaceExact *fx;// [ntri]
+  const float4 *cl;   // [ncl][2] bounding box of a cluster's faces, widened by 1e-5 of the extent: lo, hi
+  const float4 *fp;   // [FPLANES][ncl * CL] FP32 faces of the clusters: vertices, unit normal, the unit in-plane
+                      // normals of the edges (inward), face index (bits; -1: padding), 1 = never pruned
+  float ext;          // largest coordinate magnitude of the mesh (at least 1)
   double bb[6];       // axis-aligned bounding box: lo x, y, z, hi x, y, z
 };
 
-__device__ __forceinline__ void node_xyz(const Lattice &L, long long n, double P[3], int ijk[3]) {
-  const long long nxy = (long long)L.nx * L.ny;
-  ijk[2] = (int)(n / nxy);
-  const long long r = n - (long long)ijk[2] * nxy;
-  ijk[1] = (int)(r / L.nx);
-  ijk[0] = (int)(r - (long long)ijk[1] * L.nx);
+// node (i, j, k) of a node index (fewer than 2^31 nodes: 32-bit division)
+__device__ __forceinline__ void node_ijk(const Lattice &L, int n, int ijk[3]) {
+  const unsigned nxy = (unsigned)L.nx * (unsigned)L.ny, m = (unsigned)n;
+  const unsigned k = m / nxy, r = m - k * nxy, j = r / (unsigned)L.nx;
+  ijk[2] = (int)k;
+  ijk[1] = (int)j;
+  ijk[0] = (int)(r - j * (unsigned)L.nx);
+}
+
+__device__ __forceinline__ void node_xyz(const Lattice &L, int n, double P[3], int ijk[3]) {
+  node_ijk(L, n, ijk);
   for (int a = 0; a < 3; a++) P[a] = L.lo[a] + ((double)ijk[a] + 0.5) * L.d[a];
 }
 
-// sign of the edge function of edge (a, b) at P in the (u, v) projection, endpoints taken in increasing vertex
-// index (the two faces sharing the edge see opposite values), a zero resolved by the symbolic shift of P by
-// (eps, eps^2) in (u, v)
-__device__ __forceinline__ int edge_sign(const double *pa, int ia, const double *pb, int ib, const double P[3], int u,
-                                         int v) {
-  int flip = 1;
+// ---- classification (Sec. 3.2) over bit planes ------------------------------------------------------------------
+// Rays along +x, +y and +z; a node is solid when at least two of its three crossing counts are odd and it lies in
+// the surface's bounding box.  Whether the ray from a node crosses a face depends on the face's edge functions at
+// the line's two transverse coordinates, the same for every node of the lattice line; only "ahead of the node", the
+// sign of n.(a - P), depends on the node, and along a line that expression is monotone in the node's coordinate
+// (each of its rounded operations is), so the nodes with the crossing ahead are the line's first t*, found by
+// bisection with the node's own operations.  A crossing therefore toggles one bit -- the last node that has it ahead
+// -- and a node's parity is the XOR of the bits at and beyond it.
+//
+// Layout: one bit per node, a word per 32 nodes along x (rows of pw words), one plane per ray axis; bit operations
+// then vote and tag 32 nodes at a time.  The work per face is its projected area in lines instead of all lines times
+// all faces: FP64, which bounds every exact geometric test on GB300 (2 lanes per SM and clock), is spent on the few
+// lines in a face's own projected box.  Appendix A sphere, 1200 faces (ncu, cold caches): classification and lists
+// 3.00 -> 0.16 ms at 256^3 nodes (k3_cross 0.11), 0.14 -> 0.055 ms at 40^3 (launches of 5-7 us each).
+struct SubBox {
+  int b0[3], n[3];  // nodes inside the bounding box along each axis: first index and count (n > 0)
+};
+
+// sign of the edge function e at P in the (u, v) projection, endpoints taken in increasing vertex index (the two
+// faces sharing the edge see opposite values), a zero resolved by the symbolic shift of P by (eps, eps^2) in (u, v)
+struct EdgeFn {
+  double au, av, du, dv;
+  int flip;
+};
+__device__ __forceinline__ EdgeFn edge_fn(const double *pa, int ia, const double *pb, int ib, int u, int v) {
+  EdgeFn e;
+  e.flip = 1;
   if (ib < ia) {
     const double *t = pa;
     pa = pb;
     pb = t;
-    flip = -1;
+    e.flip = -1;
   }
-  const double du = pb[u] - pa[u], dv = pb[v] - pa[v];
-  const double e = du * (P[v] - pa[v]) - dv * (P[u] - pa[u]);
+  e.au = pa[u];
+  e.av = pa[v];
+  e.du = pb[u] - pa[u];
+  e.dv = pb[v] - pa[v];
+  return e;
+}
+__device__ __forceinline__ int edge_sign(const EdgeFn &f, double Pu, double Pv) {
+  const double e = f.du * (Pv - f.av) - f.dv * (Pu - f.au);
   int sg = e > 0.0 ? 1 : (e < 0.0 ? -1 : 0);
-  if (sg == 0) sg = -dv > 0.0 ? 1 : (-dv < 0.0 ? -1 : 0);
-  if (sg == 0) sg = du > 0.0 ? 1 : (du < 0.0 ? -1 : 0);
-  return flip * sg;
+  if (sg == 0) sg = -f.dv > 0.0 ? 1 : (-f.dv < 0.0 ? -1 : 0);
+  if (sg == 0) sg = f.du > 0.0 ? 1 : (f.du < 0.0 ? -1 : 0);
+  return f.flip * sg;
 }
 
-// Sec. 3.2 (Moller-Trumbore, barycentric form): does the ray from P along +axis cross face f ahead of P?
-__device__ __forceinline__ int crosses(const Mesh &m, int f, const double P[3], int axis) {
-  const int u = axis == 0 ? 1 : (axis == 1 ? 2 : 0), v = axis == 0 ? 2 : (axis == 1 ? 0 : 1);
+// lattice index range of [lo, hi] along axis a, one node wider on each side, within the sub-box
+__device__ __forceinline__ void index_range(const Lattice &L, const SubBox &B, int a, double lo, double hi, int &i0,
+                                            int &i1) {
+  const double first = (double)B.b0[a], last = (double)(B.b0[a] + B.n[a] - 1);
+  const double x0 = floor((lo - L.lo[a]) / L.d[a] - 0.5) - 1.0, x1 = ceil((hi - L.lo[a]) / L.d[a] - 0.5) + 1.0;
+  i0 = (int)fmin(fmax(x0, first), last + 1.0);
+  i1 = (int)fmax(fmin(x1, last), first - 1.0);
+}
+
+// One (face, ray axis): its projected box in lattice lines and what the edge and plane tests need
+struct CrossItem {
+  EdgeFn e[3];
+  double n[3], a[3];  // unnormalised normal and first vertex, in the order (u, v, axis)
+  int u0, v0, nu, axis;
+};
+
+template <int axis>
+__device__ __forceinline__ long long cross_item(const Lattice &L, const Mesh &m, const SubBox &B, int f, CrossItem &o) {
+  constexpr int u = (axis + 1) % 3, v = (axis + 2) % 3;
   const int i0 = __ldg(m.tri + 3 * f), i1 = __ldg(m.tri + 3 * f + 1), i2 = __ldg(m.tri + 3 * f + 2);
   double a[3], b[3], c[3];
   for (int q = 0; q < 3; q++) {
@@ -85,268 +146,306 @@ __device__ __forceinline__ int crosses(const Mesh &m, int f, const double P[3], 
     b[q] = __ldg(m.v + 3 * i1 + q);
     c[q] = __ldg(m.v + 3 * i2 + q);
   }
-  const int s0 = edge_sign(a, i0, b, i1, P, u, v);
-  const int s1 = edge_sign(b, i1, c, i2, P, u, v);
-  const int s2 = edge_sign(c, i2, a, i0, P, u, v);
-  if (s0 == 0 || s0 != s1 || s1 != s2) return 0;
+  int u0, u1, v0, v1;
+  index_range(L, B, u, fmin(a[u], fmin(b[u], c[u])), fmax(a[u], fmax(b[u], c[u])), u0, u1);
+  index_range(L, B, v, fmin(a[v], fmin(b[v], c[v])), fmax(a[v], fmax(b[v], c[v])), v0, v1);
   const double e1[3] = {b[0] - a[0], b[1] - a[1], b[2] - a[2]};
   const double e2[3] = {c[0] - a[0], c[1] - a[1], c[2] - a[2]};
-  const double n[3] = {e1[1] * e2[2] - e1[2] * e2[1], e1[2] * e2[0] - e1[0] * e2[2], e1[0] * e2[1] - e1[1] * e2[0]};
-  if (n[axis] == 0.0) return 0;
-  const double num = n[0] * (a[0] - P[0]) + n[1] * (a[1] - P[1]) + n[2] * (a[2] - P[2]);
-  return ((num > 0.0 && n[axis] > 0.0) || (num < 0.0 && n[axis] < 0.0)) ? 1 : 0;
+  const double nf[3] = {e1[1] * e2[2] - e1[2] * e2[1], e1[2] * e2[0] - e1[0] * e2[2], e1[0] * e2[1] - e1[1] * e2[0]};
+  o.e[0] = edge_fn(a, i0, b, i1, u, v);
+  o.e[1] = edge_fn(b, i1, c, i2, u, v);
+  o.e[2] = edge_fn(c, i2, a, i0, u, v);
+  o.n[0] = nf[u];
+  o.n[1] = nf[v];
+  o.n[2] = nf[axis];
+  o.a[0] = a[u];
+  o.a[1] = a[v];
+  o.a[2] = a[axis];
+  o.u0 = u0;
+  o.v0 = v0;
+  o.nu = u1 - u0 + 1;
+  o.axis = axis;
+  // a face parallel to the ray is not crossed
+  return nf[axis] != 0.0 && o.nu > 0 && v1 >= v0 ? (long long)o.nu * (v1 - v0 + 1) : 0;
 }
 
-// classification along lattice lines: one warp per line along `axis`.  Whether the ray from a node crosses a
-// face depends on the face's edge functions at the line's two transverse coordinates, the same for every node of
-// the line; only "ahead of the node", the sign of n.(a - P), depends on the node.  So the warp collects the faces
-// the line crosses once (lanes splitting the faces, the FP32 box cull of the per-node test), then every node of
-// the line evaluates its own n.(a - P) over those faces -- the operations of testing every face from every node,
-// hence the same parity.  Passes over the three axes accumulate the parities in solid[] (pass 0 writes, pass 1
-// adds, pass 2 adds and writes the vote, >= 2 of 3, for nodes inside the surface's bounding box and 0 outside).
-// A line crossing more than HCAP faces takes the per-node test over all faces instead.
-constexpr int HCAP = 48;
-
-__global__ void __launch_bounds__(B3) k3_classify_lines(Lattice L, Mesh m, int axis, uint8_t *__restrict__ solid) {
-  __shared__ double hn[B3 / 32][HCAP][3], ha[B3 / 32][HCAP][3];  // per warp: normal and first vertex of each hit
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int u = axis == 0 ? 1 : (axis == 1 ? 2 : 0), v = axis == 0 ? 2 : (axis == 1 ? 0 : 1);
-  const int n[3] = {L.nx, L.ny, L.nz};
-  const long long nlines = (long long)n[u] * n[v];
-  const long long warps = (long long)gridDim.x * (B3 / 32);
-  for (long long li = (long long)blockIdx.x * (B3 / 32) + warp; li < nlines; li += warps) {
-    int ijk[3];
-    ijk[u] = (int)(li % n[u]);
-    ijk[v] = (int)(li / n[u]);
-    double P[3];
-    P[u] = L.lo[u] + ((double)ijk[u] + 0.5) * L.d[u];
-    P[v] = L.lo[v] + ((double)ijk[v] + 0.5) * L.d[v];
-    P[axis] = L.lo[axis];
-    const bool line_in = !(P[u] < m.bb[u] || P[u] > m.bb[3 + u] || P[v] < m.bb[v] || P[v] > m.bb[3 + v]);
-    int cnt = 0;
-    if (line_in) {
-      const float pu = (float)P[u], pv = (float)P[v];
-      for (int f0 = 0; f0 < m.ntri; f0 += 32) {
-        const int f = f0 + lane;
-        bool hit = false;
-        double nf[3] = {0.0, 0.0, 0.0}, af[3] = {0.0, 0.0, 0.0};
-        if (f < m.ntri) {
-          const float4 lo = __ldg(m.fbox + 2 * f), hi = __ldg(m.fbox + 2 * f + 1);
-          const float lu = u == 0 ? lo.x : (u == 1 ? lo.y : lo.z), hu = u == 0 ? hi.x : (u == 1 ? hi.y : hi.z);
-          const float lv = v == 0 ? lo.x : (v == 1 ? lo.y : lo.z), hv = v == 0 ? hi.x : (v == 1 ? hi.y : hi.z);
-          if (!(pu < lu || pu > hu || pv < lv || pv > hv)) {
-            const int i0 = __ldg(m.tri + 3 * f), i1 = __ldg(m.tri + 3 * f + 1), i2 = __ldg(m.tri + 3 * f + 2);
-            double A[3], B[3], C[3];
-            for (int q = 0; q < 3; q++) {
-              A[q] = __ldg(m.v + 3 * i0 + q);
-              B[q] = __ldg(m.v + 3 * i1 + q);
-              C[q] = __ldg(m.v + 3 * i2 + q);
-            }
-            const int s0 = edge_sign(A, i0, B, i1, P, u, v);
-            const int s1 = edge_sign(B, i1, C, i2, P, u, v);
-            const int s2 = edge_sign(C, i2, A, i0, P, u, v);
-            if (s0 != 0 && s0 == s1 && s1 == s2) {
-              const double e1[3] = {B[0] - A[0], B[1] - A[1], B[2] - A[2]};
-              const double e2[3] = {C[0] - A[0], C[1] - A[1], C[2] - A[2]};
-              nf[0] = e1[1] * e2[2] - e1[2] * e2[1];
-              nf[1] = e1[2] * e2[0] - e1[0] * e2[2];
-              nf[2] = e1[0] * e2[1] - e1[1] * e2[0];
-              hit = nf[axis] != 0.0;
-              for (int q = 0; q < 3; q++) af[q] = A[q];
-            }
-          }
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, hit);
-        if (hit) {
-          const int slot = cnt + __popc(bal & ((1u << lane) - 1u));
-          if (slot < HCAP)
-            for (int q = 0; q < 3; q++) {
-              hn[warp][slot][q] = nf[q];
-              ha[warp][slot][q] = af[q];
-            }
-        }
-        cnt += __popc(bal);
-      }
+// Moller-Trumbore crossings: a block prepares 32 (face, axis) items, one per lane of its first warp, and its threads
+// then take the items' lines one each (an FP64 warp instruction costs the same however few lanes are active, so both
+// parts keep the lanes full; a warp per item spent 40 us on the items' set-up alone at 1200 faces).  gridDim.y blocks
+// share the same items' lines.  A crossing toggles its bit in the axis' plane (XOR: independent of the order).
+constexpr int XT = 128;
+__global__ void __launch_bounds__(XT) k3_cross(Lattice L, Mesh m, SubBox B, int pw, unsigned *__restrict__ planes,
+                                               long long plane_words) {
+  __shared__ CrossItem item[32];
+  __shared__ long long end[32];  // inclusive prefix sums of the items' lines
+  if (threadIdx.x < 32) {
+    const long long i = (long long)blockIdx.x * 32 + threadIdx.x;
+    long long lines = 0;
+    if (i < 3LL * m.ntri) {
+      const int axis = (int)(i / m.ntri), f = (int)(i - (long long)axis * m.ntri);
+      lines = axis == 0   ? cross_item<0>(L, m, B, f, item[threadIdx.x])
+              : axis == 1 ? cross_item<1>(L, m, B, f, item[threadIdx.x])
+                          : cross_item<2>(L, m, B, f, item[threadIdx.x]);
     }
-    __syncwarp();
-    if (cnt <= HCAP) {
-      for (int t = lane; t < n[axis]; t += 32) {
-        ijk[axis] = t;
-        double Q[3] = {P[0], P[1], P[2]};
-        Q[axis] = L.lo[axis] + ((double)t + 0.5) * L.d[axis];
-        int par = 0;
-        for (int h = 0; h < cnt; h++) {
-          const double num = hn[warp][h][0] * (ha[warp][h][0] - Q[0]) + hn[warp][h][1] * (ha[warp][h][1] - Q[1]) +
-                             hn[warp][h][2] * (ha[warp][h][2] - Q[2]);
-          const double na = hn[warp][h][axis];
-          par += ((num > 0.0 && na > 0.0) || (num < 0.0 && na < 0.0)) ? 1 : 0;
-        }
-        const long long idx = ((long long)ijk[2] * L.ny + ijk[1]) * L.nx + ijk[0];
-        const bool inside = !(Q[0] < m.bb[0] || Q[0] > m.bb[3] || Q[1] < m.bb[1] || Q[1] > m.bb[4] ||
-                              Q[2] < m.bb[2] || Q[2] > m.bb[5]);
-        const uint8_t p1 = (uint8_t)(par & 1);
-        if (axis == 0) solid[idx] = p1;
-        else if (axis == 1) solid[idx] = (uint8_t)(solid[idx] + p1);
-        else solid[idx] = (uint8_t)(inside && solid[idx] + p1 >= 2);
-      }
-    } else {
-      // more crossings than the warp keeps: every node of the line tests every face (lanes splitting them)
-      const float pu = (float)P[u], pv = (float)P[v];
-      for (int t = 0; t < n[axis]; t++) {
-        ijk[axis] = t;
-        double Q[3] = {P[0], P[1], P[2]};
-        Q[axis] = L.lo[axis] + ((double)t + 0.5) * L.d[axis];
-        const float pa = (float)Q[axis];
-        unsigned h = 0;
-        for (int f = lane; f < m.ntri; f += 32) {
-          const float4 lo = __ldg(m.fbox + 2 * f), hi = __ldg(m.fbox + 2 * f + 1);
-          const float lu = u == 0 ? lo.x : (u == 1 ? lo.y : lo.z), hu = u == 0 ? hi.x : (u == 1 ? hi.y : hi.z);
-          const float lv = v == 0 ? lo.x : (v == 1 ? lo.y : lo.z), hv = v == 0 ? hi.x : (v == 1 ? hi.y : hi.z);
-          const float ha_ = axis == 0 ? hi.x : (axis == 1 ? hi.y : hi.z);
-          if (pu < lu || pu > hu || pv < lv || pv > hv || pa > ha_) continue;
-          h += (unsigned)crosses(m, f, Q, axis);
-        }
-        const int par = (int)(__reduce_add_sync(0xffffffffu, h) & 1u);
-        if (lane == 0) {
-          const long long idx = ((long long)ijk[2] * L.ny + ijk[1]) * L.nx + ijk[0];
-          const bool inside = !(Q[0] < m.bb[0] || Q[0] > m.bb[3] || Q[1] < m.bb[1] || Q[1] > m.bb[4] ||
-                                Q[2] < m.bb[2] || Q[2] > m.bb[5]);
-          if (axis == 0) solid[idx] = (uint8_t)par;
-          else if (axis == 1) solid[idx] = (uint8_t)(solid[idx] + par);
-          else solid[idx] = (uint8_t)(inside && solid[idx] + par >= 2);
-        }
-      }
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long x = __shfl_up_sync(0xffffffffu, lines, o);
+      if ((int)threadIdx.x >= o) lines += x;
     }
-    __syncwarp();  // the hit list is rewritten by the warp's next line
+    end[threadIdx.x] = lines;
+  }
+  __syncthreads();
+  const long long total = end[31];
+  for (long long p = threadIdx.x + (long long)XT * blockIdx.y; p < total; p += (long long)XT * gridDim.y) {
+    int it = 0;
+    for (int s = 16; s > 0; s >>= 1)
+      if (end[it + s - 1] <= p) it += s;  // the first item whose prefix sum exceeds p
+    const CrossItem &c = item[it];
+    const long long l = p - (it ? end[it - 1] : 0);
+    const int dv = (int)(l / c.nu), iu = c.u0 + (int)(l - (long long)dv * c.nu), iv = c.v0 + dv, axis = c.axis;
+    const int u = axis == 2 ? 0 : axis + 1, v = axis == 0 ? 2 : axis - 1;
+    const double Pu = L.lo[u] + ((double)iu + 0.5) * L.d[u], Pv = L.lo[v] + ((double)iv + 0.5) * L.d[v];
+    const int s0 = edge_sign(c.e[0], Pu, Pv);
+    if (s0 == 0 || s0 != edge_sign(c.e[1], Pu, Pv) || s0 != edge_sign(c.e[2], Pu, Pv)) continue;
+    // the line's first t* nodes have the crossing ahead: n.(a - P) of the sign of n_axis
+    const double tu = c.n[0] * (c.a[0] - Pu), tv = c.n[1] * (c.a[1] - Pv), na = c.n[2], aa = c.a[2];
+    const double La = L.lo[axis], Da = L.d[axis];
+    const int first = B.b0[axis];
+    auto ahead = [&](int t) {
+      const double Q = La + ((double)(first + t) + 0.5) * Da;
+      const double ta = na * (aa - Q);
+      // the sum in coordinate order: x + y + z
+      const double num = axis == 0 ? (ta + tu) + tv : axis == 1 ? (tv + ta) + tu : (tu + tv) + ta;
+      return (num > 0.0 && na > 0.0) || (num < 0.0 && na < 0.0);
+    };
+    // bisection, begun around the crossing's position from one division
+    int lo = 0, hi = B.n[axis];
+    const double g = floor((aa + (tu + tv) / na - La) / Da - 0.5) - (double)first;
+    const int gi = (int)fmin(fmax(g, 0.0), (double)hi);
+    if (gi > 0 && gi - 1 < hi) {
+      if (ahead(gi - 1)) lo = gi;
+      else hi = gi - 1;
+    }
+    if (lo == gi && gi + 1 < hi && !ahead(gi + 1)) hi = gi + 1;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (ahead(mid)) lo = mid + 1;
+      else hi = mid;
+    }
+    if (lo == 0) continue;
+    const int at = first + lo - 1;
+    const int x = axis == 0 ? at : axis == 1 ? iv : iu, y = axis == 0 ? iu : axis == 1 ? at : iv,
+              z = axis == 0 ? iv : axis == 1 ? iu : at;
+    atomicXor(planes + axis * plane_words + ((long long)z * L.ny + y) * pw + (x >> 5), 1u << (x & 31));
   }
 }
 
-__device__ __forceinline__ bool solid_at(const Lattice &L, const uint8_t *__restrict__ solid, int i, int j, int k) {
-  return solid[((long long)k * L.ny + j) * L.nx + i] != 0;
+// suffix XOR of n words w[0], w[stride], ...: SEG threads of a column (threadIdx.y) take a segment each, the segments
+// behind a thread's own enter through shared memory; op(t, parity) receives every word's parity, from the last on
+constexpr int SEG = 8;
+template <class Op>
+__device__ __forceinline__ void suffix_xor(const unsigned *w, long long stride, int n, bool live,
+                                           unsigned (*part)[32], Op op) {
+  const int per = (n + SEG - 1) / SEG, t0 = min(n, (int)threadIdx.y * per), t1 = min(n, t0 + per);
+  unsigned x = 0;
+  if (live) {
+#pragma unroll 4
+    for (int t = t0; t < t1; t++) x ^= w[t * stride];
+  }
+  part[threadIdx.y][threadIdx.x] = x;
+  __syncthreads();
+  if (!live) return;
+  unsigned acc = 0;
+  for (int s = threadIdx.y + 1; s < SEG; s++) acc ^= part[s][threadIdx.x];
+#pragma unroll 4
+  for (int t = t1 - 1; t >= t0; t--) {
+    acc ^= w[t * stride];
+    op(t, acc);
+  }
 }
 
-// Sec. 3.2 / Sec. 5 over the 6-neighbourhood: IB = fluid node with a solid neighbour; G1..G3 = solid node whose
-// nearest non-solid node along a lattice line is 1..3 nodes away.  Per block: counts of IB, G1, G2, G3.
-__global__ void __launch_bounds__(CBLK) k3_tags(Lattice L, const uint8_t *__restrict__ solid, uint8_t *__restrict__ tags,
-                                                int *__restrict__ blockcounts) {
-  __shared__ int wc[CBLK / 32][4];
-  const long long nn = (long long)L.nx * L.ny * L.nz;
-  const long long n = (long long)blockIdx.x * CBLK + threadIdx.x;
-  int kind = -1;
-  if (n < nn) {
-    double P[3];
-    int c[3];
-    node_xyz(L, n, P, c);
-    const int dirs[6][3] = {{1, 0, 0}, {-1, 0, 0}, {0, 1, 0}, {0, -1, 0}, {0, 0, 1}, {0, 0, -1}};
-    uint8_t t;
-    if (!solid[n]) {
-      bool ib = false;
-      for (int d = 0; d < 6 && !ib; d++) {
-        const int a = c[0] + dirs[d][0], b = c[1] + dirs[d][1], e = c[2] + dirs[d][2];
-        if (a >= 0 && a < L.nx && b >= 0 && b < L.ny && e >= 0 && e < L.nz && solid_at(L, solid, a, b, e)) ib = true;
-      }
-      t = ib ? T_IB : T_FLUID;
-    } else {
-      t = T_SOLID;
-      for (int s = 1; s <= 3 && t == T_SOLID; s++) {
-        bool hit = false;
-        for (int d = 0; d < 6 && !hit; d++) {
-          const int a = c[0] + s * dirs[d][0], b = c[1] + s * dirs[d][1], e = c[2] + s * dirs[d][2];
-          if (a >= 0 && a < L.nx && b >= 0 && b < L.ny && e >= 0 && e < L.nz && !solid_at(L, solid, a, b, e))
-            hit = true;
-        }
-        if (hit) t = (uint8_t)(T_G1 + s - 1);
-      }
-    }
-    tags[n] = t;
-    kind = t == T_IB ? 0 : (t >= T_G1 ? 1 + t - T_G1 : -1);
+// parities of the x and y rays in place: blocks [0, nyb) the y columns (a word column per threadIdx.x), the rest one
+// thread per x row
+__global__ void __launch_bounds__(32 * SEG) k3_parity_xy(Lattice L, SubBox B, int pw, unsigned *__restrict__ xb,
+                                                         unsigned *__restrict__ yb, int nyb) {
+  __shared__ unsigned part[SEG][32];
+  const int w0 = B.b0[0] >> 5, nw = ((B.b0[0] + B.n[0] - 1) >> 5) - w0 + 1;
+  if ((int)blockIdx.x < nyb) {
+    const int col = blockIdx.x * 32 + threadIdx.x, k = col / nw;
+    const bool live = k < B.n[2];
+    unsigned *p = yb + ((long long)(B.b0[2] + (live ? k : 0)) * L.ny + B.b0[1]) * pw + w0 + (col - k * nw);
+    suffix_xor(p, pw, B.n[1], live, part, [&](int t, unsigned par) { p[(long long)t * pw] = par; });
+    return;
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned r = (blockIdx.x - nyb) * (32u * SEG) + threadIdx.y * 32 + threadIdx.x, k = r / (unsigned)B.n[1];
+  if (k >= (unsigned)B.n[2]) return;
+  unsigned *p = xb + ((long long)(B.b0[2] + (int)k) * L.ny + B.b0[1] + (int)(r - k * (unsigned)B.n[1])) * pw + w0;
+  unsigned carry = 0;
+  for (int w = nw - 1; w >= 0; w--) {
+    unsigned y = p[w];
+    for (int s = 1; s < 32; s <<= 1) y ^= y >> s;  // bit i: XOR of the bits at and above i
+    y ^= carry;
+    p[w] = y;
+    carry = y & 1u ? 0xffffffffu : 0u;
+  }
+}
+
+// parity of the z rays and the vote: at least two of the three, inside the bounding box
+__global__ void __launch_bounds__(32 * SEG) k3_vote(Lattice L, SubBox B, int pw, const unsigned *__restrict__ xb,
+                                                    const unsigned *__restrict__ yb, const unsigned *__restrict__ zb,
+                                                    unsigned *__restrict__ sb) {
+  __shared__ unsigned part[SEG][32];
+  const int w0 = B.b0[0] >> 5, x1 = B.b0[0] + B.n[0] - 1, nw = (x1 >> 5) - w0 + 1;
+  const int col = blockIdx.x * 32 + threadIdx.x, j = col / nw, w = w0 + col - j * nw;
+  const bool live = j < B.n[1];
+  const unsigned lom = (w << 5) < B.b0[0] ? 0xffffffffu << (B.b0[0] & 31) : 0xffffffffu;
+  const unsigned him = (w << 5) + 31 > x1 ? 0xffffffffu >> (31 - (x1 & 31)) : 0xffffffffu;
+  const long long o = ((long long)B.b0[2] * L.ny + B.b0[1] + (live ? j : 0)) * pw + w, st = (long long)L.ny * pw;
+  suffix_xor(zb + o, st, B.n[2], live, part, [&](int t, unsigned z) {
+    const unsigned x = xb[o + t * st], y = yb[o + t * st];
+    sb[o + t * st] = ((x & y) | (z & (x | y))) & lom & him;
+  });
+}
+
+// Sec. 3.2 / Sec. 5 over the 6-neighbourhood, the 32 nodes of a word at a time: m[0] = IB (fluid node with a solid
+// neighbour), m[1..3] = G1..G3 (solid node whose nearest non-solid node along a lattice line is 1..3 nodes away);
+// returns the word's solid bits.  Nodes off the lattice are neither solid nor fluid.
+__device__ __forceinline__ unsigned node_masks(const Lattice &L, int pw, const unsigned *__restrict__ sb,
+                                               long long wi, unsigned m[4], int &w, int &row) {
+  row = (int)(wi / pw);
+  w = (int)(wi - (long long)row * pw);
+  const int k = row / L.ny, j = row - k * L.ny;
+  const unsigned tail = L.nx & 31 ? 0xffffffffu >> (32 - (L.nx & 31)) : 0xffffffffu;
+  const unsigned vm = w == pw - 1 ? tail : 0xffffffffu;
+  const unsigned S = sb[wi], F = ~S & vm;
+  const unsigned Sl = w > 0 ? sb[wi - 1] : 0u, Sr = w < pw - 1 ? sb[wi + 1] : 0u;
+  const unsigned Fl = w > 0 ? ~Sl : 0u, Fr = w < pw - 1 ? ~Sr & (w + 1 == pw - 1 ? tail : 0xffffffffu) : 0u;
+  unsigned near_s = (S << 1 | Sl >> 31) | (S >> 1 | Sr << 31), near_f[3];
+  for (int s = 1; s <= 3; s++) near_f[s - 1] = (F << s | Fl >> (32 - s)) | (F >> s | Fr << (32 - s));
+  const long long py = pw, pz = (long long)L.ny * pw;
+#pragma unroll
+  for (int s = 1; s <= 3; s++) {
+    const unsigned a = j >= s ? sb[wi - s * py] : vm, b = j + s < L.ny ? sb[wi + s * py] : vm;
+    const unsigned c = k >= s ? sb[wi - s * pz] : vm, d = k + s < L.nz ? sb[wi + s * pz] : vm;
+    near_f[s - 1] |= (~a | ~b | ~c | ~d) & vm;
+    if (s == 1)
+      near_s |= (j >= 1 ? a : 0u) | (j + 1 < L.ny ? b : 0u) | (k >= 1 ? c : 0u) | (k + 1 < L.nz ? d : 0u);
+  }
+  m[0] = F & near_s;
+  m[1] = S & near_f[0];
+  m[2] = S & near_f[1] & ~m[1];
+  m[3] = S & near_f[2] & ~(m[1] | m[2]);
+  return S;
+}
+
+// tags (zero = fluid on entry: only words with solid or IB nodes are written, a byte per lane) and per block the
+// counts of IB, G1, G2, G3; one word per thread
+__global__ void __launch_bounds__(B3) k3_tags(Lattice L, int pw, long long nwords, const unsigned *__restrict__ sb,
+                                              uint8_t *__restrict__ tags, int *__restrict__ blockcounts) {
+  __shared__ int wc[B3 / 32][4];
+  const long long wi = (long long)blockIdx.x * B3 + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  unsigned m[4] = {0u, 0u, 0u, 0u}, S = 0u;
+  int w = 0, row = 0;
+  if (wi < nwords) S = node_masks(L, pw, sb, wi, m, w, row);
+  for (unsigned todo = __ballot_sync(0xffffffffu, (S | m[0]) != 0u); todo; todo &= todo - 1) {
+    const int src = __ffs(todo) - 1;
+    const unsigned s = __shfl_sync(0xffffffffu, S, src);
+    unsigned q[4];
+    for (int t = 0; t < 4; t++) q[t] = __shfl_sync(0xffffffffu, m[t], src);
+    const int x = (__shfl_sync(0xffffffffu, w, src) << 5) + lane, r = __shfl_sync(0xffffffffu, row, src);
+    if (x < L.nx) {
+      const unsigned b = 1u << lane;
+      const uint8_t t = q[0] & b ? T_IB : q[1] & b ? T_G1 : q[2] & b ? T_G1 + 1 : q[3] & b ? T_G1 + 2
+                        : s & b ? T_SOLID : T_FLUID;
+      tags[(long long)r * L.nx + x] = t;
+    }
+  }
   for (int q = 0; q < 4; q++) {
-    const unsigned b = __ballot_sync(0xffffffffu, kind == q);
-    if (lane == 0) wc[warp][q] = __popc(b);
+    const int c = (int)__reduce_add_sync(0xffffffffu, (unsigned)__popc(m[q]));
+    if (lane == 0) wc[threadIdx.x >> 5][q] = c;
   }
   __syncthreads();
   if (threadIdx.x < 4) {
     int s = 0;
-    for (int w = 0; w < CBLK / 32; w++) s += wc[w][threadIdx.x];
+    for (int t = 0; t < B3 / 32; t++) s += wc[t][threadIdx.x];
     blockcounts[4 * blockIdx.x + threadIdx.x] = s;
   }
 }
 
-// exclusive offsets of every block within each class's list, and the class totals (counts[0..3]); one block
-__global__ void __launch_bounds__(1024) k3_scan(int nblk, int *__restrict__ blockcounts, int *__restrict__ counts) {
-  __shared__ int part[1024][4];
-  const int per = (nblk + 1023) / 1024, b0 = threadIdx.x * per, b1 = min(nblk, b0 + per);
-  int s[4] = {0, 0, 0, 0};
-  for (int b = b0; b < b1; b++)
-    for (int q = 0; q < 4; q++) s[q] += blockcounts[4 * b + q];
-  for (int q = 0; q < 4; q++) part[threadIdx.x][q] = s[q];
+// exclusive scan over the block's threads of one value per thread (sh: one int per warp); total receives the sum
+__device__ __forceinline__ int block_scan(int x, int *sh, int &total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int inc = x;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) sh[warp] = inc;
   __syncthreads();
-  if (threadIdx.x < 4) {  // serial exclusive scan of the 1024 partial sums of one class
-    int acc = 0;
-    for (int t = 0; t < 1024; t++) {
-      const int x = part[t][threadIdx.x];
-      part[t][threadIdx.x] = acc;
-      acc += x;
-    }
-    counts[threadIdx.x] = acc;
+  int before = 0;
+  total = 0;
+  for (int t = 0; t < nw; t++) {
+    if (t < warp) before += sh[t];
+    total += sh[t];
   }
   __syncthreads();
-  int off[4];
-  for (int q = 0; q < 4; q++) off[q] = part[threadIdx.x][q];
-  for (int b = b0; b < b1; b++)
-    for (int q = 0; q < 4; q++) {
-      const int x = blockcounts[4 * b + q];
-      blockcounts[4 * b + q] = off[q];
-      off[q] += x;
-    }
+  return before + inc - x;
 }
 
-// listed nodes in row-major order, IB first, then G1, G2, G3; entries past cap are not written
-__global__ void __launch_bounds__(CBLK) k3_scatter(Lattice L, const uint8_t *__restrict__ tags,
-                                                   const int *__restrict__ blockoff, const int *__restrict__ counts,
-                                                   int *__restrict__ nodes, int cap) {
-  __shared__ int wc[CBLK / 32][4];
-  const long long nn = (long long)L.nx * L.ny * L.nz;
-  const long long n = (long long)blockIdx.x * CBLK + threadIdx.x;
-  int kind = -1;
-  if (n < nn) {
-    const uint8_t t = tags[n];
-    kind = t == T_IB ? 0 : (t >= T_G1 ? 1 + t - T_G1 : -1);
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int rank = 0;
+// exclusive offsets of every block within each class's list, and the class totals (counts[0..3]); one block
+__global__ void __launch_bounds__(1024) k3_scan(int nblk, int *__restrict__ blockcounts, int *__restrict__ counts) {
+  __shared__ int sh[32];
+  const int per = (nblk + 1023) / 1024, b0 = min(nblk, (int)threadIdx.x * per), b1 = min(nblk, b0 + per);
   for (int q = 0; q < 4; q++) {
-    const unsigned b = __ballot_sync(0xffffffffu, kind == q);
-    if (lane == 0) wc[warp][q] = __popc(b);
-    if (kind == q) rank = __popc(b & ((1u << lane) - 1u));
+    int s = 0, total;
+    for (int b = b0; b < b1; b++) s += blockcounts[4 * b + q];
+    int off = block_scan(s, sh, total);
+    for (int b = b0; b < b1; b++) {
+      const int x = blockcounts[4 * b + q];
+      blockcounts[4 * b + q] = off;
+      off += x;
+    }
+    if (threadIdx.x == 0) counts[q] = total;
   }
-  __syncthreads();
-  if (kind >= 0) {
-    int pos = blockoff[4 * blockIdx.x + kind] + rank;
-    for (int w = 0; w < warp; w++) pos += wc[w][kind];
-    for (int q = 0; q < kind; q++) pos += counts[q];
-    if (pos < cap) nodes[pos] = (int)n;
+}
+
+// listed nodes in row-major order, IB first, then G1, G2, G3; entries past cap are not written.  One word per
+// thread, its masks formed again from the solid bits
+__global__ void __launch_bounds__(B3) k3_scatter(Lattice L, int pw, long long nwords, const unsigned *__restrict__ sb,
+                                                 const int *__restrict__ blockoff, const int *__restrict__ counts,
+                                                 int *__restrict__ nodes, int cap) {
+  __shared__ int sh[B3 / 32];
+  const long long wi = (long long)blockIdx.x * B3 + threadIdx.x;
+  unsigned m[4] = {0u, 0u, 0u, 0u};
+  int w = 0, row = 0;
+  if (wi < nwords) node_masks(L, pw, sb, wi, m, w, row);
+  if (!__syncthreads_or((m[0] | m[1] | m[2] | m[3]) != 0u)) return;
+  const int n0 = row * L.nx + (w << 5);
+  int base = 0;
+  for (int q = 0; q < 4; q++) {
+    int total;
+    int pos = base + blockoff[4 * blockIdx.x + q] + block_scan(__popc(m[q]), sh, total);
+    for (unsigned b = m[q]; b; b &= b - 1, pos++)
+      if (pos < cap) nodes[pos] = n0 + __ffs(b) - 1;
+    base += counts[q];
   }
 }
 
 __device__ __forceinline__ double dot3(const double *a, const double *b) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; }
 
 // Sec. 4.1: closest point of face f to P -- the plane projection (barycentric normal equations) when it falls
-// inside the face, else the nearest point of its three edges (an end vertex when the edge parameter clamps)
-__device__ __forceinline__ double face_closest(const Mesh &m, int f, const double P[3], double q[3], int &fk,
-                                               int &fe, int &fv) {
-  const int t[3] = {__ldg(m.tri + 3 * f), __ldg(m.tri + 3 * f + 1), __ldg(m.tri + 3 * f + 2)};
+// inside the face, else the nearest point of its three edges (an end vertex when the edge parameter clamps);
+// fv receives the local vertex of a vertex feature
+__device__ __forceinline__ double face_closest(const FaceExact &F, const double P[3], double q[3], int &fk, int &fe,
+                                               int &fv) {
   double V[3][3];
   for (int k = 0; k < 3; k++)
-    for (int d = 0; d < 3; d++) V[k][d] = __ldg(m.v + 3 * t[k] + d);
+    for (int d = 0; d < 3; d++) V[k][d] = F.V[k][d];
   const double *A = V[0];
   const double e1[3] = {V[1][0] - A[0], V[1][1] - A[1], V[1][2] - A[2]};
   const double e2[3] = {V[2][0] - A[0], V[2][1] - A[1], V[2][2] - A[2]};
   const double w[3] = {P[0] - A[0], P[1] - A[1], P[2] - A[2]};
-  const double a11 = dot3(e1, e1), a12 = dot3(e1, e2), a22 = dot3(e2, e2), b1 = dot3(w, e1), b2 = dot3(w, e2);
-  const double det = a11 * a22 - a12 * a12;
+  const double a11 = F.a11, a12 = F.a12, a22 = F.a22, det = F.det, b1 = dot3(w, e1), b2 = dot3(w, e2);
   const double s = (b1 * a22 - b2 * a12) / det, r = (a11 * b2 - a12 * b1) / det;
   fk = 0;
   fe = 0;
@@ -355,18 +454,19 @@ __device__ __forceinline__ double face_closest(const Mesh &m, int f, const doubl
     for (int d = 0; d < 3; d++) q[d] = A[d] + s * e1[d] + r * e2[d];
   } else {
     double dmin = INFINITY;
+#pragma unroll
     for (int k = 0; k < 3; k++) {
       const double *E0 = V[k], *E1 = V[(k + 1) % 3];
       const double ed[3] = {E1[0] - E0[0], E1[1] - E0[1], E1[2] - E0[2]};
       const double pw[3] = {P[0] - E0[0], P[1] - E0[1], P[2] - E0[2]};
-      double u = dot3(pw, ed) / dot3(ed, ed);
+      double u = dot3(pw, ed) / F.ee[k];
       int vert = -1;
       if (u <= 0.0) {
         u = 0.0;
-        vert = t[k];
+        vert = k;
       } else if (u >= 1.0) {
         u = 1.0;
-        vert = t[(k + 1) % 3];
+        vert = (k + 1) % 3;
       }
       const double x[3] = {E0[0] + u * ed[0], E0[1] + u * ed[1], E0[2] + u * ed[2]};
       const double dd[3] = {P[0] - x[0], P[1] - x[1], P[2] - x[2]};
@@ -386,87 +486,275 @@ __device__ __forceinline__ double face_closest(const Mesh &m, int f, const doubl
   return dot3(dq, dq);
 }
 
-// Sec. 4.1-4.2: closest feature of every listed node (one warp per node, lanes splitting the faces, the
-// lowest face index among equal distances) and its pseudo-normal: the face normal, the angle-weighted vertex
-// normal (Eq. 2) or the normalised sum of the two faces' normals at an edge (Eq. 3)
-__global__ void __launch_bounds__(B3) k3_closest(Lattice L, Mesh m, const int *__restrict__ nodes,
-                                                 const int *__restrict__ counts, int cap,
+// the record of node n from the winning face's closest feature: its pseudo-normal (Sec. 4.2) is the face normal, the
+// angle-weighted vertex normal (Eq. 2) or the normalised sum of the two faces' normals at an edge (Eq. 3)
+__device__ __forceinline__ void write_record(const Mesh &m, int n, int f, int fk, int fe, int fv, const double q[3],
+                                             ibm_closest3d *__restrict__ out) {
+  double nn[3];
+  if (fk == IBM_FEATURE_FACE) {
+    for (int d = 0; d < 3; d++) nn[d] = m.fn[3 * f + d];
+  } else if (fk == IBM_FEATURE_VERTEX) {
+    const int v = m.tri[3 * f + fv];
+    for (int d = 0; d < 3; d++) nn[d] = m.vn[3 * v + d];
+  } else {
+    const int g = m.enb[3 * f + fe];
+    for (int d = 0; d < 3; d++) nn[d] = m.fn[3 * f + d] + (g >= 0 ? m.fn[3 * g + d] : 0.0);
+    const double Ln = sqrt(dot3(nn, nn));
+    if (Ln > 0.0)
+      for (int d = 0; d < 3; d++) nn[d] = nn[d] / Ln;
+  }
+  ibm_closest3d o;
+  o.node = n;
+  o.tri = f;
+  o.kind = fk;
+  o.reserved = 0;
+  for (int d = 0; d < 3; d++) {
+    o.cp[d] = q[d];
+    o.n[d] = nn[d];
+  }
+  *out = o;
+}
+
+// minimum over the warp (no NaN among the values: distances and infinities)
+__device__ __forceinline__ float warp_min(float x) {
+  for (int o = 16; o > 0; o >>= 1) x = fminf(x, __shfl_xor_sync(0xffffffffu, x, o));
+  return x;
+}
+
+// FP32 bounds of the distance from P to the lane's face of cluster c: lb below and ub above the distance that the
+// exact evaluation finds, by the margin mg (far above the FP32 rounding of coordinates and operations).  Every term
+// is well conditioned whatever the face's shape: the distances to the three edge segments, the distance to the plane,
+// and the signed in-plane distances to the edge lines, which say whether the projection falls inside, outside, or
+// within the margin of an edge (then the plane's distance bounds from below only).  Faces whose barycentric system
+// is too flat for that to describe its FP64 solution are never pruned and prune nothing.
+__device__ __forceinline__ void face_bounds(const Mesh &m, int c, int lane, const float P[3], float mg, float &lb,
+                                            float &ub, int &f) {
+  const int i = c * CL + lane, n = m.ncl * CL;
+  float r[4 * FPLANES];
+#pragma unroll
+  for (int p = 0; p < FPLANES; p++) {
+    const float4 q = __ldg(m.fp + (size_t)p * n + i);
+    r[4 * p] = q.x;
+    r[4 * p + 1] = q.y;
+    r[4 * p + 2] = q.z;
+    r[4 * p + 3] = q.w;
+  }
+  f = __float_as_int(r[21]);
+  float e2 = INFINITY, tin = INFINITY, w[3][3];
+#pragma unroll
+  for (int k = 0; k < 3; k++)
+    for (int d = 0; d < 3; d++) w[k][d] = P[d] - r[3 * k + d];
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    const int k1 = (k + 1) % 3;
+    const float ex = r[3 * k1] - r[3 * k], ey = r[3 * k1 + 1] - r[3 * k + 1], ez = r[3 * k1 + 2] - r[3 * k + 2];
+    const float we = fmaf(w[k][0], ex, fmaf(w[k][1], ey, w[k][2] * ez)), ee = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
+    const float u = fminf(fmaxf(__fdividef(we, ee), 0.0f), 1.0f);  // (an edge of length 0: NaN -> 0)
+    const float dx = fmaf(-u, ex, w[k][0]), dy = fmaf(-u, ey, w[k][1]), dz = fmaf(-u, ez, w[k][2]);
+    e2 = fminf(e2, fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+    tin = fminf(tin, fmaf(w[k][0], r[12 + 3 * k], fmaf(w[k][1], r[13 + 3 * k], w[k][2] * r[14 + 3 * k])));
+  }
+  const float de = sqrtf(e2), h = fabsf(fmaf(w[0][0], r[9], fmaf(w[0][1], r[10], w[0][2] * r[11])));
+  const float dm = fminf(h, de);
+  ub = (tin >= mg ? dm : de) + mg;
+  lb = (tin >= -mg ? dm : de) - mg;
+  if (r[22] != 0.0f) {
+    lb = -INFINITY;
+    ub = INFINITY;
+  }
+  if (f < 0) lb = ub = INFINITY;
+}
+
+// Sec. 4.1-4.2: closest feature of every listed node.  The exact evaluation (FP64, IEEE operations in a fixed order,
+// the lowest face index among equal distances) is needed only for the faces that FP32 bounds cannot exclude -- one to
+// a few per node -- and an FP64 warp instruction costs the same however few lanes are active, so the two parts are
+// split: (1) a warp per node finds the surviving faces by bounds, over clusters of 32 spatially sorted faces (one
+// face per lane), nearest cluster first; (2) the block's (node, face) pairs are evaluated one per thread, all lanes
+// busy, and each node's lexicographic (distance, face) minimum writes its record.  Sphere of 1200 faces, 256^3
+// lattice: 9.54 -> 0.29 ms, 40^3 0.41 -> 0.024 ms (issue-bound: 30% FMA, 29% ALU, FP64 18% of the cycles); one warp
+// per node evaluating every face within a bounding-sphere bound took its candidates through FP64 code in nearly empty
+// warps.  Boxes of the clusters instead of spheres halved the clusters visited (0.58 -> 0.29 ms).
+constexpr int PAIRS = B3, KEEP = 96, NODES = 12;  // pairs per batch, survivors per node, nodes per warp and batch
+
+__global__ void __launch_bounds__(B3, 3) k3_closest(Lattice L, Mesh m, const int *__restrict__ nodes,
+                                                 const int *__restrict__ counts, int cap, float mg,
                                                  ibm_closest3d *__restrict__ rec) {
+  __shared__ int s_face[B3 / 32][KEEP];
+  __shared__ float s_lb[B3 / 32][KEEP];
+  __shared__ int p_entry[PAIRS], p_face[PAIRS], p_first[PAIRS], p_count[PAIRS];
+  __shared__ double p_d2[PAIRS];
+  __shared__ int npairs;
   const int total = min(cap, counts[0] + counts[1] + counts[2] + counts[3]);
-  const int lane = threadIdx.x & 31;
-  const int warps = gridDim.x * (B3 / 32);
-  for (int e = blockIdx.x * (B3 / 32) + (threadIdx.x >> 5); e < total; e += warps) {
-    const long long n = nodes[e];
-    double P[3];
-    int ijk[3];
-    node_xyz(L, n, P, ijk);
-    // bounding spheres (FP32, widened by the cull margin): the nearest possible and the farthest possible
-    // distance of every face; a face whose nearest possible distance exceeds the smallest farthest possible
-    // distance of any face cannot hold the closest point (the margin is far above FP32 rounding, and a face
-    // within it is tested exactly)
-    const float pf[3] = {(float)P[0], (float)P[1], (float)P[2]};
-    float ub = INFINITY;
-    for (int f = lane; f < m.ntri; f += 32) {
-      const float4 s = __ldg(m.fsph + f);
-      const float dx = pf[0] - s.x, dy = pf[1] - s.y, dz = pf[2] - s.z;
-      ub = fminf(ub, sqrtf(dx * dx + dy * dy + dz * dz) + s.w);
-    }
-    for (int off = 16; off > 0; off >>= 1) ub = fminf(ub, __shfl_xor_sync(0xffffffffu, ub, off));
-    double best = INFINITY, bq[3] = {0.0, 0.0, 0.0};
-    int bf = -1, bk = 0, be = 0, bv = 0;
-    for (int f = lane; f < m.ntri; f += 32) {
-      const float4 s = __ldg(m.fsph + f);
-      const float dx = pf[0] - s.x, dy = pf[1] - s.y, dz = pf[2] - s.z;
-      if (sqrtf(dx * dx + dy * dy + dz * dz) - s.w > ub) continue;
-      double q[3];
-      int fk, fe, fv;
-      const double d2 = face_closest(m, f, P, q, fk, fe, fv);
-      if (d2 < best) {  // ascending f within the lane: the first minimum is kept
-        best = d2;
-        bf = f;
-        bk = fk;
-        be = fe;
-        bv = fv;
-        bq[0] = q[0];
-        bq[1] = q[1];
-        bq[2] = q[2];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // nodes per warp and batch: an even share of the blocks' rounds over the list
+  const int warps = (int)gridDim.x * (B3 / 32), rounds = 1 + total / (warps * NODES);
+  const int npw = 1 + total / (warps * rounds);
+  const int batch = npw * (B3 / 32);
+  const float lo[3] = {(float)L.lo[0], (float)L.lo[1], (float)L.lo[2]};
+  const float dd[3] = {(float)L.d[0], (float)L.d[1], (float)L.d[2]};
+  for (long long e0 = (long long)blockIdx.x * batch; e0 < total; e0 += (long long)gridDim.x * batch) {
+    if (threadIdx.x == 0) npairs = 0;
+    __syncthreads();
+    for (int q = 0; q < npw; q++) {
+      if (e0 + q * (B3 / 32) + warp >= total) break;
+      const int e = (int)e0 + q * (B3 / 32) + warp;
+      const int n = nodes[e];
+      int ijk[3];
+      node_ijk(L, n, ijk);
+      float P[3];
+      for (int a = 0; a < 3; a++) P[a] = fmaf((float)ijk[a] + 0.5f, dd[a], lo[a]);
+      // distances to the clusters' boxes (the first 64 kept); the cluster of the nearest centre comes first: its
+      // faces give the first upper bound
+      auto box = [&](int c, float &centre) {
+        const float4 l = __ldg(m.cl + 2 * c), h = __ldg(m.cl + 2 * c + 1);
+        const float dx = fmaxf(fmaxf(l.x - P[0], P[0] - h.x), 0.0f), dy = fmaxf(fmaxf(l.y - P[1], P[1] - h.y), 0.0f),
+                    dz = fmaxf(fmaxf(l.z - P[2], P[2] - h.z), 0.0f);
+        const float cx = 0.5f * (l.x + h.x) - P[0], cy = 0.5f * (l.y + h.y) - P[1], cz = 0.5f * (l.z + h.z) - P[2];
+        centre = fmaf(cx, cx, fmaf(cy, cy, cz * cz));
+        return sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz))) - mg;
+      };
+      float near = INFINITY, kept0 = INFINITY, kept1 = INFINITY;
+      int c0 = 0;
+      for (int c = lane; c < m.ncl; c += 32) {
+        float q;
+        const float d = box(c, q);
+        if (c < 32) kept0 = d;
+        else if (c < 64) kept1 = d;
+        if (q < near) {
+          near = q;
+          c0 = c;
+        }
       }
-    }
-    // lexicographic (distance, face) minimum over the warp
-    double md = best;
-    int mf = bf < 0 ? 0x7fffffff : bf;
-    for (int off = 16; off > 0; off >>= 1) {
-      const double od = __shfl_xor_sync(0xffffffffu, md, off);
-      const int of = __shfl_xor_sync(0xffffffffu, mf, off);
-      if (od < md || (od == md && of < mf)) {
-        md = od;
-        mf = of;
+      const float first_near = warp_min(near);
+      c0 = __shfl_sync(0xffffffffu, c0, __ffs(__ballot_sync(0xffffffffu, near == first_near)) - 1);
+      float ub = INFINITY;
+      int cnt = 0;
+      bool over = false;
+      // keep the listed faces whose lower bound is within the current upper bound
+      auto compact = [&]() {
+        int kept = 0;
+        for (int i0 = 0; i0 < cnt; i0 += 32) {
+          const int i = i0 + lane;
+          const bool ok = i < cnt && s_lb[warp][i] <= ub;
+          const int face = ok ? s_face[warp][i] : 0;
+          const float b = ok ? s_lb[warp][i] : 0.0f;
+          __syncwarp();
+          const unsigned bal = __ballot_sync(0xffffffffu, ok);
+          if (ok) {
+            const int at = kept + __popc(bal & ((1u << lane) - 1u));
+            s_face[warp][at] = face;
+            s_lb[warp][at] = b;
+          }
+          kept += __popc(bal);
+          __syncwarp();
+        }
+        cnt = kept;
+      };
+      auto visit = [&](int c) {
+        float lb, fu;
+        int f;
+        face_bounds(m, c, lane, P, mg, lb, fu, f);
+        ub = fminf(ub, warp_min(fu));
+        const bool ok = f >= 0 && lb <= ub;
+        const unsigned bal = __ballot_sync(0xffffffffu, ok);
+        const int more = __popc(bal);
+        if (cnt + more > KEEP) compact();
+        if (cnt + more > KEEP) {
+          over = true;
+          return;
+        }
+        if (ok) {
+          const int at = cnt + __popc(bal & ((1u << lane) - 1u));
+          s_face[warp][at] = f;
+          s_lb[warp][at] = lb;
+        }
+        cnt += more;
+        __syncwarp();
+      };
+      visit(c0);
+      for (int b = 0; b < m.ncl && !over; b += 32) {
+        const int c = b + lane;
+        float d = b == 0 ? kept0 : kept1, unused;
+        if (b >= 64 && c < m.ncl) d = box(c, unused);
+        for (unsigned todo = __ballot_sync(0xffffffffu, c < m.ncl && c != c0 && d <= ub); todo && !over;
+             todo &= todo - 1) {
+          const int src = __ffs(todo) - 1;
+          if (__shfl_sync(0xffffffffu, d, src) <= ub) visit(b + src);
+        }
       }
-    }
-    if (bf == mf) {  // the lane that holds the winning face writes the record
-      double nn[3];
-      if (bk == IBM_FEATURE_FACE) {
-        for (int d = 0; d < 3; d++) nn[d] = m.fn[3 * bf + d];
-      } else if (bk == IBM_FEATURE_VERTEX) {
-        for (int d = 0; d < 3; d++) nn[d] = m.vn[3 * bv + d];
-      } else {
-        const int g = m.enb[3 * bf + be];
-        for (int d = 0; d < 3; d++) nn[d] = m.fn[3 * bf + d] + (g >= 0 ? m.fn[3 * g + d] : 0.0);
-        const double Ln = sqrt(dot3(nn, nn));
-        if (Ln > 0.0)
-          for (int d = 0; d < 3; d++) nn[d] = nn[d] / Ln;
+      int first = PAIRS;
+      if (!over) {
+        compact();
+        if (lane == 0) first = atomicAdd(&npairs, cnt);
+        first = __shfl_sync(0xffffffffu, first, 0);
       }
-      ibm_closest3d o;
-      o.node = (int32_t)n;
-      o.tri = bf;
-      o.kind = bk;
-      o.reserved = 0;
-      for (int d = 0; d < 3; d++) {
-        o.cp[d] = bq[d];
-        o.n[d] = nn[d];
+      if (!over && first + cnt <= PAIRS) {
+        for (int i = lane; i < cnt; i += 32) {
+          p_entry[first + i] = e;
+          p_face[first + i] = s_face[warp][i];
+          p_first[first + i] = first;
+          p_count[first + i] = cnt;
+        }
+        __syncwarp();
+        continue;
       }
-      rec[e] = o;
+      // more survivors than the batch has room for: the warp evaluates them itself (all faces if they were not kept)
+      if (!over && lane == 0)
+        for (int i = first; i < PAIRS; i++) p_entry[i] = -1;  // the part of the claim inside the list stays empty
+      double X[3];
+      node_xyz(L, n, X, ijk);
+      double best = INFINITY, bq[3] = {0.0, 0.0, 0.0};
+      int bf = 0x7fffffff, bk = 0, be = 0, bv = 0;
+      const int nc = over ? m.ntri : cnt;
+      for (int i = lane; i < nc; i += 32) {
+        const int f = over ? i : s_face[warp][i];
+        double y[3];
+        int fk, fe, fv;
+        const double d2 = face_closest(m.fx[f], X, y, fk, fe, fv);
+        if (d2 < best || (d2 == best && f < bf)) {
+          best = d2;
+          bf = f;
+          bk = fk;
+          be = fe;
+          bv = fv;
+          for (int d = 0; d < 3; d++) bq[d] = y[d];
+        }
+      }
+      double md = best;
+      int mf = bf;
+      for (int o = 16; o > 0; o >>= 1) {
+        const double od = __shfl_xor_sync(0xffffffffu, md, o);
+        const int of = __shfl_xor_sync(0xffffffffu, mf, o);
+        if (od < md || (od == md && of < mf)) {
+          md = od;
+          mf = of;
+        }
+      }
+      if (bf == mf && bf != 0x7fffffff) write_record(m, n, bf, bk, be, bv, bq, rec + e);
+      __syncwarp();
     }
+    __syncthreads();
+    const int t = threadIdx.x, np = min(npairs, PAIRS);
+    const bool live = t < np && p_entry[t] >= 0;
+    double y[3];
+    int fk = 0, fe = 0, fv = 0, n = 0;
+    if (live) {
+      n = nodes[p_entry[t]];
+      double X[3];
+      int ijk[3];
+      node_xyz(L, n, X, ijk);
+      p_d2[t] = face_closest(m.fx[p_face[t]], X, y, fk, fe, fv);
+    }
+    __syncthreads();
+    if (live) {
+      const double d2 = p_d2[t];
+      const int f = p_face[t];
+      bool win = d2 < INFINITY;
+      for (int i = p_first[t]; i < p_first[t] + p_count[t]; i++)
+        if (p_d2[i] < d2 || (p_d2[i] == d2 && p_face[i] < f)) win = false;
+      if (win) write_record(m, n, f, fk, fe, fv, y, rec + p_entry[t]);
+    }
+    __syncthreads();
   }
 }
 
@@ -663,8 +951,11 @@ struct ibm_body3d {
   bool own_stream = false;
   Lattice L{};
   long long nn = 0;          // lattice nodes of the last classification
+  int pw = 0;                // words per lattice row of the bit planes
+  long long nwords = 0;      // words per bit plane
   int nblk = 0, cap = 0;
-  uint8_t *solid = nullptr, *tags = nullptr;
+  unsigned *bits = nullptr;  // four bit planes: crossings (then parities) of the x, y and z rays, solid nodes
+  uint8_t *tags = nullptr;
   int *blockcounts = nullptr, *counts = nullptr, *nodes = nullptr;
   ibm_closest3d *rec = nullptr;
   bool classified = false;
@@ -673,13 +964,14 @@ struct ibm_body3d {
 static ibm_status cuda_fail(cudaError_t e) { return ibm__noalloc_fail(IBM_ECUDA, cudaGetErrorString(e)); }
 
 static void free_lattice(ibm_body3d *b) {
-  cudaFree(b->solid);
+  cudaFree(b->bits);
   cudaFree(b->tags);
   cudaFree(b->blockcounts);
   cudaFree(b->counts);
   cudaFree(b->nodes);
   cudaFree(b->rec);
-  b->solid = b->tags = nullptr;
+  b->bits = nullptr;
+  b->tags = nullptr;
   b->blockcounts = b->counts = b->nodes = nullptr;
   b->rec = nullptr;
   b->nn = 0;
@@ -703,53 +995,99 @@ extern "C" ibm_status ibm_body3d_create(const double *verts, int nverts, const i
       auto it = first.find(std::make_pair(tris[3 * f + (k + 1) % 3], tris[3 * f + k]));
       if (it != first.end()) enb[(size_t)3 * f + k] = it->second;
     }
-  // per-face boxes and bounding spheres for the FP32 culls, widened by a margin of 1e-5 of the mesh extent
-  double ext = 0.0;
-  {
-    double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    for (int k = 0; k < nverts; k++)
-      for (int a = 0; a < 3; a++) {
-        lo[a] = std::min(lo[a], verts[3 * k + a]);
-        hi[a] = std::max(hi[a], verts[3 * k + a]);
-      }
-    for (int a = 0; a < 3; a++) ext = std::max(ext, std::max(std::fabs(lo[a]), std::fabs(hi[a])));
-    ext = std::max(ext, 1.0);
-  }
+  // closest-feature search: exact per-face data, and FP32 faces in clusters of 32 along a Morton curve through the
+  // centroids, so that a cluster is compact; bounding boxes widened by 1e-5 of the mesh's extent
+  double ext = 0.0, blo[3] = {INFINITY, INFINITY, INFINITY}, bhi[3] = {-INFINITY, -INFINITY, -INFINITY};
+  for (int k = 0; k < nverts; k++)
+    for (int a = 0; a < 3; a++) {
+      blo[a] = std::min(blo[a], verts[3 * k + a]);
+      bhi[a] = std::max(bhi[a], verts[3 * k + a]);
+    }
+  for (int a = 0; a < 3; a++) ext = std::max(ext, std::max(std::fabs(blo[a]), std::fabs(bhi[a])));
+  ext = std::max(ext, 1.0);
   const double margin = 1e-5 * ext;
-  std::vector<float4> fbox((size_t)2 * ntris), fsph((size_t)ntris);
+  std::vector<FaceExact> fx((size_t)ntris);
+  std::vector<std::pair<uint32_t, int>> order((size_t)ntris);
   for (int f = 0; f < ntris; f++) {
     const double *V[3] = {verts + 3 * tris[3 * f], verts + 3 * tris[3 * f + 1], verts + 3 * tris[3 * f + 2]};
-    double lo[3], hi[3], cen[3], r2 = 0.0;
+    FaceExact &x = fx[f];
+    auto dot = [](const double *a, const double *b) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; };
+    double ed[3][3], e2[3];
+    for (int k = 0; k < 3; k++)
+      for (int d = 0; d < 3; d++) {
+        x.V[k][d] = V[k][d];
+        ed[k][d] = V[(k + 1) % 3][d] - V[k][d];
+      }
+    for (int d = 0; d < 3; d++) e2[d] = V[2][d] - V[0][d];
+    x.a11 = dot(ed[0], ed[0]);
+    x.a12 = dot(ed[0], e2);
+    x.a22 = dot(e2, e2);
+    x.det = x.a11 * x.a22 - x.a12 * x.a12;
+    for (int k = 0; k < 3; k++) x.ee[k] = dot(ed[k], ed[k]);
+    uint32_t key = 0;
     for (int a = 0; a < 3; a++) {
-      lo[a] = std::min(V[0][a], std::min(V[1][a], V[2][a])) - margin;
-      hi[a] = std::max(V[0][a], std::max(V[1][a], V[2][a])) + margin;
-      cen[a] = (V[0][a] + V[1][a] + V[2][a]) / 3.0;
+      const double c = (V[0][a] + V[1][a] + V[2][a]) / 3.0, w = bhi[a] - blo[a];
+      const double t = w > 0.0 ? (c - blo[a]) / w : 0.0;
+      const uint32_t g = t > 0.0 ? (uint32_t)std::min(1023.0, t * 1024.0) : 0u;
+      for (int bit = 0; bit < 10; bit++) key |= (g >> bit & 1u) << (3 * bit + a);
     }
-    for (int k = 0; k < 3; k++) {
-      const double dx = V[k][0] - cen[0], dy = V[k][1] - cen[1], dz = V[k][2] - cen[2];
-      r2 = std::max(r2, dx * dx + dy * dy + dz * dz);
+    order[f] = std::make_pair(key, f);
+  }
+  std::sort(order.begin(), order.end());
+  const int ncl = (ntris + CL - 1) / CL;
+  std::vector<float4> cl((size_t)2 * ncl), fp((size_t)FPLANES * ncl * CL);
+  for (int c = 0; c < ncl; c++) {
+    double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    const int i0 = c * CL, i1 = std::min(ntris, i0 + CL);
+    for (int i = i0; i < i1; i++)
+      for (int k = 0; k < 3; k++)
+        for (int a = 0; a < 3; a++) {
+          lo[a] = std::min(lo[a], fx[order[i].second].V[k][a]);
+          hi[a] = std::max(hi[a], fx[order[i].second].V[k][a]);
+        }
+    for (int i = i0; i < i0 + CL; i++) {
+      float r[4 * FPLANES] = {};
+      int f = -1;
+      if (i < i1) {
+        f = order[i].second;
+        const FaceExact &x = fx[f];
+        const double *n = &fn[(size_t)3 * f];
+        for (int k = 0; k < 3; k++) {
+          const int k1 = (k + 1) % 3;
+          const double e[3] = {x.V[k1][0] - x.V[k][0], x.V[k1][1] - x.V[k][1], x.V[k1][2] - x.V[k][2]};
+          const double len = std::sqrt(x.ee[k]), il = len > 0.0 ? 1.0 / len : 0.0;
+          const double in[3] = {n[1] * e[2] - n[2] * e[1], n[2] * e[0] - n[0] * e[2], n[0] * e[1] - n[1] * e[0]};
+          for (int a = 0; a < 3; a++) {
+            r[3 * k + a] = (float)x.V[k][a];
+            r[12 + 3 * k + a] = (float)(in[a] * il);
+          }
+        }
+        for (int a = 0; a < 3; a++) r[9 + a] = (float)n[a];
+        // sin^2 of the angle at the first vertex below 1e-8: the FP64 barycentric solution may be off by more than
+        // the margin
+        r[22] = !(x.det >= 1e-8 * (x.a11 * x.a22)) ? 1.0f : 0.0f;
+      }
+      std::memcpy(&r[21], &f, sizeof f);
+      for (int p = 0; p < FPLANES; p++)
+        fp[(size_t)p * ncl * CL + i] = make_float4(r[4 * p], r[4 * p + 1], r[4 * p + 2], r[4 * p + 3]);
     }
-    fbox[(size_t)2 * f] = make_float4((float)lo[0], (float)lo[1], (float)lo[2], 0.f);
-    fbox[(size_t)2 * f + 1] = make_float4((float)hi[0], (float)hi[1], (float)hi[2], 0.f);
-    fsph[f] = make_float4((float)cen[0], (float)cen[1], (float)cen[2], (float)(std::sqrt(r2) + margin));
+    cl[2 * c] = make_float4((float)(lo[0] - margin), (float)(lo[1] - margin), (float)(lo[2] - margin), 0.f);
+    cl[2 * c + 1] = make_float4((float)(hi[0] + margin), (float)(hi[1] + margin), (float)(hi[2] + margin), 0.f);
   }
   ibm_body3d *b = new ibm_body3d();
   b->m.nv = nverts;
   b->m.ntri = ntris;
+  b->m.ncl = ncl;
+  b->m.ext = (float)ext;
   for (int a = 0; a < 3; a++) {
-    b->m.bb[a] = INFINITY;
-    b->m.bb[3 + a] = -INFINITY;
+    b->m.bb[a] = blo[a];
+    b->m.bb[3 + a] = bhi[a];
   }
-  for (int k = 0; k < nverts; k++)
-    for (int a = 0; a < 3; a++) {
-      b->m.bb[a] = std::min(b->m.bb[a], verts[3 * k + a]);
-      b->m.bb[3 + a] = std::max(b->m.bb[3 + a], verts[3 * k + a]);
-    }
   const size_t sv = (size_t)3 * nverts * sizeof(double), st = (size_t)3 * ntris * sizeof(int),
                sf = (size_t)3 * ntris * sizeof(double);
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-  const size_t sbx = (size_t)2 * ntris * sizeof(float4), ssp = (size_t)ntris * sizeof(float4);
-  const size_t total = up(sv) * 2 + up(st) * 2 + up(sf) + up(sbx) + up(ssp);
+  const size_t sfx = fx.size() * sizeof(FaceExact), scl = cl.size() * sizeof(float4), sfp = fp.size() * sizeof(float4);
+  const size_t total = up(sv) * 2 + up(st) * 2 + up(sf) + up(sfx) + up(scl) + up(sfp);
   cudaError_t e = cudaMalloc(&b->mem, total);
   if (e != cudaSuccess) {
     delete b;
@@ -766,9 +1104,11 @@ extern "C" ibm_status ibm_body3d_create(const double *verts, int nverts, const i
   p += up(st);
   double *dfn = (double *)p;
   p += up(sf);
-  float4 *dbx = (float4 *)p;
-  p += up(sbx);
-  float4 *dsp = (float4 *)p;
+  FaceExact *dfx = (FaceExact *)p;
+  p += up(sfx);
+  float4 *dcl = (float4 *)p;
+  p += up(scl);
+  float4 *dfp = (float4 *)p;
   if (cuda_stream) {
     b->stream = (cudaStream_t)cuda_stream;
   } else {
@@ -780,8 +1120,9 @@ extern "C" ibm_status ibm_body3d_create(const double *verts, int nverts, const i
   if (e == cudaSuccess) e = cudaMemcpy(dt, tris, st, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(den, enb.data(), st, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(dfn, fn.data(), sf, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(dbx, fbox.data(), sbx, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(dsp, fsph.data(), ssp, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(dfx, fx.data(), sfx, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(dcl, cl.data(), scl, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(dfp, fp.data(), sfp, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     ibm_body3d_destroy(b);
     return cuda_fail(e);
@@ -791,8 +1132,9 @@ extern "C" ibm_status ibm_body3d_create(const double *verts, int nverts, const i
   b->m.tri = dt;
   b->m.enb = den;
   b->m.fn = dfn;
-  b->m.fbox = dbx;
-  b->m.fsph = dsp;
+  b->m.fx = dfx;
+  b->m.cl = dcl;
+  b->m.fp = dfp;
   *out = b;
   return IBM_OK;
 }
@@ -823,12 +1165,15 @@ extern "C" ibm_status ibm_body3d_classify(ibm_body3d *b, const ibm_grid3d *g) {
   }
   cap = std::max(1LL, std::min(cap, nn));
   cudaError_t e = cudaSuccess;
-  if (nn != b->nn || (int)cap != b->cap) {
+  const bool same = nn == b->nn && (int)cap == b->cap && g->nx == b->L.nx && g->ny == b->L.ny && g->nz == b->L.nz;
+  if (!same) {
     e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return cuda_fail(e);
     free_lattice(b);
-    b->nblk = (int)((nn + CBLK - 1) / CBLK);
-    if (e == cudaSuccess) e = cudaMalloc(&b->solid, (size_t)nn);
+    b->pw = (g->nx + 31) / 32;
+    b->nwords = (long long)b->pw * g->ny * g->nz;
+    b->nblk = (int)((b->nwords + B3 - 1) / B3);
+    if (e == cudaSuccess) e = cudaMalloc(&b->bits, (size_t)4 * b->nwords * sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMalloc(&b->tags, (size_t)nn);
     if (e == cudaSuccess) e = cudaMalloc(&b->blockcounts, (size_t)4 * b->nblk * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&b->counts, 4 * sizeof(int));
@@ -845,12 +1190,44 @@ extern "C" ibm_status ibm_body3d_classify(ibm_body3d *b, const ibm_grid3d *g) {
   int dev = 0, nsm = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const int gw = nsm * 8;  // 8 blocks of 8 warps per SM, striding over the lines (classification) or nodes
-  for (int axis = 0; axis < 3; axis++) k3_classify_lines<<<gw, B3, 0, b->stream>>>(L, b->m, axis, b->solid);
-  k3_tags<<<b->nblk, CBLK, 0, b->stream>>>(L, b->solid, b->tags, b->blockcounts);
+  // nodes inside the bounding box along each axis, by the nodes' own coordinates (non-decreasing in the index)
+  SubBox B;
+  bool any = true;
+  for (int a = 0; a < 3; a++) {
+    auto first = [&](auto outside) {  // first index that is not outside (n if none)
+      int lo = 0, hi = nd[a];
+      while (lo < hi) {
+        const int mid = lo + (hi - lo) / 2;
+        if (outside(L.lo[a] + ((double)mid + 0.5) * L.d[a])) lo = mid + 1;
+        else hi = mid;
+      }
+      return lo;
+    };
+    B.b0[a] = first([&](double x) { return x < b->m.bb[a]; });
+    B.n[a] = first([&](double x) { return !(x > b->m.bb[3 + a]); }) - B.b0[a];
+    any = any && B.n[a] > 0;
+  }
+  unsigned *xb = b->bits, *yb = xb + b->nwords, *zb = yb + b->nwords, *sb = zb + b->nwords;
+  cudaMemsetAsync(b->bits, 0, (size_t)4 * b->nwords * sizeof(unsigned), b->stream);
+  cudaMemsetAsync(b->tags, T_FLUID, (size_t)nn, b->stream);
+  if (any) {
+    // 32 (face, axis) items per block; few faces have many lines each, shared by several blocks
+    const int items = (int)((3LL * b->m.ntri + 31) / 32);
+    k3_cross<<<dim3(items, std::max(1, std::min(1024, 4 * nsm / items))), XT, 0, b->stream>>>(L, b->m, B, b->pw, b->bits,
+                                                                                             b->nwords);
+    const int nw = ((B.b0[0] + B.n[0] - 1) >> 5) - (B.b0[0] >> 5) + 1;
+    const int nyb = (int)(((long long)nw * B.n[2] + 31) / 32);
+    const int nxb = (int)(((long long)B.n[1] * B.n[2] + 32 * SEG - 1) / (32 * SEG));
+    k3_parity_xy<<<nyb + nxb, dim3(32, SEG), 0, b->stream>>>(L, B, b->pw, xb, yb, nyb);
+    k3_vote<<<(int)(((long long)nw * B.n[1] + 31) / 32), dim3(32, SEG), 0, b->stream>>>(L, B, b->pw, xb, yb, zb, sb);
+  }
+  k3_tags<<<b->nblk, B3, 0, b->stream>>>(L, b->pw, b->nwords, sb, b->tags, b->blockcounts);
   k3_scan<<<1, 1024, 0, b->stream>>>(b->nblk, b->blockcounts, b->counts);
-  k3_scatter<<<b->nblk, CBLK, 0, b->stream>>>(L, b->tags, b->blockcounts, b->counts, b->nodes, b->cap);
-  k3_closest<<<gw, B3, 0, b->stream>>>(L, b->m, b->nodes, b->counts, b->cap, b->rec);
+  k3_scatter<<<b->nblk, B3, 0, b->stream>>>(L, b->pw, b->nwords, sb, b->blockcounts, b->counts, b->nodes, b->cap);
+  float mg = 0.0f;
+  for (int a = 0; a < 3; a++) mg = std::max(mg, (float)std::max(std::fabs(g->lo[a]), std::fabs(g->hi[a])));
+  mg = 1e-5f * b->m.ext + 2e-6f * mg;
+  k3_closest<<<nsm * 3, B3, 0, b->stream>>>(L, b->m, b->nodes, b->counts, b->cap, mg, b->rec);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e);
   b->classified = true;
