@@ -6,6 +6,9 @@
 // rho v, rho E), each (ny + 6) rows of `pitch` doubles; cell (i, j) of the
 // interior sits at (j + 3) * pitch + (i + 3).  Rows are padded to a multiple
 // of 32 elements so every row starts 256-byte aligned.
+#include <algorithm>
+
+#include "fp64_math.cuh"
 #include "ibm_internal.cuh"
 
 namespace ibm {
@@ -21,15 +24,15 @@ __global__ void __launch_bounds__(256) k_dt(Consts k, const double *__restrict__
                                             const uint8_t *__restrict__ tag, DevState *ds) {
   const int ncell = k.nx * k.ny;
   double lmax = 0.0;
-  const double vis = (2.0 * k.gamma * k.mu / k.prandtl) * (1.0 / (k.dx * k.dx) + 1.0 / (k.dy * k.dy));
+  const double idx = 1.0 / k.dx, idy = 1.0 / k.dy;
+  const double vis = (2.0 * k.gamma * k.mu / k.prandtl) * fma(idx, idx, idy * idy);
   for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < ncell; n += gridDim.x * blockDim.x) {
     if (tag[n] != FLUID && !(k.ib_advance && tag[n] == IB)) continue;
     long long id = cidx(k, n % k.nx, n / k.nx);
-    double r = A[id], u = A[id + k.plane] / r, v = A[id + 2 * k.plane] / r;
-    double p = (k.gamma - 1.0) * (A[id + 3 * k.plane] - 0.5 * r * (u * u + v * v));
-    double c = sqrt(k.gamma * p / r);
-    double lam = (fabs(u) + c) / k.dx + (fabs(v) + c) / k.dy + vis / r;
-    lmax = fmax(lmax, lam);
+    const double r = A[id], ir = rcp64(r), u = A[id + k.plane] * ir, v = A[id + 2 * k.plane] * ir;
+    const double p = (k.gamma - 1.0) * fma(-0.5 * r, fma(u, u, v * v), A[id + 3 * k.plane]);
+    const double c = sqrt64(k.gamma * p * ir);
+    lmax = fmax(lmax, fma(fabs(u) + c, idx, fma(fabs(v) + c, idy, vis * ir)));
   }
   for (int off = 16; off > 0; off >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, off));
   __shared__ double wm[8];
@@ -201,199 +204,167 @@ void launch_recon_f64(const Consts &k, double *U, const ibm_stencil *st, int cap
 }
 
 // ---------------------------------------------------------------------------
-// Sec. 2: fifth-order WENO (Jiang-Shu smoothness indicators, linear weights
-// 1/10, 6/10, 3/10, eps = 1e-6); value at the face right of f2.
-// ---------------------------------------------------------------------------
-template <typename R>
-__device__ __forceinline__ R weno5(R f0, R f1, R f2, R f3, R f4) {
-  const R eps = R(1e-6);
-  R a = f0 - R(2) * f1 + f2, b = f0 - R(4) * f1 + R(3) * f2;
-  R b0 = R(13.0 / 12.0) * a * a + R(0.25) * b * b;
-  a = f1 - R(2) * f2 + f3;
-  b = f1 - f3;
-  R b1 = R(13.0 / 12.0) * a * a + R(0.25) * b * b;
-  a = f2 - R(2) * f3 + f4;
-  b = R(3) * f2 - R(4) * f3 + f4;
-  R b2 = R(13.0 / 12.0) * a * a + R(0.25) * b * b;
-  R q0 = (R(2) * f0 - R(7) * f1 + R(11) * f2) * R(1.0 / 6.0);
-  R q1 = (-f1 + R(5) * f2 + R(2) * f3) * R(1.0 / 6.0);
-  R q2 = (R(2) * f2 + R(5) * f3 - f4) * R(1.0 / 6.0);
-  R e0 = eps + b0, e1 = eps + b1, e2 = eps + b2;
-  // a_k = d_k / e_k^2, normalised; one division for all three weights
-  R e01 = e0 * e1, e12 = e1 * e2, e02 = e0 * e2;
-  R a0 = R(0.1) * e12 * e12, a1 = R(0.6) * e02 * e02, a2 = R(0.3) * e01 * e01;
-  return (a0 * q0 + a1 * q1 + a2 * q2) / (a0 + a1 + a2);
-}
-
-// Sec. 2, the second-order TVD scheme: MUSCL with the minmod limiter; value at the face right of f1
-template <typename R>
-__device__ __forceinline__ R tvd2(R f0, R f1, R f2) {
-  const R a = f1 - f0, b = f2 - f1;
-  R m = R(0);
-  if (a > R(0) && b > R(0)) m = a < b ? a : b;
-  else if (a < R(0) && b < R(0)) m = a > b ? a : b;
-  return f1 + R(0.5) * m;
-}
-
-// ---------------------------------------------------------------------------
-// Sec. 2: LDFSS(0) face flux (plain, Mr^2 = 1: explicit time stepping does
-// not precondition the dissipation).  States (rho, u, v, p); normal along
-// the first velocity component un, tangential ut.  F = (mass, normal
-// momentum, tangential momentum, energy).
-// ---------------------------------------------------------------------------
-template <bool PRE>
-__device__ __forceinline__ void ldfss_f64(double rL, double unL, double utL, double pL, double rR, double unR,
-                                          double utR, double pR, double gamma, double mr2, double F[4]) {
-  const double gg = gamma / (gamma - 1.0);
-  const double cL = sqrt(gamma * pL / rL), cR = sqrt(gamma * pR / rR);
-  const double HL = gg * pL / rL + 0.5 * (unL * unL + utL * utL);
-  const double HR = gg * pR / rR + 0.5 * (unR * unR + utR * utR);
-  const double cb = 0.5 * (cL + cR);
-  double cs = cb;
-  if (PRE) {  // low-Mach numerical sound speed c' = 1/2 sqrt((1-Mr^2)^2 un^2 + 4 Mr^2 c^2)
-    const double ub = 0.5 * (unL + unR), om = 1.0 - mr2;
-    cs = 0.5 * sqrt(om * om * ub * ub + 4.0 * mr2 * cb * cb);
-  }
-  const double ics = 1.0 / cs;
-  const double ML = unL * ics, MR = unR * ics;
-  const double aL = ML >= 0.0 ? 1.0 : 0.0;
-  const double aR = MR >= 0.0 ? 0.0 : 1.0;
-  const double tL = 1.0 - floor(fabs(ML)), tR = 1.0 - floor(fabs(MR));
-  const double bL = -fmax(tL, 0.0), bR = -fmax(tR, 0.0);
-  const double MpL = 0.25 * (ML + 1.0) * (ML + 1.0);
-  const double MmR = -0.25 * (MR - 1.0) * (MR - 1.0);
-  const double CVL = aL * (1.0 + bL) * ML - bL * MpL;
-  const double CVR = aR * (1.0 + bR) * MR - bR * MmR;
-  const double sq = sqrt(0.5 * (ML * ML + MR * MR)) - 1.0;
-  const double Mh = 0.25 * bL * bR * sq * sq;
-  const double dp = pL - pR, adp = fabs(dp);
-  const double ic2 = 0.5 * ics * ics;
-  const double MhP = Mh * (1.0 - (dp + adp) * ic2 / rL);
-  const double MhM = Mh * (1.0 - (adp - dp) * ic2 / rR);
-  const double Cp = CVL - MhP, Cm = CVR + MhM;
-  double DL, DR;
-  if (PRE && mr2 < 1.0) {  // pressure split with the physical Mach numbers (its dissipation scaled below)
-    const double ic = 1.0 / cb;
-    const double mL = unL * ic, mR = unR * ic;
-    const double paL = mL >= 0.0 ? 1.0 : 0.0, paR = mR >= 0.0 ? 0.0 : 1.0;
-    const double pbL = -fmax(1.0 - floor(fabs(mL)), 0.0), pbR = -fmax(1.0 - floor(fabs(mR)), 0.0);
-    const double PpL = 0.25 * (mL + 1.0) * (mL + 1.0) * (2.0 - mL);
-    const double PmR = 0.25 * (mR - 1.0) * (mR - 1.0) * (2.0 + mR);
-    DL = paL * (1.0 + pbL) - pbL * PpL;
-    DR = paR * (1.0 + pbR) - pbR * PmR;
-  } else {
-    const double PpL = MpL * (2.0 - ML);
-    const double PmR = -MmR * (2.0 + MR);
-    DL = aL * (1.0 + bL) - bL * PpL;
-    DR = aR * (1.0 + bR) - bR * PmR;
-  }
-  const double mL = rL * cs * Cp, mR = rR * cs * Cm;
-  double ph = DL * pL + DR * pR;
-  if (PRE && mr2 < 1.0) {
-    // low-Mach scaling: the split's departure from the face mean (its rho c du dissipation) times c'/c
-    const double fa = cs / cb;
-    ph = 0.5 * (pL + pR) + fa * ((DL - 0.5) * pL + (DR - 0.5) * pR);
-  }
-  F[0] = mL + mR;
-  F[1] = mL * unL + mR * unR + ph;
-  F[2] = mL * utL + mR * utR;
-  F[3] = mL * HL + mR * HR;
-}
-
-// ---------------------------------------------------------------------------
-// Fused residual + stage update, FP64.  One 16x16 tile of cells per block:
-// the tile and its 3-cell halo are loaded once, converted to primitives in
-// shared memory; every x- and y-face of the tile is computed once (WENO5 +
-// LDFSS + central viscous flux); each fluid cell then takes the flux
-// divergence and applies its SSP-RK3 stage:
+// Fused residual + stage update, FP64.  One TX x TY tile of cells per block,
+// one thread per cell: the tile and its 3-cell halo are loaded once and
+// converted to primitives in shared memory; WENO5 (or TVD-2) runs along tile
+// lines -- an item is one variable of one row or column, or half of one, and
+// its consecutive windows share their differences (Weno64); every face then
+// takes its LDFSS + central viscous flux, and each fluid cell its flux
+// divergence and SSP-RK3 stage
 //   stage 1: out = Un + dt L(in)
 //   stage 2: out = 3/4 Un + 1/4 (in + dt L(in))
 //   stage 3: out = 1/3 Un + 2/3 (in + dt L(in))
-// Tiles without a fluid cell exit at once.
+// or, in dual time, its point-implicit pseudo stage.  Tiles without a fluid
+// cell exit at once.
+//
+// The kernel is bound by the FP64 pipe (fp64_math.cuh; 85% busy in ncu):
+// a window per state with IEEE divisions took about 2,000 FP64 instructions
+// per cell and stage, the shared windows and reciprocals about 540.  768 x 384
+// wedge: 1.15 -> 0.39 ms per stage, two steps 6.90 -> 3.07 ms.
 // ---------------------------------------------------------------------------
-constexpr int TX = 16, TY = 16, HX = TX + 2 * NG, HY = TY + 2 * NG;
+struct F64Consts {
+  double idx, idy, g1, ig1, iR;
+  double xx, xy, xs, xv, xk;  // x face: mu 4/3 / dx, mu 2/3 / (4 dy), mu / (4 dy), mu / dx, kappa / dx
+  double yy, yx, ys, yu, yk;  // y face: the same with x and y exchanged
+  double munu2x, munu2y;      // (mu / dx)^2, (mu / dy)^2
+  // dual time: mu / min(dx, dy), 2 gamma mu / Pr (1 / dx^2 + 1 / dy^2), 1 / CFL_tau, 1 / cp
+  double nud, dif, icfl, icp;
+};
 
-// Low-Mach preconditioning parameter at a face (dual time): reference velocity
-// Ur = min(c, max(|V|, U_ref, nu/dn)) from face-averaged c, |V|, rho;
-// returns Mr^2 = (Ur/c)^2.  States (rho, u, v, p).
-__device__ __forceinline__ double face_mr2(const Consts &k, const double qL[4], const double qR[4], double dn) {
-  const double cb = 0.5 * (sqrt(k.gamma * qL[3] / qL[0]) + sqrt(k.gamma * qR[3] / qR[0]));
-  const double ub = 0.5 * (qL[1] + qR[1]), vb = 0.5 * (qL[2] + qR[2]);
-  const double Vm = sqrt(ub * ub + vb * vb);
-  const double rb = 0.5 * (qL[0] + qR[0]);
-  double Ur = fmax(fmax(Vm, 1.0), k.mu / rb / dn);
-  Ur = fmin(Ur, cb);
-  const double m = (Ur / cb) * (Ur / cb);
-  return fmin(m, 1.0);
+static F64Consts f64_consts(const Consts &k) {
+  F64Consts c;
+  c.idx = 1.0 / k.dx;
+  c.idy = 1.0 / k.dy;
+  c.g1 = k.gamma - 1.0;
+  c.ig1 = k.ig1;
+  c.iR = k.iR;
+  c.xx = k.mu * (4.0 / 3.0) * c.idx;
+  c.xy = k.mu * (2.0 / 3.0) * 0.25 * c.idy;
+  c.xs = k.mu * 0.25 * c.idy;
+  c.xv = k.mu * c.idx;
+  c.xk = k.kappa * c.idx;
+  c.yy = k.mu * (4.0 / 3.0) * c.idy;
+  c.yx = k.mu * (2.0 / 3.0) * 0.25 * c.idx;
+  c.ys = k.mu * 0.25 * c.idx;
+  c.yu = k.mu * c.idy;
+  c.yk = k.kappa * c.idy;
+  c.munu2x = (k.mu * c.idx) * (k.mu * c.idx);
+  c.munu2y = (k.mu * c.idy) * (k.mu * c.idy);
+  c.nud = k.mu / k.dmin;
+  c.dif = (2.0 * k.gamma * k.mu / k.prandtl) * (c.idx * c.idx + c.idy * c.idy);
+  c.icfl = k.cfl_tau > 0.0 ? 1.0 / k.cfl_tau : 0.0;
+  c.icp = 1.0 / k.cp;
+  return c;
 }
 
-// Weiss-Smith matrix in Q = (p, u, v, T) with first-column parameter theta:
-// Gamma (theta = 1/Ur^2 - rT/(r cp)) or dW/dQ (theta = 1/(R T)); row major
-__device__ __forceinline__ void wq_matrix(double theta, double p, double u, double v, double T, double r, double cpv,
-                                          double M[16]) {
-  const double rT = -r / T;
-  const double H = cpv * T + 0.5 * (u * u + v * v);
-  M[0] = theta;           M[1] = 0.0;    M[2] = 0.0;    M[3] = rT;
-  M[4] = theta * u;       M[5] = r;      M[6] = 0.0;    M[7] = rT * u;
-  M[8] = theta * v;       M[9] = 0.0;    M[10] = r;     M[11] = rT * v;
-  M[12] = theta * H - 1.0; M[13] = r * u; M[14] = r * v; M[15] = rT * H + r * cpv;
-  (void)p;
-}
+template <int TX, int TY>
+struct Tile64 {
+  double sq[4][TY + 2 * NG][TX + 2 * NG];  // rho, u, v, p
+  double sT[TY + 2 * NG][TX + 2 * NG];
+  double Lx[4][TY][TX + 1], Rx[4][TY][TX + 1];  // x-face states; Lx then the x flux
+  double Ly[4][TY + 1][TX], Ry[4][TY + 1][TX];  // y-face states; Ly then the y flux
+};
 
-// Gaussian elimination with partial pivoting; false if singular
-__device__ __forceinline__ bool solve4(double A[16], double b[4], double x[4]) {
-#pragma unroll
-  for (int col = 0; col < 4; col++) {
-    int piv = col;
-#pragma unroll
-    for (int i = col + 1; i < 4; i++)
-      if (fabs(A[4 * i + col]) > fabs(A[4 * piv + col])) piv = i;
-    if (A[4 * piv + col] == 0.0) return false;
-    if (piv != col) {
-#pragma unroll
-      for (int j = 0; j < 4; j++) {
-        const double t = A[4 * col + j];
-        A[4 * col + j] = A[4 * piv + j];
-        A[4 * piv + j] = t;
-      }
-      const double t = b[col];
-      b[col] = b[piv];
-      b[piv] = t;
+// one line of windows, centres p0 .. p0 + N - 1 of the values at lp[ls *]: both states of every window to
+// put(centre, qL, qR)
+template <int N, class Put>
+__device__ __forceinline__ void line64(const double *lp, int ls, int p0, bool tvd, Put put) {
+  if (tvd) {
+    // Sec. 2, the second-order TVD scheme: MUSCL with the minmod limiter
+    double f1 = lp[(p0 - 1) * ls], f2 = lp[p0 * ls];
+    for (int i = 0; i < N; i++) {
+      const double f3 = lp[(p0 + i + 1) * ls], a = f2 - f1, b = f3 - f2;
+      double m = 0.0;
+      if (a > 0.0 && b > 0.0) m = a < b ? a : b;
+      else if (a < 0.0 && b < 0.0) m = a > b ? a : b;
+      put(p0 + i, fma(0.5, m, f2), fma(-0.5, m, f2));
+      f1 = f2;
+      f2 = f3;
     }
-#pragma unroll
-    for (int i = col + 1; i < 4; i++) {
-      const double f = A[4 * i + col] / A[4 * col + col];
-#pragma unroll
-      for (int j = col; j < 4; j++) A[4 * i + j] -= f * A[4 * col + j];
-      b[i] -= f * b[col];
-    }
+    return;
   }
+  Weno64 w;
+  double f3 = lp[(p0 + 1) * ls];
+  w.start(lp[(p0 - 2) * ls], lp[(p0 - 1) * ls], lp[p0 * ls], f3);
 #pragma unroll
-  for (int i = 3; i >= 0; i--) {
-    double s = b[i];
-#pragma unroll
-    for (int j = i + 1; j < 4; j++) s -= A[4 * i + j] * x[j];
-    x[i] = s / A[4 * i + i];
+  for (int i = 0; i < N; i++) {
+    const double f4 = lp[(p0 + i + 2) * ls];
+    double qL, qR;
+    w.next(f3, f4, qL, qR);
+    put(p0 + i, qL, qR);
+    f3 = f4;
   }
-  return true;
 }
 
-template <int STAGE, bool DUAL>
-__global__ void __launch_bounds__(256) k_stage_f64(Consts k, const double *Un, const double *__restrict__ In,
-                                                   double *Out, const double *__restrict__ Wn,
-                                                   const double *__restrict__ Wm, const uint8_t *__restrict__ tag,
-                                                   DevState *ds) {
-  __shared__ double sq[4][HY][HX];  // rho, u, v, p
-  __shared__ double sT[HY][HX];     // temperature
-  __shared__ double sfx[4][TY][TX + 1];
-  __shared__ double sfy[4][TY + 1][TX];
+// Dual time (Sec. 2): pseudo-time stage of the point-implicit preconditioned update
+//   [Gamma/dtau + a dW/dQ] dQ = -(R + BDF(W)),  a = 3/(2 dt) (BDF2) or 1/dt (first step),
+// combined with the sub-iteration's start Q0 (held in A) as SSP-RK3 stage STAGE.  Gamma and dW/dQ are Weiss-Smith
+// matrices that differ in their first column's parameter only (1/Ur^2 + 1/(T cp) and 1/(R T)), so the sum is s times
+// such a matrix, s = 1/dtau + a, and its rows less multiples of the first solve in closed form: the momentum rows give
+// du, dv, the energy row r cp dT - dp = Y, and the first row dT.  Rv: flux divergence.
+template <int STAGE>
+__device__ __forceinline__ void dual_cell64(const Consts &k, const F64Consts &c, const double *A, const double *In,
+                                            double *Out, const double *__restrict__ Wn, const double *__restrict__ Wm,
+                                            long long id, const double Rv[4], bool bdf2) {
+  const long long P = k.plane;
+  double W[4], S[4];
+  for (int v = 0; v < 4; v++) W[v] = In[id + v * P];
+  const double r = W[0], ir = rcp64(r), u = W[1] * ir, v = W[2] * ir, V2 = fma(u, u, v * v);
+  const double pr = c.g1 * fma(-0.5 * r, V2, W[3]), T = pr * ir * c.iR;
+  const double aw = bdf2 ? 1.5 * k.idt_phys : k.idt_phys;
+  for (int q = 0; q < 4; q++) {
+    const long long o = id + q * P;
+    const double t = bdf2 ? k.idt_phys * fma(0.5, Wm[o], fma(1.5, W[q], -2.0 * Wn[o])) : k.idt_phys * (W[q] - Wn[o]);
+    S[q] = -(Rv[q] + t);
+  }
+  // pseudo-time step of the preconditioned eigenvalues, reference velocity by squares
+  const double c2 = k.gamma * pr * ir, vis = c.nud * ir;
+  const double ur2 = fmin(fmax(fmax(V2, 1.0), vis * vis), c2), ic2 = rcp64(c2);
+  const double mr2 = ur2 * ic2, t = 0.5 * (1.0 - mr2), Vm = sqrt64(V2), cq = sqrt64(fma(t * t, V2, ur2));
+  const double lam = fma(fma(0.5 * Vm, 1.0 + mr2, cq), c.idx + c.idy, c.dif * ir);
+  const double idtau = lam * c.icfl, s = idtau + aw;
+  const double iT = rcp64(T), rT = -r * iT;
+  const double th = fma(idtau, fma(iT, c.icp, rcp64(ur2)), aw * c.iR * iT);
+  const double is = rcp64(s), isr = is * ir, H = fma(k.cp, T, 0.5 * V2);
+  const double du = (S[1] - u * S[0]) * isr, dv = (S[2] - v * S[0]) * isr;
+  const double rcp_ = r * k.cp;
+  const double Y = fma(S[3] - H * S[0], is, -r * fma(u, du, v * dv));
+  const double dT = fma(th, Y, S[0]) * rcp64(fma(th, rcp_, s * rT));
+  const double dQ[4] = {fma(rcp_, dT, -Y), du, dv, dT}, Qk[4] = {pr, u, v, T};
+  double Qn[4];
+  if (STAGE == 1) {
+    for (int q = 0; q < 4; q++) Qn[q] = Qk[q] + dQ[q];
+  } else {
+    const double r0 = A[id], ir0 = rcp64(r0), u0 = A[id + P] * ir0, v0 = A[id + 2 * P] * ir0;
+    const double p0 = c.g1 * fma(-0.5 * r0, fma(u0, u0, v0 * v0), A[id + 3 * P]);
+    const double Q0[4] = {p0, u0, v0, p0 * ir0 * c.iR};
+    const double w0 = STAGE == 2 ? 0.75 : 1.0 / 3.0, w1 = STAGE == 2 ? 0.25 : 2.0 / 3.0;
+    for (int q = 0; q < 4; q++) Qn[q] = fma(w0, Q0[q], w1 * (Qk[q] + dQ[q]));
+  }
+  const double rn = Qn[0] * c.iR * rcp64(Qn[3]);
+  Out[id] = rn;
+  Out[id + P] = rn * Qn[1];
+  Out[id + 2 * P] = rn * Qn[2];
+  Out[id + 3 * P] = fma(Qn[0], c.ig1, 0.5 * rn * fma(Qn[1], Qn[1], Qn[2] * Qn[2]));
+}
+
+template <int STAGE, bool DUAL, int TX, int TY>
+__global__ void __launch_bounds__(TX *TY) k_stage_f64(Consts k, F64Consts c, const double *Un,
+                                                      const double *__restrict__ In, double *Out,
+                                                      const double *__restrict__ Wn, const double *__restrict__ Wm,
+                                                      const uint8_t *__restrict__ tag, DevState *ds) {
+  constexpr int HX = TX + 2 * NG, HY = TY + 2 * NG, NT = TX * TY;
+  extern __shared__ __align__(16) unsigned char smem64[];
+  Tile64<TX, TY> &sm = *reinterpret_cast<Tile64<TX, TY> *>(smem64);
+  auto &sq = sm.sq;
+  auto &sT = sm.sT;
   const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY;
   const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
   const int ci = i0 + tx, cj = j0 + ty;
   const bool inside = ci < k.nx && cj < k.ny;
   // cells the flux update advances: fluid cells, and IB nodes when the ghost layers alone impose the wall
   const bool fluid = inside && (tag[cj * k.nx + ci] == FLUID || (k.ib_advance && tag[cj * k.nx + ci] == IB));
-  const double dt = ds->dt;
+  const double dt = DUAL ? 0.0 : ds->dt;
   if (!DUAL && STAGE == 3 && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
     // end of the step (no other kernel of this stage reads t)
     ds->t = ds->t + dt;
@@ -402,8 +373,7 @@ __global__ void __launch_bounds__(256) k_stage_f64(Consts k, const double *Un, c
   if (!__syncthreads_or(fluid)) return;
 
   const long long P = k.plane;
-  const double g1 = k.gamma - 1.0;
-  for (int m = threadIdx.x; m < HX * HY; m += 256) {
+  for (int m = threadIdx.x; m < HX * HY; m += NT) {
     const int a = m % HX, b = m / HX;
     int gi = i0 - NG + a, gj = j0 - NG + b;
     double U0, U1, U2, U3;
@@ -419,171 +389,141 @@ __global__ void __launch_bounds__(256) k_stage_f64(Consts k, const double *Un, c
       U2 = k.Uinf[2];
       U3 = k.Uinf[3];
     }
-    const double r = U0;
-    const double ir = 1.0 / r;
+    const double ir = rcp64(U0);
     const double u = U1 * ir, v = U2 * ir;
-    const double p = g1 * (U3 - 0.5 * r * (u * u + v * v));
-    sq[0][b][a] = r;
+    const double p = c.g1 * fma(-0.5 * U0, fma(u, u, v * v), U3);
+    sq[0][b][a] = U0;
     sq[1][b][a] = u;
     sq[2][b][a] = v;
     sq[3][b][a] = p;
-    sT[b][a] = p * ir / k.R;
+    sT[b][a] = p * ir * c.iR;
   }
   __syncthreads();
 
-  const double mu = k.mu, kap = k.kappa;
-  const double idx = 1.0 / k.dx, idy = 1.0 / k.dy;
-  // x-faces: face f sits between local columns f+2 and f+3 (global i0-1+f, i0+f)
-  for (int m = threadIdx.x; m < (TX + 1) * TY; m += 256) {
-    const int f = m % (TX + 1), row = m / (TX + 1);
-    const int b = row + NG;
-    double qL[4], qR[4];
-    for (int v = 0; v < 4; v++) {
-      const double *s = &sq[v][b][f];
-      if (k.tvd2) {
-        qL[v] = tvd2(s[1], s[2], s[3]);
-        qR[v] = tvd2(s[4], s[3], s[2]);
-      } else {
-        qL[v] = weno5(s[0], s[1], s[2], s[3], s[4]);
-        qR[v] = weno5(s[5], s[4], s[3], s[2], s[1]);
-      }
-    }
-    if (!(qL[0] > 0.0) || !(qL[3] > 0.0) || !(qR[0] > 0.0) || !(qR[3] > 0.0)) {
-      for (int v = 0; v < 4; v++) {
-        qL[v] = sq[v][b][f + 2];
-        qR[v] = sq[v][b][f + 3];
-      }
-    }
-    double F[4];
-    ldfss_f64<DUAL>(qL[0], qL[1], qL[2], qL[3], qR[0], qR[1], qR[2], qR[3], k.gamma,
-                    DUAL ? face_mr2(k, qL, qR, k.dx) : 1.0, F);
-    const int a = f + 2, a1 = f + 3;
-    const double ux = (sq[1][b][a1] - sq[1][b][a]) * idx;
-    const double vx = (sq[2][b][a1] - sq[2][b][a]) * idx;
-    const double Tx = (sT[b][a1] - sT[b][a]) * idx;
-    const double uy = (sq[1][b + 1][a] - sq[1][b - 1][a] + sq[1][b + 1][a1] - sq[1][b - 1][a1]) * (0.25 * idy);
-    const double vy = (sq[2][b + 1][a] - sq[2][b - 1][a] + sq[2][b + 1][a1] - sq[2][b - 1][a1]) * (0.25 * idy);
-    const double txx = mu * ((4.0 / 3.0) * ux - (2.0 / 3.0) * vy);
-    const double txy = mu * (uy + vx);
-    const double uf = 0.5 * (sq[1][b][a] + sq[1][b][a1]), vf = 0.5 * (sq[2][b][a] + sq[2][b][a1]);
-    sfx[0][row][f] = F[0];
-    sfx[1][row][f] = F[1] - txx;
-    sfx[2][row][f] = F[2] - txy;
-    sfx[3][row][f] = F[3] - (uf * txx + vf * txy + kap * Tx);
+  // face states along lines: TX (TY) + 2 windows per row (column), in two halves of nine or one of ten
+  constexpr int NX = TX == 16 ? 9 : 10, HFX = TX == 16 ? 2 : 1, NY = TY == 16 ? 9 : 10, HFY = TY == 16 ? 2 : 1;
+  static_assert(4 * TY * HFX + 4 * TX * HFY == NT, "one item per thread");
+  if (threadIdx.x < 4 * TY * HFX) {
+    const int u = threadIdx.x, half = u % HFX, line = u / HFX % TY, v = u / (HFX * TY);
+    line64<NX>(&sq[v][NG + line][0], 1, 2 + NX * half, k.tvd2, [&](int pc, double qL, double qR) {
+      if (pc - 2 <= TX) sm.Lx[v][line][pc - 2] = qL;  // face between pc and pc + 1
+      if (pc >= 3) sm.Rx[v][line][pc - 3] = qR;       // face between pc - 1 and pc
+    });
+  } else {
+    const int u = threadIdx.x - 4 * TY * HFX, line = u % TX, half = u / TX % HFY, v = u / (TX * HFY);
+    line64<NY>(&sq[v][0][NG + line], HX, 2 + NY * half, k.tvd2, [&](int pc, double qL, double qR) {
+      if (pc - 2 <= TY) sm.Ly[v][pc - 2][line] = qL;
+      if (pc >= 3) sm.Ry[v][pc - 3][line] = qR;
+    });
   }
-  // y-faces: face f sits between local rows f+2 and f+3
-  for (int m = threadIdx.x; m < TX * (TY + 1); m += 256) {
-    const int col = m % TX, f = m / TX;
-    const int a = col + NG;
-    double qL[4], qR[4];
-    for (int v = 0; v < 4; v++) {
-      const double s0 = sq[v][f][a], s1 = sq[v][f + 1][a], s2 = sq[v][f + 2][a];
-      const double s3 = sq[v][f + 3][a], s4 = sq[v][f + 4][a], s5 = sq[v][f + 5][a];
-      if (k.tvd2) {
-        qL[v] = tvd2(s1, s2, s3);
-        qR[v] = tvd2(s4, s3, s2);
-      } else {
-        qL[v] = weno5(s0, s1, s2, s3, s4);
-        qR[v] = weno5(s5, s4, s3, s2, s1);
-      }
-    }
-    if (!(qL[0] > 0.0) || !(qL[3] > 0.0) || !(qR[0] > 0.0) || !(qR[3] > 0.0)) {
-      for (int v = 0; v < 4; v++) {
-        qL[v] = sq[v][f + 2][a];
-        qR[v] = sq[v][f + 3][a];
-      }
-    }
+  __syncthreads();
+
+  // face fluxes: inviscid (first order where a reconstructed density or pressure is not positive) less viscous
+  for (int m = threadIdx.x; m < (TX + 1) * TY + TX * (TY + 1); m += NT) {
     double F[4];
-    // normal velocity v, tangential u
-    ldfss_f64<DUAL>(qL[0], qL[2], qL[1], qL[3], qR[0], qR[2], qR[1], qR[3], k.gamma,
-                    DUAL ? face_mr2(k, qL, qR, k.dy) : 1.0, F);
-    const int b = f + 2, b1 = f + 3;
-    const double uy = (sq[1][b1][a] - sq[1][b][a]) * idy;
-    const double vy = (sq[2][b1][a] - sq[2][b][a]) * idy;
-    const double Ty = (sT[b1][a] - sT[b][a]) * idy;
-    const double ux = (sq[1][b][a + 1] - sq[1][b][a - 1] + sq[1][b1][a + 1] - sq[1][b1][a - 1]) * (0.25 * idx);
-    const double vx = (sq[2][b][a + 1] - sq[2][b][a - 1] + sq[2][b1][a + 1] - sq[2][b1][a - 1]) * (0.25 * idx);
-    const double tyy = mu * ((4.0 / 3.0) * vy - (2.0 / 3.0) * ux);
-    const double txy = mu * (uy + vx);
-    const double uf = 0.5 * (sq[1][b][a] + sq[1][b1][a]), vf = 0.5 * (sq[2][b][a] + sq[2][b1][a]);
-    sfy[0][f][col] = F[0];
-    sfy[1][f][col] = F[2] - txy;
-    sfy[2][f][col] = F[1] - tyy;
-    sfy[3][f][col] = F[3] - (uf * txy + vf * tyy + kap * Ty);
+    if (m < (TX + 1) * TY) {
+      const int f = m % (TX + 1), row = m / (TX + 1), b = row + NG, a = f + 2, a1 = f + 3;
+      double qL[4], qR[4];
+      for (int v = 0; v < 4; v++) {
+        qL[v] = sm.Lx[v][row][f];
+        qR[v] = sm.Rx[v][row][f];
+      }
+      if (!positive(qL[0]) || !positive(qL[3]) || !positive(qR[0]) || !positive(qR[3])) {
+        for (int v = 0; v < 4; v++) {
+          qL[v] = sq[v][b][a];
+          qR[v] = sq[v][b][a1];
+        }
+      }
+      ldfss64<DUAL, 1>(qL[0], qL[1], &qL[2], qL[3], qR[0], qR[1], &qR[2], qR[3], k.gamma, c.ig1, c.munu2x, F);
+      const double u0 = sq[1][b][a], u1 = sq[1][b][a1], v0 = sq[2][b][a], v1 = sq[2][b][a1];
+      const double us = (sq[1][b + 1][a] - sq[1][b - 1][a]) + (sq[1][b + 1][a1] - sq[1][b - 1][a1]);
+      const double vs = (sq[2][b + 1][a] - sq[2][b - 1][a]) + (sq[2][b + 1][a1] - sq[2][b - 1][a1]);
+      const double txx = fma(c.xx, u1 - u0, -c.xy * vs), txy = fma(c.xs, us, c.xv * (v1 - v0));
+      const double w = fma(u0 + u1, txx, (v0 + v1) * txy);
+      sm.Lx[0][row][f] = F[0];
+      sm.Lx[1][row][f] = F[1] - txx;
+      sm.Lx[2][row][f] = F[2] - txy;
+      sm.Lx[3][row][f] = fma(-c.xk, sT[b][a1] - sT[b][a], fma(-0.5, w, F[3]));
+    } else {
+      const int mm = m - (TX + 1) * TY, col = mm % TX, f = mm / TX, a = col + NG, b = f + 2, b1 = f + 3;
+      double qL[4], qR[4];
+      for (int v = 0; v < 4; v++) {
+        qL[v] = sm.Ly[v][f][col];
+        qR[v] = sm.Ry[v][f][col];
+      }
+      if (!positive(qL[0]) || !positive(qL[3]) || !positive(qR[0]) || !positive(qR[3])) {
+        for (int v = 0; v < 4; v++) {
+          qL[v] = sq[v][b][a];
+          qR[v] = sq[v][b1][a];
+        }
+      }
+      // normal velocity v, tangential u
+      ldfss64<DUAL, 1>(qL[0], qL[2], &qL[1], qL[3], qR[0], qR[2], &qR[1], qR[3], k.gamma, c.ig1, c.munu2y, F);
+      const double u0 = sq[1][b][a], u1 = sq[1][b1][a], v0 = sq[2][b][a], v1 = sq[2][b1][a];
+      const double us = (sq[1][b][a + 1] - sq[1][b][a - 1]) + (sq[1][b1][a + 1] - sq[1][b1][a - 1]);
+      const double vs = (sq[2][b][a + 1] - sq[2][b][a - 1]) + (sq[2][b1][a + 1] - sq[2][b1][a - 1]);
+      const double tyy = fma(c.yy, v1 - v0, -c.yx * us), txy = fma(c.ys, vs, c.yu * (u1 - u0));
+      const double w = fma(u0 + u1, txy, (v0 + v1) * tyy);
+      sm.Ly[0][f][col] = F[0];
+      sm.Ly[1][f][col] = F[2] - txy;
+      sm.Ly[2][f][col] = F[1] - tyy;
+      sm.Ly[3][f][col] = fma(-c.yk, sT[b1][a] - sT[b][a], fma(-0.5, w, F[3]));
+    }
   }
   __syncthreads();
   if (!fluid) return;
   const long long id = cidx(k, ci, cj);
-  if (!DUAL) {
-    for (int v = 0; v < 4; v++) {
-      const double L = -((sfx[v][ty][tx + 1] - sfx[v][ty][tx]) * idx + (sfy[v][ty + 1][tx] - sfy[v][ty][tx]) * idy);
-      const long long o = id + v * P;
-      double r;
-      if (STAGE == 1) r = Un[o] + dt * L;
-      else if (STAGE == 2) r = 0.75 * Un[o] + 0.25 * (In[o] + dt * L);
-      else r = (1.0 / 3.0) * Un[o] + (2.0 / 3.0) * (In[o] + dt * L);
-      Out[o] = r;
-    }
+  double Rv[4];
+  for (int v = 0; v < 4; v++)
+    Rv[v] = fma(sm.Lx[v][ty][tx + 1] - sm.Lx[v][ty][tx], c.idx, (sm.Ly[v][ty + 1][tx] - sm.Ly[v][ty][tx]) * c.idy);
+  if (DUAL) {
+    dual_cell64<STAGE>(k, c, Un, In, Out, Wn, Wm, id, Rv, ds->steps > 0);
     return;
   }
-  // Dual time (Sec. 2): pseudo-time stage of the point-implicit preconditioned update
-  //   [Gamma/dtau + a dW/dQ] dQ = -(R + BDF(W)),  a = 3/(2 dt) (BDF2) or 1/dt (first step)
-  // combined with the sub-iteration's start Q0 as SSP-RK3 stage STAGE.  FP64 4x4 solve.
-  const bool bdf2 = ds->steps > 0;
-  const double dtp = k.dt_phys;
-  double W[4], S[4];
-  for (int v = 0; v < 4; v++) W[v] = In[id + v * P];
-  const double r = W[0], iu = W[1] / r, iv = W[2] / r;
-  const double pr = g1 * (W[3] - 0.5 * r * (iu * iu + iv * iv));
-  const double T = pr / (r * k.R);
   for (int v = 0; v < 4; v++) {
-    const double Rv = (sfx[v][ty][tx + 1] - sfx[v][ty][tx]) / k.dx + (sfy[v][ty + 1][tx] - sfy[v][ty][tx]) / k.dy;
     const long long o = id + v * P;
-    const double tdt = bdf2 ? (3.0 * W[v] - 4.0 * Wn[o] + Wm[o]) / (2.0 * dtp) : (W[v] - Wn[o]) / dtp;
-    S[v] = -(Rv + tdt);
+    if (STAGE == 1) Out[o] = fma(-dt, Rv[v], Un[o]);
+    else if (STAGE == 2) Out[o] = fma(0.75, Un[o], 0.25 * fma(-dt, Rv[v], In[o]));
+    else Out[o] = fma(1.0 / 3.0, Un[o], (2.0 / 3.0) * fma(-dt, Rv[v], In[o]));
   }
-  const double cs = sqrt(k.gamma * pr / r);
-  const double Vm = sqrt(iu * iu + iv * iv);
-  double Ur = fmax(fmax(Vm, 1.0), k.mu / r / k.dmin);
-  Ur = fmin(Ur, cs);
-  const double mr2 = (Ur / cs) * (Ur / cs);
-  const double up = 0.5 * Vm * (1.0 + mr2);
-  const double om = 1.0 - mr2;
-  const double cp_ = 0.5 * sqrt(om * om * Vm * Vm + 4.0 * Ur * Ur);
-  const double vis = (2.0 * k.gamma * k.mu / k.prandtl) * (1.0 / (k.dx * k.dx) + 1.0 / (k.dy * k.dy));
-  const double lam = (up + cp_) * (1.0 / k.dx + 1.0 / k.dy) + vis / r;
-  const double dtau = k.cfl_tau / lam;
-  const double theta = 1.0 / (Ur * Ur) - (-r / T) / (r * k.cp);
-  double G[16], J[16];
-  wq_matrix(theta, pr, iu, iv, T, r, k.cp, G);
-  wq_matrix(1.0 / (k.R * T), pr, iu, iv, T, r, k.cp, J);
-  const double a = bdf2 ? 1.5 / dtp : 1.0 / dtp;
-  for (int q = 0; q < 16; q++) G[q] = G[q] / dtau + a * J[q];
-  double dQ[4];
-  if (!solve4(G, S, dQ)) return;
-  // Q0 of the sub-iteration (held in Un = A)
-  const double r0 = Un[id], u0 = Un[id + P] / r0, v0 = Un[id + 2 * P] / r0;
-  const double p0 = g1 * (Un[id + 3 * P] - 0.5 * r0 * (u0 * u0 + v0 * v0));
-  const double Q0[4] = {p0, u0, v0, p0 / (r0 * k.R)};
-  const double Qk[4] = {pr, iu, iv, T};
-  double Qn[4];
-  for (int v = 0; v < 4; v++) {
-    const double e = Qk[v] + dQ[v];
-    Qn[v] = STAGE == 1 ? e : (STAGE == 2 ? 0.75 * Q0[v] + 0.25 * e : (1.0 / 3.0) * Q0[v] + (2.0 / 3.0) * e);
-  }
-  const double rn = Qn[0] / (k.R * Qn[3]);
-  Out[id] = rn;
-  Out[id + P] = rn * Qn[1];
-  Out[id + 2 * P] = rn * Qn[2];
-  Out[id + 3 * P] = Qn[0] / (k.gamma - 1.0) + 0.5 * rn * (Qn[1] * Qn[1] + Qn[2] * Qn[2]);
+}
+
+template <int STAGE, bool DUAL, int TX, int TY>
+static void launch_tile_f64(const Consts &k, const double *Un, const double *In, double *Out, const double *Wn,
+                            const double *Wm, const uint8_t *tag, DevState *ds, cudaStream_t s) {
+  constexpr int bytes = (int)sizeof(Tile64<TX, TY>);
+  if (bytes > 48 * 1024)
+    cudaFuncSetAttribute(k_stage_f64<STAGE, DUAL, TX, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  k_stage_f64<STAGE, DUAL, TX, TY><<<dim3((k.nx + TX - 1) / TX, (k.ny + TY - 1) / TY), TX * TY, bytes, s>>>(
+      k, f64_consts(k), Un, In, Out, Wn, Wm, tag, ds);
+}
+
+// Tile shape by the work of the fullest SM: an SM's time is its tiles' FP64 instructions (halo cells, windows and
+// faces included: 1, 0.53 and 0.30 of the 16 x 16 tile), and the tiles are dealt evenly, so a grid of few tiles takes
+// the shape whose last round is fullest -- 257 x 131 cells are 153 tiles of 16 x 16 on 152 SMs, 289 of 16 x 8: a
+// dual-time pseudo stage there went from 374 us (16 x 16, the arithmetic before) to 77.
+template <bool DUAL>
+static void launch_tiles_f64(const Consts &k, int stage, const double *Un, const double *In, double *Out,
+                             const double *Wn, const double *Wm, const uint8_t *tag, DevState *ds, cudaStream_t s) {
+  const auto cost = [&](int tx, int ty, double work) {
+    const long long tiles = (long long)((k.nx + tx - 1) / tx) * ((k.ny + ty - 1) / ty);
+    return (double)((tiles + 151) / 152) * work;
+  };
+  const double c0 = cost(16, 16, 1.0), c1 = cost(16, 8, 0.53), c2 = cost(8, 8, 0.30);
+  const int shape = c0 <= c1 && c0 <= c2 ? 0 : c1 <= c2 ? 1 : 2;
+#define IBM_F64(S)                                                                                    \
+  (shape == 0   ? launch_tile_f64<S, DUAL, 16, 16>(k, Un, In, Out, Wn, Wm, tag, ds, s)                \
+   : shape == 1 ? launch_tile_f64<S, DUAL, 16, 8>(k, Un, In, Out, Wn, Wm, tag, ds, s)                 \
+                : launch_tile_f64<S, DUAL, 8, 8>(k, Un, In, Out, Wn, Wm, tag, ds, s))
+  if (stage == 1) IBM_F64(1);
+  else if (stage == 2) IBM_F64(2);
+  else IBM_F64(3);
+#undef IBM_F64
 }
 
 void launch_dual_f64(const Consts &k, int stage, const double *A, const double *In, double *Out, const double *Wn,
                      const double *Wm, const uint8_t *tag, DevState *ds, cudaStream_t s) {
-  dim3 grid((k.nx + TX - 1) / TX, (k.ny + TY - 1) / TY);
-  if (stage == 1) k_stage_f64<1, true><<<grid, 256, 0, s>>>(k, A, In, Out, Wn, Wm, tag, ds);
-  else if (stage == 2) k_stage_f64<2, true><<<grid, 256, 0, s>>>(k, A, In, Out, Wn, Wm, tag, ds);
-  else k_stage_f64<3, true><<<grid, 256, 0, s>>>(k, A, In, Out, Wn, Wm, tag, ds);
+  launch_tiles_f64<true>(k, stage, A, In, Out, Wn, Wm, tag, ds, s);
 }
 
 __global__ void k_dual_end(Consts k, DevState *ds) {
@@ -595,10 +535,7 @@ void launch_dual_end(const Consts &k, DevState *ds, cudaStream_t s) { k_dual_end
 
 void launch_stage_f64(const Consts &k, int stage, const double *Un, const double *In, double *Out,
                       const uint8_t *tag, DevState *ds, cudaStream_t s) {
-  dim3 grid((k.nx + TX - 1) / TX, (k.ny + TY - 1) / TY);
-  if (stage == 1) k_stage_f64<1, false><<<grid, 256, 0, s>>>(k, Un, In, Out, nullptr, nullptr, tag, ds);
-  else if (stage == 2) k_stage_f64<2, false><<<grid, 256, 0, s>>>(k, Un, In, Out, nullptr, nullptr, tag, ds);
-  else k_stage_f64<3, false><<<grid, 256, 0, s>>>(k, Un, In, Out, nullptr, nullptr, tag, ds);
+  launch_tiles_f64<false>(k, stage, Un, In, Out, nullptr, nullptr, tag, ds, s);
 }
 
 }  // namespace ibm

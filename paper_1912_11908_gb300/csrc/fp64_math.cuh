@@ -1,0 +1,159 @@
+// FP64 arithmetic of the residuals (2-D and 3-D).  GB300 retires two FP64 lanes per SM and clock (1.056 TFLOP/s
+// measured, 1/70 of its FP32 rate), so an FP64 residual is bound by the number of FP64 instructions, and everything
+// here is written to issue few of them: reciprocals and square roots as the hardware's approximation (relative error
+// about 2^-20) and one third-order correction (Householder's method: the new error is the old one cubed, below
+// 2^-58) in place of the IEEE sequences with their range checks -- the arguments are densities, pressures, speeds and
+// smoothness weights in the normal range; one reciprocal shared where several quotients stand side by side; signs and
+// magnitudes against 1 tested on the integer bits, off the FP64 pipe.
+#pragma once
+
+namespace ibm {
+
+// 1 / x for normal x
+__device__ __forceinline__ double rcp64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);  // y (1 + e + e^2)
+}
+
+// 1 / sqrt(x) for normal x > 0 (NaN for x < 0)
+__device__ __forceinline__ double rsqrt64(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);  // y (1 + e / 2 + 3 e^2 / 8)
+}
+
+__device__ __forceinline__ int hi64(double x) { return __double2hiint(x); }
+
+// sqrt(x) for x >= 0; 0 for zero and subnormal x (squares of speeds below 1e-154), where the approximation is infinite
+__device__ __forceinline__ double sqrt64(double x) {
+  return (unsigned)hi64(x) < 0x00100000u ? 0.0 : x * rsqrt64(x);
+}
+
+// |x| < 1 (exact: the biased exponent is below 1023); false for NaN
+__device__ __forceinline__ bool below_one(double x) { return (hi64(x) & 0x7fffffff) < 0x3ff00000; }
+// x positive, normal and finite
+__device__ __forceinline__ bool positive(double x) { return (unsigned)(hi64(x) - 1) < 0x7fefffffu; }
+__device__ __forceinline__ bool negative(double x) { return hi64(x) < 0; }
+
+// Sec. 2: fifth-order WENO (Jiang-Shu smoothness indicators, linear weights 1/10, 6/10, 3/10, eps = 1e-6) of one
+// five-point window, both of its values: the left state at the centre's right face and, mirrored, the right state at
+// its left face.  With first differences g and second differences d of the line, the indicators are
+//   eps + beta_k = [eps + 13/12 d^2] + (first-difference term / 2)^2,
+// whose bracket three windows share; the candidates are taken relative to the centre's value and the nonlinear
+// weights d_k / (eps + beta_k)^2 cleared of their common denominator, so that each value is f + N / D and one
+// reciprocal of D_L D_R serves both.  About 40 FP64 instructions for two states.
+struct Weno64 {
+  double f, g, hg, d0, d1, e0, e1;  // centre value; g = f(c) - f(c-1) and half of it; second differences at c - 1 and
+                                    // c; their brackets
+  // window centred at f2; the first advance() moves to it
+  __device__ __forceinline__ void start(double f0, double f1, double f2, double f3) {
+    const double ga = f1 - f0, gb = f2 - f1, gc = f3 - f2;
+    f = f2;
+    g = gb;
+    hg = 0.5 * gb;
+    d0 = gb - ga;
+    d1 = gc - gb;
+    e0 = fma((13.0 / 12.0) * d0, d0, 1e-6);
+    e1 = fma((13.0 / 12.0) * d1, d1, 1e-6);
+  }
+  // the two states of the window at f, f3 and f4 the values one and two beyond it; then moves the window on
+  __device__ __forceinline__ void next(double f3, double f4, double &qL, double &qR) {
+    const double g0 = f3 - f, hg0 = 0.5 * g0, d2 = (f4 - f3) - g0, e2 = fma((13.0 / 12.0) * d2, d2, 1e-6);
+    const double b0 = fma(0.5, d0, g), b1 = fma(0.5, d1, g), b2 = fma(0.5, d2, -g0);
+    const double i0 = fma(b0, b0, e0), i1 = fma(b1, b1, e1), i2 = fma(b2, b2, e2);
+    const double t0 = i0 * i0, t1 = i1 * i1, t2 = i2 * i2;
+    const double s12 = t1 * t2, s02 = t0 * t2, s01 = t0 * t1;
+    // left: candidates less f times (1, 6, 3), the linear weights in units of 1/10
+    const double l0 = fma(1.0 / 3.0, d0, hg), l1 = fma(3.0, g0, -d1), l2 = hg0 - b2;
+    const double NL = fma(s12, l0, fma(s02, l1, s01 * l2)), DL = fma(6.0, s02, fma(3.0, s01, s12));
+    const double r0 = fma(1.0 / 3.0, d2, -hg0), r1 = fma(-3.0, g, -d1), r2 = -hg - b0;
+    const double NR = fma(s01, r0, fma(s02, r1, s12 * r2)), DR = fma(6.0, s02, fma(3.0, s12, s01));
+    const double inv = rcp64(DL * DR);
+    qL = fma(NL * DR, inv, f);
+    qR = fma(NR * DL, inv, f);
+    f = f3;
+    g = g0;
+    hg = hg0;
+    d0 = d1;
+    d1 = d2;
+    e0 = e1;
+    e1 = e2;
+  }
+};
+
+// Sec. 2, LDFSS(0) with D tangential velocity components: face flux of the states (rho, un, ut..., p), F = (mass,
+// normal momentum, tangential momenta..., energy).  PRE: the dual-time low-Mach form -- numerical sound speed
+// c' = 1/2 sqrt((1 - Mr^2)^2 un^2 + 4 Mr^2 c^2) of the reference velocity Ur = min(c, max(|V|, U_ref, nu/dn)) (face
+// averages; taken by squares), pressure split in the physical Mach numbers with its departure from the face mean
+// scaled by c'/c.  munu2 = (mu / dn)^2.
+template <bool PRE, int D>
+__device__ __forceinline__ void ldfss64(double rL, double unL, const double utL[D], double pL, double rR, double unR,
+                                        const double utR[D], double pR, double gamma, double ig1, double munu2,
+                                        double F[3 + D]) {
+  const double irr = rcp64(rL * rR), irL = irr * rR, irR = irr * rL;
+  const double c2L = gamma * pL * irL, c2R = gamma * pR * irR;
+  const double cL = c2L * rsqrt64(c2L), cR = c2R * rsqrt64(c2R);
+  double kL = unL * unL, kR = unR * unR;
+#pragma unroll
+  for (int d = 0; d < D; d++) {
+    kL = fma(utL[d], utL[d], kL);
+    kR = fma(utR[d], utR[d], kR);
+  }
+  const double HL = fma(0.5, kL, c2L * ig1), HR = fma(0.5, kR, c2R * ig1);  // gamma/(gamma-1) p/rho = c^2/(gamma-1)
+  const double cb = 0.5 * (cL + cR), icb = rcp64(cb);
+  double cs = cb, ics = icb;
+  bool low = false;
+  if (PRE) {
+    const double ub = 0.5 * (unL + unR);
+    double v2 = ub * ub;
+#pragma unroll
+    for (int d = 0; d < D; d++) {
+      const double vb = 0.5 * (utL[d] + utR[d]);
+      v2 = fma(vb, vb, v2);
+    }
+    const double rb = 0.5 * (rL + rR), rb2 = rb * rb, cb2 = cb * cb;
+    double ur2 = fmax(v2, 1.0);
+    if (munu2 > ur2 * rb2) ur2 = munu2 * rcp64(rb2);
+    if (ur2 < cb2) {
+      low = true;
+      const double t = 0.5 * fma(-ur2 * icb, icb, 1.0) * ub;
+      const double x = fma(t, t, ur2);
+      ics = rsqrt64(x);
+      cs = x * ics;
+    }
+  }
+  const double ML = unL * ics, MR = unR * ics;
+  const bool subL = below_one(ML), subR = below_one(MR);
+  const double aL = ML + 1.0, aR = MR - 1.0;
+  const double MpL = 0.25 * aL * aL, MmR = -0.25 * aR * aR;
+  const double CL = subL ? MpL : (negative(ML) ? 0.0 : ML), CR = subR ? MmR : (negative(MR) ? MR : 0.0);
+  const double sq = sqrt64(0.5 * fma(ML, ML, MR * MR)) - 1.0;
+  const double Mh = subL && subR ? 0.25 * sq * sq : 0.0;
+  // only the side that the pressure falls to is weighted: M_1/2 (1 - |dp| / (rho c'^2))
+  const double dp = pL - pR;
+  const bool up = negative(dp);
+  const double Mw = Mh * fma(-fabs(dp), (up ? irR : irL) * (ics * ics), 1.0);
+  const double Cp = CL - (up ? Mh : Mw), Cm = CR + (up ? Mw : Mh);
+  double DL, DR, ph;
+  if (PRE && low) {
+    const double mL = unL * icb, mR = unR * icb, bL = mL + 1.0, bR = mR - 1.0;
+    DL = below_one(mL) ? 0.25 * bL * bL * (2.0 - mL) : (negative(mL) ? 0.0 : 1.0);
+    DR = below_one(mR) ? 0.25 * bR * bR * (2.0 + mR) : (negative(mR) ? 1.0 : 0.0);
+    ph = fma(cs * icb, fma(DL - 0.5, pL, (DR - 0.5) * pR), 0.5 * (pL + pR));
+  } else {
+    DL = subL ? MpL * (2.0 - ML) : (negative(ML) ? 0.0 : 1.0);
+    DR = subR ? -MmR * (2.0 + MR) : (negative(MR) ? 1.0 : 0.0);
+    ph = fma(DL, pL, DR * pR);
+  }
+  const double mL = rL * cs * Cp, mR = rR * cs * Cm;
+  F[0] = mL + mR;
+  F[1] = fma(mL, unL, fma(mR, unR, ph));
+#pragma unroll
+  for (int d = 0; d < D; d++) F[2 + d] = fma(mL, utL[d], mR * utR[d]);
+  F[2 + D] = fma(mL, HL, mR * HR);
+}
+
+}  // namespace ibm
