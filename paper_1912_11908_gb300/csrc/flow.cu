@@ -219,39 +219,37 @@ void launch_recon_f64(const Consts &k, double *U, const ibm_stencil *st, int cap
 //
 // The kernel is bound by the FP64 pipe (fp64_math.cuh; 85% busy in ncu):
 // a window per state with IEEE divisions took about 2,000 FP64 instructions
-// per cell and stage, the shared windows and reciprocals about 540.  768 x 384
-// wedge: 1.15 -> 0.39 ms per stage, two steps 6.90 -> 3.07 ms.
+// per cell and stage, the shared windows and reciprocals about 540, with
+// products on the integer pipes 370.  768 x 384 wedge: 1.15 -> 0.39 -> 0.245
+// ms per stage, two steps 6.90 -> 3.07 -> 2.21 ms.
 // ---------------------------------------------------------------------------
 struct F64Consts {
-  double idx, idy, g1, ig1, iR;
-  double xx, xy, xs, xv, xk;  // x face: mu 4/3 / dx, mu 2/3 / (4 dy), mu / (4 dy), mu / dx, kappa / dx
-  double yy, yx, ys, yu, yk;  // y face: the same with x and y exchanged
-  double munu2x, munu2y;      // (mu / dx)^2, (mu / dy)^2
+  double ih[2], g1, ig1, iR;
+  // viscous terms of the x and y faces, h the spacing along the normal and t along the tangent: mu 4/3 / h,
+  // mu 2/3 / (4 t), mu / (4 t), mu / h, kappa / h, and (mu / h)^2
+  double nn[2], nt[2], ts[2], tv[2], kt[2], munu2[2];
   // dual time: mu / min(dx, dy), 2 gamma mu / Pr (1 / dx^2 + 1 / dy^2), 1 / CFL_tau, 1 / cp
   double nud, dif, icfl, icp;
 };
 
 static F64Consts f64_consts(const Consts &k) {
   F64Consts c;
-  c.idx = 1.0 / k.dx;
-  c.idy = 1.0 / k.dy;
+  c.ih[0] = 1.0 / k.dx;
+  c.ih[1] = 1.0 / k.dy;
   c.g1 = k.gamma - 1.0;
   c.ig1 = k.ig1;
   c.iR = k.iR;
-  c.xx = k.mu * (4.0 / 3.0) * c.idx;
-  c.xy = k.mu * (2.0 / 3.0) * 0.25 * c.idy;
-  c.xs = k.mu * 0.25 * c.idy;
-  c.xv = k.mu * c.idx;
-  c.xk = k.kappa * c.idx;
-  c.yy = k.mu * (4.0 / 3.0) * c.idy;
-  c.yx = k.mu * (2.0 / 3.0) * 0.25 * c.idx;
-  c.ys = k.mu * 0.25 * c.idx;
-  c.yu = k.mu * c.idy;
-  c.yk = k.kappa * c.idy;
-  c.munu2x = (k.mu * c.idx) * (k.mu * c.idx);
-  c.munu2y = (k.mu * c.idy) * (k.mu * c.idy);
+  for (int d = 0; d < 2; d++) {
+    const double in = c.ih[d], it = c.ih[1 - d];
+    c.nn[d] = k.mu * (4.0 / 3.0) * in;
+    c.nt[d] = k.mu * (2.0 / 3.0) * 0.25 * it;
+    c.ts[d] = k.mu * 0.25 * it;
+    c.tv[d] = k.mu * in;
+    c.kt[d] = k.kappa * in;
+    c.munu2[d] = (k.mu * in) * (k.mu * in);
+  }
   c.nud = k.mu / k.dmin;
-  c.dif = (2.0 * k.gamma * k.mu / k.prandtl) * (c.idx * c.idx + c.idy * c.idy);
+  c.dif = (2.0 * k.gamma * k.mu / k.prandtl) * (c.ih[0] * c.ih[0] + c.ih[1] * c.ih[1]);
   c.icfl = k.cfl_tau > 0.0 ? 1.0 / k.cfl_tau : 0.0;
   c.icp = 1.0 / k.cp;
   return c;
@@ -265,33 +263,38 @@ struct Tile64 {
   double Ly[4][TY + 1][TX], Ry[4][TY + 1][TX];  // y-face states; Ly then the y flux
 };
 
-// one line of windows, centres p0 .. p0 + N - 1 of the values at lp[ls *]: both states of every window to
-// put(centre, qL, qR)
-template <int N, class Put>
-__device__ __forceinline__ void line64(const double *lp, int ls, int p0, bool tvd, Put put) {
+// n windows of a line, the first centred at lp[0] (stride ls): a window's left state to L[i], its right state to
+// R[i] for i < nl and i >= 1 of the line's windows i0 + 0 .. n - 1 (stride os).  The loop stays rolled: unrolled, the
+// integer multiplications overflow the instruction cache.
+__device__ __forceinline__ void line64(const double *lp, int ls, int n, double *L, double *R, int os, int i0, int nl,
+                                       bool tvd) {
+  double f3 = lp[ls];
   if (tvd) {
     // Sec. 2, the second-order TVD scheme: MUSCL with the minmod limiter
-    double f1 = lp[(p0 - 1) * ls], f2 = lp[p0 * ls];
-    for (int i = 0; i < N; i++) {
-      const double f3 = lp[(p0 + i + 1) * ls], a = f2 - f1, b = f3 - f2;
+    double f1 = lp[-ls], f2 = lp[0];
+#pragma unroll 1
+    for (int i = 0; i < n; i++) {
+      f3 = lp[(i + 1) * ls];
+      const double a = f2 - f1, b = f3 - f2;
       double m = 0.0;
       if (a > 0.0 && b > 0.0) m = a < b ? a : b;
       else if (a < 0.0 && b < 0.0) m = a > b ? a : b;
-      put(p0 + i, fma(0.5, m, f2), fma(-0.5, m, f2));
+      if (i0 + i < nl) L[(i0 + i) * os] = fma(0.5, m, f2);
+      if (i0 + i >= 1) R[(i0 + i - 1) * os] = fma(-0.5, m, f2);
       f1 = f2;
       f2 = f3;
     }
     return;
   }
   Weno64 w;
-  double f3 = lp[(p0 + 1) * ls];
-  w.start(lp[(p0 - 2) * ls], lp[(p0 - 1) * ls], lp[p0 * ls], f3);
-#pragma unroll
-  for (int i = 0; i < N; i++) {
-    const double f4 = lp[(p0 + i + 2) * ls];
+  w.start(lp[-2 * ls], lp[-ls], lp[0], f3);
+#pragma unroll 1
+  for (int i = 0; i < n; i++) {
+    const double f4 = lp[(i + 2) * ls];
     double qL, qR;
     w.next(f3, f4, qL, qR);
-    put(p0 + i, qL, qR);
+    if (i0 + i < nl) L[(i0 + i) * os] = qL;
+    if (i0 + i >= 1) R[(i0 + i - 1) * os] = qR;
     f3 = f4;
   }
 }
@@ -321,7 +324,7 @@ __device__ __forceinline__ void dual_cell64(const Consts &k, const F64Consts &c,
   const double c2 = k.gamma * pr * ir, vis = c.nud * ir;
   const double ur2 = fmin(fmax(fmax(V2, 1.0), vis * vis), c2), ic2 = rcp64(c2);
   const double mr2 = ur2 * ic2, t = 0.5 * (1.0 - mr2), Vm = sqrt64(V2), cq = sqrt64(fma(t * t, V2, ur2));
-  const double lam = fma(fma(0.5 * Vm, 1.0 + mr2, cq), c.idx + c.idy, c.dif * ir);
+  const double lam = fma(fma(half64(Vm), 1.0 + mr2, cq), c.ih[0] + c.ih[1], mul64(c.dif, ir));
   const double idtau = lam * c.icfl, s = idtau + aw;
   const double iT = rcp64(T), rT = -r * iT;
   const double th = fma(idtau, fma(iT, c.icp, rcp64(ur2)), aw * c.iR * iT);
@@ -390,92 +393,74 @@ __global__ void __launch_bounds__(TX *TY) k_stage_f64(Consts k, F64Consts c, con
       U3 = k.Uinf[3];
     }
     const double ir = rcp64(U0);
-    const double u = U1 * ir, v = U2 * ir;
-    const double p = c.g1 * fma(-0.5 * U0, fma(u, u, v * v), U3);
+    const double u = mul64(U1, ir), v = mul64(U2, ir);
+    const double p = mul64(c.g1, fma(-half64(U0), fma(u, u, mul64(v, v)), U3));
     sq[0][b][a] = U0;
     sq[1][b][a] = u;
     sq[2][b][a] = v;
     sq[3][b][a] = p;
-    sT[b][a] = p * ir * c.iR;
+    sT[b][a] = mul64(mul64(p, ir), c.iR);
   }
   __syncthreads();
 
-  // face states along lines: TX (TY) + 2 windows per row (column), in two halves of nine or one of ten
+  // face states along lines: TX (TY) + 2 windows per row (column), in two halves of nine or one of ten; one code
+  // path for both directions
   constexpr int NX = TX == 16 ? 9 : 10, HFX = TX == 16 ? 2 : 1, NY = TY == 16 ? 9 : 10, HFY = TY == 16 ? 2 : 1;
   static_assert(4 * TY * HFX + 4 * TX * HFY == NT, "one item per thread");
-  if (threadIdx.x < 4 * TY * HFX) {
-    const int u = threadIdx.x, half = u % HFX, line = u / HFX % TY, v = u / (HFX * TY);
-    line64<NX>(&sq[v][NG + line][0], 1, 2 + NX * half, k.tvd2, [&](int pc, double qL, double qR) {
-      if (pc - 2 <= TX) sm.Lx[v][line][pc - 2] = qL;  // face between pc and pc + 1
-      if (pc >= 3) sm.Rx[v][line][pc - 3] = qR;       // face between pc - 1 and pc
-    });
-  } else {
-    const int u = threadIdx.x - 4 * TY * HFX, line = u % TX, half = u / TX % HFY, v = u / (TX * HFY);
-    line64<NY>(&sq[v][0][NG + line], HX, 2 + NY * half, k.tvd2, [&](int pc, double qL, double qR) {
-      if (pc - 2 <= TY) sm.Ly[v][pc - 2][line] = qL;
-      if (pc >= 3) sm.Ry[v][pc - 3][line] = qR;
-    });
+  {
+    const bool xd = threadIdx.x < 4 * TY * HFX;
+    const int u = xd ? threadIdx.x : threadIdx.x - 4 * TY * HFX;
+    const int half = xd ? u % HFX : u / TX % HFY, line = xd ? u / HFX % TY : u % TX,
+              v = xd ? u / (HFX * TY) : u / (TX * HFY);
+    const int i0w = half * (xd ? NX : NY);
+    line64(xd ? &sq[v][NG + line][2 + i0w] : &sq[v][2 + i0w][NG + line], xd ? 1 : HX, xd ? NX : NY,
+           xd ? &sm.Lx[v][line][0] : &sm.Ly[v][0][line], xd ? &sm.Rx[v][line][0] : &sm.Ry[v][0][line], xd ? 1 : TX, i0w,
+           (xd ? TX : TY) + 1, k.tvd2);
   }
   __syncthreads();
 
-  // face fluxes: inviscid (first order where a reconstructed density or pressure is not positive) less viscous
+  // face fluxes: inviscid (first order where a reconstructed density or pressure is not positive) less viscous; d the
+  // direction, un / ut the velocity components along the normal and the tangent, sn / st the strides
   for (int m = threadIdx.x; m < (TX + 1) * TY + TX * (TY + 1); m += NT) {
-    double F[4];
-    if (m < (TX + 1) * TY) {
-      const int f = m % (TX + 1), row = m / (TX + 1), b = row + NG, a = f + 2, a1 = f + 3;
-      double qL[4], qR[4];
-      for (int v = 0; v < 4; v++) {
-        qL[v] = sm.Lx[v][row][f];
-        qR[v] = sm.Rx[v][row][f];
-      }
-      if (!positive(qL[0]) || !positive(qL[3]) || !positive(qR[0]) || !positive(qR[3])) {
-        for (int v = 0; v < 4; v++) {
-          qL[v] = sq[v][b][a];
-          qR[v] = sq[v][b][a1];
-        }
-      }
-      ldfss64<DUAL, 1>(qL[0], qL[1], &qL[2], qL[3], qR[0], qR[1], &qR[2], qR[3], k.gamma, c.ig1, c.munu2x, F);
-      const double u0 = sq[1][b][a], u1 = sq[1][b][a1], v0 = sq[2][b][a], v1 = sq[2][b][a1];
-      const double us = (sq[1][b + 1][a] - sq[1][b - 1][a]) + (sq[1][b + 1][a1] - sq[1][b - 1][a1]);
-      const double vs = (sq[2][b + 1][a] - sq[2][b - 1][a]) + (sq[2][b + 1][a1] - sq[2][b - 1][a1]);
-      const double txx = fma(c.xx, u1 - u0, -c.xy * vs), txy = fma(c.xs, us, c.xv * (v1 - v0));
-      const double w = fma(u0 + u1, txx, (v0 + v1) * txy);
-      sm.Lx[0][row][f] = F[0];
-      sm.Lx[1][row][f] = F[1] - txx;
-      sm.Lx[2][row][f] = F[2] - txy;
-      sm.Lx[3][row][f] = fma(-c.xk, sT[b][a1] - sT[b][a], fma(-0.5, w, F[3]));
-    } else {
-      const int mm = m - (TX + 1) * TY, col = mm % TX, f = mm / TX, a = col + NG, b = f + 2, b1 = f + 3;
-      double qL[4], qR[4];
-      for (int v = 0; v < 4; v++) {
-        qL[v] = sm.Ly[v][f][col];
-        qR[v] = sm.Ry[v][f][col];
-      }
-      if (!positive(qL[0]) || !positive(qL[3]) || !positive(qR[0]) || !positive(qR[3])) {
-        for (int v = 0; v < 4; v++) {
-          qL[v] = sq[v][b][a];
-          qR[v] = sq[v][b1][a];
-        }
-      }
-      // normal velocity v, tangential u
-      ldfss64<DUAL, 1>(qL[0], qL[2], &qL[1], qL[3], qR[0], qR[2], &qR[1], qR[3], k.gamma, c.ig1, c.munu2y, F);
-      const double u0 = sq[1][b][a], u1 = sq[1][b1][a], v0 = sq[2][b][a], v1 = sq[2][b1][a];
-      const double us = (sq[1][b][a + 1] - sq[1][b][a - 1]) + (sq[1][b1][a + 1] - sq[1][b1][a - 1]);
-      const double vs = (sq[2][b][a + 1] - sq[2][b][a - 1]) + (sq[2][b1][a + 1] - sq[2][b1][a - 1]);
-      const double tyy = fma(c.yy, v1 - v0, -c.yx * us), txy = fma(c.ys, vs, c.yu * (u1 - u0));
-      const double w = fma(u0 + u1, txy, (v0 + v1) * tyy);
-      sm.Ly[0][f][col] = F[0];
-      sm.Ly[1][f][col] = F[2] - txy;
-      sm.Ly[2][f][col] = F[1] - tyy;
-      sm.Ly[3][f][col] = fma(-c.yk, sT[b1][a] - sT[b][a], fma(-0.5, w, F[3]));
+    const int d = m < (TX + 1) * TY ? 0 : 1, mm = d ? m - (TX + 1) * TY : m;
+    const int f = d ? mm / TX : mm % (TX + 1), line = d ? mm % TX : mm / (TX + 1);
+    const int at = d ? (f + 2) * HX + line + NG : (line + NG) * HX + f + 2, sn = d ? HX : 1, st = d ? 1 : HX;
+    const double *q0 = &sq[0][0][0] + at, *qn = q0 + (1 + d) * HX * HY, *qt = q0 + (2 - d) * HX * HY,
+                 *q3 = q0 + 3 * HX * HY, *T = &sT[0][0] + at;
+    double *o = (d ? &sm.Ly[0][0][0] : &sm.Lx[0][0][0]) + mm;
+    const double *r = (d ? &sm.Ry[0][0][0] : &sm.Rx[0][0][0]) + mm;
+    const int vs = d ? (TY + 1) * TX : TY * (TX + 1);  // values per variable
+    double rL = o[0], uL = o[(1 + d) * vs], vL = o[(2 - d) * vs], pL = o[3 * vs];
+    double rR = r[0], uR = r[(1 + d) * vs], vR = r[(2 - d) * vs], pR = r[3 * vs];
+    if (!positive(rL) || !positive(pL) || !positive(rR) || !positive(pR)) {
+      rL = q0[0];
+      uL = qn[0];
+      vL = qt[0];
+      pL = q3[0];
+      rR = q0[sn];
+      uR = qn[sn];
+      vR = qt[sn];
+      pR = q3[sn];
     }
+    double F[4];
+    ldfss64<DUAL, 1>(rL, uL, &vL, pL, rR, uR, &vR, pR, k.gamma, c.ig1, c.munu2[d], F);
+    const double u0 = qn[0], u1 = qn[sn], v0 = qt[0], v1 = qt[sn];
+    const double us = (qn[st] - qn[-st]) + (qn[sn + st] - qn[sn - st]);
+    const double ws = (qt[st] - qt[-st]) + (qt[sn + st] - qt[sn - st]);
+    const double tn = fma(c.nn[d], u1 - u0, -mul64(c.nt[d], ws)), tt = fma(c.ts[d], us, mul64(c.tv[d], v1 - v0));
+    const double w = fma(u0 + u1, tn, mul64(v0 + v1, tt));
+    o[0] = F[0];
+    o[(1 + d) * vs] = F[1] - tn;
+    o[(2 - d) * vs] = F[2] - tt;
+    o[3 * vs] = fma(-c.kt[d], T[sn] - T[0], fma(-0.5, w, F[3]));
   }
   __syncthreads();
   if (!fluid) return;
   const long long id = cidx(k, ci, cj);
   double Rv[4];
   for (int v = 0; v < 4; v++)
-    Rv[v] = fma(sm.Lx[v][ty][tx + 1] - sm.Lx[v][ty][tx], c.idx, (sm.Ly[v][ty + 1][tx] - sm.Ly[v][ty][tx]) * c.idy);
+    Rv[v] = fma(sm.Lx[v][ty][tx + 1] - sm.Lx[v][ty][tx], c.ih[0],
+                mul64(sm.Ly[v][ty + 1][tx] - sm.Ly[v][ty][tx], c.ih[1]));
   if (DUAL) {
     dual_cell64<STAGE>(k, c, Un, In, Out, Wn, Wm, id, Rv, ds->steps > 0);
     return;
@@ -483,8 +468,8 @@ __global__ void __launch_bounds__(TX *TY) k_stage_f64(Consts k, F64Consts c, con
   for (int v = 0; v < 4; v++) {
     const long long o = id + v * P;
     if (STAGE == 1) Out[o] = fma(-dt, Rv[v], Un[o]);
-    else if (STAGE == 2) Out[o] = fma(0.75, Un[o], 0.25 * fma(-dt, Rv[v], In[o]));
-    else Out[o] = fma(1.0 / 3.0, Un[o], (2.0 / 3.0) * fma(-dt, Rv[v], In[o]));
+    else if (STAGE == 2) Out[o] = fma(0.75, Un[o], half64(half64(fma(-dt, Rv[v], In[o]))));
+    else Out[o] = fma(1.0 / 3.0, Un[o], mul64(2.0 / 3.0, fma(-dt, Rv[v], In[o])));
   }
 }
 
@@ -501,7 +486,7 @@ static void launch_tile_f64(const Consts &k, const double *Un, const double *In,
 // Tile shape by the work of the fullest SM: an SM's time is its tiles' FP64 instructions (halo cells, windows and
 // faces included: 1, 0.53 and 0.30 of the 16 x 16 tile), and the tiles are dealt evenly, so a grid of few tiles takes
 // the shape whose last round is fullest -- 257 x 131 cells are 153 tiles of 16 x 16 on 152 SMs, 289 of 16 x 8: a
-// dual-time pseudo stage there went from 374 us (16 x 16, the arithmetic before) to 77.
+// dual-time pseudo stage there went from 374 us (16 x 16, the arithmetic before) to 55.
 template <bool DUAL>
 static void launch_tiles_f64(const Consts &k, int stage, const double *Un, const double *In, double *Out,
                              const double *Wn, const double *Wm, const uint8_t *tag, DevState *ds, cudaStream_t s) {

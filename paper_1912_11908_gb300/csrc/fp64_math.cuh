@@ -9,6 +9,42 @@
 
 namespace ibm {
 
+__device__ __forceinline__ int hi64(double x) { return __double2hiint(x); }
+
+// a * b on the integer pipes.  An FP64 instruction holds its pipe for 16 cycles per warp, 64 issue slots of the SM's
+// four schedulers, which an FP64-bound kernel leaves 93% idle; this takes about 40.  The 53-bit
+// mantissas are multiplied as 64-bit integers (the partial product of the low words, below 2^-10 ulp, is left out) and
+// rounded to nearest, so the result is within 0.501 ulp of the product, equal to the hardware's but for ties.
+// Subnormal operands and results are zero; an infinite or NaN operand, or a product above the range, gives NaN.  (No
+// branch to the hardware multiplication: the compiler would issue it for every call.)
+__device__ __forceinline__ double mul64(double a, double b) {
+  const unsigned ah = __double2hiint(a), al = __double2loint(a), bh = __double2hiint(b), bl = __double2loint(b);
+  const unsigned ea = ah & 0x7ff00000u, eb = bh & 0x7ff00000u, es = ea + eb;
+  const unsigned xh = 0x80000000u | __funnelshift_l(al, ah, 11), xl = al << 11;
+  const unsigned yh = 0x80000000u | __funnelshift_l(bl, bh, 11), yl = bl << 11;
+  const unsigned long long m1 = (unsigned long long)xl * yh, m2 = (unsigned long long)xh * yl + (unsigned)m1;
+  unsigned long long P = (unsigned long long)xh * yh + (m1 >> 32) + (m2 >> 32);  // in [2^62, 2^64)
+  const bool top = (long long)P < 0;
+  if (!top) P += P;
+  const unsigned long long q = (P >> 11) + ((unsigned)P >> 10 & 1u);  // the leading one adds 1 to the exponent
+  const unsigned sign = (ah ^ bh) & 0x80000000u;
+  unsigned hi = (unsigned)(q >> 32) + (es - 0x40000000u) + (top ? 0x00100000u : 0u) + sign, lo = (unsigned)q;
+  const bool nan = max(ea, eb) >= 0x7ff00000u || es > 0xbfa00000u;  // operand not finite, or exponent above the range
+  const bool zero = min(ea, eb) == 0u || es < 0x40000000u;          // operand or product subnormal
+  if (zero) hi = sign;
+  if (nan) hi = 0x7ff80000u;
+  if (zero || nan) lo = 0u;
+  return __hiloint2double((int)hi, (int)lo);
+}
+
+// x / 2 on the integer pipe (exact; subnormal results are zero, infinities and NaN stay)
+__device__ __forceinline__ double half64(double x) {
+  const unsigned h = __double2hiint(x), e = h & 0x7ff00000u;
+  const bool tiny = e < 0x00200000u;
+  const unsigned hi = tiny ? h & 0x80000000u : e == 0x7ff00000u ? h : h - 0x00100000u;
+  return __hiloint2double((int)hi, tiny ? 0 : __double2loint(x));
+}
+
 // 1 / x for normal x
 __device__ __forceinline__ double rcp64(double x) {
   double y;
@@ -21,15 +57,13 @@ __device__ __forceinline__ double rcp64(double x) {
 __device__ __forceinline__ double rsqrt64(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-(x * y), y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);  // y (1 + e / 2 + 3 e^2 / 8)
+  const double e = fma(-mul64(x, y), y, 1.0);
+  return fma(mul64(y, e), fma(0.375, e, 0.5), y);  // y (1 + e / 2 + 3 e^2 / 8)
 }
-
-__device__ __forceinline__ int hi64(double x) { return __double2hiint(x); }
 
 // sqrt(x) for x >= 0; 0 for zero and subnormal x (squares of speeds below 1e-154), where the approximation is infinite
 __device__ __forceinline__ double sqrt64(double x) {
-  return (unsigned)hi64(x) < 0x00100000u ? 0.0 : x * rsqrt64(x);
+  return (unsigned)hi64(x) < 0x00100000u ? 0.0 : mul64(x, rsqrt64(x));
 }
 
 // |x| < 1 (exact: the biased exponent is below 1023); false for NaN
@@ -53,27 +87,27 @@ struct Weno64 {
     const double ga = f1 - f0, gb = f2 - f1, gc = f3 - f2;
     f = f2;
     g = gb;
-    hg = 0.5 * gb;
+    hg = half64(gb);
     d0 = gb - ga;
     d1 = gc - gb;
-    e0 = fma((13.0 / 12.0) * d0, d0, 1e-6);
-    e1 = fma((13.0 / 12.0) * d1, d1, 1e-6);
+    e0 = fma(mul64(13.0 / 12.0, d0), d0, 1e-6);
+    e1 = fma(mul64(13.0 / 12.0, d1), d1, 1e-6);
   }
   // the two states of the window at f, f3 and f4 the values one and two beyond it; then moves the window on
   __device__ __forceinline__ void next(double f3, double f4, double &qL, double &qR) {
-    const double g0 = f3 - f, hg0 = 0.5 * g0, d2 = (f4 - f3) - g0, e2 = fma((13.0 / 12.0) * d2, d2, 1e-6);
+    const double g0 = f3 - f, hg0 = half64(g0), d2 = (f4 - f3) - g0, e2 = fma(mul64(13.0 / 12.0, d2), d2, 1e-6);
     const double b0 = fma(0.5, d0, g), b1 = fma(0.5, d1, g), b2 = fma(0.5, d2, -g0);
     const double i0 = fma(b0, b0, e0), i1 = fma(b1, b1, e1), i2 = fma(b2, b2, e2);
-    const double t0 = i0 * i0, t1 = i1 * i1, t2 = i2 * i2;
-    const double s12 = t1 * t2, s02 = t0 * t2, s01 = t0 * t1;
+    const double t0 = mul64(i0, i0), t1 = mul64(i1, i1), t2 = mul64(i2, i2);
+    const double s12 = mul64(t1, t2), s02 = mul64(t0, t2), s01 = mul64(t0, t1);
     // left: candidates less f times (1, 6, 3), the linear weights in units of 1/10
     const double l0 = fma(1.0 / 3.0, d0, hg), l1 = fma(3.0, g0, -d1), l2 = hg0 - b2;
-    const double NL = fma(s12, l0, fma(s02, l1, s01 * l2)), DL = fma(6.0, s02, fma(3.0, s01, s12));
+    const double NL = fma(s12, l0, fma(s02, l1, mul64(s01, l2))), DL = fma(6.0, s02, fma(3.0, s01, s12));
     const double r0 = fma(1.0 / 3.0, d2, -hg0), r1 = fma(-3.0, g, -d1), r2 = -hg - b0;
-    const double NR = fma(s01, r0, fma(s02, r1, s12 * r2)), DR = fma(6.0, s02, fma(3.0, s12, s01));
-    const double inv = rcp64(DL * DR);
-    qL = fma(NL * DR, inv, f);
-    qR = fma(NR * DL, inv, f);
+    const double NR = fma(s01, r0, fma(s02, r1, mul64(s12, r2))), DR = fma(6.0, s02, fma(3.0, s12, s01));
+    const double inv = rcp64(mul64(DL, DR));
+    qL = fma(mul64(NL, DR), inv, f);
+    qR = fma(mul64(NR, DL), inv, f);
     f = f3;
     g = g0;
     hg = hg0;
@@ -93,67 +127,67 @@ template <bool PRE, int D>
 __device__ __forceinline__ void ldfss64(double rL, double unL, const double utL[D], double pL, double rR, double unR,
                                         const double utR[D], double pR, double gamma, double ig1, double munu2,
                                         double F[3 + D]) {
-  const double irr = rcp64(rL * rR), irL = irr * rR, irR = irr * rL;
-  const double c2L = gamma * pL * irL, c2R = gamma * pR * irR;
-  const double cL = c2L * rsqrt64(c2L), cR = c2R * rsqrt64(c2R);
-  double kL = unL * unL, kR = unR * unR;
+  const double irr = rcp64(mul64(rL, rR)), irL = mul64(irr, rR), irR = mul64(irr, rL);
+  const double c2L = mul64(mul64(gamma, pL), irL), c2R = mul64(mul64(gamma, pR), irR);
+  const double cL = mul64(c2L, rsqrt64(c2L)), cR = mul64(c2R, rsqrt64(c2R));
+  double kL = mul64(unL, unL), kR = mul64(unR, unR);
 #pragma unroll
   for (int d = 0; d < D; d++) {
     kL = fma(utL[d], utL[d], kL);
     kR = fma(utR[d], utR[d], kR);
   }
-  const double HL = fma(0.5, kL, c2L * ig1), HR = fma(0.5, kR, c2R * ig1);  // gamma/(gamma-1) p/rho = c^2/(gamma-1)
-  const double cb = 0.5 * (cL + cR), icb = rcp64(cb);
+  const double HL = fma(0.5, kL, mul64(c2L, ig1)), HR = fma(0.5, kR, mul64(c2R, ig1));  // gamma/(gamma-1) p/rho = c^2/(gamma-1)
+  const double cb = half64(cL + cR), icb = rcp64(cb);
   double cs = cb, ics = icb;
   bool low = false;
   if (PRE) {
-    const double ub = 0.5 * (unL + unR);
-    double v2 = ub * ub;
+    const double ub = half64(unL + unR);
+    double v2 = mul64(ub, ub);
 #pragma unroll
     for (int d = 0; d < D; d++) {
-      const double vb = 0.5 * (utL[d] + utR[d]);
+      const double vb = half64(utL[d] + utR[d]);
       v2 = fma(vb, vb, v2);
     }
-    const double rb = 0.5 * (rL + rR), rb2 = rb * rb, cb2 = cb * cb;
+    const double rb = half64(rL + rR), rb2 = mul64(rb, rb), cb2 = mul64(cb, cb);
     double ur2 = fmax(v2, 1.0);
-    if (munu2 > ur2 * rb2) ur2 = munu2 * rcp64(rb2);
+    if (munu2 > mul64(ur2, rb2)) ur2 = mul64(munu2, rcp64(rb2));
     if (ur2 < cb2) {
       low = true;
-      const double t = 0.5 * fma(-ur2 * icb, icb, 1.0) * ub;
+      const double t = mul64(half64(fma(-mul64(ur2, icb), icb, 1.0)), ub);
       const double x = fma(t, t, ur2);
       ics = rsqrt64(x);
-      cs = x * ics;
+      cs = mul64(x, ics);
     }
   }
-  const double ML = unL * ics, MR = unR * ics;
+  const double ML = mul64(unL, ics), MR = mul64(unR, ics);
   const bool subL = below_one(ML), subR = below_one(MR);
-  const double aL = ML + 1.0, aR = MR - 1.0;
-  const double MpL = 0.25 * aL * aL, MmR = -0.25 * aR * aR;
+  const double aL = half64(ML + 1.0), aR = half64(MR - 1.0);
+  const double MpL = mul64(aL, aL), MmR = -mul64(aR, aR);
   const double CL = subL ? MpL : (negative(ML) ? 0.0 : ML), CR = subR ? MmR : (negative(MR) ? MR : 0.0);
-  const double sq = sqrt64(0.5 * fma(ML, ML, MR * MR)) - 1.0;
-  const double Mh = subL && subR ? 0.25 * sq * sq : 0.0;
+  const double sq = half64(sqrt64(half64(fma(ML, ML, mul64(MR, MR)))) - 1.0);
+  const double Mh = subL && subR ? mul64(sq, sq) : 0.0;
   // only the side that the pressure falls to is weighted: M_1/2 (1 - |dp| / (rho c'^2))
   const double dp = pL - pR;
   const bool up = negative(dp);
-  const double Mw = Mh * fma(-fabs(dp), (up ? irR : irL) * (ics * ics), 1.0);
+  const double Mw = mul64(Mh, fma(-fabs(dp), mul64(up ? irR : irL, mul64(ics, ics)), 1.0));
   const double Cp = CL - (up ? Mh : Mw), Cm = CR + (up ? Mw : Mh);
   double DL, DR, ph;
   if (PRE && low) {
-    const double mL = unL * icb, mR = unR * icb, bL = mL + 1.0, bR = mR - 1.0;
-    DL = below_one(mL) ? 0.25 * bL * bL * (2.0 - mL) : (negative(mL) ? 0.0 : 1.0);
-    DR = below_one(mR) ? 0.25 * bR * bR * (2.0 + mR) : (negative(mR) ? 1.0 : 0.0);
-    ph = fma(cs * icb, fma(DL - 0.5, pL, (DR - 0.5) * pR), 0.5 * (pL + pR));
+    const double mL = mul64(unL, icb), mR = mul64(unR, icb), bL = half64(mL + 1.0), bR = half64(mR - 1.0);
+    DL = below_one(mL) ? mul64(mul64(bL, bL), 2.0 - mL) : (negative(mL) ? 0.0 : 1.0);
+    DR = below_one(mR) ? mul64(mul64(bR, bR), 2.0 + mR) : (negative(mR) ? 1.0 : 0.0);
+    ph = fma(mul64(cs, icb), fma(DL - 0.5, pL, mul64(DR - 0.5, pR)), half64(pL + pR));
   } else {
-    DL = subL ? MpL * (2.0 - ML) : (negative(ML) ? 0.0 : 1.0);
-    DR = subR ? -MmR * (2.0 + MR) : (negative(MR) ? 1.0 : 0.0);
-    ph = fma(DL, pL, DR * pR);
+    DL = subL ? mul64(MpL, 2.0 - ML) : (negative(ML) ? 0.0 : 1.0);
+    DR = subR ? -mul64(MmR, 2.0 + MR) : (negative(MR) ? 1.0 : 0.0);
+    ph = fma(DL, pL, mul64(DR, pR));
   }
-  const double mL = rL * cs * Cp, mR = rR * cs * Cm;
+  const double mL = mul64(mul64(rL, cs), Cp), mR = mul64(mul64(rR, cs), Cm);
   F[0] = mL + mR;
   F[1] = fma(mL, unL, fma(mR, unR, ph));
 #pragma unroll
-  for (int d = 0; d < D; d++) F[2 + d] = fma(mL, utL[d], mR * utR[d]);
-  F[2 + D] = fma(mL, HL, mR * HR);
+  for (int d = 0; d < D; d++) F[2 + d] = fma(mL, utL[d], mul64(mR, utR[d]));
+  F[2 + D] = fma(mL, HL, mul64(mR, HR));
 }
 
 }  // namespace ibm
