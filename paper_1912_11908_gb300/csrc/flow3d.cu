@@ -1,14 +1,14 @@
 // 3-D flow on the GPU in FP64 (Sec. 2-6 of arXiv 1912.11908 on one uniform 3-D block around a static closed
 // triangulated body): explicit SSP-RK3 steps, each stage
 //   IB nodes from their probes and the three ghost layers from their image points (Sec. 4.3-4.6, Sec. 5),
-//   domain halos, primitives, the face fluxes of the three directions (WENO5 on (rho, u, v, w, p), LDFSS(0),
-//   central viscous flux with the Stokes hypothesis; Sec. 2) and the stage update of the fluid cells,
+//   domain halos, primitives, and the residual by a sweep per direction (WENO5 on (rho, u, v, w, p), LDFSS(0),
+//   central viscous flux with the Stokes hypothesis; Sec. 2), the last with the stage update of the fluid cells,
 // and Eq. 9's force over the triangles.  Classification, tags, lists and the stencils of the listed nodes and
 // of the force probes come from the 3-D pre-processing (geometry3d.cu), once at creation (the body is static).
 //
 // Layout: structure of arrays over the cells with three halo layers, cell (i, j, k) of the (nx + 6) x (ny + 6)
-// x (nz + 6) array at ((k + 3) H + j + 3) W + i + 3; face i + 1/2 (j + 1/2, k + 1/2) of a direction is stored
-// at its lower cell.  One thread per cell, per face or per listed node.
+// x (nz + 6) array at ((k + 3) H + j + 3) W + i + 3.  One thread per cell, per window of a sweep or per corner of a
+// listed node's cube.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -17,6 +17,7 @@
 #include <cstring>
 #include <vector>
 
+#include "fp64_math.cuh"
 #include "ibm.h"
 
 extern "C" ibm_status ibm__noalloc_fail(ibm_status s, const char *msg);
@@ -27,6 +28,11 @@ ibm_status ibm__surface3d_stencils(ibm_body3d *b, const double *mn, int ntri, do
 int ibm__body3d_capacity(const ibm_body3d *b);
 
 namespace {
+
+using ibm::half64;
+using ibm::mul64;
+using ibm::rcp64;
+using ibm::sqrt64;
 
 constexpr int NG = 3;
 constexpr int TB = 256;        // threads per block of the list kernels
@@ -44,6 +50,7 @@ struct Grid3 {
 
 struct Phys3 {
   double gamma, R, mu, kappa, prandtl, cfl, pinf, dt_fixed;
+  double g1, ig1, iR, dif;  // gamma - 1, 1 / (gamma - 1), 1 / R; 2 gamma mu / Pr (1/dx^2 + 1/dy^2 + 1/dz^2)
   double Uinf[5];
 };
 
@@ -58,66 +65,15 @@ __device__ __forceinline__ long long cid(const Grid3 &g, int i, int j, int k) {
   return ((long long)(k + NG) * g.H + (j + NG)) * g.W + (i + NG);
 }
 
-// Sec. 2: WENO5 (Jiang-Shu indicators, linear weights 1/10, 6/10, 3/10, eps = 1e-6), left-biased value at the
-// face between f[2] and f[3] of f[0..4]
-__device__ __forceinline__ double weno5(double f0, double f1, double f2, double f3, double f4) {
-  const double eps = 1e-6;
-  double a = f0 - 2.0 * f1 + f2, b = f0 - 4.0 * f1 + 3.0 * f2;
-  const double b0 = (13.0 / 12.0) * a * a + 0.25 * b * b;
-  a = f1 - 2.0 * f2 + f3;
-  b = f1 - f3;
-  const double b1 = (13.0 / 12.0) * a * a + 0.25 * b * b;
-  a = f2 - 2.0 * f3 + f4;
-  b = 3.0 * f2 - 4.0 * f3 + f4;
-  const double b2 = (13.0 / 12.0) * a * a + 0.25 * b * b;
-  const double q0 = (2.0 * f0 - 7.0 * f1 + 11.0 * f2) * (1.0 / 6.0);
-  const double q1 = (-f1 + 5.0 * f2 + 2.0 * f3) * (1.0 / 6.0);
-  const double q2 = (2.0 * f2 + 5.0 * f3 - f4) * (1.0 / 6.0);
-  const double e0 = eps + b0, e1 = eps + b1, e2 = eps + b2;
-  // alpha_k = d_k / e_k^2 over a common denominator: one division
-  const double s0 = e1 * e1 * e2 * e2, s1 = e0 * e0 * e2 * e2, s2 = e0 * e0 * e1 * e1;
-  const double a0 = 0.1 * s0, a1 = 0.6 * s1, a2 = 0.3 * s2;
-  return (a0 * q0 + a1 * q1 + a2 * q2) / (a0 + a1 + a2);
-}
-
-// Sec. 2: LDFSS(0) across a face of unit normal along axis DIR (plain: Mr = 1, so c' = (c_L + c_R) / 2);
-// q = (rho, u, v, w, p)
-template <int DIR>
-__device__ __forceinline__ void ldfss(const double qL[5], const double qR[5], double gamma, double F[5]) {
-  const double rL = qL[0], pL = qL[4], rR = qR[0], pR = qR[4];
-  const double irL = 1.0 / rL, irR = 1.0 / rR;
-  const double cL = sqrt(gamma * pL * irL), cR = sqrt(gamma * pR * irR);
-  const double gg = gamma / (gamma - 1.0);
-  const double HL = gg * pL * irL + 0.5 * (qL[1] * qL[1] + qL[2] * qL[2] + qL[3] * qL[3]);
-  const double HR = gg * pR * irR + 0.5 * (qR[1] * qR[1] + qR[2] * qR[2] + qR[3] * qR[3]);
-  const double unL = qL[1 + DIR], unR = qR[1 + DIR];
-  const double cs = 0.5 * (cL + cR), ics = 1.0 / cs;
-  const double ML = unL * ics, MR = unR * ics;
-  const double aL = ML >= 0.0 ? 1.0 : 0.0, aR = MR >= 0.0 ? 0.0 : 1.0;
-  const double tL = 1.0 - floor(fabs(ML)), tR = 1.0 - floor(fabs(MR));
-  const double bL = -fmax(tL, 0.0), bR = -fmax(tR, 0.0);
-  const double MpL = 0.25 * (ML + 1.0) * (ML + 1.0);
-  const double MmR = -0.25 * (MR - 1.0) * (MR - 1.0);
-  const double CVL = aL * (1.0 + bL) * ML - bL * MpL;
-  const double CVR = aR * (1.0 + bR) * MR - bR * MmR;
-  const double sq = sqrt(0.5 * (ML * ML + MR * MR)) - 1.0;
-  const double Mh = 0.25 * bL * bR * sq * sq;
-  const double dp = pL - pR, adp = fabs(dp), ic2 = 0.5 * ics * ics;
-  const double MhP = Mh * (1.0 - (dp + adp) * ic2 * irL);
-  const double MhM = Mh * (1.0 - (-dp + adp) * ic2 * irR);
-  const double Cp = CVL - MhP, Cm = CVR + MhM;
-  const double PpL = 0.25 * (ML + 1.0) * (ML + 1.0) * (2.0 - ML);
-  const double PmR = 0.25 * (MR - 1.0) * (MR - 1.0) * (2.0 + MR);
-  const double DL = aL * (1.0 + bL) - bL * PpL;
-  const double DR = aR * (1.0 + bR) - bR * PmR;
-  const double mL = rL * cs * Cp, mR = rR * cs * Cm;
-  const double ph = DL * pL + DR * pR;
-  F[0] = mL + mR;
-  F[1] = mL * qL[1] + mR * qR[1];
-  F[2] = mL * qL[2] + mR * qR[2];
-  F[3] = mL * qL[3] + mR * qR[3];
-  F[1 + DIR] += ph;
-  F[4] = mL * HL + mR * HR;
+// primitives of one cell (products on the integer pipes: the per-cell kernels are bound by the FP64 pipe too)
+__device__ __forceinline__ void cell_prim(const Phys3 &ph, const F5 &U, long long m, double &r, double &ir, double &u,
+                                          double &v, double &w, double &p) {
+  r = U.v[0][m];
+  ir = rcp64(r);
+  u = mul64(U.v[1][m], ir);
+  v = mul64(U.v[2][m], ir);
+  w = mul64(U.v[3][m], ir);
+  p = mul64(ph.g1, fma(-half64(r), fma(u, u, fma(v, v, mul64(w, w))), U.v[4][m]));
 }
 
 // primitives (rho, u, v, w, p) and T of every cell, halos included
@@ -125,98 +81,14 @@ __global__ void __launch_bounds__(TC) k3_prim(Grid3 g, Phys3 ph, F5 U, F6 Q) {
   const int x = blockIdx.x * BX + threadIdx.x, y = blockIdx.y * BY + threadIdx.y;
   if (x >= g.W || y >= g.H) return;
   const long long m = ((long long)blockIdx.z * g.H + y) * g.W + x;
-  const double r = U.v[0][m], ir = 1.0 / r;
-  const double u = U.v[1][m] * ir, v = U.v[2][m] * ir, w = U.v[3][m] * ir;
-  const double p = (ph.gamma - 1.0) * (U.v[4][m] - 0.5 * r * (u * u + v * v + w * w));
+  double r, ir, u, v, w, p;
+  cell_prim(ph, U, m, r, ir, u, v, w, p);
   Q.v[0][m] = r;
   Q.v[1][m] = u;
   Q.v[2][m] = v;
   Q.v[3][m] = w;
   Q.v[4][m] = p;
-  Q.v[5][m] = p * ir / ph.R;
-}
-
-// face fluxes of direction DIR: inviscid (WENO5 states, first order where a density or pressure is not
-// positive; LDFSS) minus viscous (normal derivatives across the face, tangential ones from four-cell central
-// averages)
-template <int DIR>
-__global__ void __launch_bounds__(TC) k3_flux(Grid3 g, Phys3 ph, F6 Q, F5 Fo) {
-  // faces i + 1/2 (DIR 0) for i in [-1, nx - 1], likewise along y and z; one thread per face
-  int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
-  if (i >= g.nx + (DIR == 0) || j >= g.ny + (DIR == 1)) return;
-  if (DIR == 0) i -= 1;
-  if (DIR == 1) j -= 1;
-  if (DIR == 2) k -= 1;
-  const long long st = DIR == 0 ? 1 : DIR == 1 ? (long long)g.W : g.plane;
-  const long long a = cid(g, i, j, k), b = a + st;
-  double qL[5], qR[5];
-  for (int v = 0; v < 5; v++) {
-    const double *q = Q.v[v];
-    const double f0 = q[a - 2 * st], f1 = q[a - st], f2 = q[a], f3 = q[b], f4 = q[b + st], f5 = q[b + 2 * st];
-    qL[v] = weno5(f0, f1, f2, f3, f4);
-    qR[v] = weno5(f5, f4, f3, f2, f1);
-  }
-  if (!(qL[0] > 0.0) || !(qL[4] > 0.0) || !(qR[0] > 0.0) || !(qR[4] > 0.0)) {
-    for (int v = 0; v < 5; v++) {
-      qL[v] = Q.v[v][a];
-      qR[v] = Q.v[v][b];
-    }
-  }
-  double F[5];
-  ldfss<DIR>(qL, qR, ph.gamma, F);
-  if (ph.mu > 0.0) {
-    // the two tangential directions t1 < t2 and their strides and inverse spacings
-    const int t1 = DIR == 0 ? 1 : 0, t2 = DIR == 2 ? 1 : 2;
-    const long long s1 = t1 == 0 ? 1 : (long long)g.W, s2 = t2 == 1 ? (long long)g.W : g.plane;
-    const double ih[3] = {g.idx, g.idy, g.idz};
-    const double in = ih[DIR], i1 = 0.25 * ih[t1], i2 = 0.25 * ih[t2];
-    const double *T = Q.v[5];
-    double dn[3], d1[3], d2[3];  // d(u, v, w)/dn and the tangential derivatives
-    for (int c = 0; c < 3; c++) {
-      const double *q = Q.v[1 + c];
-      dn[c] = (q[b] - q[a]) * in;
-      d1[c] = (q[a + s1] - q[a - s1] + q[b + s1] - q[b - s1]) * i1;
-      d2[c] = (q[a + s2] - q[a - s2] + q[b + s2] - q[b - s2]) * i2;
-    }
-    // velocity gradient G[c][e] = d u_c / d x_e
-    double G[3][3];
-    for (int c = 0; c < 3; c++) {
-      G[c][DIR] = dn[c];
-      G[c][t1] = d1[c];
-      G[c][t2] = d2[c];
-    }
-    const double div = G[0][0] + G[1][1] + G[2][2];
-    double tau[3];  // row DIR of the viscous stress
-    for (int c = 0; c < 3; c++) tau[c] = ph.mu * (G[c][DIR] + G[DIR][c]);
-    tau[DIR] = ph.mu * (2.0 * G[DIR][DIR] - (2.0 / 3.0) * div);
-    const double qn = -ph.kappa * (T[b] - T[a]) * in;
-    double work = 0.0;
-    for (int c = 0; c < 3; c++) {
-      F[1 + c] -= tau[c];
-      work += 0.5 * (Q.v[1 + c][a] + Q.v[1 + c][b]) * tau[c];
-    }
-    F[4] -= work - qn;
-  }
-  for (int v = 0; v < 5; v++) Fo.v[v][a] = F[v];
-}
-
-// SSP-RK3 stage on the fluid cells: out = Un + dt L, 3/4 Un + 1/4 (in + dt L), 1/3 Un + 2/3 (in + dt L)
-__global__ void __launch_bounds__(TC) k3_update(Grid3 g, int stage, F5 Fx, F5 Fy, F5 Fz, F5 Un, F5 In, F5 Out,
-                                                const uint8_t *__restrict__ tags, const double *__restrict__ dtp) {
-  const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
-  if (i >= g.nx || j >= g.ny) return;
-  if (tags[((long long)k * g.ny + j) * g.nx + i] != TAG_FLUID) return;
-  const long long m = cid(g, i, j, k);
-  const double dt = *dtp;
-  for (int v = 0; v < 5; v++) {
-    const double L = -((Fx.v[v][m] - Fx.v[v][m - 1]) * g.idx + (Fy.v[v][m] - Fy.v[v][m - g.W]) * g.idy +
-                       (Fz.v[v][m] - Fz.v[v][m - g.plane]) * g.idz);
-    double o;
-    if (stage == 1) o = Un.v[v][m] + dt * L;
-    else if (stage == 2) o = 0.75 * Un.v[v][m] + 0.25 * (In.v[v][m] + dt * L);
-    else o = (1.0 / 3.0) * Un.v[v][m] + (2.0 / 3.0) * (In.v[v][m] + dt * L);
-    Out.v[v][m] = o;
-  }
+  Q.v[5][m] = mul64(mul64(p, ir), ph.iR);
 }
 
 // CFL rule: the largest (|u|+c)/dx + (|v|+c)/dy + (|w|+c)/dz + 2 gamma mu/(Pr rho)(1/dx^2 + 1/dy^2 + 1/dz^2)
@@ -227,12 +99,10 @@ __global__ void __launch_bounds__(TC) k3_lambda(Grid3 g, Phys3 ph, F5 U, const u
   double lam = 0.0;
   if (i < g.nx && j < g.ny && tags[((long long)k * g.ny + j) * g.nx + i] == TAG_FLUID) {
     const long long m = cid(g, i, j, k);
-    const double r = U.v[0][m], ir = 1.0 / r;
-    const double u = U.v[1][m] * ir, v = U.v[2][m] * ir, w = U.v[3][m] * ir;
-    const double p = (ph.gamma - 1.0) * (U.v[4][m] - 0.5 * r * (u * u + v * v + w * w));
-    const double c = sqrt(ph.gamma * ph.R * (p * ir / ph.R));
-    lam = (fabs(u) + c) * g.idx + (fabs(v) + c) * g.idy + (fabs(w) + c) * g.idz +
-          (2.0 * ph.gamma * ph.mu / (ph.prandtl * r)) * (g.idx * g.idx + g.idy * g.idy + g.idz * g.idz);
+    double r, ir, u, v, w, p;
+    cell_prim(ph, U, m, r, ir, u, v, w, p);
+    const double c = sqrt64(mul64(mul64(ph.gamma, p), ir));
+    lam = fma(fabs(u) + c, g.idx, fma(fabs(v) + c, g.idy, fma(fabs(w) + c, g.idz, mul64(ph.dif, ir))));
   }
   for (int o = 16; o > 0; o >>= 1) lam = fmax(lam, __shfl_xor_sync(0xffffffffu, lam, o));
   if ((threadIdx.x & 31) == 0 && lam > 0.0) atomicMax(lmax, (unsigned long long)__double_as_longlong(lam));
@@ -299,29 +169,28 @@ __global__ void __launch_bounds__(128) k3_reconstruct(Grid3 g, Phys3 ph, F5 U, c
   double q[5] = {0.0, 0.0, 0.0, 0.0, 0.0};  // this corner's weighted p, u, v, w, T
   if (mask >> b & 1) {
     const long long id = cid(g, sp->i0 + (b & 1), sp->j0 + (b >> 1 & 1), sp->k0 + (b >> 2));
-    const double r = U.v[0][id], ir = 1.0 / r;
-    const double u = U.v[1][id] * ir, v = U.v[2][id] * ir, w = U.v[3][id] * ir;
-    const double p = (ph.gamma - 1.0) * (U.v[4][id] - 0.5 * r * (u * u + v * v + w * w));
+    double r, ir, u, v, w, p;
+    cell_prim(ph, U, id, r, ir, u, v, w, p);
     const double wb = sp->w[b];
-    q[0] = wb * p;
-    q[1] = wb * u;
-    q[2] = wb * v;
-    q[3] = wb * w;
-    q[4] = wb * (p * ir / ph.R);
+    q[0] = mul64(wb, p);
+    q[1] = mul64(wb, u);
+    q[2] = mul64(wb, v);
+    q[3] = mul64(wb, w);
+    q[4] = mul64(wb, mul64(mul64(p, ir), ph.iR));
   }
   for (int o = 4; o > 0; o >>= 1)
     for (int v = 0; v < 5; v++) q[v] += __shfl_xor_sync(0xffffffffu, q[v], o);
   if (!live || b != 0 || mask == 0) return;
-  const double ratio = sp->xi_node / sp->xi_probe;
-  const double u = q[1] * ratio, v = q[2] * ratio, w = q[3] * ratio;
-  const double r = q[0] / (ph.R * q[4]);
+  const double ratio = mul64(sp->xi_node, rcp64(sp->xi_probe));
+  const double u = mul64(q[1], ratio), v = mul64(q[2], ratio), w = mul64(q[3], ratio);
+  const double r = mul64(q[0], mul64(ph.iR, rcp64(q[4])));
   const int node = sp->node;
   const long long id = cid(g, node % g.nx, (node / g.nx) % g.ny, node / (g.nx * g.ny));
   U.v[0][id] = r;
-  U.v[1][id] = r * u;
-  U.v[2][id] = r * v;
-  U.v[3][id] = r * w;
-  U.v[4][id] = q[0] / (ph.gamma - 1.0) + 0.5 * r * (u * u + v * v + w * w);
+  U.v[1][id] = mul64(r, u);
+  U.v[2][id] = mul64(r, v);
+  U.v[3][id] = mul64(r, w);
+  U.v[4][id] = fma(q[0], ph.ig1, mul64(half64(r), fma(u, u, fma(v, v, mul64(w, w)))));
 }
 
 // Eq. 9 per triangle (tri: area per triangle; st: its probe): (-(p_s - p_inf) n + mu (u - (u.n) n) / xi) A
@@ -387,10 +256,11 @@ __global__ void k3_step_end(const double *__restrict__ dtp, double *__restrict__
 // last stage, which accumulates its FP32 increment onto the master and refreshes the mirror from it.
 
 struct P32 {
-  float pinf, ipinf, gamma, gg, igm1, mu, kappa, ipr, u0[3], u2;  // gg = gamma / (gamma - 1), igm1 = 1 / (gamma - 1),
+  float pinf, ipinf, gamma, gg, igm1, mu, ipr, u0[3], u2;  // gg = gamma / (gamma - 1), igm1 = 1 / (gamma - 1),
                                                                    // ipr = 1 / Pr, u2 = |U_inf|^2
   float ih[3], ih2;  // inverse spacings 1/dx, 1/dy, 1/dz and 1/dx^2 + 1/dy^2 + 1/dz^2
   float Hinf;        // free-stream total enthalpy
+  float vn[3], vt[3], kq[3];  // mu / h, mu / (4 h), kappa / h per axis
 };
 
 struct F5f {
@@ -565,173 +435,11 @@ __global__ void __launch_bounds__(TB) k3_halo32(Grid3 g, F5f U) {
   }
 }
 
-__device__ __forceinline__ float weno5f(float f0, float f1, float f2, float f3, float f4) {
-  const float eps = 1e-6f;
-  float a = f0 - 2.0f * f1 + f2, b = f0 - 4.0f * f1 + 3.0f * f2;
-  const float b0 = (13.0f / 12.0f) * a * a + 0.25f * b * b;
-  a = f1 - 2.0f * f2 + f3;
-  b = f1 - f3;
-  const float b1 = (13.0f / 12.0f) * a * a + 0.25f * b * b;
-  a = f2 - 2.0f * f3 + f4;
-  b = 3.0f * f2 - 4.0f * f3 + f4;
-  const float b2 = (13.0f / 12.0f) * a * a + 0.25f * b * b;
-  const float q0 = (2.0f * f0 - 7.0f * f1 + 11.0f * f2) * (1.0f / 6.0f);
-  const float q1 = (-f1 + 5.0f * f2 + 2.0f * f3) * (1.0f / 6.0f);
-  const float q2 = (2.0f * f2 + 5.0f * f3 - f4) * (1.0f / 6.0f);
-  // alpha_k = d_k / (eps + beta_k)^2 through FP32 reciprocals (in range for beta_k up to ~1e19)
-  const float e0 = eps + b0, e1 = eps + b1, e2 = eps + b2;
-  const float i0 = __fdividef(1.0f, e0 * e0), i1 = __fdividef(1.0f, e1 * e1), i2 = __fdividef(1.0f, e2 * e2);
-  const float a0 = 0.1f * i0, a1 = 0.6f * i1, a2 = 0.3f * i2;
-  return __fdividef(a0 * q0 + a1 * q1 + a2 * q2, a0 + a1 + a2);
-}
+}  // namespace
 
-// LDFSS(0) (Mr = 1) on perturbation states q' = (rho', u', v', w', p'); F = mass, momentum less p_inf n,
-// rho u H'
-template <int DIR>
-__device__ __forceinline__ void ldfss32(const float qL[5], const float qR[5], const P32 &c, float F[5]) {
-  const float rL = 1.0f + qL[0], rR = 1.0f + qR[0];
-  const float irL = __fdividef(1.0f, rL), irR = __fdividef(1.0f, rR);
-  const float pL = c.pinf + qL[4], pR = c.pinf + qR[4];
-  const float c2L = c.gamma * pL * irL, c2R = c.gamma * pR * irR;
-  const float cL = c2L * rsqrtf(c2L), cR = c2R * rsqrtf(c2R);  // sound speeds (approximate square roots)
-  float uL[3], uR[3];
-  for (int a = 0; a < 3; a++) {
-    uL[a] = c.u0[a] + qL[1 + a];
-    uR[a] = c.u0[a] + qR[1 + a];
-  }
-  // H' = gamma/(gamma-1) (p / rho - p_inf) + (|u|^2 - |U_inf|^2) / 2
-  float kL = 0.0f, kR = 0.0f;
-  for (int a = 0; a < 3; a++) {
-    kL += qL[1 + a] * (2.0f * c.u0[a] + qL[1 + a]);
-    kR += qR[1 + a] * (2.0f * c.u0[a] + qR[1 + a]);
-  }
-  const float HL = c.gg * (qL[4] - c.pinf * qL[0]) * irL + 0.5f * kL;
-  const float HR = c.gg * (qR[4] - c.pinf * qR[0]) * irR + 0.5f * kR;
-  const float unL = uL[DIR], unR = uR[DIR];
-  const float cs = 0.5f * (cL + cR), ics = __fdividef(1.0f, cs);
-  const float ML = unL * ics, MR = unR * ics;
-  const float aL = ML >= 0.0f ? 1.0f : 0.0f, aR = MR >= 0.0f ? 0.0f : 1.0f;
-  const float bL = -fmaxf(1.0f - floorf(fabsf(ML)), 0.0f), bR = -fmaxf(1.0f - floorf(fabsf(MR)), 0.0f);
-  const float MpL = 0.25f * (ML + 1.0f) * (ML + 1.0f);
-  const float MmR = -0.25f * (MR - 1.0f) * (MR - 1.0f);
-  const float CVL = aL * (1.0f + bL) * ML - bL * MpL;
-  const float CVR = aR * (1.0f + bR) * MR - bR * MmR;
-  const float m2 = 0.5f * (ML * ML + MR * MR);
-  const float sq = (m2 > 0.0f ? m2 * rsqrtf(m2) : 0.0f) - 1.0f;
-  const float Mh = 0.25f * bL * bR * sq * sq;
-  const float dp = qL[4] - qR[4], adp = fabsf(dp), ic2 = 0.5f * ics * ics;
-  const float MhP = Mh * (1.0f - (dp + adp) * ic2 * irL);
-  const float MhM = Mh * (1.0f - (-dp + adp) * ic2 * irR);
-  const float Cp = CVL - MhP, Cm = CVR + MhM;
-  const float PpL = 0.25f * (ML + 1.0f) * (ML + 1.0f) * (2.0f - ML);
-  const float PmR = 0.25f * (MR - 1.0f) * (MR - 1.0f) * (2.0f + MR);
-  const float DL = aL * (1.0f + bL) - bL * PpL;
-  const float DR = aR * (1.0f + bR) - bR * PmR;
-  const float mL = rL * cs * Cp, mR = rR * cs * Cm;
-  const float php = c.pinf * ((DL + DR) - 1.0f) + (DL * qL[4] + DR * qR[4]);
-  F[0] = mL + mR;
-  for (int a = 0; a < 3; a++) F[1 + a] = mL * uL[a] + mR * uR[a];
-  F[1 + DIR] += php;
-  F[4] = mL * HL + mR * HR;
-}
+#include "flow3d_sweep.cuh"
 
-template <int DIR>
-__global__ void __launch_bounds__(TC) k3_flux32(Grid3 g, P32 c, F6f Q, F5f Fo) {
-  // faces i + 1/2 (DIR 0) for i in [-1, nx - 1], likewise along y and z; one thread per face
-  int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
-  if (i >= g.nx + (DIR == 0) || j >= g.ny + (DIR == 1)) return;
-  if (DIR == 0) i -= 1;
-  if (DIR == 1) j -= 1;
-  if (DIR == 2) k -= 1;
-  const long long st = DIR == 0 ? 1 : DIR == 1 ? (long long)g.W : g.plane;
-  const long long a = cid(g, i, j, k), b = a + st;
-  float qL[5], qR[5];
-  for (int v = 0; v < 5; v++) {
-    const float *q = Q.v[v];
-    const float f0 = q[a - 2 * st], f1 = q[a - st], f2 = q[a], f3 = q[b], f4 = q[b + st], f5 = q[b + 2 * st];
-    qL[v] = weno5f(f0, f1, f2, f3, f4);
-    qR[v] = weno5f(f5, f4, f3, f2, f1);
-  }
-  if (!(1.0f + qL[0] > 0.0f) || !(c.pinf + qL[4] > 0.0f) || !(1.0f + qR[0] > 0.0f) || !(c.pinf + qR[4] > 0.0f)) {
-    for (int v = 0; v < 5; v++) {
-      qL[v] = Q.v[v][a];
-      qR[v] = Q.v[v][b];
-    }
-  }
-  float F[5];
-  ldfss32<DIR>(qL, qR, c, F);
-  if (c.mu > 0.0f) {
-    const int t1 = DIR == 0 ? 1 : 0, t2 = DIR == 2 ? 1 : 2;
-    const long long s1 = t1 == 0 ? 1 : (long long)g.W, s2 = t2 == 1 ? (long long)g.W : g.plane;
-    const float in = c.ih[DIR], i1 = 0.25f * c.ih[t1], i2 = 0.25f * c.ih[t2];
-    float G[3][3];
-    for (int cc = 0; cc < 3; cc++) {
-      const float *q = Q.v[1 + cc];
-      G[cc][DIR] = (q[b] - q[a]) * in;
-      G[cc][t1] = (q[a + s1] - q[a - s1] + q[b + s1] - q[b - s1]) * i1;
-      G[cc][t2] = (q[a + s2] - q[a - s2] + q[b + s2] - q[b - s2]) * i2;
-    }
-    const float div = G[0][0] + G[1][1] + G[2][2];
-    float tau[3];
-    for (int cc = 0; cc < 3; cc++) tau[cc] = c.mu * (G[cc][DIR] + G[DIR][cc]);
-    tau[DIR] = c.mu * (2.0f * G[DIR][DIR] - (2.0f / 3.0f) * div);
-    const float qn = -c.kappa * (Q.v[5][b] - Q.v[5][a]) * in;
-    float work = 0.0f;
-    for (int cc = 0; cc < 3; cc++) {
-      F[1 + cc] -= tau[cc];
-      work += (c.u0[cc] + 0.5f * (Q.v[1 + cc][a] + Q.v[1 + cc][b])) * tau[cc];
-    }
-    F[4] -= work - qn;
-  }
-  for (int v = 0; v < 5; v++) Fo.v[v][a] = F[v];
-}
-
-// SSP-RK3 stages 1 and 2 on the fluid cells in FP32 from the flux divergence (L(rho E) = L' + H_inf L(rho)),
-// on perturbations: out = M + dt L, M + ((In - M) + dt L) / 4, with M the mirror of U^n
-__device__ __forceinline__ void flux_div32(const Grid3 &g, const P32 &c, const F5f &Fx, const F5f &Fy, const F5f &Fz,
-                                           long long m, float L[5]) {
-  const float ix = c.ih[0], iy = c.ih[1], iz = c.ih[2], Hinf = c.Hinf;
-  for (int v = 0; v < 5; v++)
-    L[v] = -((Fx.v[v][m] - Fx.v[v][m - 1]) * ix + (Fy.v[v][m] - Fy.v[v][m - g.W]) * iy +
-             (Fz.v[v][m] - Fz.v[v][m - g.plane]) * iz);
-  L[4] += Hinf * L[0];
-}
-
-__global__ void __launch_bounds__(TC) k3_update32(Grid3 g, P32 c, int stage, F5f Fx, F5f Fy, F5f Fz, F5f M,
-                                                  F5f In, F5f Out, const uint8_t *__restrict__ tags,
-                                                  const double *__restrict__ dtp) {
-  const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
-  if (i >= g.nx || j >= g.ny) return;
-  if (tags[((long long)k * g.ny + j) * g.nx + i] != TAG_FLUID) return;
-  const long long m = cid(g, i, j, k);
-  const float dt = (float)*dtp;
-  float L[5];
-  flux_div32(g, c, Fx, Fy, Fz, m, L);
-  for (int v = 0; v < 5; v++) {
-    const float mv = M.v[v][m];
-    Out.v[v][m] = stage == 1 ? mv + dt * L[v] : mv + 0.25f * ((In.v[v][m] - mv) + dt * L[v]);
-  }
-}
-
-// SSP-RK3 stage 3: the increment 2/3 ((In - M) + dt L) in FP32, accumulated onto the FP64 master, whose new
-// value refreshes the mirror
-__global__ void __launch_bounds__(TC) k3_update32_last(Grid3 g, Phys3 ph, P32 c, F5f Fx, F5f Fy, F5f Fz, F5 A,
-                                                       F5f M, F5f In, const uint8_t *__restrict__ tags,
-                                                       const double *__restrict__ dtp) {
-  const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
-  if (i >= g.nx || j >= g.ny) return;
-  if (tags[((long long)k * g.ny + j) * g.nx + i] != TAG_FLUID) return;
-  const long long m = cid(g, i, j, k);
-  const float dt = (float)*dtp;
-  float L[5];
-  flux_div32(g, c, Fx, Fy, Fz, m, L);
-  for (int v = 0; v < 5; v++) {
-    const float d = (2.0f / 3.0f) * ((In.v[v][m] - M.v[v][m]) + dt * L[v]);
-    const double a = A.v[v][m] + (double)d;
-    A.v[v][m] = a;
-    M.v[v][m] = (float)(a - ph.Uinf[v]);
-  }
-}
+namespace {
 
 inline unsigned nblk(long long n) { return (unsigned)((n + TB - 1) / TB); }
 inline dim3 cells(int ex, int ey, int ez) { return dim3((ex + BX - 1) / BX, (ey + BY - 1) / BY, ez); }
@@ -747,7 +455,7 @@ struct ibm_case3d {
   ibm_body3d *body = nullptr;
   int ntri = 0;
   char *mem = nullptr;  // one allocation for every array below
-  F5 A{}, B{}, C{}, Fx{}, Fy{}, Fz{};
+  F5 A{}, B{}, C{}, D{};          // U^n and two stages; flux divergence of the sweeps so far
   F6 Q{};
   uint8_t *tags = nullptr;        // the body's tags, or the case's own (all fluid) without a body
   uint8_t *own_tags = nullptr;
@@ -764,9 +472,11 @@ struct ibm_case3d {
   int precision = IBM_PREC_FP64;
   P32 p32{};
   double Hinf = 0.0;
-  // FP32-bulk views into the storage of the FP64 stage, primitive and flux arrays: the mirror of the master
-  // and the two intermediate stage sets (perturbations), primitives, face fluxes
-  F5f mirror{}, s1{}, s2{}, fx32{}, fy32{}, fz32{};
+  P64 p64{};
+  int rows_y = 0, rows_z = 0;     // rows of the y and z sweeps' blocks
+  // FP32-bulk views into the storage of the FP64 stage, primitive and divergence arrays: the mirror of the master
+  // and the two intermediate stage sets (perturbations), primitives, flux divergence
+  F5f mirror{}, s1{}, s2{}, d32{};
   F6f q32{};
   int64_t launches = 0;
 };
@@ -831,6 +541,10 @@ extern "C" ibm_status ibm_case3d_create(const double *verts, int nverts, const i
   ph.mu = fl->re > 0.0 ? 1.0 / fl->re : 0.0;
   ph.kappa = ph.mu * (fl->gamma * ph.R / (fl->gamma - 1.0)) / fl->prandtl;
   ph.prandtl = fl->prandtl;
+  ph.g1 = fl->gamma - 1.0;
+  ph.ig1 = 1.0 / ph.g1;
+  ph.iR = 1.0 / ph.R;
+  ph.dif = (2.0 * ph.gamma * ph.mu / ph.prandtl) * (g.idx * g.idx + g.idy * g.idy + g.idz * g.idz);
   ph.cfl = fl->cfl;
   ph.dt_fixed = fl->dt_fixed;
   const double u = fl->uinf[0], v = fl->uinf[1], w = fl->uinf[2];
@@ -853,8 +567,22 @@ extern "C" ibm_status ibm_case3d_create(const double *verts, int nverts, const i
   c->p32.gamma = (float)fl->gamma;
   c->p32.gg = (float)(fl->gamma / (fl->gamma - 1.0));
   c->p32.mu = (float)ph.mu;
-  c->p32.kappa = (float)ph.kappa;
   for (int a = 0; a < 3; a++) c->p32.u0[a] = (float)fl->uinf[a];
+  c->p64.gamma = ph.gamma;
+  c->p64.ig1 = 1.0 / (ph.gamma - 1.0);
+  c->p64.mu = ph.mu;
+  const double ih[3] = {g.idx, g.idy, g.idz};
+  for (int a = 0; a < 3; a++) {
+    c->p64.ih[a] = ih[a];
+    c->p64.vn[a] = ph.mu * ih[a];
+    c->p64.vt[a] = 0.25 * ph.mu * ih[a];
+    c->p64.kq[a] = ph.kappa * ih[a];
+    c->p32.vn[a] = (float)c->p64.vn[a];
+    c->p32.vt[a] = (float)c->p64.vt[a];
+    c->p32.kq[a] = (float)c->p64.kq[a];
+  }
+  c->rows_y = sweep_rows(g.ny);
+  c->rows_z = sweep_rows(g.nz);
   cudaError_t e = cudaSuccess;
   if (cuda_stream) {
     c->stream = (cudaStream_t)cuda_stream;
@@ -890,14 +618,14 @@ extern "C" ibm_status ibm_case3d_create(const double *verts, int nverts, const i
     }
     cap = ibm__body3d_capacity(c->body);
   }
-  // one allocation: 3 x 5 state arrays, 6 primitive arrays, 3 x 5 flux arrays, stencils, triangles, forces
+  // one allocation: 3 x 5 state arrays, 6 primitive arrays, 5 divergence arrays, stencils, triangles, forces
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t arr = up((size_t)g.ncell * sizeof(double));
   const size_t s_st = up((size_t)std::max(cap, 1) * sizeof(ibm_stencil3d));
   const size_t s_sst = up((size_t)std::max(ntris, 1) * sizeof(ibm_stencil3d));
   const size_t s_tri = up((size_t)std::max(ntris, 1) * 7 * sizeof(double));
   const size_t s_f = up(((size_t)std::max(ntris, 1) * 3 + 3) * sizeof(double));
-  const size_t total = arr * 36 + s_st + s_sst + s_tri + s_f + 256 * 4;
+  const size_t total = arr * 26 + s_st + s_sst + s_tri + s_f + 256 * 4;
   e = cudaMalloc(&c->mem, total);
   if (e != cudaSuccess) {
     ibm_case3d_destroy(c);
@@ -913,9 +641,7 @@ extern "C" ibm_status ibm_case3d_create(const double *verts, int nverts, const i
     c->A.v[v] = (double *)take(arr);
     c->B.v[v] = (double *)take(arr);
     c->C.v[v] = (double *)take(arr);
-    c->Fx.v[v] = (double *)take(arr);
-    c->Fy.v[v] = (double *)take(arr);
-    c->Fz.v[v] = (double *)take(arr);
+    c->D.v[v] = (double *)take(arr);
   }
   for (int v = 0; v < 6; v++) c->Q.v[v] = (double *)take(arr);
   c->st = (ibm_stencil3d *)take(s_st);
@@ -941,9 +667,7 @@ extern "C" ibm_status ibm_case3d_create(const double *verts, int nverts, const i
     c->mirror.v[v] = (float *)c->B.v[v];
     c->s2.v[v] = (float *)c->B.v[v] + g.ncell;
     c->s1.v[v] = (float *)c->C.v[v];
-    c->fx32.v[v] = (float *)c->Fx.v[v];
-    c->fy32.v[v] = (float *)c->Fy.v[v];
-    c->fz32.v[v] = (float *)c->Fz.v[v];
+    c->d32.v[v] = (float *)c->D.v[v];
   }
   for (int v = 0; v < 6; v++) c->q32.v[v] = (float *)c->Q.v[v];
   if (e == cudaSuccess && c->precision == IBM_PREC_FP32_BULK) {
@@ -1034,7 +758,9 @@ extern "C" ibm_status ibm_case3d_step(ibm_case3d *c, int nsteps) {
   const int nib = c->counts[0], ngh = c->counts[1] + c->counts[2] + c->counts[3];
   cudaStream_t s = c->stream;
   const bool f32 = c->precision == IBM_PREC_FP32_BULK;
-  const dim3 bx = cells(g.nx + 1, g.ny, g.nz), by = cells(g.nx, g.ny + 1, g.nz), bz = cells(g.nx, g.ny, g.nz + 1);
+  const dim3 gx((g.nx + XCELLS - 1) / XCELLS, (g.ny + BY - 1) / BY, g.nz);
+  const dim3 gy((g.nx + SLANES - 1) / SLANES, g.nz, (g.ny + c->rows_y - 3) / (c->rows_y - 2)), sy(SLANES, c->rows_y, 1);
+  const dim3 gz((g.nx + SLANES - 1) / SLANES, g.ny, (g.nz + c->rows_z - 3) / (c->rows_z - 2)), sz(SLANES, c->rows_z, 1);
   const dim3 ball = cells(g.W, g.H, g.D), bint = cells(g.nx, g.ny, g.nz);
   const unsigned bhalo = nblk(2LL * NG * ((long long)g.W * g.H + (long long)g.nz * g.W + (long long)g.nz * g.ny));
   // eight lanes per listed node (one cube corner each), 16 nodes per block
@@ -1057,16 +783,16 @@ extern "C" ibm_status ibm_case3d_step(ibm_case3d *c, int nsteps) {
         if (ngh) k3_reconstruct32<<<bgh, 128, 0, s>>>(g, ph, c->p32, in[k], c->st, nib, ngh, c->A, k == 0);
         k3_halo32<<<bhalo, TB, 0, s>>>(g, in[k]);
         k3_prim32<<<ball, CB, 0, s>>>(g, c->p32, in[k], c->q32);
-        k3_flux32<0><<<bx, CB, 0, s>>>(g, c->p32, c->q32, c->fx32);
-        k3_flux32<1><<<by, CB, 0, s>>>(g, c->p32, c->q32, c->fy32);
-        k3_flux32<2><<<bz, CB, 0, s>>>(g, c->p32, c->q32, c->fz32);
-        if (k < 2)
-          k3_update32<<<bint, CB, 0, s>>>(g, c->p32, k + 1, c->fx32, c->fy32, c->fz32, c->mirror, in[k],
-                                          k == 0 ? c->s1 : c->s2, c->tags, c->dt);
+        k3_sweep_yz<1, float><<<gy, sy, 0, s>>>(g, c->p32, c->q32, c->d32);
+        k3_sweep_yz<2, float><<<gz, sz, 0, s>>>(g, c->p32, c->q32, c->d32);
+        const F5f &out = k == 0 ? c->s1 : c->s2;  // (stage 3 writes the master and its mirror)
+        if (k == 0)
+          k3_sweep_x32<1><<<gx, CB, 0, s>>>(g, ph, c->p32, c->q32, c->d32, c->mirror, in[k], out, c->A, c->tags, c->dt);
+        else if (k == 1)
+          k3_sweep_x32<2><<<gx, CB, 0, s>>>(g, ph, c->p32, c->q32, c->d32, c->mirror, in[k], out, c->A, c->tags, c->dt);
         else
-          k3_update32_last<<<bint, CB, 0, s>>>(g, ph, c->p32, c->fx32, c->fy32, c->fz32, c->A, c->mirror,
-                                               in[k], c->tags, c->dt);
-        c->launches += 6 + (nib ? 1 : 0) + (ngh ? 1 : 0);
+          k3_sweep_x32<3><<<gx, CB, 0, s>>>(g, ph, c->p32, c->q32, c->d32, c->mirror, in[k], out, c->A, c->tags, c->dt);
+        c->launches += 5 + (nib ? 1 : 0) + (ngh ? 1 : 0);
       }
     } else {
       F5 in[3] = {c->A, c->B, c->C}, out[3] = {c->B, c->C, c->A};
@@ -1075,11 +801,12 @@ extern "C" ibm_status ibm_case3d_step(ibm_case3d *c, int nsteps) {
         if (ngh) k3_reconstruct<<<bgh, 128, 0, s>>>(g, ph, in[k], c->st, nib, ngh);
         k3_halo<<<bhalo, TB, 0, s>>>(g, ph, in[k]);
         k3_prim<<<ball, CB, 0, s>>>(g, ph, in[k], c->Q);
-        k3_flux<0><<<bx, CB, 0, s>>>(g, ph, c->Q, c->Fx);
-        k3_flux<1><<<by, CB, 0, s>>>(g, ph, c->Q, c->Fy);
-        k3_flux<2><<<bz, CB, 0, s>>>(g, ph, c->Q, c->Fz);
-        k3_update<<<bint, CB, 0, s>>>(g, k + 1, c->Fx, c->Fy, c->Fz, c->A, in[k], out[k], c->tags, c->dt);
-        c->launches += 6 + (nib ? 1 : 0) + (ngh ? 1 : 0);
+        k3_sweep_yz<1, double><<<gy, sy, 0, s>>>(g, c->p64, c->Q, c->D);
+        k3_sweep_yz<2, double><<<gz, sz, 0, s>>>(g, c->p64, c->Q, c->D);
+        if (k == 0) k3_sweep_x<1><<<gx, CB, 0, s>>>(g, c->p64, c->Q, c->D, c->A, in[k], out[k], c->tags, c->dt);
+        else if (k == 1) k3_sweep_x<2><<<gx, CB, 0, s>>>(g, c->p64, c->Q, c->D, c->A, in[k], out[k], c->tags, c->dt);
+        else k3_sweep_x<3><<<gx, CB, 0, s>>>(g, c->p64, c->Q, c->D, c->A, in[k], out[k], c->tags, c->dt);
+        c->launches += 5 + (nib ? 1 : 0) + (ngh ? 1 : 0);
       }
     }
     k3_step_end<<<1, 1, 0, s>>>(c->dt, c->time);
