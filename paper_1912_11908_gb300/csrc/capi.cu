@@ -313,6 +313,9 @@ static void init_case(ibm_case *c, const ibm_geometry *geo, const ibm_grid *gr, 
   k.Uinf[2] = fl->uinf[1];
   k.Uinf[3] = k.pinf / (k.gamma - 1.0) + 0.5 * (fl->uinf[0] * fl->uinf[0] + fl->uinf[1] * fl->uinf[1]);
   k.Hinf = k.gamma / (k.gamma - 1.0) * k.pinf + 0.5 * (fl->uinf[0] * fl->uinf[0] + fl->uinf[1] * fl->uinf[1]);
+  k.g1 = k.gamma - 1.0;
+  k.hq = k.Hinf - 0.5 * (fl->uinf[0] * fl->uinf[0] + fl->uinf[1] * fl->uinf[1]);
+  k.g1hq = k.g1 * k.hq;
   for (int s = 0; s < 4; s++) k.bc[s] = gr->bc[s];
   k.motion.kind = mo ? mo->kind : IBM_MOTION_STATIC;
   for (int d = 0; d < 2; d++) {

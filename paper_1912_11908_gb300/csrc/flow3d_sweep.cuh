@@ -1,9 +1,10 @@
 // 3-D residual by directional sweeps, FP64 and FP32-bulk (included by flow3d.cu).
 //
 // A sweep forms the face fluxes of one direction -- WENO5 states, LDFSS(0), central viscous flux (Sec. 2) -- and adds
-// their difference to the cells' flux divergence; the z sweep, the last, applies the stage update.  No face flux goes
-// to memory, and a WENO window is formed once per cell and direction: it gives the left state of the cell's upper face
-// and the right state of its lower face from shared differences.
+// their difference to the cells' flux divergence: y first, then z, then x with the stage update (its warps need no
+// block barrier, so the update's operands load while others compute).  No face flux goes to memory, and a WENO window
+// is formed once per cell and direction: it gives the left state of the cell's upper face and the right state of its
+// lower face from shared differences.
 // Lanes run along x in every sweep (coalesced); the neighbouring window's state and the neighbouring face's flux come
 //   x: by shuffles -- a warp's 32 windows give 31 faces and 30 cells;
 //   y, z: through shared memory -- a block's rows of windows give one face less and two cells less.

@@ -47,9 +47,9 @@ struct DevState {
   int pad3;
 };
 
-// IB / ghost lists up to this capacity are rebuilt by a single 1024-thread
-// block per stage (IB nodes, barrier, ghost nodes); larger lists use two
-// launches.
+// FP64: IB / ghost lists up to this capacity are rebuilt by a single cluster
+// of blocks per stage (IB nodes, cluster barrier, ghost nodes); larger lists
+// use two launches.
 constexpr int RECON_ONE_BLOCK_MAX = 1 << 16;
 
 constexpr int ERR_CAPACITY = 1;
@@ -81,6 +81,7 @@ struct Consts {
   double dt_phys;   // dual time: physical step
   double cfl_tau;   // dual time: pseudo-time CFL number
   double iR, ig1;   // 1/R and 1/(gamma - 1)
+  double g1, hq, g1hq;  // gamma - 1; H_inf - |u_inf|^2 / 2 and gamma - 1 times it
   double idt_phys;  // dual time: 1/dt_phys
   int tvd2;         // face reconstruction: TVD-2 (MUSCL, minmod) instead of WENO5
   int quad;         // IB / ghost reconstruction: quadratic along the normal (IBM_INTERP_QUADRATIC)
