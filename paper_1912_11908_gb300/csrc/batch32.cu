@@ -19,8 +19,9 @@ namespace ibm {
 // TVD / QUAD: the TVD-2 reconstruction and / or the quadratic IB / ghost reconstruction compiled in (a group
 // holds cases of one variant)
 template <int STAGE, bool TVD, bool QUAD>
-__global__ void __launch_bounds__(256, 6) k_stage_f32_batch_one(const __grid_constant__ StageBatch b) {
+__global__ void __launch_bounds__(NTH, 8) k_stage_f32_batch_one(const __grid_constant__ StageBatch b) {
   __shared__ TileSmem sm;
+  __shared__ StageCase sc;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int nbody = b.body_start[b.n], total = nbody + b.plain_start[b.n];
@@ -30,7 +31,7 @@ __global__ void __launch_bounds__(256, 6) k_stage_f32_batch_one(const __grid_con
     const int ee = body ? e : e - nbody;
     int q = 0;
     while (q + 1 < b.n && start[q + 1] <= ee) q++;
-    const StageCase &sc = b.cs[q];
+    load_case(sc, b.cs[q]);
     const float *In = STAGE == 1 ? sc.M : (STAGE == 2 ? sc.F1 : sc.F2);
     float *Out = STAGE == 1 ? sc.F1 : (STAGE == 2 ? sc.F2 : nullptr);
     if (body)
@@ -52,7 +53,7 @@ cudaError_t launch_stage_f32_batch_one(const StageBatch &b, int stage, int grid,
   if (total == 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)(grid > 0 && grid < total ? grid : total));
-  cfg.blockDim = dim3(256);
+  cfg.blockDim = dim3(NTH);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -10,7 +10,7 @@ namespace ibm {
 // Dual-time pseudo stage of one case (FP32 residual, FP64 point-implicit
 // update): plain tiles and body tiles as for the explicit stages.
 template <int STAGE, bool BODY>
-__global__ void __launch_bounds__(256) k_dual_f32(Consts k, PertConsts c, const float *__restrict__ In,
+__global__ void __launch_bounds__(NTH) k_dual_f32(Consts k, PertConsts c, const float *__restrict__ In,
                                                   float *Out32, double *D, const uint8_t *__restrict__ tag,
                                                   const int *__restrict__ sid, const RStencil32 *__restrict__ rs,
                                                   const uint8_t *__restrict__ tile_body,
@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(256) k_dual_f32(Consts k, PertConsts c, const 
 // reconstruction compiled in: body-tile slots [0, nb) first, then one block per tile (every launch form of such
 // a case)
 template <int STAGE, bool TVD, bool QUAD>
-__global__ void __launch_bounds__(256) k_dual_f32_var(Consts k, PertConsts c, const float *__restrict__ In,
+__global__ void __launch_bounds__(NTH) k_dual_f32_var(Consts k, PertConsts c, const float *__restrict__ In,
                                                       float *Out32, double *D, const uint8_t *__restrict__ tag,
                                                       const int *__restrict__ sid,
                                                       const RStencil32 *__restrict__ rs,
@@ -63,7 +63,7 @@ cudaError_t launch_dual_f32_var(const Consts &k, int stage, const float *In32, f
   dp.Q0 = Q0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)(nt + nb));
-  cfg.blockDim = dim3(256);
+  cfg.blockDim = dim3(NTH);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -93,8 +93,9 @@ cudaError_t launch_dual_f32_var(const Consts &k, int stage, const float *In32, f
 // previous pseudo stage's last blocks finish (they wait at the top for it to
 // complete).
 template <int STAGE>
-__global__ void __launch_bounds__(256, 4) k_dual_f32_batch_one(const __grid_constant__ StageBatch b) {
+__global__ void __launch_bounds__(NTH, 8) k_dual_f32_batch_one(const __grid_constant__ StageBatch b) {
   __shared__ TileSmem sm;
+  __shared__ StageCase sc;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int nbody = b.body_start[b.n], total = nbody + b.plain_start[b.n];
@@ -104,7 +105,7 @@ __global__ void __launch_bounds__(256, 4) k_dual_f32_batch_one(const __grid_cons
     const int ee = body ? e : e - nbody;
     int q = 0;
     while (q + 1 < b.n && start[q + 1] <= ee) q++;
-    const StageCase &sc = b.cs[q];
+    load_case(sc, b.cs[q]);
     const float *In = STAGE == 1 ? sc.M : (STAGE == 2 ? sc.F1 : sc.F2);
     float *Out = STAGE == 1 ? sc.F1 : (STAGE == 2 ? sc.F2 : sc.M);
     DualPtrs dp;
@@ -127,7 +128,7 @@ cudaError_t launch_dual_f32_batch_one(const StageBatch &b, int stage, int grid, 
   if (total == 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)(grid > 0 && grid < total ? grid : total));
-  cfg.blockDim = dim3(256);
+  cfg.blockDim = dim3(NTH);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -176,9 +177,9 @@ void launch_dual_f32(const Consts &k, int stage, const float *In32, float *Out32
 #define IBM_DUAL_PAIR(S)                                                                                          \
   do {                                                                                                            \
     if (nb)                                                                                                       \
-      k_dual_f32<S, true><<<nb, 256, 0, sb>>>(k, c, In32, Out32, D, tag, sid, rs, tile_body, body_tiles, ds, ncfl, \
+      k_dual_f32<S, true><<<nb, NTH, 0, sb>>>(k, c, In32, Out32, D, tag, sid, rs, tile_body, body_tiles, ds, ncfl, \
                                               dp);                                                                \
-    k_dual_f32<S, false><<<nt, 256, 0, s>>>(k, c, In32, Out32, D, tag, sid, rs, tile_body, body_tiles, ds, ncfl,   \
+    k_dual_f32<S, false><<<nt, NTH, 0, s>>>(k, c, In32, Out32, D, tag, sid, rs, tile_body, body_tiles, ds, ncfl,   \
                                             dp);                                                                  \
   } while (0)
   if (stage == 1) IBM_DUAL_PAIR(1);

@@ -109,11 +109,10 @@ void launch_compact_stencils(const Consts &k, const ibm_stencil *st, RStencil32 
 }
 
 // A case stepped on its own: one block per tile (plain) or body-tile slot.
-// MINB: resident blocks per SM the register allocation must allow (0: left to
-// the compiler, 40 registers; 5: 48 registers; 4: about 60 registers) -- the
-// autotuner picks one per grid size.
+// MINB: resident blocks per SM the register allocation must allow (8: 64 registers and the most that shared memory
+// holds; 7: 72; 6: 80) -- the autotuner picks one per grid size.
 template <int STAGE, bool BODY, int MINB>
-__global__ void __launch_bounds__(256, MINB) k_stage_f32(Consts k, PertConsts c, float *Mn, const float *__restrict__ In,
+__global__ void __launch_bounds__(NTH, MINB) k_stage_f32(Consts k, PertConsts c, float *Mn, const float *__restrict__ In,
                                                    float *Out, double *D, const uint8_t *__restrict__ tag,
                                                    const int *__restrict__ sid, const RStencil32 *__restrict__ rs,
                                                    const uint8_t *__restrict__ tile_body,
@@ -133,12 +132,14 @@ __global__ void __launch_bounds__(256, MINB) k_stage_f32(Consts k, PertConsts c,
 // grid to complete and its stores to become visible, so the next stage's
 // blocks are resident when the tail of this one ends.
 template <int STAGE, int MINB>
-__global__ void __launch_bounds__(256, MINB)
+__global__ void __launch_bounds__(NTH, MINB)
     k_stage_f32_one(Consts k, PertConsts c, float *Mn, const float *__restrict__ In, float *Out, double *D,
                     const uint8_t *__restrict__ tag, const int *__restrict__ sid, const RStencil32 *__restrict__ rs,
                     const uint8_t *__restrict__ tile_body, const int *__restrict__ body_tiles, int nb, DevState *ds,
                     bool fuse_cfl, unsigned int ncfl, const __grid_constant__ CUtensorMap tmap, int use_tma) {
   __shared__ TileSmem sm;
+  if (threadIdx.x == 0 && use_tma)  // the tensor map is a kernel parameter: on its way before the stage it waits for ends
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap) : "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int b = (int)blockIdx.x;
@@ -154,13 +155,15 @@ __global__ void __launch_bounds__(256, MINB)
 // (Sec. 4.5, Sec. 5) compiled in: a case with either takes this kernel in every launch form (the two-stream
 // form runs it as one launch on the case stream), so that the default kernels carry neither.
 template <int STAGE, bool TVD, bool QUAD>
-__global__ void __launch_bounds__(256, 6)
+__global__ void __launch_bounds__(NTH, 7)
     k_stage_f32_var(Consts k, PertConsts c, float *Mn, const float *__restrict__ In, float *Out, double *D,
                     const uint8_t *__restrict__ tag, const int *__restrict__ sid, const RStencil32 *__restrict__ rs,
                     const uint8_t *__restrict__ tile_body, const int *__restrict__ body_tiles, int nb, DevState *ds,
                     bool fuse_cfl, unsigned int ncfl, const __grid_constant__ CUtensorMap tmap, int use_tma,
                     const RStencilQ *__restrict__ rsq) {
   __shared__ TileSmem sm;
+  if (threadIdx.x == 0 && use_tma)  // the tensor map is a kernel parameter: on its way before the stage it waits for ends
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap) : "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int b = (int)blockIdx.x;
@@ -275,13 +278,13 @@ void launch_stage_f32(const Consts &k, int stage, float *Mn, const float *In, fl
 #define IBM_ARGS k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, ds, fuse_cfl, ncfl, tm, ut
 #define IBM_STAGE_PAIR(S)                                                      \
   do {                                                                         \
-    if (nb && with_body) k_stage_f32<S, true, 0><<<nb, 256, 0, sb>>>(IBM_ARGS); \
+    if (nb && with_body) k_stage_f32<S, true, 0><<<nb, NTH, 0, sb>>>(IBM_ARGS); \
     if (plain_variant == 1)                                                    \
-      k_stage_f32<S, false, 5><<<nt, 256, 0, s>>>(IBM_ARGS);                   \
+      k_stage_f32<S, false, 7><<<nt, NTH, 0, s>>>(IBM_ARGS);                   \
     else if (plain_variant == 2)                                               \
-      k_stage_f32<S, false, 4><<<nt, 256, 0, s>>>(IBM_ARGS);                   \
+      k_stage_f32<S, false, 6><<<nt, NTH, 0, s>>>(IBM_ARGS);                   \
     else                                                                       \
-      k_stage_f32<S, false, 0><<<nt, 256, 0, s>>>(IBM_ARGS);                   \
+      k_stage_f32<S, false, 8><<<nt, NTH, 0, s>>>(IBM_ARGS);                   \
   } while (0)
   if (stage == 1) IBM_STAGE_PAIR(1);
   else if (stage == 2) IBM_STAGE_PAIR(2);
@@ -305,7 +308,7 @@ cudaError_t launch_stage_f32_one(const Consts &k, int stage, float *Mn, const fl
   const int ut = tmap ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)(nt + nb));
-  cfg.blockDim = dim3(256);
+  cfg.blockDim = dim3(NTH);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -315,7 +318,7 @@ cudaError_t launch_stage_f32_one(const Consts &k, int stage, float *Mn, const fl
 #define IBM_ONE(S, MB)                                                                                        \
   cudaLaunchKernelEx(&cfg, k_stage_f32_one<S, MB>, k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, nb, \
                      ds, fuse_cfl, ncfl, tm, ut)
-#define IBM_ONE_V(S) (plain_variant == 1 ? IBM_ONE(S, 5) : plain_variant == 2 ? IBM_ONE(S, 4) : IBM_ONE(S, 6))
+#define IBM_ONE_V(S) (plain_variant == 1 ? IBM_ONE(S, 7) : plain_variant == 2 ? IBM_ONE(S, 6) : IBM_ONE(S, 8))
 #define IBM_VAR(S, T, Q)                                                                                       \
   cudaLaunchKernelEx(&cfg, k_stage_f32_var<S, T, Q>, k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, nb, \
                      ds, fuse_cfl, ncfl, tm, ut, rsq)

@@ -398,9 +398,9 @@ __host__ inline PertConsts pert_consts(const Consts &k) {
 // covers the listed body tiles and rebuilds IB and ghost nodes from rs / sid
 // while it loads a tile (no separate reconstruction launch).  plain_variant
 // selects the plain kernel's register budget, i.e. its resident blocks per SM
-// (0: compiler's choice, 40 registers, six blocks; 1: 48 registers, five
-// blocks; 2: about 60 registers, four blocks); with_body = false launches the
-// plain kernel only (autotuning).
+// (0: 64 registers, eight blocks; 1: 72 registers, seven blocks; 2: 80
+// registers, six blocks); with_body = false launches the plain kernel only
+// (autotuning).
 constexpr int PLAIN_VARIANTS = 3;
 void launch_stage_f32(const Consts &k, int stage, float *Mn, const float *In, float *Out, double *D,
                       const uint8_t *tag, const int *sid, const RStencil32 *rs, const uint8_t *tile_body,
@@ -435,7 +435,7 @@ struct StepSched {
   unsigned int pad;
   // followed by one completion count per tile
 };
-constexpr int STEP_VARIANTS = 2;  // register budget: 0 -> 40 registers (six blocks per SM), 1 -> 48 (five)
+constexpr int STEP_VARIANTS = 2;  // register budget: 0 -> 72 registers (seven blocks per SM), 1 -> 80 (six)
 size_t step_sched_bytes(const Consts &k);
 // grid of the persistent kernel: resident blocks per SM x SMs, at most 3 x tiles
 int step_f32_grid(const Consts &k, int variant);

@@ -20,6 +20,7 @@
 
 #include <cuda.h>  // CUtensorMap
 
+#include "f32x2.cuh"
 #include "dual_update.cuh"  // FP64 point-implicit update of the dual-time pseudo stages
 #include "ibm_internal.cuh"
 
@@ -37,6 +38,19 @@ __device__ __forceinline__ void pert_prim(const PertConsts &c, float dr, float d
   const float ke = 0.5f * (dr * (u * u + v * v) + dq);  // (rho |u|^2 - rho_inf |u_inf|^2) / 2
   pp = c.g1 * (W + c.Hinf * dr - ke);
   Tp = (pp - c.R * dr) * ir / c.R;
+}
+
+// the same for two cells
+__device__ __forceinline__ void pert_prim2(const PertConsts &c, f2 dr, f2 dmx, f2 dmy, f2 W, f2 &u, f2 &v, f2 &pp,
+                                           f2 &Tp) {
+  const f2 ir = rcp2(1.f + dr);
+  const f2 du = fma2(-c.ux, dr, dmx) * ir, dv = fma2(-c.uy, dr, dmy) * ir;
+  u = c.ux + du;
+  v = c.uy + dv;
+  const f2 dq = fma2(du, c.ux + u, dv * (c.uy + v));
+  const f2 ke2 = fma2(dr, fma2(u, u, v * v), dq);
+  pp = c.g1 * fma2(-0.5f, ke2, fma2(c.Hinf, dr, W));
+  Tp = (fma2(-c.R, dr, pp) * ir) * both(__fdividef(1.f, c.R));
 }
 
 // (p', u, v, T') -> perturbation conserved
@@ -62,74 +76,84 @@ __device__ __forceinline__ void prim_pert(const PertConsts &c, float pp, float u
 // scales the mass-flux (dissipation) part; the pressure split takes the
 // physical face Mach numbers and its departure from the face mean (the
 // rho c du dissipation) is scaled by c'/c, as in the FP64 path.
+//
+// Two faces at a time in packed arithmetic (f32x2.cuh); the reciprocals, square roots, extrema and selects are scalar.
 template <bool PRE = false>
-__device__ __forceinline__ void ldfss_pert(const PertConsts &c, float drL, float unL, float utL, float ppL,
-                                           float drR, float unR, float utR, float ppR, float un_inf, float ut_inf,
-                                           float F[4], float idn = 0.f) {
-  const float rL = 1.f + drL, rR = 1.f + drR;
-  const float irL = 1.f / rL, irR = 1.f / rR;
-  const float cL = sqrtf(c.gamma * (c.R + ppL) * irL), cR = sqrtf(c.gamma * (c.R + ppR) * irR);
-  const float HL = c.gg * (ppL - c.R * drL) * irL +
-                   0.5f * ((unL - un_inf) * (unL + un_inf) + (utL - ut_inf) * (utL + ut_inf));
-  const float HR = c.gg * (ppR - c.R * drR) * irR +
-                   0.5f * ((unR - un_inf) * (unR + un_inf) + (utR - ut_inf) * (utR + ut_inf));
-  const float cb = 0.5f * (cL + cR);
-  float cs = cb, mr2 = 1.f;
+__device__ __forceinline__ void ldfss_pert2(const PertConsts &c, f2 drL, f2 unL, f2 utL, f2 ppL, f2 drR, f2 unR,
+                                            f2 utR, f2 ppR, float un_inf, float ut_inf, f2 F[4], float idn = 0.f) {
+  const f2 rL = 1.f + drL, rR = 1.f + drR;
+  const f2 irL = rcp2(rL), irR = rcp2(rR);
+  const float gR = c.gamma * c.R;
+  const f2 cL = sqrt2(fma2(c.gamma, ppL, both(gR)) * irL), cR = sqrt2(fma2(c.gamma, ppR, both(gR)) * irR);
+  const f2 kL = fma2(unL - both(un_inf), un_inf + unL, (utL - both(ut_inf)) * (ut_inf + utL));
+  const f2 kR = fma2(unR - both(un_inf), un_inf + unR, (utR - both(ut_inf)) * (ut_inf + utR));
+  const f2 HL = fma2(c.gg, fma2(-c.R, drL, ppL) * irL, 0.5f * kL);
+  const f2 HR = fma2(c.gg, fma2(-c.R, drR, ppR) * irR, 0.5f * kR);
+  const f2 cb = 0.5f * (cL + cR);
+  f2 cs = cb, mr2 = both(1.f);
   if (PRE) {
-    const float ub = 0.5f * (unL + unR), vb = 0.5f * (utL + utR);
-    const float Vm = sqrtf(ub * ub + vb * vb);
-    const float rb = 0.5f * (rL + rR);
-    float Ur = fmaxf(fmaxf(Vm, 1.f), c.mu / rb * idn);
-    Ur = fminf(Ur, cb);
-    mr2 = fminf((Ur / cb) * (Ur / cb), 1.f);
-    const float om = 1.f - mr2;
-    cs = 0.5f * sqrtf(om * om * ub * ub + 4.f * mr2 * cb * cb);
+    const f2 ub = 0.5f * (unL + unR), vb = 0.5f * (utL + utR);
+    const f2 Vm = sqrt2(fma2(ub, ub, vb * vb)), nu = (c.mu * idn) * rcp2(0.5f * (rL + rR));
+    const f2 Ur = min2(max2(max2(Vm, both(1.f)), nu), cb);
+    const f2 q = Ur * rcp2(cb);
+    mr2 = min2(q * q, both(1.f));
+    const f2 om = both(1.f) - mr2, w = om * ub;
+    cs = 0.5f * sqrt2(fma2(w, w, (4.f * mr2) * (cb * cb)));
   }
-  const float ics = 1.f / cs;
-  const float ML = unL * ics, MR = unR * ics;
+  const f2 ics = rcp2(cs), ML = unL * ics, MR = unR * ics;
   // the split functions' subsonic / supersonic branches as selects: alpha = 1 (0) for M >= 0 (< 0) on the
   // left, the reverse on the right; beta = -1 subsonic, 0 supersonic
-  const bool subL = fabsf(ML) < 1.f, subR = fabsf(MR) < 1.f;
-  const float MpL = 0.25f * (ML + 1.f) * (ML + 1.f);
-  const float MmR = -0.25f * (MR - 1.f) * (MR - 1.f);
-  const float CVL = subL ? MpL : fmaxf(ML, 0.f);
-  const float CVR = subR ? MmR : fminf(MR, 0.f);
-  const float sq = sqrtf(0.5f * (ML * ML + MR * MR)) - 1.f;
-  const float Mh = subL && subR ? 0.25f * sq * sq : 0.f;
-  const float dp = ppL - ppR, adp = fabsf(dp);
-  const float ic2 = 0.5f * ics * ics;
-  const float MhP = Mh * (1.f - (dp + adp) * ic2 * irL);
-  const float MhM = Mh * (1.f - (adp - dp) * ic2 * irR);
-  const float Cp = CVL - MhP, Cm = CVR + MhM;
-  float DL, DR, Dm1;
-  if (PRE && mr2 < 1.f) {
-    // pressure split with the physical face Mach numbers
-    const float icb = 1.f / cb;
-    const float pML = unL * icb, pMR = unR * icb;
-    const bool psL = fabsf(pML) < 1.f, psR = fabsf(pMR) < 1.f;
-    const float PpL = 0.25f * (pML + 1.f) * (pML + 1.f) * (2.f - pML);
-    const float PmR = 0.25f * (pMR - 1.f) * (pMR - 1.f) * (2.f + pMR);
-    DL = psL ? PpL : (pML >= 0.f ? 1.f : 0.f);
-    DR = psR ? PmR : (pMR >= 0.f ? 0.f : 1.f);
-    Dm1 = (psL && psR) ? 0.25f * (pMR - pML) * (pMR * pMR + pMR * pML + pML * pML - 3.f) : (DL + DR - 1.f);
-  } else {
-    const float PpL = MpL * (2.f - ML);
-    const float PmR = -MmR * (2.f + MR);
-    DL = subL ? PpL : (ML >= 0.f ? 1.f : 0.f);
-    DR = subR ? PmR : (MR >= 0.f ? 0.f : 1.f);
-    Dm1 = (subL && subR) ? 0.25f * (MR - ML) * (MR * MR + MR * ML + ML * ML - 3.f) : (DL + DR - 1.f);
+  const bool sLx = fabsf(ML.x) < 1.f, sLy = fabsf(ML.y) < 1.f, sRx = fabsf(MR.x) < 1.f, sRy = fabsf(MR.y) < 1.f;
+  const f2 hL = fma2(0.5f, ML, both(0.5f)), hR = fma2(0.5f, MR, both(-0.5f));
+  const f2 MpL = hL * hL, MmR = hR * hR;  // M+ and -M-
+  const f2 CVL = {sLx ? MpL.x : fmaxf(ML.x, 0.f), sLy ? MpL.y : fmaxf(ML.y, 0.f)};
+  const f2 CVR = {sRx ? -MmR.x : fminf(MR.x, 0.f), sRy ? -MmR.y : fminf(MR.y, 0.f)};
+  const f2 mm = fma2(MR, MR, ML * ML);
+  const f2 sq = fma2(0.5f, sqrt2(0.5f * mm), both(-0.5f)), sq2 = sq * sq;
+  const f2 Mh = {sLx && sRx ? sq2.x : 0.f, sLy && sRy ? sq2.y : 0.f};
+  const f2 dp = ppL - ppR, ic2 = ics * ics;
+  // -(dp + |dp|) / 2 and -(|dp| - dp) / 2
+  const f2 dpL = {fminf(-dp.x, 0.f), fminf(-dp.y, 0.f)}, dpR = {fminf(dp.x, 0.f), fminf(dp.y, 0.f)};
+  const f2 Cp = CVL - Mh * fma2(dpL, ic2 * irL, both(1.f));
+  const f2 Cm = fma2(Mh, fma2(dpR, ic2 * irR, both(1.f)), CVR);
+  const f2 mL = rL * (cs * Cp), mR = rR * (cs * Cm);
+  // p_inf (D_L + D_R - 1) + D_L p'_L + D_R p'_R; with low-Mach scaling (pressure split with the physical face Mach
+  // numbers) the departure from the face mean 1/2 (p'_L + p'_R) is scaled by c'/c
+  f2 ph;
+  bool low_x = false, low_y = false;
+  if (PRE) low_x = mr2.x < 1.f, low_y = mr2.y < 1.f;
+  {
+    f2 m1 = ML, m2 = MR, kLs = hL, kRs = hR, q3 = mm;
+    bool pLx = sLx, pLy = sLy, pRx = sRx, pRy = sRy;
+    f2 icb = both(1.f);
+    if (PRE) {
+      icb = rcp2(cb);
+      const f2 f = {low_x ? icb.x : ics.x, low_y ? icb.y : ics.y};
+      m1 = unL * f;
+      m2 = unR * f;
+      pLx = fabsf(m1.x) < 1.f, pLy = fabsf(m1.y) < 1.f, pRx = fabsf(m2.x) < 1.f, pRy = fabsf(m2.y) < 1.f;
+      kLs = fma2(0.5f, m1, both(0.5f));
+      kRs = fma2(0.5f, m2, both(-0.5f));
+      q3 = fma2(m2, m2, m1 * m1);
+    }
+    const f2 PpL = (PRE ? kLs * kLs : MpL) * (both(2.f) - m1), PmR = (PRE ? kRs * kRs : MmR) * (2.f + m2);
+    // outside |M| < 1: 1 or 0 by the sign of M
+    const f2 DL = {pLx ? PpL.x : __saturatef(m1.x), pLy ? PpL.y : __saturatef(m1.y)};
+    const f2 DR = {pRx ? PmR.x : __saturatef(-m2.x), pRy ? PmR.y : __saturatef(-m2.y)};
+    const f2 cub = (0.25f * (m2 - m1)) * (-3.f + fma2(m2, m1, q3)), sup = -1.f + (DL + DR);
+    const f2 Dm1 = {pLx && pRx ? cub.x : sup.x, pLy && pRy ? cub.y : sup.y};
+    if (PRE) {
+      const f2 dep = fma2(c.R, Dm1, fma2(-0.5f + DL, ppL, (-0.5f + DR) * ppR)), mean = 0.5f * (ppL + ppR);
+      const f2 sc = cs * icb;
+      ph = fma2(f2{low_x ? sc.x : 1.f, low_y ? sc.y : 1.f}, dep, mean);
+    } else {
+      ph = fma2(c.R, Dm1, fma2(DL, ppL, DR * ppR));
+    }
   }
-  const float mL = rL * cs * Cp, mR = rR * cs * Cm;
-  // p_inf (D_L + D_R - 1) + D_L p'_L + D_R p'_R; with low-Mach scaling the departure from the face mean
-  // 1/2 (p'_L + p'_R) is scaled by c'/c
   F[0] = mL + mR;
-  if (PRE && mr2 < 1.f)
-    F[1] = mL * unL + mR * unR +
-           (0.5f * (ppL + ppR) + (cs / cb) * (c.R * Dm1 + (DL - 0.5f) * ppL + (DR - 0.5f) * ppR));
-  else
-    F[1] = mL * unL + mR * unR + c.R * Dm1 + DL * ppL + DR * ppR;
-  F[2] = mL * utL + mR * utR;
-  F[3] = mL * HL + mR * HR;
+  F[1] = fma2(mL, unL, fma2(mR, unR, ph));
+  F[2] = fma2(mL, utL, mR * utR);
+  F[3] = fma2(mL, HL, mR * HR);
 }
 
 // ---------------------------------------------------------------------------
@@ -137,8 +161,25 @@ __device__ __forceinline__ void ldfss_pert(const PertConsts &c, float drL, float
 // the FP64 kernel.  Stage 3 accumulates U^{n+1} in FP64 and refreshes the
 // FP32 mirror of U^{n+1}.
 // ---------------------------------------------------------------------------
+// A block is 128 threads on a 16 x 16 tile, every thread with one reconstruction item, two or three flux items of two
+// faces and two cells.  The stage was bound by issue slots (86% busy, 1303 thread instructions per cell at
+// 3072 x 1536); packed arithmetic took it to about 840.  256 threads with half of them idle in the reconstruction left
+// too few warps (3072 x 1536, four steps: 3.31 ms; scalar 3.03 ms; 128 threads, seven blocks per SM 2.95 ms).  With the
+// faces' values free of bank conflicts, the update's operands read ahead of its barrier and stores, and the lists in
+// the face storage (eight blocks of 27.5 KB per SM) it is 2.56 ms: issue slots 71% busy, FP32 pipe 57%, the rest the
+// phases' barriers.
+constexpr int NTH = 128;
 constexpr int TX = STAGE_TILE, TY = STAGE_TILE, HX = TX + 2 * NG, HY = TY + 2 * NG;
-constexpr int NFX = 4 * TY * (TX + 1), NFY = 4 * (TY + 1) * TX;  // x-face and y-face values of a tile
+// Shared memory is laid out for pairs: a thread reconstructs two adjacent rows (x direction) or columns (y direction)
+// and forms the fluxes of their two faces with packed arithmetic.  The face values of a direction are [variable][face
+// along the line][line], the two lines of a pair adjacent (8-byte accesses), the eight pairs of a face permuted by the
+// face's number (face_slot): reads and writes of a face's pairs, of two faces, and of one line along the faces (the
+// stage update) all fall in different banks.  VP is the pitch of the cell planes: with 498, the reads of
+// 8 row pairs x 2 halves x 2 variables fall in 32 banks.
+constexpr int FP = TX, NF1 = (TX + 1) * FP, NFD = 4 * NF1;  // one variable's, one direction's and side's face values
+constexpr int VP = 498;
+constexpr int CELLS = TX * TY / NTH, CROWS = NTH / TX;  // cells a thread updates, rows between them
+static_assert(CELLS == 2 && TX == TY && VP >= HY * HX && VP % 2 == 0 && HX % 2 == 0, "pairs are 8-byte aligned");
 constexpr int RB_MAX = 192;  // IB / ghost nodes a body tile's loaded region may hold
 
 // Shared memory of one tile.  face holds, in turn: the TMA box of the tile's
@@ -146,18 +187,21 @@ constexpr int RB_MAX = 192;  // IB / ghost nodes a body tile's loaded region may
 // the WENO face states, the face fluxes; each use ends behind a barrier
 // before the next begins.
 struct TileSmem {
-  alignas(128) float face[2 * (NFX + NFY)];
-  float sq[4][HY][HX];  // rho', u, v, p' of the loaded region
-  float sT[HY][HX];     // T'
+  alignas(128) float face[4 * NFD];  // x left, x right, y left, y right
+  alignas(8) float q[5][VP];         // rho', u, v, p', T' of the loaded region, HY x HX each
   unsigned long long mbar;
   unsigned int mbar_phase;  // persistent kernel: parity of the barrier's next phase (barrier initialised once)
+  // float offset of line l (a pair's first if even) of face f of a variable
+  static __device__ __forceinline__ int face_slot(int f, int l) { return f * FP + (l ^ (f & 14)); }
+  // body tiles: cell and stencil of the listed nodes, in the face storage behind the TMA box and the stencils
+  __device__ __forceinline__ int *rbm() { return reinterpret_cast<int *>(face) + RB_MAX * (int)sizeof(RStencil32) / 4; }
+  __device__ __forceinline__ int *rbe() { return rbm() + RB_MAX; }
   float wm[7];    // wall velocity and acceleration at the stage time; 1 if Eq. 7 applies (else 0); the rotation
                   // rate and its rate of change of a pitching body (else 0)
-  float lred[8];  // per-warp maxima of the CFL reduction
+  float lred[NTH / 32];  // per-warp maxima of the CFL reduction
   int nrb;        // listed IB / ghost nodes (body tiles)
-  int rbm[RB_MAX], rbe[RB_MAX];
 };
-static_assert(RB_MAX * sizeof(RStencil32) <= sizeof(float) * 2 * (NFX + NFY), "node stencils fit the face storage");
+static_assert(RB_MAX * (sizeof(RStencil32) + 2 * sizeof(int)) <= sizeof(float) * 4 * NFD, "node stencils fit the face storage");
 
 // ---------------------------------------------------------------------------
 // TMA staging of a tile (Blackwell bulk tensor copy, inline PTX).  The FP32
@@ -230,7 +274,7 @@ __device__ __forceinline__ float cfl_lambda(const Consts &k, const PertConsts &c
   return (fabsf(u) + cs) * c.idx + (fabsf(v) + cs) * c.idy + c.vis / r;
 }
 
-// block maximum of lam (all 256 threads call), then the grid-wide maximum and
+// block maximum of lam (all threads call), then the grid-wide maximum and
 // dt through the last-block pattern
 __device__ __forceinline__ void cfl_block_max(const Consts &k, float lam, float *red, DevState *ds,
                                               unsigned int nblocks, bool defer) {
@@ -239,11 +283,14 @@ __device__ __forceinline__ void cfl_block_max(const Consts &k, float lam, float 
   __syncthreads();
   if (threadIdx.x == 0) {
     float m = red[0];
-    for (int w = 1; w < 8; w++) m = fmaxf(m, red[w]);
+    for (int w = 1; w < NTH / 32; w++) m = fmaxf(m, red[w]);
     atomicMax(&ds->lmax_bits, (unsigned long long)__double_as_longlong((double)m));
     finish_cfl(k, ds, nblocks, defer);
   }
 }
+
+// cells the flux update advances: fluid cells, and IB nodes when the ghost layers alone impose the wall
+__device__ __forceinline__ bool advanced(const Consts &k, uint8_t t) { return t == FLUID || (k.ib_advance && t == IB); }
 
 // load of a value that other blocks of the same launch may have written (CG:
 // through L2, never the non-coherent read-only path)
@@ -323,10 +370,17 @@ static __device__ __noinline__ void rebuild_ib(const Consts &k, const PertConsts
                                                const RStencil32 &s, const RStencilQ *t, const float *wm,
                                                float q[4]) {
   float qp[4] = {0.f, 0.f, 0.f, 0.f};
+  float raw[4][4];  // the corners' loads in flight together (bits 0-3 of the mask: valid corners; bit 4: IB node)
+#pragma unroll
+  for (int b = 0; b < 4; b++)
+#pragma unroll
+    for (int v = 0; v < 4; v++)
+      raw[b][v] = s.mask >> b & 1 ? ld_stage<CG>(U + s.corner + (b & 1) + (b >> 1) * k.pitch + v * k.plane) : 0.f;
+#pragma unroll
   for (int b = 0; b < 4; b++) {
-    if (!(s.mask >> b & 1)) continue;  // bits 0-3: valid corners (bit 4: IB node)
+    if (!(s.mask >> b & 1)) continue;
     float cq[4];
-    raw_prim<CG>(c, U, s.corner + (b & 1) + (b >> 1) * k.pitch, k.plane, cq);
+    pert_prim(c, raw[b][0], raw[b][1], raw[b][2], raw[b][3], cq[1], cq[2], cq[0], cq[3]);
     for (int v = 0; v < 4; v++) qp[v] += s.w[b] * cq[v];
   }
   if (QUAD && t->mask) {
@@ -378,15 +432,10 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
                                            DevState *ds, bool fuse_cfl, unsigned int ncfl, int blk, TileSmem &sm,
                                            const DualPtrs &dp = DualPtrs{}, const CUtensorMap *tmap = nullptr,
                                            const RStencilQ *__restrict__ rsq = nullptr) {
-  static_assert(!TMA || 4 * HY * TMA_W <= 2 * (NFX + NFY), "TMA box must fit in the face-state storage");
+  static_assert(!TMA || 4 * HY * TMA_W <= RB_MAX * (int)sizeof(RStencil32) / 4, "TMA box ahead of the listed nodes");
   float *s_face = sm.face;
   unsigned long long &s_mbar = sm.mbar;
-  float(&sq)[4][HY][HX] = sm.sq;
-  float(&sT)[HY][HX] = sm.sT;
-  float(*fLx)[TY][TX + 1] = reinterpret_cast<float(*)[TY][TX + 1]>(s_face);  // x-face states; fLx then x flux
-  float(*fRx)[TY][TX + 1] = reinterpret_cast<float(*)[TY][TX + 1]>(s_face + NFX);
-  float(*fLy)[TY + 1][TX] = reinterpret_cast<float(*)[TY + 1][TX]>(s_face + 2 * NFX);  // y-face states; then y flux
-  float(*fRy)[TY + 1][TX] = reinterpret_cast<float(*)[TY + 1][TX]>(s_face + 2 * NFX + NFY);
+  auto sq = [&sm](int v, int b, int a) -> float & { return sm.q[v][b * HX + a]; };
   float(*s_raw)[HY][TMA_W] = reinterpret_cast<float(*)[HY][TMA_W]>(s_face);  // TMA box
   float *wm = sm.wm;
   float *lred = sm.lred;
@@ -400,7 +449,7 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
   } else if (BODY) {
     tile = blk < ds->nbody_tiles ? body_tiles[blk] : -1;
   } else {
-    tile = tile_body[blk] ? -1 : blk;
+    tile = blk;
     if (!DUAL && blk == 0 && threadIdx.x == 0) {
       if (STAGE == 1) {  // stage times for the body kernels of stages 2 and 3
         ds->tst[0] = ds->t + dtd;
@@ -411,20 +460,45 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
       }
     }
   }
-  if (tile < 0) {
+  // plain launch: a listed tile is left to its body block; its tags are on their way before the answer is known
+  const bool listed = !PERSIST && !BODY && tile_body[blk];
+  if (BODY && tile < 0) {
     if (STAGE == 3 && fuse_cfl && threadIdx.x == 0) finish_cfl(k, ds, ncfl, PERSIST);
     return;
   }
   const int i0 = (tile % ntx) * TX, j0 = (tile / ntx) * TY;
-  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
-  const int ci = i0 + tx, cj = j0 + ty;
-  const bool inside = ci < k.nx && cj < k.ny;
-  const uint8_t mytag = inside ? tag[cj * k.nx + ci] : (uint8_t)SOLID;
-  // cells the flux update advances: fluid cells, and IB nodes when the ghost layers alone impose the wall
-  const bool fluid = mytag == FLUID || (k.ib_advance && mytag == IB);
-  // stages 1 and 3 also keep the IB / ghost nodes of U^n current; stage 2 only needs fluid cells
-  const bool work = STAGE == 2 ? fluid : (mytag != SOLID);
+  const int tx = threadIdx.x % TX, ty0 = threadIdx.x / TX;  // the thread's cells: rows ty0, ty0 + CROWS, ...
+  uint8_t tags[CELLS];
+  bool work = false;
+#pragma unroll
+  for (int h = 0; h < CELLS; h++) {
+    const int ci = i0 + tx, cj = j0 + ty0 + h * CROWS;
+    tags[h] = ci < k.nx && cj < k.ny ? tag[cj * k.nx + ci] : (uint8_t)SOLID;
+    // stages 1 and 3 also keep the IB / ghost nodes of U^n current; stage 2 only needs the cells it advances
+    work |= STAGE == 2 ? advanced(k, tags[h]) : tags[h] != SOLID;
+  }
+  // interior tile (the loaded region needs no domain mapping): one tensor copy stages it,
+  // issued before the tags are read
+  const bool interior = i0 >= NG && j0 >= NG && i0 + TX + NG <= k.nx && j0 + TY + NG <= k.ny;
+  const bool tma = TMA && tmap != nullptr && interior;
+  if (listed) {
+    if (STAGE == 3 && fuse_cfl && threadIdx.x == 0) finish_cfl(k, ds, ncfl, PERSIST);
+    return;
+  }
+  if (TMA && tma && threadIdx.x == 0) {
+    if (PERSIST) {
+      // the box may hold values other blocks of this launch wrote: order the tensor copy after them
+      asm volatile("fence.proxy.async.global;" ::: "memory");
+    } else {
+      tma_init(&s_mbar);
+    }
+    tma_load(s_face, tmap, i0, j0, &s_mbar);
+  }
   if (!__syncthreads_or(work)) {
+    if (TMA && tma && threadIdx.x == 0) {  // the copy on its way still writes the box
+      if (!tma_wait(&s_mbar, PERSIST ? sm.mbar_phase : 0u)) atomicOr(&ds->err, ERR_TIMEOUT);
+      if (PERSIST) sm.mbar_phase ^= 1u;
+    }
     if (STAGE == 3 && fuse_cfl && threadIdx.x == 0) finish_cfl(k, ds, ncfl, PERSIST);
     return;
   }
@@ -458,16 +532,16 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
     wm[5] = (float)om;
     wm[6] = (float)al;
   }
-  // interior tile (the loaded region needs no domain mapping): one tensor copy stages it
-  const bool tma = TMA && tmap != nullptr && i0 >= NG && j0 >= NG && i0 + TX + NG <= k.nx && j0 + TY + NG <= k.ny;
-  if (TMA && tma && threadIdx.x == 0) {
-    if (PERSIST) {
-      // the box may hold values other blocks of this launch wrote: order the tensor copy after them
-      asm volatile("fence.proxy.async.global;" ::: "memory");
-    } else {
-      tma_init(&s_mbar);
+  // body tiles: the listed nodes of the thread's cells, on their way while the copy is
+  int esid[(HX * HY / 2 + NTH - 1) / NTH][2];
+  if (BODY && interior) {
+#pragma unroll
+    for (int r = 0; r < (HX * HY / 2 + NTH - 1) / NTH; r++) {
+      const int m = min((int)threadIdx.x + r * NTH, HX * HY / 2 - 1), b = m / (HX / 2), a = 2 * (m - b * (HX / 2));
+      const int *ps = sid + (j0 - NG + b) * k.nx + i0 - NG + a;
+      esid[r][0] = ps[0];
+      esid[r][1] = ps[1];
     }
-    tma_load(s_face, tmap, i0, j0, &s_mbar);
   }
   __syncthreads();
   if (TMA && tma) {
@@ -489,66 +563,90 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
   // body tiles: every IB / ghost node of the loaded region, with its stencil staged in shared memory (in the
   // face storage, after the TMA box has been consumed)
   int &s_nrb = sm.nrb;
-  int *s_rbm = sm.rbm, *s_rbe = sm.rbe;
+  int *s_rbm = sm.rbm(), *s_rbe = sm.rbe();
   RStencil32 *s_rs = reinterpret_cast<RStencil32 *>(s_face);
   if (BODY && threadIdx.x == 0) s_nrb = 0;
   if (BODY) __syncthreads();
-  for (int m = threadIdx.x; m < HX * HY; m += 256) {
-    const int a = m % HX, b = m / HX;
-    int gi = i0 - NG + a, gj = j0 - NG + b;
-    float q[4] = {0.f, c.ux, c.uy, 0.f};  // (p', u, v, T'); free stream: zero perturbation
-    float dr = 0.f;
-    if (TMA && tma) {
-      float u, v, pp, Tp;
-      dr = s_raw[0][b][a];
-      pert_prim(c, dr, s_raw[1][b][a], s_raw[2][b][a], s_raw[3][b][a], u, v, pp, Tp);
-      q[0] = pp;
-      q[1] = u;
-      q[2] = v;
-      q[3] = Tp;
-      if (BODY) {
-        const int e = sid[gj * k.nx + gi];
-        if (e >= 0) {
-          const int slot = atomicAdd(&s_nrb, 1);
-          if (slot < RB_MAX) {
-            s_rbm[slot] = m;
-            s_rbe[slot] = e;
-          }
+  // a listed node of the loaded region (body tiles)
+  auto list_node = [&](int m, int e) {
+    if (e < 0) return;
+    const int slot = atomicAdd(&s_nrb, 1);
+    if (slot < RB_MAX) {
+      s_rbm[slot] = m;
+      s_rbe[slot] = e;
+    }
+  };
+  if (interior) {  // no domain mapping: two cells at a time, from the tensor copy's box or from memory
+    constexpr int NC = (HX * HY / 2 + NTH - 1) / NTH;
+#pragma unroll
+    for (int r = 0; r < NC; r++) {
+      const int m = threadIdx.x + r * NTH, b = m / (HX / 2), a = 2 * (m - b * (HX / 2));
+      if (m >= HX * HY / 2) break;
+      f2 w[4], u, v, pp, Tp;
+      if (TMA && tma) {
+        for (int q = 0; q < 4; q++) w[q] = ld2(&s_raw[q][b][a]);
+      } else {
+        const float *p = In + cidx(k, i0 - NG + a, j0 - NG + b);  // an even column of the padded row
+        for (int q = 0; q < 4; q++) {
+          const float2 t = ld_stage<PERSIST>(reinterpret_cast<const float2 *>(p + q * P));
+          w[q] = f2{t.x, t.y};
         }
       }
-    } else if (halo_map(k, gi, gj)) {
-      const long long id = cidx(k, gi, gj);
-      int e = -1;
-      if (BODY) e = sid[gj * k.nx + gi];
-      dr = ld_stage<PERSIST>(In + id);
-      raw_prim<PERSIST>(c, In, id, P, q);
-      if (BODY && e >= 0) {
-        const int slot = atomicAdd(&s_nrb, 1);
-        if (slot < RB_MAX) {
-          s_rbm[slot] = m;
-          s_rbe[slot] = e;
-        }
+      pert_prim2(c, w[0], w[1], w[2], w[3], u, v, pp, Tp);
+      float *o = &sm.q[0][b * HX + a];
+      st2(o, w[0]);
+      st2(o + VP, u);
+      st2(o + 2 * VP, v);
+      st2(o + 3 * VP, pp);
+      st2(o + 4 * VP, Tp);
+      if (BODY) {
+        list_node(b * HX + a, esid[r][0]);
+        list_node(b * HX + a + 1, esid[r][1]);
       }
     }
-    sq[0][b][a] = dr;
-    sq[1][b][a] = q[1];
-    sq[2][b][a] = q[2];
-    sq[3][b][a] = q[0];
-    sT[b][a] = q[3];
+  } else {
+    // every load of the thread's cells before the first use
+    constexpr int NC = (HX * HY + NTH - 1) / NTH;
+    float w[NC][4];
+    int e[NC];
+#pragma unroll
+    for (int r = 0; r < NC; r++) {
+      const int m = threadIdx.x + r * NTH;
+      int gi = i0 - NG + m % HX, gj = j0 - NG + m / HX;
+      const bool in = m < HX * HY && halo_map(k, gi, gj);
+      const float *p = In + cidx(k, gi, gj);
+      e[r] = BODY && in ? sid[gj * k.nx + gi] : -1;
+#pragma unroll
+      for (int q = 0; q < 4; q++) w[r][q] = in ? ld_stage<PERSIST>(p + q * P) : 0.f;  // free stream: zero perturbation
+    }
+#pragma unroll
+    for (int r = 0; r < NC; r++) {
+      const int m = threadIdx.x + r * NTH;
+      if (m >= HX * HY) break;
+      float u, v, pp, Tp;
+      pert_prim(c, w[r][0], w[r][1], w[r][2], w[r][3], u, v, pp, Tp);
+      float *o = &sm.q[0][m];
+      o[0] = w[r][0];
+      o[VP] = u;
+      o[2 * VP] = v;
+      o[3 * VP] = pp;
+      o[4 * VP] = Tp;
+      if (BODY) list_node(m, e[r]);
+    }
   }
   __syncthreads();
   // every thread has waited on this phase: the next tile's copy completes the other parity
   if (PERSIST && TMA && tma && threadIdx.x == 0) sm.mbar_phase ^= 1u;
   if (BODY) {
     const int nrb = min(s_nrb, RB_MAX);
-    for (int r = threadIdx.x; r < nrb; r += 256) s_rs[r] = rs[s_rbe[r]];
+    for (int r = threadIdx.x; r < nrb; r += NTH) s_rs[r] = rs[s_rbe[r]];
     __syncthreads();
     // rebuild the listed nodes in place: IB nodes, barrier, ghost nodes (whose image points may use IB
     // nodes); corners inside the loaded region come from shared memory
     // four lanes per node, one stencil corner each, so that corners outside the loaded region (chains of
     // dependent global loads) overlap; the node's first lane sums the corners in stencil order
     for (int pass = k.ib_advance ? 1 : 0; pass < 2; pass++) {  // IB nodes (pass 0) unless advanced
-      for (int t0 = 0; t0 < 4 * nrb; t0 += 256) {  // block-uniform: every lane takes part in the shuffles
+      for (int t0 = 0; t0 < 4 * nrb; t0 += NTH) {  // block-uniform: every lane takes part in the shuffles
         const int r = (t0 + (int)threadIdx.x) >> 2, cq = threadIdx.x & 3;
         bool node = false;
         float v4[4] = {0.f, 0.f, 0.f, 0.f};
@@ -559,10 +657,10 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
             const int cn = st.ccell + (cq & 1) + (cq >> 1) * k.nx;
             const int la = cn % k.nx - (i0 - NG), lb = cn / k.nx - (j0 - NG);
             if (la >= 0 && la < HX && lb >= 0 && lb < HY) {
-              v4[0] = sq[3][lb][la];
-              v4[1] = sq[1][lb][la];
-              v4[2] = sq[2][lb][la];
-              v4[3] = sT[lb][la];
+              v4[0] = sq(3, lb, la);
+              v4[1] = sq(1, lb, la);
+              v4[2] = sq(2, lb, la);
+              v4[3] = sq(4, lb, la);
             } else {
               // corner outside the loaded region: fluid value, or an IB node rebuilt from its own stencil
               const int e2 = pass == 1 ? sid[cn] : -1;
@@ -581,10 +679,10 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
             const int cn = tq->ccell + (cq & 1) + (cq >> 1) * k.nx;
             const int la = cn % k.nx - (i0 - NG), lb = cn / k.nx - (j0 - NG);
             if (la >= 0 && la < HX && lb >= 0 && lb < HY) {
-              v4b[0] = sq[3][lb][la];
-              v4b[1] = sq[1][lb][la];
-              v4b[2] = sq[2][lb][la];
-              v4b[3] = sT[lb][la];
+              v4b[0] = sq(3, lb, la);
+              v4b[1] = sq(1, lb, la);
+              v4b[2] = sq(2, lb, la);
+              v4b[3] = sq(4, lb, la);
             } else {
               const int e2 = pass == 1 ? sid[cn] : -1;
               if (!k.ib_advance && e2 >= 0 && (rs[e2].mask & 15))
@@ -620,11 +718,11 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
         float q[4];
         if (QUAD && tq->mask) wall_bc_quad(c, st, *tq, qp, qb, wm, q);
         else wall_bc(c, st, qp, wm, q);
-        sq[0][b][a] = (q[0] - c.R * q[3]) / (c.R * (1.f + q[3]));
-        sq[1][b][a] = q[1];
-        sq[2][b][a] = q[2];
-        sq[3][b][a] = q[0];
-        sT[b][a] = q[3];
+        sq(0, b, a) = (q[0] - c.R * q[3]) / (c.R * (1.f + q[3]));
+        sq(1, b, a) = q[1];
+        sq(2, b, a) = q[2];
+        sq(3, b, a) = q[0];
+        sq(4, b, a) = q[3];
         const bool own = a >= NG && a < NG + TX && b >= NG && b < NG + TY;
         if (own && STAGE == 1) {  // U^n on this node for output and for a node that turns fluid
           float d0, d1, d2, d3;
@@ -639,196 +737,219 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
     }
     if (threadIdx.x == 0 && s_nrb > RB_MAX) atomicOr(&ds->err, ERR_CAPACITY);
   }
-  // WENO5 (Sec. 2) along lines: an item is one variable of one interior tile row (x) or column (y) and one of
-  // its two halves -- nine consecutive window centres, local 2..10 or 11..19, the cells whose faces the tile
-  // needs.  The smoothness indicators are written with the second differences d2 and first differences g of the
+  // WENO5 (Sec. 2) along lines: an item is one variable of a pair of adjacent interior tile rows (x) or columns (y)
+  // and one of its two halves -- nine consecutive window centres, local 2..10 or 11..19, the cells whose faces the
+  // tile needs.  The smoothness indicators are written with the second differences d2 and first differences g of the
   // line, beta_0 = 13/12 d2(c-1)^2 + 1/4 (d2(c-1) + 2 g(c-1))^2, beta_1 = 13/12 d2(c)^2 + 1/4 (g(c-1) + g(c))^2,
   // beta_2 = 13/12 d2(c+1)^2 + 1/4 (d2(c+1) - 2 g(c))^2 with g(j) = f(j+1) - f(j), so that each centre loads one
   // value and forms one new squared second difference, shared by three windows.  The three candidate
   // polynomials and the nonlinear weights of a window give the left state at its right face and, mirrored, the
   // right state at its left face.
-  static_assert(TX == 16 && TY == 16, "one item per thread: 2 directions x 16 lines x 4 variables x 2 halves");
-  if (TVD) {
-    // the second-order TVD scheme (Sec. 2): MUSCL with the minmod limiter over the same items; differences
-    // of perturbations equal differences of the variables, so the limiter sees what it would in absolute form
-    const int u = threadIdx.x & 127;
-    const bool xdir = threadIdx.x < 128;
-    const int half = u & 1, line = (u >> 1) & 15, v = u >> 5;
-    const float *lp = xdir ? &sq[v][NG + line][0] : &sq[v][0][NG + line];
-    const int ls = xdir ? 1 : HX;
+  // Every operation of the window is one packed instruction for both lines (40 and 4 reciprocals for 4 face states),
+  // and the results are stored as pairs.
+  static_assert(TX == 16 && TY == 16, "items: 2 directions x 4 variables x 2 halves x 8 line pairs");
+  static_assert(NTH == 128, "one item per thread");
+  {
+    const int lp = threadIdx.x & 7, half = threadIdx.x >> 3 & 1, v = threadIdx.x >> 4 & 3;
+    const bool xdir = threadIdx.x < 64;
+    const int ls = xdir ? 1 : HX, ps = xdir ? HX : 1;  // strides along the line and between the pair's lines
     const int p0 = 2 + 9 * half;
-    float f1 = lp[(p0 - 1) * ls], f2 = lp[p0 * ls];
+    const float *lp0 = &sm.q[v][xdir ? (NG + 2 * lp) * HX : NG + 2 * lp] + (p0 - 2) * ls, *lp1 = lp0 + ps;
+    // left state of face pc - 2 (between cells pc and pc + 1), right state of face pc - 3
+    // at face_slot(p0 - 2 + i, 2 lp), formed from the slot's bits: p0 - 2 = 9 half is half mod 2
+    float *const of = s_face + (xdir ? 0 : 2 * NFD) + v * NF1 + (p0 - 2) * FP;
+    const int slot0 = 2 * lp ^ 8 * half, hp = 2 * half;
+    auto store = [&](int i, f2 qL, f2 qR, float *&prev) {
+      float *const p = of + i * FP + (slot0 ^ (i & 1 ? (i & 14) + hp : i & 14));
+      if (i < 8 || half == 0) st2(p, qL);
+      if (i > 0) st2(prev + NFD, qR);
+      else if (half == 1) st2(of - FP + (2 * lp ^ 8) + NFD, qR);  // face 8
+      prev = p;
+    };
+    float *prev = nullptr;
+    if (TVD) {
+      // the second-order TVD scheme (Sec. 2): MUSCL with the minmod limiter over the same items; differences
+      // of perturbations equal differences of the variables, so the limiter sees what it would in absolute form
+      f2 f1 = {lp0[ls], lp1[ls]}, f2c = {lp0[2 * ls], lp1[2 * ls]};
+      auto minmod = [](float a, float b) {
+        float m = 0.f;
+        if (a > 0.f && b > 0.f) m = a < b ? a : b;
+        else if (a < 0.f && b < 0.f) m = a > b ? a : b;
+        return m;
+      };
 #pragma unroll
-    for (int i = 0; i < 9; i++) {
-      const int pc = p0 + i;
-      const float f3 = lp[(pc + 1) * ls];
-      const float a = f2 - f1, b = f3 - f2;
-      // minmod(a, b) for the left state at the right face, minmod(-b, -a) = -minmod(a, b) for the right state
-      float m = 0.f;
-      if (a > 0.f && b > 0.f) m = a < b ? a : b;
-      else if (a < 0.f && b < 0.f) m = a > b ? a : b;
-      const float qL = f2 + 0.5f * m, qR = f2 - 0.5f * m;
-      if (xdir) {
-        if (pc - 2 <= TX) fLx[v][line][pc - 2] = qL;
-        if (pc >= 3) fRx[v][line][pc - 3] = qR;
-      } else {
-        if (pc - 2 <= TY) fLy[v][pc - 2][line] = qL;
-        if (pc >= 3) fRy[v][pc - 3][line] = qR;
+      for (int i = 0; i < 9; i++) {
+        const f2 f3 = {lp0[(i + 3) * ls], lp1[(i + 3) * ls]};
+        const f2 a = f2c - f1, b = f3 - f2c;
+        // minmod(a, b) for the left state at the right face, minmod(-b, -a) = -minmod(a, b) for the right state
+        const f2 m = {minmod(a.x, b.x), minmod(a.y, b.y)};
+        store(i, fma2(0.5f, m, f2c), fma2(-0.5f, m, f2c), prev);
+        f1 = f2c;
+        f2c = f3;
       }
-      f1 = f2;
-      f2 = f3;
-    }
-  } else {
-    const int u = threadIdx.x & 127;
-    const bool xdir = threadIdx.x < 128;
-    const int half = u & 1, line = (u >> 1) & 15, v = u >> 5;
-    const float *lp = xdir ? &sq[v][NG + line][0] : &sq[v][0][NG + line];
-    const int ls = xdir ? 1 : HX;  // stride along the line
-    const int p0 = 2 + 9 * half;
-    // the indicators are written as e_k = eps + beta_k = [eps + 13/12 d2^2] + (b_k / 2)^2: eps rides in the
-    // sliding 13/12 d2^2 terms and the first-difference combinations are halved, so each e_k is one FMA
-    const float eps = 1e-6f;
-    float f0 = lp[(p0 - 2) * ls], f1 = lp[(p0 - 1) * ls], f2 = lp[p0 * ls], f3 = lp[(p0 + 1) * ls];
-    float d2m = f0 - 2.f * f1 + f2, d2c = f1 - 2.f * f2 + f3;  // second differences centred at c - 1 and c
-    float am = fmaf((13.f / 12.f) * d2m, d2m, eps), ac = fmaf((13.f / 12.f) * d2c, d2c, eps);
+    } else {
+      // smoothness indicators e_k = eps + beta_k = [eps + 13/12 d2^2] + (b_k / 2)^2; candidates as differences from
+      // the centre value, in x = g / 2 and y = d2 / 6: left (2 y_m + x_m, x_0 - y_c, x_0 - y_p), right (mirrored) minus
+      // (x_0 - 2 y_p, x_m + y_c, x_m + y_m), with linear weights (1/6, 1, 1/2); the nonlinear weights d_k / e_k^2
+      // cleared of their common denominator (s12 for k = 0, s02, s01)
+      const f2 eps = both(1e-6f);
+      f2 fa = {lp0[0], lp1[0]}, fb = {lp0[ls], lp1[ls]}, fc = {lp0[2 * ls], lp1[2 * ls]}, fd = {lp0[3 * ls], lp1[3 * ls]};
+      f2 gm = fc - fb, g0 = fd - fc;
+      f2 dm = gm - (fb - fa), dc = g0 - gm;  // second differences centred at c - 1 and c
+      f2 am = fma2((13.f / 12.f) * dm, dm, eps), ac = fma2((13.f / 12.f) * dc, dc, eps);
+      f2 xm = 0.5f * gm, x0 = 0.5f * g0, ym = (1.f / 6.f) * dm, yc = (1.f / 6.f) * dc;
 #pragma unroll
-    for (int i = 0; i < 9; i++) {
-      const int pc = p0 + i;
-      const float f4 = lp[(pc + 2) * ls];
-      const float d2p = f2 - 2.f * f3 + f4, ap = fmaf((13.f / 12.f) * d2p, d2p, eps);
-      const float gm = f2 - f1, g0 = f3 - f2;
-      const float hb0 = fmaf(0.5f, d2m, gm), hb1 = 0.5f * (gm + g0), hb2 = fmaf(0.5f, d2p, -g0);
-      const float e0 = fmaf(hb0, hb0, am), e1 = fmaf(hb1, hb1, ac), e2 = fmaf(hb2, hb2, ap);
-      const float e01 = e0 * e1, e12 = e1 * e2, e02 = e0 * e2;
-      const float s01 = e01 * e01, s12 = e12 * e12, s02 = e02 * e02;
-      // left state at the cell's right face: the candidates (2 f0 - 7 f1 + 11 f2, -f1 + 5 f2 + 2 f3,
-      // 2 f2 + 5 f3 - f4) / 6 with the linear weights (0.1, 0.6, 0.3) folded into their coefficients, the
-      // nonlinear weights d_k / e_k^2 cleared of their common denominator (s12 for k = 0, s02, s01)
-      const float hf2 = 0.5f * f2;
-      const float l0 = (1.f / 30.f) * f0 - (7.f / 60.f) * f1 + (11.f / 60.f) * f2;
-      const float l1 = fmaf(-0.1f, f1, fmaf(0.2f, f3, hf2));
-      const float l2 = 0.1f * f2 + 0.25f * f3 - 0.05f * f4;
-      const float qL = __fdividef(fmaf(s12, l0, fmaf(s02, l1, s01 * l2)),
-                                  fmaf(0.1f, s12, fmaf(0.6f, s02, 0.3f * s01)));
-      // right state at the cell's left face: mirrored window, indicators reversed
-      const float r0 = (1.f / 30.f) * f4 - (7.f / 60.f) * f3 + (11.f / 60.f) * f2;
-      const float r1 = fmaf(-0.1f, f3, fmaf(0.2f, f1, hf2));
-      const float r2 = 0.1f * f2 + 0.25f * f1 - 0.05f * f0;
-      const float qR = __fdividef(fmaf(s01, r0, fmaf(s02, r1, s12 * r2)),
-                                  fmaf(0.1f, s01, fmaf(0.6f, s02, 0.3f * s12)));
-      if (xdir) {
-        if (pc - 2 <= TX) fLx[v][line][pc - 2] = qL;  // face between pc and pc+1
-        if (pc >= 3) fRx[v][line][pc - 3] = qR;        // face between pc-1 and pc
-      } else {
-        if (pc - 2 <= TY) fLy[v][pc - 2][line] = qL;
-        if (pc >= 3) fRy[v][pc - 3][line] = qR;
+      for (int i = 0; i < 9; i++) {
+        const f2 fe = {lp0[(i + 4) * ls], lp1[(i + 4) * ls]};
+        const f2 g1 = fe - fd, dn = g1 - g0;
+        const f2 an = fma2((13.f / 12.f) * dn, dn, eps), yp = (1.f / 6.f) * dn;
+        const f2 b0 = fma2(0.5f, dm, gm), b1 = xm + x0, b2 = fma2(-0.5f, dn, g0);
+        const f2 e0 = fma2(b0, b0, am), e1 = fma2(b1, b1, ac), e2 = fma2(b2, b2, an);
+        const f2 e01 = e0 * e1, e12 = e1 * e2, e02 = e0 * e2;
+        const f2 s01 = e01 * e01, s12 = e12 * e12, s02 = e02 * e02;
+        const f2 a1 = (1.f / 6.f) * s12, a3 = 0.5f * s01, c1 = (1.f / 6.f) * s01, c3 = 0.5f * s12;
+        const f2 nL = fma2(a1, fma2(2.f, ym, xm), fma2(s02, x0 - yc, a3 * (x0 - yp)));
+        const f2 nR = fma2(c1, fma2(-2.f, yp, x0), fma2(s02, xm + yc, c3 * (xm + ym)));
+        const f2 qL = fma2(nL, rcp2((a1 + s02) + a3), fc), qR = fc - nR * rcp2((c1 + s02) + c3);
+        store(i, qL, qR, prev);
+        fc = fd;
+        fd = fe;
+        gm = g0;
+        g0 = g1;
+        dm = dc;
+        dc = dn;
+        am = ac;
+        ac = an;
+        xm = x0;
+        x0 = 0.5f * g1;
+        ym = yc;
+        yc = yp;
       }
-      f0 = f1;
-      f1 = f2;
-      f2 = f3;
-      f3 = f4;
-      d2m = d2c;
-      d2c = d2p;
-      am = ac;
-      ac = ap;
     }
   }
   __syncthreads();
 
   const float mu = c.mu, kap = c.kappa, idx = c.idx, idy = c.idy;
-  for (int m = threadIdx.x; m < (TX + 1) * TY + TX * (TY + 1); m += 256) {
-    const bool xdir = m < (TX + 1) * TY;
-    float qL[4], qR[4], F[4];
-    if (xdir) {
-      const int f = m % (TX + 1), row = m / (TX + 1);
-      const int b = row + NG, a = f + 2, a1 = f + 3;
+  // an item is the faces of two adjacent rows (x direction) or columns (y direction) at one place of the line
+  for (int m = threadIdx.x; m < 2 * (TX + 1) * (TX / 2); m += NTH) {
+    const bool xdir = m < (TX + 1) * (TX / 2);
+    const int mm = xdir ? m : m - (TX + 1) * (TX / 2), f = mm >> 3, l = 2 * (mm & 7);
+    float *fl = s_face + (xdir ? 0 : 2 * NFD) + sm.face_slot(f, l);  // left states, then the flux; right states NFD further
+    const int n = xdir ? 1 : 2, t = 3 - n;  // variables: velocity along the normal and the tangent
+    const float *fn = fl + n * NF1, *ft = fl + t * NF1;
+    f2 rL = ld2(fl), unL = ld2(fn), utL = ld2(ft), pL = ld2(fl + 3 * NF1);
+    f2 rR = ld2(fl + NFD), unR = ld2(fn + NFD), utR = ld2(ft + NFD), pR = ld2(fl + NFD + 3 * NF1);
+    // the first cells of the pair's faces; the second cells are ls further, the other line ps
+    const int ls = xdir ? 1 : HX, ps = xdir ? HX : 1;
+    const float *qa = &sm.q[0][xdir ? (NG + l) * HX + f + 2 : (f + 2) * HX + NG + l];
+    const float *qn = qa + n * VP, *qt = qa + t * VP, *qT = qa + 4 * VP;
+    if (!(rL.x > -1.f && rL.y > -1.f && rR.x > -1.f && rR.y > -1.f && pL.x > -c.R && pL.y > -c.R && pR.x > -c.R &&
+          pR.y > -c.R)) {  // first-order states on the faces where a density or pressure is not positive
+      if (!(rL.x > -1.f) || !(pL.x > -c.R) || !(rR.x > -1.f) || !(pR.x > -c.R)) {
+        rL.x = qa[0], unL.x = qn[0], utL.x = qt[0], pL.x = qa[3 * VP];
+        rR.x = qa[ls], unR.x = qn[ls], utR.x = qt[ls], pR.x = qa[3 * VP + ls];
+      }
+      if (!(rL.y > -1.f) || !(pL.y > -c.R) || !(rR.y > -1.f) || !(pR.y > -c.R)) {
+        rL.y = qa[ps], unL.y = qn[ps], utL.y = qt[ps], pL.y = qa[3 * VP + ps];
+        rR.y = qa[ls + ps], unR.y = qn[ls + ps], utR.y = qt[ls + ps], pR.y = qa[3 * VP + ls + ps];
+      }
+    }
+    const float idn = xdir ? idx : idy, idt = xdir ? idy : idx;
+    f2 F[4];  // mass, momentum along the normal and the tangent, energy
+    ldfss_pert2<DUAL>(c, rL, unL, utL, pL, rR, unR, utR, pR, xdir ? c.ux : c.uy, xdir ? c.uy : c.ux, F, idn);
+    // viscous part from the cells before and after the face, lines (before, first) and (second, after) of the pair:
+    // differences along the normal, sums, and differences across the lines of the two cells' sums
+    f2 dn[2], av[2], dt2[2];
+#pragma unroll
+    for (int w = 0; w < 2; w++) {
+      const float *q = w ? qt : qn;
+      f2 lo0, hi0, lo1, hi1;
+      if (xdir) {
+        lo0 = f2{q[-HX], q[0]}, hi0 = f2{q[HX], q[2 * HX]};
+        lo1 = f2{q[1 - HX], q[1]}, hi1 = f2{q[1 + HX], q[1 + 2 * HX]};
+      } else {
+        lo0 = ld2(q - 1), hi0 = ld2(q + 1), lo1 = ld2(q + HX - 1), hi1 = ld2(q + HX + 1);
+      }
+      const f2 lo = lo0 + lo1, hi = hi0 + hi1;
+      dt2[w] = hi - lo;
+      av[w] = f2{lo.y, hi.x};
+      dn[w] = f2{lo1.y, hi1.x} - f2{lo0.y, hi0.x};
+    }
+    const f2 Tn = f2{qT[ls], qT[ls + ps]} - f2{qT[0], qT[ps]};
+    const f2 tnn = fma2((4.f / 3.f) * mu * idn, dn[0], ((-1.f / 6.f) * mu * idt) * dt2[1]);
+    const f2 tnt = fma2(0.25f * mu * idt, dt2[0], (mu * idn) * dn[1]);
+    const f2 work = 0.5f * fma2(av[0], tnn, av[1] * tnt);
+    st2(fl, F[0]);
+    st2(fl + n * NF1, F[1] - tnn);
+    st2(fl + t * NF1, F[2] - tnt);
+    st2(fl + 3 * NF1, F[3] - fma2(kap * idn, Tn, work));
+  }
+  // the update's operands: read ahead of the barrier and of the stores (which may alias them), all in flight together
+  float um[CELLS][4], ui[CELLS][4];
+  double ud[CELLS][4];
+  if constexpr (!DUAL) {
+#pragma unroll
+    for (int h = 0; h < CELLS; h++) {
+      const bool adv = advanced(k, tags[h]);
+      const long long id = cidx(k, i0 + tx, j0 + ty0 + h * CROWS);
+#pragma unroll
       for (int v = 0; v < 4; v++) {
-        qL[v] = fLx[v][row][f];
-        qR[v] = fRx[v][row][f];
+        if (adv) um[h][v] = Mn[id + v * P];
+        if (STAGE >= 2 && adv) ui[h][v] = ld_stage<PERSIST>(In + id + v * P);
+        if (STAGE == 3 && (adv || (BODY && tags[h] != SOLID))) ud[h][v] = ld_stage<PERSIST>(D + id + v * P);
       }
-      if (!(qL[0] > -1.f) || !(qL[3] > -c.R) || !(qR[0] > -1.f) || !(qR[3] > -c.R)) {
-        for (int v = 0; v < 4; v++) {
-          qL[v] = sq[v][b][a];
-          qR[v] = sq[v][b][a1];
-        }
-      }
-      ldfss_pert<DUAL>(c, qL[0], qL[1], qL[2], qL[3], qR[0], qR[1], qR[2], qR[3], c.ux, c.uy, F, idx);
-      const float ux = (sq[1][b][a1] - sq[1][b][a]) * idx;
-      const float vx = (sq[2][b][a1] - sq[2][b][a]) * idx;
-      const float Tx = (sT[b][a1] - sT[b][a]) * idx;
-      const float uy = (sq[1][b + 1][a] - sq[1][b - 1][a] + sq[1][b + 1][a1] - sq[1][b - 1][a1]) * (0.25f * idy);
-      const float vy = (sq[2][b + 1][a] - sq[2][b - 1][a] + sq[2][b + 1][a1] - sq[2][b - 1][a1]) * (0.25f * idy);
-      const float txx = mu * ((4.f / 3.f) * ux - (2.f / 3.f) * vy);
-      const float txy = mu * (uy + vx);
-      const float uf = 0.5f * (sq[1][b][a] + sq[1][b][a1]), vf = 0.5f * (sq[2][b][a] + sq[2][b][a1]);
-      fLx[0][row][f] = F[0];
-      fLx[1][row][f] = F[1] - txx;
-      fLx[2][row][f] = F[2] - txy;
-      fLx[3][row][f] = F[3] - (uf * txx + vf * txy + kap * Tx);
-    } else {
-      const int mm = m - (TX + 1) * TY;
-      const int col = mm % TX, f = mm / TX;
-      const int a = col + NG, b = f + 2, b1 = f + 3;
-      for (int v = 0; v < 4; v++) {
-        qL[v] = fLy[v][f][col];
-        qR[v] = fRy[v][f][col];
-      }
-      if (!(qL[0] > -1.f) || !(qL[3] > -c.R) || !(qR[0] > -1.f) || !(qR[3] > -c.R)) {
-        for (int v = 0; v < 4; v++) {
-          qL[v] = sq[v][b][a];
-          qR[v] = sq[v][b1][a];
-        }
-      }
-      ldfss_pert<DUAL>(c, qL[0], qL[2], qL[1], qL[3], qR[0], qR[2], qR[1], qR[3], c.uy, c.ux, F, idy);
-      const float uy = (sq[1][b1][a] - sq[1][b][a]) * idy;
-      const float vy = (sq[2][b1][a] - sq[2][b][a]) * idy;
-      const float Ty = (sT[b1][a] - sT[b][a]) * idy;
-      const float ux = (sq[1][b][a + 1] - sq[1][b][a - 1] + sq[1][b1][a + 1] - sq[1][b1][a - 1]) * (0.25f * idx);
-      const float vx = (sq[2][b][a + 1] - sq[2][b][a - 1] + sq[2][b1][a + 1] - sq[2][b1][a - 1]) * (0.25f * idx);
-      const float tyy = mu * ((4.f / 3.f) * vy - (2.f / 3.f) * ux);
-      const float txy = mu * (uy + vx);
-      const float uf = 0.5f * (sq[1][b][a] + sq[1][b1][a]), vf = 0.5f * (sq[2][b][a] + sq[2][b1][a]);
-      fLy[0][f][col] = F[0];
-      fLy[1][f][col] = F[2] - txy;
-      fLy[2][f][col] = F[1] - tyy;
-      fLy[3][f][col] = F[3] - (uf * txy + vf * tyy + kap * Ty);
     }
   }
   __syncthreads();
 
   float lam = 0.f;
-  const long long id = cidx(k, ci, cj);
-  if (fluid) {
-    float L[4];
-    for (int v = 0; v < 4; v++)
-      L[v] = -((fLx[v][ty][tx + 1] - fLx[v][ty][tx]) * idx + (fLy[v][ty + 1][tx] - fLy[v][ty][tx]) * idy);
-    if (DUAL) {
-      dual_update_cell<STAGE>(k, c, id, P, L, dp, Out, ds->steps > 0);
-    } else if (STAGE == 1) {
-      for (int v = 0; v < 4; v++) Out[id + v * P] = Mn[id + v * P] + dt * L[v];
-    } else if (STAGE == 2) {
+#pragma unroll(DUAL ? 1 : CELLS)
+  for (int h = 0; h < CELLS; h++) {
+    const int ty = ty0 + h * CROWS;
+    const long long id = cidx(k, i0 + tx, j0 + ty);
+    const uint8_t mytag = h == 0 ? tags[0] : tags[CELLS - 1];
+    if (advanced(k, mytag)) {
+      float L[4];
+      const float *x0 = s_face + sm.face_slot(tx, ty), *x1 = s_face + sm.face_slot(tx + 1, ty);
+      const float *y0 = s_face + 2 * NFD + sm.face_slot(ty, tx), *y1 = s_face + 2 * NFD + sm.face_slot(ty + 1, tx);
       for (int v = 0; v < 4; v++)
-        Out[id + v * P] = 0.75f * Mn[id + v * P] + 0.25f * (ld_stage<PERSIST>(In + id + v * P) + dt * L[v]);
-    } else {
-      // FP64 accumulation: dU^{n+1} = dU^n + (double)[2/3 ((dU^(2) - dU^n) + dt L)]
-      float mnew[4];
-      for (int v = 0; v < 4; v++) {
-        const long long o = id + v * P;
-        const float inc = (2.f / 3.f) * ((ld_stage<PERSIST>(In + o) - Mn[o]) + dt * L[v]);
-        const double dn = ld_stage<PERSIST>(D + o) + (double)inc;
-        D[o] = dn;
-        mnew[v] = (float)dn;
-        Mn[o] = mnew[v];
+        L[v] = -((x1[v * NF1] - x0[v * NF1]) * idx + (y1[v * NF1] - y0[v * NF1]) * idy);
+      if (DUAL) {
+        dual_update_cell<STAGE>(k, c, id, P, L, dp, Out, ds->steps > 0);
+      } else if (STAGE == 1) {
+        for (int v = 0; v < 4; v++) Out[id + v * P] = um[h][v] + dt * L[v];
+      } else if (STAGE == 2) {
+        for (int v = 0; v < 4; v++)
+          Out[id + v * P] = 0.75f * um[h][v] + 0.25f * (ui[h][v] + dt * L[v]);
+      } else {
+        // FP64 accumulation: dU^{n+1} = dU^n + (double)[2/3 ((dU^(2) - dU^n) + dt L)]
+        float mnew[4];
+        for (int v = 0; v < 4; v++) {
+          const long long o = id + v * P;
+          const float inc = (2.f / 3.f) * ((ui[h][v] - um[h][v]) + dt * L[v]);
+          const double dn = ud[h][v] + (double)inc;
+          D[o] = dn;
+          mnew[v] = (float)dn;
+          Mn[o] = mnew[v];
+        }
+        if (fuse_cfl) lam = fmaxf(lam, cfl_lambda(k, c, mnew));
       }
-      if (fuse_cfl) lam = cfl_lambda(k, c, mnew);
+    } else if (!DUAL && BODY && STAGE == 3 && mytag != SOLID) {
+      // IB / ghost node: the mirror of U^{n+1} takes the value rebuilt at stage 1
+      for (int v = 0; v < 4; v++) Mn[id + v * P] = f64_to_f32(ud[h][v]);
     }
-  } else if (!DUAL && BODY && STAGE == 3 && inside && mytag != SOLID) {
-    // IB / ghost node: the mirror of U^{n+1} takes the value rebuilt at stage 1
-    for (int v = 0; v < 4; v++) Mn[id + v * P] = (float)ld_stage<PERSIST>(D + id + v * P);
   }
   // one call site for the whole block (the reduction has a barrier)
   if (STAGE == 3 && fuse_cfl) cfl_block_max(k, lam, lred, ds, ncfl, PERSIST);
 }
 
+// The block's copy of a table entry's case.  Indexed in the kernel's parameters, the constants and pointers were read
+// early and held across the tile in spilled registers; shared memory is read where a value is used.
+__device__ __forceinline__ void load_case(StageCase &dst, const StageCase &src) {
+  static_assert(sizeof(StageCase) % 8 == 0, "copied in 8-byte words");
+  for (int i = threadIdx.x; i < (int)(sizeof(StageCase) / 8); i += NTH)
+    reinterpret_cast<unsigned long long *>(&dst)[i] = reinterpret_cast<const unsigned long long *>(&src)[i];
+  __syncthreads();
+}
 
 }  // namespace ibm

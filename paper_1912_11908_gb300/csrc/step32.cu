@@ -70,10 +70,10 @@ __device__ __forceinline__ void wait_neighbours(const Consts &k, const unsigned 
   __syncthreads();
 }
 
-// MINB: resident blocks per SM the register allocation must allow (6: 40
-// registers, 5: 48 registers).
+// MINB: resident blocks per SM the register allocation must allow (7: 72
+// registers, 6: 80 registers).
 template <int MINB>
-__global__ void __launch_bounds__(256, MINB)
+__global__ void __launch_bounds__(NTH, MINB)
     k_step_f32(Consts k, PertConsts c, float *M, float *F1, float *F2, double *D, const uint8_t *__restrict__ tag,
                const int *__restrict__ sid, const RStencil32 *__restrict__ rs, const uint8_t *__restrict__ tile_body,
                const int *__restrict__ body_tiles, int body_cap, DevState *ds, StepSched *sch, bool fuse_cfl,
@@ -161,8 +161,8 @@ int step_f32_grid(const Consts &k, int variant) {
   int dev = 0, sms = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (variant == 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_step_f32<5>, 256, 0);
-  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_step_f32<6>, 256, 0);
+  if (variant == 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_step_f32<6>, NTH, 0);
+  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_step_f32<7>, NTH, 0);
   long long g = (long long)per * sms;
   const long long items = 3LL * stage_tiles(k);
   if (g > items) g = items;
@@ -182,7 +182,7 @@ cudaError_t launch_step_f32(const Consts &k, float *M, float *F1, float *F2, dou
   // all blocks resident at once
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)grid);
-  cfg.blockDim = dim3(256);
+  cfg.blockDim = dim3(NTH);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -191,9 +191,9 @@ cudaError_t launch_step_f32(const Consts &k, float *M, float *F1, float *F2, dou
   cfg.attrs = at;
   cfg.numAttrs = 1;
   if (variant == 1)
-    return cudaLaunchKernelEx(&cfg, k_step_f32<5>, k, c, M, F1, F2, D, tag, sid, rs, tile_body, body_tiles, body_cap,
+    return cudaLaunchKernelEx(&cfg, k_step_f32<6>, k, c, M, F1, F2, D, tag, sid, rs, tile_body, body_tiles, body_cap,
                               ds, sch, fuse_cfl, tm[0], tm[1], tm[2], ut, s_first, s_last);
-  return cudaLaunchKernelEx(&cfg, k_step_f32<6>, k, c, M, F1, F2, D, tag, sid, rs, tile_body, body_tiles, body_cap,
+  return cudaLaunchKernelEx(&cfg, k_step_f32<7>, k, c, M, F1, F2, D, tag, sid, rs, tile_body, body_tiles, body_cap,
                             ds, sch, fuse_cfl, tm[0], tm[1], tm[2], ut, s_first, s_last);
 }
 
