@@ -55,8 +55,8 @@ __device__ __forceinline__ float f64_to_f32(double d) {
 // The update below is bound by the FP64 pipe: reciprocals and the products that no fused multiply-add holds follow
 // fp64_math.cuh (integer pipes), and the kinetic terms are written with dq = |u|^2 - |u_inf|^2 alone,
 //   rho |u|^2 - |u_inf|^2 = drho |u_inf|^2 + rho dq,
-// so that p' = (gamma - 1) [W + (H_inf - |u_inf|^2 / 2) drho - rho dq / 2].  About 57 FP64 instructions per cell and
-// pseudo stage (93 before).  2048 x 1024, M = 0.001: 454 -> 309 us per pseudo stage.
+// so that p' = (gamma - 1) [W + (H_inf - |u_inf|^2 / 2) drho - rho dq / 2].  About 48 FP64 instructions per cell and
+// pseudo stage (93 before).  2048 x 1024, M = 0.001: 454 -> 283 us per pseudo stage, FP64 pipe 82% busy.
 //
 // FP64 perturbation conserved -> (p', u', v', T') with u' = u - u_inf; dr = rho - 1, r = rho, ir = 1 / rho
 __device__ __forceinline__ void pert_prim64(const Consts &k, const double W[4], double q[4], double &r, double &ir,

@@ -321,43 +321,45 @@ __device__ __forceinline__ void dual_cell64(const Consts &k, const F64Consts &c,
   const long long P = k.plane;
   double W[4], S[4];
   for (int v = 0; v < 4; v++) W[v] = In[id + v * P];
-  const double r = W[0], ir = rcp64(r), u = W[1] * ir, v = W[2] * ir, V2 = fma(u, u, v * v);
-  const double pr = c.g1 * fma(-0.5 * r, V2, W[3]), T = pr * ir * c.iR;
+  const double r = W[0], ir = rcp64(r), u = mul64(W[1], ir), v = mul64(W[2], ir), V2 = fma(u, u, mul64(v, v));
+  const double pr = mul64(c.g1, fma(-half64(r), V2, W[3])), T = mul64(mul64(pr, ir), c.iR);
   const double aw = bdf2 ? 1.5 * k.idt_phys : k.idt_phys;
   for (int q = 0; q < 4; q++) {
     const long long o = id + q * P;
-    const double t = bdf2 ? k.idt_phys * fma(0.5, Wm[o], fma(1.5, W[q], -2.0 * Wn[o])) : k.idt_phys * (W[q] - Wn[o]);
-    S[q] = -(Rv[q] + t);
+    const double t = bdf2 ? fma(0.5, Wm[o], fma(1.5, W[q], mul64(-2.0, Wn[o]))) : W[q] - Wn[o];
+    S[q] = fma(-k.idt_phys, t, -Rv[q]);
   }
   // pseudo-time step of the preconditioned eigenvalues, reference velocity by squares
-  const double c2 = k.gamma * pr * ir, vis = c.nud * ir;
-  const double ur2 = fmin(fmax(fmax(V2, 1.0), vis * vis), c2), ic2 = rcp64(c2);
-  const double mr2 = ur2 * ic2, t = 0.5 * (1.0 - mr2), Vm = sqrt64(V2), cq = sqrt64(fma(t * t, V2, ur2));
+  const double c2 = mul64(mul64(k.gamma, pr), ir), vis = mul64(c.nud, ir);
+  const double ur2 = fmin(fmax(fmax(V2, 1.0), mul64(vis, vis)), c2), ic2 = rcp64(c2);
+  const double mr2 = mul64(ur2, ic2), t = half64(1.0 - mr2), Vm = sqrt64(V2), cq = sqrt64(fma(mul64(t, t), V2, ur2));
   const double lam = fma(fma(half64(Vm), 1.0 + mr2, cq), c.ih[0] + c.ih[1], mul64(c.dif, ir));
-  const double idtau = lam * c.icfl, s = idtau + aw;
-  const double iT = rcp64(T), rT = -r * iT;
-  const double th = fma(idtau, fma(iT, c.icp, rcp64(ur2)), aw * c.iR * iT);
-  const double is = rcp64(s), isr = is * ir, H = fma(k.cp, T, 0.5 * V2);
-  const double du = (S[1] - u * S[0]) * isr, dv = (S[2] - v * S[0]) * isr;
-  const double rcp_ = r * k.cp;
-  const double Y = fma(S[3] - H * S[0], is, -r * fma(u, du, v * dv));
-  const double dT = fma(th, Y, S[0]) * rcp64(fma(th, rcp_, s * rT));
+  const double idtau = mul64(lam, c.icfl), s = idtau + aw;
+  const double iT = rcp64(T), rT = mul64(-r, iT);
+  const double th = fma(idtau, fma(iT, c.icp, rcp64(ur2)), mul64(mul64(aw, c.iR), iT));
+  const double is = rcp64(s), isr = mul64(is, ir), H = fma(k.cp, T, half64(V2));
+  const double du = mul64(fma(-u, S[0], S[1]), isr), dv = mul64(fma(-v, S[0], S[2]), isr);
+  const double rcp_ = mul64(r, k.cp);
+  const double Y = fma(fma(-H, S[0], S[3]), is, mul64(-r, fma(u, du, mul64(v, dv))));
+  const double dT = mul64(fma(th, Y, S[0]), rcp64(fma(th, rcp_, mul64(s, rT))));
   const double dQ[4] = {fma(rcp_, dT, -Y), du, dv, dT}, Qk[4] = {pr, u, v, T};
   double Qn[4];
   if (STAGE == 1) {
     for (int q = 0; q < 4; q++) Qn[q] = Qk[q] + dQ[q];
   } else {
-    const double r0 = A[id], ir0 = rcp64(r0), u0 = A[id + P] * ir0, v0 = A[id + 2 * P] * ir0;
-    const double p0 = c.g1 * fma(-0.5 * r0, fma(u0, u0, v0 * v0), A[id + 3 * P]);
-    const double Q0[4] = {p0, u0, v0, p0 * ir0 * c.iR};
-    const double w0 = STAGE == 2 ? 0.75 : 1.0 / 3.0, w1 = STAGE == 2 ? 0.25 : 2.0 / 3.0;
-    for (int q = 0; q < 4; q++) Qn[q] = fma(w0, Q0[q], w1 * (Qk[q] + dQ[q]));
+    const double r0 = A[id], ir0 = rcp64(r0), u0 = mul64(A[id + P], ir0), v0 = mul64(A[id + 2 * P], ir0);
+    const double p0 = mul64(c.g1, fma(-half64(r0), fma(u0, u0, mul64(v0, v0)), A[id + 3 * P]));
+    const double Q0[4] = {p0, u0, v0, mul64(mul64(p0, ir0), c.iR)};
+    for (int q = 0; q < 4; q++) {
+      const double e = Qk[q] + dQ[q];
+      Qn[q] = STAGE == 2 ? fma(0.75, Q0[q], half64(half64(e))) : fma(1.0 / 3.0, Q0[q], mul64(2.0 / 3.0, e));
+    }
   }
-  const double rn = Qn[0] * c.iR * rcp64(Qn[3]);
+  const double rn = mul64(mul64(Qn[0], c.iR), rcp64(Qn[3]));
   Out[id] = rn;
-  Out[id + P] = rn * Qn[1];
-  Out[id + 2 * P] = rn * Qn[2];
-  Out[id + 3 * P] = fma(Qn[0], c.ig1, 0.5 * rn * fma(Qn[1], Qn[1], Qn[2] * Qn[2]));
+  Out[id + P] = mul64(rn, Qn[1]);
+  Out[id + 2 * P] = mul64(rn, Qn[2]);
+  Out[id + 3 * P] = fma(Qn[0], c.ig1, mul64(half64(rn), fma(Qn[1], Qn[1], mul64(Qn[2], Qn[2]))));
 }
 
 template <int STAGE, bool DUAL, int TX, int TY>

@@ -1,10 +1,11 @@
 // FP64 arithmetic of the residuals (2-D and 3-D).  GB300 retires two FP64 lanes per SM and clock (1.056 TFLOP/s
 // measured, 1/70 of its FP32 rate), so an FP64 residual is bound by the number of FP64 instructions, and everything
-// here is written to issue few of them: reciprocals and square roots as the hardware's approximation (relative error
-// about 2^-20) and one third-order correction (Householder's method: the new error is the old one cubed, below
-// 2^-58) in place of the IEEE sequences with their range checks -- the arguments are densities, pressures, speeds and
-// smoothness weights in the normal range; one reciprocal shared where several quotients stand side by side; signs and
-// magnitudes against 1 tested on the integer bits, off the FP64 pipe.
+// here is written to issue few of them: plain products, reciprocals and square roots on the integer pipes (the
+// arguments are densities, pressures, speeds and smoothness weights in the normal range); one reciprocal shared where
+// several quotients stand side by side; signs and magnitudes against 1 tested on the integer bits.  With reciprocals and
+// square roots corrected on the FP64 pipe instead: 768 x 384 FP64 wedge, two steps, 1.71 ms (1.53 here); 257 x 131 FP64
+// dual time 5.80 (5.13, also with the update's products off the pipe); 96 x 48 x 48 FP64 sphere 2.94 (2.73); FP32-bulk
+// dual time 2048 x 1024 27.8 (25.5).
 #pragma once
 
 namespace ibm {
@@ -45,20 +46,50 @@ __device__ __forceinline__ double half64(double x) {
   return __hiloint2double((int)hi, tiny ? 0 : __double2loint(x));
 }
 
-// 1 / x for normal x
+// 1 / x for normal x, on the integer pipes: third-order correction of an FP32 reciprocal (Householder's method: the new
+// error is the old one cubed), about 35 instructions in place of three on the FP64 pipe (192 issue slots).  With m the 53-bit mantissa and Y the FP32
+// reciprocal as a 24-bit integer, 2^76 - m Y is the residual e = 1 - D y in units of 2^-76, exact modulo 2^64
+// (|e| < 2^-21); y (1 + e + e^2) is formed to 2^-60 and rounded to nearest: within 0.506 ulp.
+// NaN for zero, subnormal, infinite and NaN x; a result below the normal range is zero.
 __device__ __forceinline__ double rcp64(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);  // y (1 + e + e^2)
+  const unsigned h = __double2hiint(x), l = __double2loint(x), e20 = h & 0x7ff00000u;
+  float y0;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(__uint_as_float(0x3f000000u | (__funnelshift_l(l, h, 3) & 0x7fffffu))));
+  const unsigned Y = __float_as_uint(y0) - 0x3f000000u;  // 2^23 y0
+  const long long E = -(long long)((unsigned long long)l * Y + ((unsigned long long)((h & 0xfffffu | 0x100000u) * Y) << 32));
+  const int Eh = (int)(E >> 30);
+  const long long c = (E + ((long long)Eh * Eh >> 16)) >> 16;  // e + e^2 in units of 2^-60
+  const unsigned long long q = (((unsigned long long)Y << 39) + ((long long)Y * c >> 21) + 512u) >> 10;
+  unsigned hi = (unsigned)(q >> 32) + (0x7fc00000u - e20) + (h & 0x80000000u), lo = (unsigned)q;
+  const bool nan = e20 - 0x00100000u >= 0x7fe00000u, zero = e20 >= 0x7fd00000u;
+  if (zero) hi = h & 0x80000000u;
+  if (nan) hi = 0x7ff80000u;
+  if (zero || nan) lo = 0u;
+  return __hiloint2double((int)hi, (int)lo);
 }
 
-// 1 / sqrt(x) for normal x > 0 (NaN for x < 0)
+// 1 / sqrt(x) for normal x > 0, the same way: X = x 4^-k in [1, 4) as a 54-bit integer, the residual 1 - X y^2 from the
+// middle 64 bits of its product with Y^2 (|e| < 2^-21, in units of 2^-68), y (1 + e / 2 + 3 e^2 / 8): within 0.507 ulp.
+// NaN for anything else.
 __device__ __forceinline__ double rsqrt64(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-mul64(x, y), y, 1.0);
-  return fma(mul64(y, e), fma(0.375, e, 0.5), y);  // y (1 + e / 2 + 3 e^2 / 8)
+  const unsigned h = __double2hiint(x), l = __double2loint(x), odd = (h >> 20) + 1u & 1u;
+  float y0;
+  asm("rsqrt.approx.ftz.f32 %0, %1;"
+      : "=f"(y0)
+      : "f"(__uint_as_float((127u + odd << 23) | (__funnelshift_l(l, h, 3) & 0x7fffffu))));
+  const unsigned Y = __float_as_uint(y0) - 0x3e800000u;  // 2^24 y0
+  const unsigned mh = __funnelshift_l(l, h & 0xfffffu | 0x100000u, odd), ml = l << odd;
+  const unsigned long long Y2 = (unsigned long long)Y * Y;
+  const unsigned yl = (unsigned)Y2, yh = (unsigned)(Y2 >> 32);
+  const long long E = -(long long)(((unsigned long long)ml * yl >> 32) + (unsigned long long)ml * yh +
+                                   (unsigned long long)mh * yl + ((unsigned long long)(mh * yh) << 32));
+  const int Eh = (int)(E >> 24);
+  const long long c = ((E >> 1) + (3 * ((long long)Eh * Eh) >> 23)) >> 8;  // e / 2 + 3 e^2 / 8 in units of 2^-60
+  const unsigned long long q = (((unsigned long long)Y << 39) + ((long long)Y * c >> 21) + 512u) >> 10;
+  // exponent 1022 - k with k = (biased exponent - 1023 - odd) / 2; q's leading one adds 1
+  const unsigned hi = (unsigned)(q >> 32) + (0x3fd00000u + ((0x3ffu + odd) << 19) - ((h & 0x7ff00000u) >> 1));
+  const bool ok = h - 0x00100000u < 0x7fe00000u;
+  return __hiloint2double(ok ? (int)hi : 0x7ff80000, ok ? (int)(unsigned)q : 0);
 }
 
 // sqrt(x) for x >= 0; 0 for zero and subnormal x (squares of speeds below 1e-154), where the approximation is infinite
@@ -78,7 +109,7 @@ __device__ __forceinline__ bool negative(double x) { return hi64(x) < 0; }
 //   eps + beta_k = [eps + 13/12 d^2] + (first-difference term / 2)^2,
 // whose bracket three windows share; the candidates are taken relative to the centre's value and the nonlinear
 // weights d_k / (eps + beta_k)^2 cleared of their common denominator, so that each value is f + N / D and one
-// reciprocal of D_L D_R serves both.  About 40 FP64 instructions for two states.
+// reciprocal of D_L D_R serves both.  About 37 FP64 instructions for two states.
 struct Weno64 {
   double f, g, hg, d0, d1, e0, e1;  // centre value; g = f(c) - f(c-1) and half of it; second differences at c - 1 and
                                     // c; their brackets
