@@ -475,7 +475,7 @@ def run_ours(args, rank, world):
             g3["%d^3" % n3] = {"ms": e0.elapsed_time(e1) / reps, "listed_nodes": int(b3.counts().sum())}
         b3.close()
         geo3d = {"workload": "Appendix A: UV sphere of 1200 triangles, radius 0.35, in n^3 lattice nodes over the unit "
-                             "cube", "kernels": "k3_classify_lines (x3), k3_tags, k3_scan, k3_scatter, k3_closest", "gpu": g3,
+                             "cube", "kernels": "k3_cross, k3_parity_xy, k3_vote, k3_tags, k3_scan, k3_scatter, k3_closest", "gpu": g3,
                  "paper_table_a1_context": "4.296e-2 s for 40^3 nodes on one Xeon E5-2670 core (the paper's "
                                            "pre-processing; other hardware, context only)"}
 
@@ -539,7 +539,7 @@ def run_ours(args, rank, world):
 
 def flow3d_block(ibm, stream, fma, steps=10, warmup=3):
     """3-D steps of the 192 x 96 x 96 sphere case in FP32-bulk and in FP64, CUDA events on the case's stream (the
-    working set, ~600 MB, is larger than L2); the achieved rate of the step's algorithmic flops against the
+    working set, ~430 MB, is larger than L2); the achieved rate of the step's algorithmic flops against the
     measured FMA rate of the precision the fluxes run in."""
     import torch
     from paper_1912_11908_gb300 import workloads as W

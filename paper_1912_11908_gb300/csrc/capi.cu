@@ -874,13 +874,13 @@ static ibm_status tune_plain_variant(ibm_case *c) {
   float step_ms[2];
   for (int f = 0; f < nforms; f++) {
     for (int st = 0; st < 2; st++) {
-      // another budget replaces the compiler's default only when it is clearly faster: margins within the
-      // timing noise flip between runs (a 2% margin still flipped the stage-1 pick at 768 x 384 on GB300,
-      // and the pick that won by that margin made flushed-cache steps 4% slower), and the default keeps more
-      // blocks resident for cold caches
+      // another budget replaces eight blocks per SM only when it is far faster here: these timings run from a warm
+      // L2, and with caches flushed between steps the resident blocks hide the loads (768 x 384 step: eight blocks
+      // 66 us, seven 75, the pick at a 4% margin 79; warm 72.5, 72.3 and 73.4; 3072 x 1536, four steps: 2.60 ms,
+      // seven blocks 2.67)
       int b = 0;
       for (int v = 1; v < PLAIN_VARIANTS; v++)
-        if (best[f][st][v] < (b == 0 ? 0.96f : 1.f) * best[f][st][b]) b = v;
+        if (best[f][st][v] < (b == 0 ? 0.85f : 1.f) * best[f][st][b]) b = v;
       pick[f][st] = b;
     }
     step_ms[f] = best[f][0][pick[f][0]] + 2.f * best[f][1][pick[f][1]];
