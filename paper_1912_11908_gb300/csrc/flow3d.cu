@@ -759,8 +759,6 @@ extern "C" ibm_status ibm_case3d_step(ibm_case3d *c, int nsteps) {
   cudaStream_t s = c->stream;
   const bool f32 = c->precision == IBM_PREC_FP32_BULK;
   const dim3 gx((g.nx + XCELLS - 1) / XCELLS, (g.ny + BY - 1) / BY, g.nz);
-  const dim3 gy((g.nx + SLANES - 1) / SLANES, g.nz, (g.ny + c->rows_y - 3) / (c->rows_y - 2)), sy(SLANES, c->rows_y, 1);
-  const dim3 gz((g.nx + SLANES - 1) / SLANES, g.ny, (g.nz + c->rows_z - 3) / (c->rows_z - 2)), sz(SLANES, c->rows_z, 1);
   const dim3 ball = cells(g.W, g.H, g.D), bint = cells(g.nx, g.ny, g.nz);
   const unsigned bhalo = nblk(2LL * NG * ((long long)g.W * g.H + (long long)g.nz * g.W + (long long)g.nz * g.ny));
   // eight lanes per listed node (one cube corner each), 16 nodes per block
@@ -783,8 +781,8 @@ extern "C" ibm_status ibm_case3d_step(ibm_case3d *c, int nsteps) {
         if (ngh) k3_reconstruct32<<<bgh, 128, 0, s>>>(g, ph, c->p32, in[k], c->st, nib, ngh, c->A, k == 0);
         k3_halo32<<<bhalo, TB, 0, s>>>(g, in[k]);
         k3_prim32<<<ball, CB, 0, s>>>(g, c->p32, in[k], c->q32);
-        k3_sweep_yz<1, float><<<gy, sy, 0, s>>>(g, c->p32, c->q32, c->d32);
-        k3_sweep_yz<2, float><<<gz, sz, 0, s>>>(g, c->p32, c->q32, c->d32);
+        c->launches += launch_sweep_yz<1, float>(g, c->p32, c->q32, c->d32, c->rows_y, s);
+        c->launches += launch_sweep_yz<2, float>(g, c->p32, c->q32, c->d32, c->rows_z, s);
         const F5f &out = k == 0 ? c->s1 : c->s2;  // (stage 3 writes the master and its mirror)
         if (k == 0)
           k3_sweep_x32<1><<<gx, CB, 0, s>>>(g, ph, c->p32, c->q32, c->d32, c->mirror, in[k], out, c->A, c->tags, c->dt);
@@ -792,7 +790,7 @@ extern "C" ibm_status ibm_case3d_step(ibm_case3d *c, int nsteps) {
           k3_sweep_x32<2><<<gx, CB, 0, s>>>(g, ph, c->p32, c->q32, c->d32, c->mirror, in[k], out, c->A, c->tags, c->dt);
         else
           k3_sweep_x32<3><<<gx, CB, 0, s>>>(g, ph, c->p32, c->q32, c->d32, c->mirror, in[k], out, c->A, c->tags, c->dt);
-        c->launches += 5 + (nib ? 1 : 0) + (ngh ? 1 : 0);
+        c->launches += 3 + (nib ? 1 : 0) + (ngh ? 1 : 0);
       }
     } else {
       F5 in[3] = {c->A, c->B, c->C}, out[3] = {c->B, c->C, c->A};
@@ -801,12 +799,12 @@ extern "C" ibm_status ibm_case3d_step(ibm_case3d *c, int nsteps) {
         if (ngh) k3_reconstruct<<<bgh, 128, 0, s>>>(g, ph, in[k], c->st, nib, ngh);
         k3_halo<<<bhalo, TB, 0, s>>>(g, ph, in[k]);
         k3_prim<<<ball, CB, 0, s>>>(g, ph, in[k], c->Q);
-        k3_sweep_yz<1, double><<<gy, sy, 0, s>>>(g, c->p64, c->Q, c->D);
-        k3_sweep_yz<2, double><<<gz, sz, 0, s>>>(g, c->p64, c->Q, c->D);
+        c->launches += launch_sweep_yz<1, double>(g, c->p64, c->Q, c->D, c->rows_y, s);
+        c->launches += launch_sweep_yz<2, double>(g, c->p64, c->Q, c->D, c->rows_z, s);
         if (k == 0) k3_sweep_x<1><<<gx, CB, 0, s>>>(g, c->p64, c->Q, c->D, c->A, in[k], out[k], c->tags, c->dt);
         else if (k == 1) k3_sweep_x<2><<<gx, CB, 0, s>>>(g, c->p64, c->Q, c->D, c->A, in[k], out[k], c->tags, c->dt);
         else k3_sweep_x<3><<<gx, CB, 0, s>>>(g, c->p64, c->Q, c->D, c->A, in[k], out[k], c->tags, c->dt);
-        c->launches += 5 + (nib ? 1 : 0) + (ngh ? 1 : 0);
+        c->launches += 3 + (nib ? 1 : 0) + (ngh ? 1 : 0);
       }
     }
     k3_step_end<<<1, 1, 0, s>>>(c->dt, c->time);

@@ -240,6 +240,7 @@ __device__ __forceinline__ void sweep_x(const Grid3 &g, const typename Real<T>::
 // SROWS rows along DIR, one window per row; the y sweep writes
 // the cells' divergence, the z sweep adds to it.  Every thread of the block calls it.
 constexpr int SROWS = 16, SLANES = 16;
+constexpr int GRID_YZ_MAX = 65535;  // gridDim.y and gridDim.z
 template <class T>
 struct SweepSmem {
   T x[11][SROWS][SLANES];  // right states (then fluxes) and the tangential differences of the rows
@@ -343,9 +344,22 @@ __device__ __forceinline__ void sweep_yz(const Grid3 &g, const typename Real<T>:
 
 template <int DIR, class T>
 __global__ void __launch_bounds__(SLANES *SROWS) k3_sweep_yz(Grid3 g, typename Real<T>::Par c, typename Real<T>::Q Q,
-                                                          typename Real<T>::L Lo) {
+                                                          typename Real<T>::L Lo, int o0) {
   __shared__ SweepSmem<T> sm;
-  sweep_yz<DIR, T>(g, c, Q, Lo, blockIdx.x * SLANES + threadIdx.x, blockIdx.y, sm);
+  sweep_yz<DIR, T>(g, c, Q, Lo, blockIdx.x * SLANES + threadIdx.x, o0 + blockIdx.y, sm);
+}
+
+// the y (DIR 1) or z (DIR 2) sweep in blocks of `rows` rows: gridDim.y runs over the cells of the third axis, at most
+// 65,535 of them per launch (one launch for any usual grid); returns the launches
+template <int DIR, class T>
+inline int launch_sweep_yz(const Grid3 &g, const typename Real<T>::Par &c, const typename Real<T>::Q &Q,
+                           const typename Real<T>::L &Lo, int rows, cudaStream_t s) {
+  const int n = DIR == 1 ? g.ny : g.nz, no = DIR == 1 ? g.nz : g.ny;
+  int launches = 0;
+  for (int o0 = 0; o0 < no; o0 += GRID_YZ_MAX, launches++)
+    k3_sweep_yz<DIR, T><<<dim3((g.nx + SLANES - 1) / SLANES, std::min(no - o0, GRID_YZ_MAX), (n + rows - 3) / (rows - 2)),
+                          dim3(SLANES, rows), 0, s>>>(g, c, Q, Lo, o0);
+  return launches;
 }
 
 // x sweep with the SSP-RK3 stage on the fluid cells: out = Un - dt D, 3/4 Un + 1/4 (in - dt D),
