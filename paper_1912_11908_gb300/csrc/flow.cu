@@ -497,16 +497,23 @@ static void launch_tile_f64(const Consts &k, const double *Un, const double *In,
 // Tile shape by the work of the fullest SM: an SM's time is its tiles' FP64 instructions (halo cells, windows and
 // faces included: 1, 0.53 and 0.30 of the 16 x 16 tile), and the tiles are dealt evenly, so a grid of few tiles takes
 // the shape whose last round is fullest -- 257 x 131 cells are 153 tiles of 16 x 16 on 152 SMs, 289 of 16 x 8: a
-// dual-time pseudo stage there went from 374 us (16 x 16, the arithmetic before) to 55.
+// dual-time pseudo stage there went from 374 us (16 x 16, the arithmetic before) to 55.  Rows of tiles run along
+// gridDim.y, so a grid taller than 65,535 rows of eight cells keeps the 16 x 16 tile.  Returns 0: 16 x 16, 1: 16 x 8,
+// 2: 8 x 8.
+extern "C" int ibm__tile_shape_f64(int nx, int ny, int sms) {
+  if ((ny + 7) / 8 > 65535) return 0;
+  const auto cost = [&](int tx, int ty, double work) {
+    const long long tiles = (long long)((nx + tx - 1) / tx) * ((ny + ty - 1) / ty);
+    return (double)((tiles + sms - 1) / sms) * work;
+  };
+  const double c0 = cost(16, 16, 1.0), c1 = cost(16, 8, 0.53), c2 = cost(8, 8, 0.30);
+  return c0 <= c1 && c0 <= c2 ? 0 : c1 <= c2 ? 1 : 2;
+}
+
 template <bool DUAL>
 static void launch_tiles_f64(const Consts &k, int stage, const double *Un, const double *In, double *Out,
                              const double *Wn, const double *Wm, const uint8_t *tag, DevState *ds, cudaStream_t s) {
-  const auto cost = [&](int tx, int ty, double work) {
-    const long long tiles = (long long)((k.nx + tx - 1) / tx) * ((k.ny + ty - 1) / ty);
-    return (double)((tiles + 151) / 152) * work;
-  };
-  const double c0 = cost(16, 16, 1.0), c1 = cost(16, 8, 0.53), c2 = cost(8, 8, 0.30);
-  const int shape = c0 <= c1 && c0 <= c2 ? 0 : c1 <= c2 ? 1 : 2;
+  const int shape = ibm__tile_shape_f64(k.nx, k.ny, 152);
 #define IBM_F64(S)                                                                                    \
   (shape == 0   ? launch_tile_f64<S, DUAL, 16, 16>(k, Un, In, Out, Wn, Wm, tag, ds, s)                \
    : shape == 1 ? launch_tile_f64<S, DUAL, 16, 8>(k, Un, In, Out, Wn, Wm, tag, ds, s)                 \
