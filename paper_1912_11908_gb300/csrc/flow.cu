@@ -32,7 +32,15 @@ __global__ void __launch_bounds__(256) k_dt(Consts k, const double *__restrict__
     const double r = A[id], ir = rcp64(r), u = A[id + k.plane] * ir, v = A[id + 2 * k.plane] * ir;
     const double p = (k.gamma - 1.0) * fma(-0.5 * r, fma(u, u, v * v), A[id + 3 * k.plane]);
     const double c = sqrt64(k.gamma * p * ir);
-    lmax = fmax(lmax, fma(fabs(u) + c, idx, fma(fabs(v) + c, idy, vis * ir)));
+    double lam = fma(fabs(u) + c, idx, fma(fabs(v) + c, idy, vis * ir));
+    if (not_finite(lam)) {
+      // a state beyond the range of fp64_math.cuh, whose results are NaN there and would drop out of the maximum: the
+      // bound in the hardware's arithmetic, so that a cell that overflowed drives dt to zero
+      const double ui = A[id + k.plane] / r, vi = A[id + 2 * k.plane] / r;
+      const double ci = sqrt(k.gamma * ((k.gamma - 1.0) * (A[id + 3 * k.plane] - 0.5 * r * (ui * ui + vi * vi))) / r);
+      lam = (fabs(ui) + ci) / k.dx + (fabs(vi) + ci) / k.dy + vis / r;
+    }
+    lmax = fmax(lmax, lam);
   }
   for (int off = 16; off > 0; off >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, off));
   __shared__ double wm[8];

@@ -31,6 +31,7 @@ namespace {
 
 using ibm::half64;
 using ibm::mul64;
+using ibm::not_finite;
 using ibm::rcp64;
 using ibm::sqrt64;
 
@@ -103,6 +104,12 @@ __global__ void __launch_bounds__(TC) k3_lambda(Grid3 g, Phys3 ph, F5 U, const u
     cell_prim(ph, U, m, r, ir, u, v, w, p);
     const double c = sqrt64(mul64(mul64(ph.gamma, p), ir));
     lam = fma(fabs(u) + c, g.idx, fma(fabs(v) + c, g.idy, fma(fabs(w) + c, g.idz, mul64(ph.dif, ir))));
+    if (not_finite(lam)) {  // beyond the range of fp64_math.cuh: the bound in the hardware's arithmetic, as in 2-D
+      ir = 1.0 / r;
+      const double ui = U.v[1][m] * ir, vi = U.v[2][m] * ir, wi = U.v[3][m] * ir;
+      const double ci = sqrt(ph.gamma * (ph.g1 * (U.v[4][m] - 0.5 * r * (ui * ui + vi * vi + wi * wi))) * ir);
+      lam = (fabs(ui) + ci) * g.idx + (fabs(vi) + ci) * g.idy + (fabs(wi) + ci) * g.idz + ph.dif * ir;
+    }
   }
   for (int o = 16; o > 0; o >>= 1) lam = fmax(lam, __shfl_xor_sync(0xffffffffu, lam, o));
   if ((threadIdx.x & 31) == 0 && lam > 0.0) atomicMax(lmax, (unsigned long long)__double_as_longlong(lam));

@@ -102,6 +102,8 @@ __device__ __forceinline__ bool below_one(double x) { return (hi64(x) & 0x7fffff
 // x positive, normal and finite
 __device__ __forceinline__ bool positive(double x) { return (unsigned)(hi64(x) - 1) < 0x7fefffffu; }
 __device__ __forceinline__ bool negative(double x) { return hi64(x) < 0; }
+// x infinite or NaN
+__device__ __forceinline__ bool not_finite(double x) { return (hi64(x) & 0x7ff00000) == 0x7ff00000; }
 
 // Sec. 2: fifth-order WENO (Jiang-Shu smoothness indicators, linear weights 1/10, 6/10, 3/10, eps = 1e-6) of one
 // five-point window, both of its values: the left state at the centre's right face and, mirrored, the right state at
