@@ -194,13 +194,14 @@ struct TileSmem {
   unsigned int mbar_phase;  // persistent kernel: parity of the barrier's next phase (barrier initialised once)
   // float offset of line l (a pair's first if even) of face f of a variable
   static __device__ __forceinline__ int face_slot(int f, int l) { return f * FP + (l ^ (f & 14)); }
-  // body tiles: cell and stencil of the listed nodes, in the face storage behind the TMA box and the stencils
+  // body tiles: cell and stencil of the listed nodes, in the face storage behind the TMA box and the stencils; IB nodes
+  // from slot 0 up, ghost nodes from the last slot down
   __device__ __forceinline__ int *rbm() { return reinterpret_cast<int *>(face) + RB_MAX * (int)sizeof(RStencil32) / 4; }
   __device__ __forceinline__ int *rbe() { return rbm() + RB_MAX; }
   float wm[7];    // wall velocity and acceleration at the stage time; 1 if Eq. 7 applies (else 0); the rotation
                   // rate and its rate of change of a pitching body (else 0)
   float lred[NTH / 32];  // per-warp maxima of the CFL reduction
-  int nrb;        // listed IB / ghost nodes (body tiles)
+  int nrb[2];     // listed IB and ghost nodes (body tiles)
 };
 static_assert(RB_MAX * (sizeof(RStencil32) + 2 * sizeof(int)) <= sizeof(float) * 4 * NFD, "node stencils fit the face storage");
 
@@ -563,16 +564,18 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
   const long long P = k.plane;
   // body tiles: every IB / ghost node of the loaded region, with its stencil staged in shared memory (in the
   // face storage, after the TMA box has been consumed)
-  int &s_nrb = sm.nrb;
+  int *s_nrb = sm.nrb;
   int *s_rbm = sm.rbm(), *s_rbe = sm.rbe();
   RStencil32 *s_rs = reinterpret_cast<RStencil32 *>(s_face);
-  if (BODY && threadIdx.x == 0) s_nrb = 0;
+  if (BODY && threadIdx.x < 2) s_nrb[threadIdx.x] = 0;
+  const int nib_all = BODY ? ds->offset[1] : 0;  // the case's list holds its IB nodes first
   if (BODY) __syncthreads();
-  // a listed node of the loaded region (body tiles)
+  // a listed node of the loaded region (body tiles), by class: each pass of the rebuild then takes its own nodes only
   auto list_node = [&](int m, int e) {
     if (e < 0) return;
-    const int slot = atomicAdd(&s_nrb, 1);
-    if (slot < RB_MAX) {
+    const int ghost = e >= nib_all, n = atomicAdd(&s_nrb[ghost], 1);
+    if (n < RB_MAX) {
+      const int slot = ghost ? RB_MAX - 1 - n : n;
       s_rbm[slot] = m;
       s_rbe[slot] = e;
     }
@@ -639,21 +642,26 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
   // every thread has waited on this phase: the next tile's copy completes the other parity
   if (PERSIST && TMA && tma && threadIdx.x == 0) sm.mbar_phase ^= 1u;
   if (BODY) {
-    const int nrb = min(s_nrb, RB_MAX);
-    for (int r = threadIdx.x; r < nrb; r += NTH) s_rs[r] = rs[s_rbe[r]];
+    const int nib = min(s_nrb[0], RB_MAX), ngh = min(s_nrb[1], RB_MAX - nib);
+    for (int r = threadIdx.x; r < nib + ngh; r += NTH) {
+      const int slot = r < nib ? r : RB_MAX - 1 - (r - nib);
+      s_rs[slot] = rs[s_rbe[slot]];
+    }
     __syncthreads();
     // rebuild the listed nodes in place: IB nodes, barrier, ghost nodes (whose image points may use IB
     // nodes); corners inside the loaded region come from shared memory
     // four lanes per node, one stencil corner each, so that corners outside the loaded region (chains of
     // dependent global loads) overlap; the node's first lane sums the corners in stencil order
     for (int pass = k.ib_advance ? 1 : 0; pass < 2; pass++) {  // IB nodes (pass 0) unless advanced
-      for (int t0 = 0; t0 < 4 * nrb; t0 += NTH) {  // block-uniform: every lane takes part in the shuffles
-        const int r = (t0 + (int)threadIdx.x) >> 2, cq = threadIdx.x & 3;
+      const int np = pass == 0 ? nib : ngh;
+      for (int t0 = 0; t0 < 4 * np; t0 += NTH) {  // block-uniform: every lane takes part in the shuffles
+        const int t = (t0 + (int)threadIdx.x) >> 2, cq = threadIdx.x & 3, r = pass == 0 ? t : RB_MAX - 1 - t;
+        const bool listed_node = t < np;
         bool node = false;
         float v4[4] = {0.f, 0.f, 0.f, 0.f};
-        if (r < nrb) {
+        if (listed_node) {
           const RStencil32 &st = s_rs[r];
-          node = ((st.mask & 16) != 0) == (pass == 0) && (st.mask & 15);
+          node = (st.mask & 15) != 0;
           if (node && (st.mask >> cq & 1)) {
             const int cn = st.ccell + (cq & 1) + (cq >> 1) * k.nx;
             const int la = cn % k.nx - (i0 - NG), lb = cn / k.nx - (j0 - NG);
@@ -674,7 +682,7 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
         // quadratic form: the same lane also takes its corner of the second probe's square
         const RStencilQ *tq = nullptr;
         float v4b[4] = {0.f, 0.f, 0.f, 0.f};
-        if (QUAD && r < nrb && node) {
+        if (QUAD && node) {
           tq = rsq + s_rbe[r];
           if (tq->mask >> cq & 1) {
             const int cn = tq->ccell + (cq & 1) + (cq >> 1) * k.nx;
@@ -694,9 +702,9 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
         }
         const int lane0 = (int)(threadIdx.x & 31) & ~3;
         float qp[4] = {0.f, 0.f, 0.f, 0.f};
-        const unsigned int mask = r < nrb ? (unsigned int)s_rs[r].mask : 0u;
+        const unsigned int mask = listed_node ? (unsigned int)s_rs[r].mask : 0u;
         for (int j = 0; j < 4; j++) {
-          const float wj = r < nrb ? s_rs[r].w[j] : 0.f;
+          const float wj = listed_node ? s_rs[r].w[j] : 0.f;
           for (int v = 0; v < 4; v++) {
             const float x = __shfl_sync(0xffffffffu, v4[v], lane0 + j);
             if (mask >> j & 1) qp[v] += wj * x;
@@ -736,7 +744,7 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
       }
       __syncthreads();
     }
-    if (threadIdx.x == 0 && s_nrb > RB_MAX) atomicOr(&ds->err, ERR_CAPACITY);
+    if (threadIdx.x == 0 && s_nrb[0] + s_nrb[1] > RB_MAX) atomicOr(&ds->err, ERR_CAPACITY);
   }
   // WENO5 (Sec. 2) along lines: an item is one variable of a pair of adjacent interior tile rows (x) or columns (y)
   // and one of its two halves -- nine consecutive window centres, local 2..10 or 11..19, the cells whose faces the
