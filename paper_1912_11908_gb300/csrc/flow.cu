@@ -54,6 +54,17 @@ __global__ void __launch_bounds__(256) k_dt(Consts k, const double *__restrict__
   }
 }
 
+int sm_count() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
+    cudaGetLastError();
+    return 152;
+  }
+  return sms;
+}
+extern "C" int ibm__sm_count() { return sm_count(); }
+
 void launch_dt(const Consts &k, const double *A, const uint8_t *tag, DevState *ds, cudaStream_t s, int *nlaunch) {
   if (k.dt_fixed > 0.0) return;  // ds->dt was set at creation
   int ncell = k.nx * k.ny;
@@ -521,7 +532,7 @@ extern "C" int ibm__tile_shape_f64(int nx, int ny, int sms) {
 template <bool DUAL>
 static void launch_tiles_f64(const Consts &k, int stage, const double *Un, const double *In, double *Out,
                              const double *Wn, const double *Wm, const uint8_t *tag, DevState *ds, cudaStream_t s) {
-  const int shape = ibm__tile_shape_f64(k.nx, k.ny, 152);
+  const int shape = ibm__tile_shape_f64(k.nx, k.ny, sm_count());
 #define IBM_F64(S)                                                                                    \
   (shape == 0   ? launch_tile_f64<S, DUAL, 16, 16>(k, Un, In, Out, Wn, Wm, tag, ds, s)                \
    : shape == 1 ? launch_tile_f64<S, DUAL, 16, 8>(k, Un, In, Out, Wn, Wm, tag, ds, s)                 \

@@ -287,6 +287,9 @@ void launch_body_end(DevState *ds, cudaStream_t s);
 void launch_forces_f64(const Consts &k, const Geom &g, const uint8_t *tag, const double *A, bool pert,
                        DevState *ds, cudaStream_t s, bool set_accel = false, double *surf = nullptr);
 
+// multiprocessors of the current device
+int sm_count();
+
 // ---- launchers (flow.cu) ----
 void launch_dt(const Consts &k, const double *A, const uint8_t *tag, DevState *ds, cudaStream_t s, int *nlaunch);
 void launch_recon_f64(const Consts &k, double *U, const ibm_stencil *st, int cap, const DevState *ds,
