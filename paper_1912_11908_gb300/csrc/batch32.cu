@@ -18,8 +18,8 @@ namespace ibm {
 // complete).
 // TVD / QUAD: the TVD-2 reconstruction and / or the quadratic IB / ghost reconstruction compiled in (a group
 // holds cases of one variant)
-template <int STAGE, bool TVD, bool QUAD>
-__global__ void __launch_bounds__(NTH, 8) k_stage_f32_batch_one(const __grid_constant__ StageBatch b) {
+template <int STAGE, bool TVD, bool QUAD, int NT>
+__global__ void __launch_bounds__(NT, NT == NTH ? BATCH_BLOCKS : WIDE_BLOCKS) k_stage_f32_batch_one(const __grid_constant__ StageBatch b) {
   __shared__ TileSmem sm;
   __shared__ StageCase sc;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -31,16 +31,16 @@ __global__ void __launch_bounds__(NTH, 8) k_stage_f32_batch_one(const __grid_con
     const int ee = body ? e : e - nbody;
     int q = 0;
     while (q + 1 < b.n && start[q + 1] <= ee) q++;
-    load_case(sc, b.cs[q]);
+    load_case<NT>(sc, b.cs[q]);
     const float *In = STAGE == 1 ? sc.M : (STAGE == 2 ? sc.F1 : sc.F2);
     float *Out = STAGE == 1 ? sc.F1 : (STAGE == 2 ? sc.F2 : nullptr);
     if (body)
-      stage_tile<STAGE, true, false, false, false, TVD, QUAD>(sc.k, sc.c, sc.M, In, Out, sc.D, sc.tag, sc.sid, sc.rs,
+      stage_tile<STAGE, true, false, false, false, TVD, QUAD, NT>(sc.k, sc.c, sc.M, In, Out, sc.D, sc.tag, sc.sid, sc.rs,
                                                               sc.tile_body, sc.body_tiles, sc.ds, sc.fuse_cfl != 0,
                                                               sc.ncfl, ee - start[q], sm, DualPtrs{}, nullptr,
                                                               sc.rsq);
     else
-      stage_tile<STAGE, false, false, false, false, TVD, QUAD>(sc.k, sc.c, sc.M, In, Out, sc.D, sc.tag, sc.sid,
+      stage_tile<STAGE, false, false, false, false, TVD, QUAD, NT>(sc.k, sc.c, sc.M, In, Out, sc.D, sc.tag, sc.sid,
                                                                sc.rs, sc.tile_body, sc.body_tiles, sc.ds,
                                                                sc.fuse_cfl != 0, sc.ncfl, ee - start[q], sm,
                                                                DualPtrs{}, nullptr, sc.rsq);
@@ -53,7 +53,8 @@ cudaError_t launch_stage_f32_batch_one(const StageBatch &b, int stage, int grid,
   if (total == 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)(grid > 0 && grid < total ? grid : total));
-  cfg.blockDim = dim3(NTH);
+  const bool wide = stage_wide(b.plain_start[b.n], b.body_start[b.n]);
+  cfg.blockDim = dim3(wide ? WIDE : NTH);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -64,7 +65,9 @@ cudaError_t launch_stage_f32_batch_one(const StageBatch &b, int stage, int grid,
   if (quad)
     for (int q = 0; q < b.n; q++)
       if (!b.cs[q].rsq) return cudaErrorInvalidValue;  // the quadratic kernels read the second probes
-#define IBM_BATCH(S, T, Q) cudaLaunchKernelEx(&cfg, k_stage_f32_batch_one<S, T, Q>, b)
+#define IBM_BATCH(S, T, Q)                                                  \
+  (wide ? cudaLaunchKernelEx(&cfg, k_stage_f32_batch_one<S, T, Q, WIDE>, b) \
+        : cudaLaunchKernelEx(&cfg, k_stage_f32_batch_one<S, T, Q, NTH>, b))
 #define IBM_BATCH_S(S)                                                                                          \
   (tvd ? (quad ? IBM_BATCH(S, true, true) : IBM_BATCH(S, true, false))                                          \
        : (quad ? IBM_BATCH(S, false, true) : IBM_BATCH(S, false, false)))

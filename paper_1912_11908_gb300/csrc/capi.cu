@@ -52,7 +52,7 @@ struct ibm_case {
   int stage_launch = 2;               // FP32-bulk explicit stages: 0 plain + body kernels on two streams, 1 one
                                       // kernel, 2 one kernel chained by programmatic launch (ibm_stage_launches)
   bool launch_pinned = false;         // stage_launch set by the caller (else the autotuner picks 0 or 2)
-  int step_variant = 0;               // register budget of the persistent kernel
+  int step_variant = 0;               // persistent kernel: step_f32_variant
   int step_grid = 0;                  // its grid (0: not computed yet)
   bool autotune = true;
   int box_w = 0, box_h = 0;      // cells spanned by the body's bounding box (any pose), for classification
@@ -416,6 +416,7 @@ extern "C" ibm_status ibm_create_case(const ibm_geometry *geo, const ibm_grid *g
   }
   init_case(c, geo, gr, fl, mo);
   const Consts &k = c->k;
+  c->step_variant = step_f32_variant(k);
   const int nv = geo->nverts;
   const size_t ncell = (size_t)k.nx * k.ny;
   const size_t plane = (size_t)k.plane;
@@ -818,6 +819,8 @@ static ibm_status tune_plain_variant(ibm_case *c) {
       return IBM_OK;
     }
   }
+  // (wide blocks have one budget)
+  const int nvar = stage_wide(stage_tiles(c->k), c->body_cap) ? 1 : PLAIN_VARIANTS;
   int forms[2] = {c->stage_launch, -1}, nforms = 1;
   if (!c->launch_pinned) {
     forms[0] = 2;
@@ -855,7 +858,7 @@ static ibm_status tune_plain_variant(ibm_case *c) {
   for (int round = 0; round < ROUNDS && e == cudaSuccess; round++)
     for (int f = 0; f < nforms && e == cudaSuccess; f++)
       for (int st = 0; st < 2 && e == cudaSuccess; st++)
-        for (int v = 0; v < PLAIN_VARIANTS && e == cudaSuccess; v++) {
+        for (int v = 0; v < nvar && e == cudaSuccess; v++) {
           pair(st + 1, v, forms[f]);  // warm-up
           cudaEventRecord(e0, s);
           for (int rep = 0; rep < REPS; rep++) pair(st + 1, v, forms[f]);

@@ -7,25 +7,35 @@
 
 namespace ibm {
 
+// Wide blocks (stage32.cuh) for the pseudo stage of nt tiles of one case or of several.  The update is the longest chain of all: two cells per
+// thread in turn where tiles are few last twice as long, and eight blocks of 128 threads per SM, chained by programmatic
+// launch, settle on few SMs.  A step of 10 sub-iterations, 128 threads against 288 (the step before the packed tile in
+// brackets): 64 x 64 625 us, 417 (558), 512 x 256 1445, 829 (1270), 768 x 384 1662, 1570 (2320), 1024 x 512 2684, 2650
+// (3924), 2048 x 1024 8970, 9210 (14270): there more blocks overlap one's update with others' fluxes.  Groups share the
+// GPU with each other: 16 requests 11.3 ms with wide blocks up to six tiles per SM, 11.5 up to 16; two to eight requests
+// 4 to 18% less than without.
+extern "C" int ibm__dual_wide(int nt, int cases, int sms) { return nt <= (cases > 1 ? 6 : 16) * sms; }
+static bool dual_wide(int nt, int cases = 1) { return ibm__dual_wide(nt, cases, sm_count()) != 0; }
+
 // Dual-time pseudo stage of one case (FP32 residual, FP64 point-implicit
 // update): plain tiles and body tiles as for the explicit stages.
-template <int STAGE, bool BODY>
-__global__ void __launch_bounds__(NTH) k_dual_f32(Consts k, PertConsts c, const float *__restrict__ In,
+template <int STAGE, bool BODY, int NT>
+__global__ void __launch_bounds__(NT, NT == NTH ? 6 : WIDE_BLOCKS) k_dual_f32(Consts k, PertConsts c, const float *__restrict__ In,
                                                   float *Out32, double *D, const uint8_t *__restrict__ tag,
                                                   const int *__restrict__ sid, const RStencil32 *__restrict__ rs,
                                                   const uint8_t *__restrict__ tile_body,
                                                   const int *__restrict__ body_tiles, DevState *ds, unsigned int ncfl,
                                                   DualPtrs dp) {
   __shared__ TileSmem sm;
-  stage_tile<STAGE, BODY, true>(k, c, nullptr, In, Out32, D, tag, sid, rs, tile_body, body_tiles, ds, false, ncfl,
+  stage_tile<STAGE, BODY, true, false, false, false, false, NT>(k, c, nullptr, In, Out32, D, tag, sid, rs, tile_body, body_tiles, ds, false, ncfl,
                                 (int)blockIdx.x, sm, dp);
 }
 
 // one launch of the pseudo stage of a case with the TVD-2 reconstruction and / or the quadratic IB / ghost
 // reconstruction compiled in: body-tile slots [0, nb) first, then one block per tile (every launch form of such
 // a case)
-template <int STAGE, bool TVD, bool QUAD>
-__global__ void __launch_bounds__(NTH) k_dual_f32_var(Consts k, PertConsts c, const float *__restrict__ In,
+template <int STAGE, bool TVD, bool QUAD, int NT>
+__global__ void __launch_bounds__(NT, NT == NTH ? 6 : WIDE_BLOCKS) k_dual_f32_var(Consts k, PertConsts c, const float *__restrict__ In,
                                                       float *Out32, double *D, const uint8_t *__restrict__ tag,
                                                       const int *__restrict__ sid,
                                                       const RStencil32 *__restrict__ rs,
@@ -38,10 +48,10 @@ __global__ void __launch_bounds__(NTH) k_dual_f32_var(Consts k, PertConsts c, co
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int b = (int)blockIdx.x;
   if (b < nb)
-    stage_tile<STAGE, true, true, false, false, TVD, QUAD>(k, c, nullptr, In, Out32, D, tag, sid, rs, tile_body,
+    stage_tile<STAGE, true, true, false, false, TVD, QUAD, NT>(k, c, nullptr, In, Out32, D, tag, sid, rs, tile_body,
                                                            body_tiles, ds, false, ncfl, b, sm, dp, nullptr, rsq);
   else
-    stage_tile<STAGE, false, true, false, false, TVD, QUAD>(k, c, nullptr, In, Out32, D, tag, sid, rs, tile_body,
+    stage_tile<STAGE, false, true, false, false, TVD, QUAD, NT>(k, c, nullptr, In, Out32, D, tag, sid, rs, tile_body,
                                                             body_tiles, ds, false, ncfl, b - nb, sm, dp, nullptr,
                                                             rsq);
 }
@@ -63,15 +73,17 @@ cudaError_t launch_dual_f32_var(const Consts &k, int stage, const float *In32, f
   dp.Q0 = Q0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)(nt + nb));
-  cfg.blockDim = dim3(NTH);
+  const bool wide = dual_wide(nt);
+  cfg.blockDim = dim3(wide ? WIDE : NTH);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = pdl ? 1 : 0;
-#define IBM_DUAL_VAR(S, T, Q)                                                                                 \
-  cudaLaunchKernelEx(&cfg, k_dual_f32_var<S, T, Q>, k, c, In32, Out32, D, tag, sid, rs, tile_body, body_tiles, nb, \
+#define IBM_DUAL_VAR(S, T, Q) (wide ? IBM_DUAL_VAR_N(S, T, Q, WIDE) : IBM_DUAL_VAR_N(S, T, Q, NTH))
+#define IBM_DUAL_VAR_N(S, T, Q, N)                                                                            \
+  cudaLaunchKernelEx(&cfg, k_dual_f32_var<S, T, Q, N>, k, c, In32, Out32, D, tag, sid, rs, tile_body, body_tiles, nb, \
                      ds, ncfl, dp, rsq)
 #define IBM_DUAL_VAR_S(S)                                                                                       \
   (k.tvd2 && k.quad ? IBM_DUAL_VAR(S, true, true)                                                              \
@@ -79,6 +91,7 @@ cudaError_t launch_dual_f32_var(const Consts &k, int stage, const float *In32, f
   const cudaError_t e = stage == 1 ? IBM_DUAL_VAR_S(1) : stage == 2 ? IBM_DUAL_VAR_S(2) : IBM_DUAL_VAR_S(3);
 #undef IBM_DUAL_VAR_S
 #undef IBM_DUAL_VAR
+#undef IBM_DUAL_VAR_N
   return e;
 }
 
@@ -92,8 +105,8 @@ cudaError_t launch_dual_f32_var(const Consts &k, int stage, const float *In32, f
 // With programmatic dependent launch its blocks are resident while the
 // previous pseudo stage's last blocks finish (they wait at the top for it to
 // complete).
-template <int STAGE>
-__global__ void __launch_bounds__(NTH, 8) k_dual_f32_batch_one(const __grid_constant__ StageBatch b) {
+template <int STAGE, int NT>
+__global__ void __launch_bounds__(NT, NT == NTH ? BATCH_BLOCKS : WIDE_BLOCKS) k_dual_f32_batch_one(const __grid_constant__ StageBatch b) {
   __shared__ TileSmem sm;
   __shared__ StageCase sc;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -105,7 +118,7 @@ __global__ void __launch_bounds__(NTH, 8) k_dual_f32_batch_one(const __grid_cons
     const int ee = body ? e : e - nbody;
     int q = 0;
     while (q + 1 < b.n && start[q + 1] <= ee) q++;
-    load_case(sc, b.cs[q]);
+    load_case<NT>(sc, b.cs[q]);
     const float *In = STAGE == 1 ? sc.M : (STAGE == 2 ? sc.F1 : sc.F2);
     float *Out = STAGE == 1 ? sc.F1 : (STAGE == 2 ? sc.F2 : sc.M);
     DualPtrs dp;
@@ -114,10 +127,10 @@ __global__ void __launch_bounds__(NTH, 8) k_dual_f32_batch_one(const __grid_cons
     dp.G = sc.G;
     dp.Q0 = sc.Q0;
     if (body)
-      stage_tile<STAGE, true, true>(sc.k, sc.c, nullptr, In, Out, sc.D, sc.tag, sc.sid, sc.rs, sc.tile_body,
+      stage_tile<STAGE, true, true, false, false, false, false, NT>(sc.k, sc.c, nullptr, In, Out, sc.D, sc.tag, sc.sid, sc.rs, sc.tile_body,
                                     sc.body_tiles, sc.ds, false, sc.ncfl, ee - start[q], sm, dp);
     else
-      stage_tile<STAGE, false, true>(sc.k, sc.c, nullptr, In, Out, sc.D, sc.tag, sc.sid, sc.rs, sc.tile_body,
+      stage_tile<STAGE, false, true, false, false, false, false, NT>(sc.k, sc.c, nullptr, In, Out, sc.D, sc.tag, sc.sid, sc.rs, sc.tile_body,
                                      sc.body_tiles, sc.ds, false, sc.ncfl, ee - start[q], sm, dp);
     __syncthreads();  // shared memory is reused by the next entry
   }
@@ -128,16 +141,18 @@ cudaError_t launch_dual_f32_batch_one(const StageBatch &b, int stage, int grid, 
   if (total == 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)(grid > 0 && grid < total ? grid : total));
-  cfg.blockDim = dim3(NTH);
+  const bool wide = dual_wide(b.plain_start[b.n], b.n);
+  cfg.blockDim = dim3(wide ? WIDE : NTH);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = pdl ? 1 : 0;
-  if (stage == 1) return cudaLaunchKernelEx(&cfg, k_dual_f32_batch_one<1>, b);
-  if (stage == 2) return cudaLaunchKernelEx(&cfg, k_dual_f32_batch_one<2>, b);
-  return cudaLaunchKernelEx(&cfg, k_dual_f32_batch_one<3>, b);
+#define IBM_DUAL_BATCH(S) \
+  (wide ? cudaLaunchKernelEx(&cfg, k_dual_f32_batch_one<S, WIDE>, b) : cudaLaunchKernelEx(&cfg, k_dual_f32_batch_one<S, NTH>, b))
+  return stage == 1 ? IBM_DUAL_BATCH(1) : stage == 2 ? IBM_DUAL_BATCH(2) : IBM_DUAL_BATCH(3);
+#undef IBM_DUAL_BATCH
 }
 
 // Start of a physical step: one thread per FP64 word of the 4-plane state.
@@ -174,18 +189,25 @@ void launch_dual_f32(const Consts &k, int stage, const float *In32, float *Out32
   dp.Out64 = Out64;
   dp.G = G;
   dp.Q0 = Q0;
-#define IBM_DUAL_PAIR(S)                                                                                          \
+#define IBM_DUAL_PAIR_N(S, N)                                                                                     \
   do {                                                                                                            \
     if (nb)                                                                                                       \
-      k_dual_f32<S, true><<<nb, NTH, 0, sb>>>(k, c, In32, Out32, D, tag, sid, rs, tile_body, body_tiles, ds, ncfl, \
-                                              dp);                                                                \
-    k_dual_f32<S, false><<<nt, NTH, 0, s>>>(k, c, In32, Out32, D, tag, sid, rs, tile_body, body_tiles, ds, ncfl,   \
-                                            dp);                                                                  \
+      k_dual_f32<S, true, N><<<nb, N, 0, sb>>>(k, c, In32, Out32, D, tag, sid, rs, tile_body, body_tiles, ds,      \
+                                               ncfl, dp);                                                         \
+    k_dual_f32<S, false, N><<<nt, N, 0, s>>>(k, c, In32, Out32, D, tag, sid, rs, tile_body, body_tiles, ds, ncfl,  \
+                                             dp);                                                                 \
   } while (0)
+#define IBM_DUAL_PAIR(S)            \
+  do {                              \
+    if (wide) IBM_DUAL_PAIR_N(S, WIDE); \
+    else IBM_DUAL_PAIR_N(S, NTH);   \
+  } while (0)
+  const bool wide = dual_wide(nt);
   if (stage == 1) IBM_DUAL_PAIR(1);
   else if (stage == 2) IBM_DUAL_PAIR(2);
   else IBM_DUAL_PAIR(3);
 #undef IBM_DUAL_PAIR
+#undef IBM_DUAL_PAIR_N
 }
 
 // Self-check of f32_to_f64 / f64_to_f32 against the hardware conversions of

@@ -123,23 +123,24 @@ __device__ __forceinline__ void dual_update_cell(const Consts &k, const PertCons
   // -(R' + BDF') with R' = -L and the BDF term aw W + G: BDF2 (3 W - 4 W^n + W^{n-1}) / (2 dt), BDF1 (W - W^n) / dt
   for (int q = 0; q < 4; q++) S[q] = fma(-aw, W[q], f32_to_f64(L[q]) - dp.G[id + q * P]);
   // pseudo-time coefficients (local dtau, preconditioning parameter) in FP32: they set the pseudo-time path,
-  // not the fixed point R' + BDF' = 0
+  // not the fixed point R' + BDF' = 0.  (Sums of products written out as fused multiply-adds here and in the divergence, so
+  // that blocks of either width give a case the same bits.)
   const float rf = f64_to_f32(r), irf = 1.f / rf, uf = f64_to_f32(u), vf = f64_to_f32(v);
   const float Tf = 1.f + f64_to_f32(Qk[3]), iTf = 1.f / Tf;
   const float csf = sqrtf(c.gamma * (c.R + f64_to_f32(Qk[0])) * irf), icsf = 1.f / csf;
-  const float Vm = sqrtf(uf * uf + vf * vf);
+  const float Vm = sqrtf(__fmaf_rn(uf, uf, __fmul_rn(vf, vf)));
   float Ur = fmaxf(fmaxf(Vm, 1.f), c.mu * irf / c.dmin);
   Ur = fminf(Ur, csf);
-  const float mr2 = (Ur * icsf) * (Ur * icsf);
-  const float up = 0.5f * Vm * (1.f + mr2);
-  const float om = 1.f - mr2;
-  const float cp_ = 0.5f * sqrtf(om * om * Vm * Vm + 4.f * Ur * Ur);
-  const float lam = (up + cp_) * (c.idx + c.idy) + c.vis * irf;
+  const float ui = __fmul_rn(Ur, icsf), mr2 = __fmul_rn(ui, ui);
+  const float up = __fmul_rn(__fmul_rn(0.5f, Vm), 1.f + mr2);
+  const float om = __fsub_rn(1.f, mr2), ov = __fmul_rn(om, Vm), ur = __fmul_rn(2.f, Ur);
+  const float cp_ = __fmul_rn(0.5f, sqrtf(__fmaf_rn(ov, ov, __fmul_rn(ur, ur))));
+  const float lam = __fmaf_rn(__fadd_rn(up, cp_), c.idx + c.idy, __fmul_rn(c.vis, irf));
   const float idtau = lam / c.cfl_tau;
-  const float af = bdf2 ? 1.5f * c.idt_phys : c.idt_phys;
-  const float thG = 1.f / (Ur * Ur) + iTf / c.cp, thJ = iTf / c.R;
-  const float sf = idtau + af;
-  const float tau = (thG * idtau + af * thJ) / sf;
+  const float af = bdf2 ? __fmul_rn(1.5f, c.idt_phys) : c.idt_phys;
+  const float thG = __fadd_rn(1.f / __fmul_rn(Ur, Ur), iTf / c.cp), thJ = iTf / c.R;
+  const float sf = __fadd_rn(idtau, af);
+  const float tau = __fmaf_rn(thG, idtau, __fmul_rn(af, thJ)) / sf;
   const double dH = fma(k.cp, Qk[3], half64(dq));
   double dQ[4];
   solve_precond(f32_to_f64(1.f / sf), f32_to_f64(tau), r, ir, u, v, -f32_to_f64(rf * iTf), k.cp, dH, S, dQ);

@@ -111,8 +111,8 @@ void launch_compact_stencils(const Consts &k, const ibm_stencil *st, RStencil32 
 // A case stepped on its own: one block per tile (plain) or body-tile slot.
 // MINB: resident blocks per SM the register allocation must allow (8: 64 registers and the most that shared memory
 // holds; 7: 72; 6: 80) -- the autotuner picks one per grid size.
-template <int STAGE, bool BODY, int MINB>
-__global__ void __launch_bounds__(NTH, MINB) k_stage_f32(Consts k, PertConsts c, float *Mn, const float *__restrict__ In,
+template <int STAGE, bool BODY, int MINB, int NT = NTH>
+__global__ void __launch_bounds__(NT, MINB) k_stage_f32(Consts k, PertConsts c, float *Mn, const float *__restrict__ In,
                                                    float *Out, double *D, const uint8_t *__restrict__ tag,
                                                    const int *__restrict__ sid, const RStencil32 *__restrict__ rs,
                                                    const uint8_t *__restrict__ tile_body,
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_stage_f32(Consts k, PertConsts c,
                                                    unsigned int ncfl, const __grid_constant__ CUtensorMap tmap,
                                                    int use_tma) {
   __shared__ TileSmem sm;
-  stage_tile<STAGE, BODY, false, true>(k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, ds, fuse_cfl, ncfl,
+  stage_tile<STAGE, BODY, false, true, false, false, false, NT>(k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, ds, fuse_cfl, ncfl,
                                        (int)blockIdx.x, sm, DualPtrs{}, use_tma ? &tmap : nullptr);
 }
 
@@ -131,8 +131,8 @@ __global__ void __launch_bounds__(NTH, MINB) k_stage_f32(Consts k, PertConsts c,
 // block of this one has started; its blocks then wait at the top for this
 // grid to complete and its stores to become visible, so the next stage's
 // blocks are resident when the tail of this one ends.
-template <int STAGE, int MINB>
-__global__ void __launch_bounds__(NTH, MINB)
+template <int STAGE, int MINB, int NT = NTH>
+__global__ void __launch_bounds__(NT, MINB)
     k_stage_f32_one(Consts k, PertConsts c, float *Mn, const float *__restrict__ In, float *Out, double *D,
                     const uint8_t *__restrict__ tag, const int *__restrict__ sid, const RStencil32 *__restrict__ rs,
                     const uint8_t *__restrict__ tile_body, const int *__restrict__ body_tiles, int nb, DevState *ds,
@@ -144,18 +144,18 @@ __global__ void __launch_bounds__(NTH, MINB)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int b = (int)blockIdx.x;
   if (b < nb)
-    stage_tile<STAGE, true, false, true>(k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, ds, fuse_cfl,
+    stage_tile<STAGE, true, false, true, false, false, false, NT>(k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, ds, fuse_cfl,
                                          ncfl, b, sm, DualPtrs{}, use_tma ? &tmap : nullptr);
   else
-    stage_tile<STAGE, false, false, true>(k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, ds, fuse_cfl,
+    stage_tile<STAGE, false, false, true, false, false, false, NT>(k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, ds, fuse_cfl,
                                           ncfl, b - nb, sm, DualPtrs{}, use_tma ? &tmap : nullptr);
 }
 
 // The same stage with the TVD-2 reconstruction (Sec. 2) and / or the quadratic IB / ghost reconstruction
 // (Sec. 4.5, Sec. 5) compiled in: a case with either takes this kernel in every launch form (the two-stream
 // form runs it as one launch on the case stream), so that the default kernels carry neither.
-template <int STAGE, bool TVD, bool QUAD>
-__global__ void __launch_bounds__(NTH, 7)
+template <int STAGE, bool TVD, bool QUAD, int NT = NTH>
+__global__ void __launch_bounds__(NT, NT == NTH ? 7 : WIDE_BLOCKS)
     k_stage_f32_var(Consts k, PertConsts c, float *Mn, const float *__restrict__ In, float *Out, double *D,
                     const uint8_t *__restrict__ tag, const int *__restrict__ sid, const RStencil32 *__restrict__ rs,
                     const uint8_t *__restrict__ tile_body, const int *__restrict__ body_tiles, int nb, DevState *ds,
@@ -168,14 +168,24 @@ __global__ void __launch_bounds__(NTH, 7)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int b = (int)blockIdx.x;
   if (b < nb)
-    stage_tile<STAGE, true, false, true, false, TVD, QUAD>(k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles,
+    stage_tile<STAGE, true, false, true, false, TVD, QUAD, NT>(k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles,
                                                            ds, fuse_cfl, ncfl, b, sm, DualPtrs{},
                                                            use_tma ? &tmap : nullptr, rsq);
   else
-    stage_tile<STAGE, false, false, true, false, TVD, QUAD>(k, c, Mn, In, Out, D, tag, sid, rs, tile_body,
+    stage_tile<STAGE, false, false, true, false, TVD, QUAD, NT>(k, c, Mn, In, Out, D, tag, sid, rs, tile_body,
                                                             body_tiles, ds, fuse_cfl, ncfl, b - nb, sm, DualPtrs{},
                                                             use_tma ? &tmap : nullptr, rsq);
 }
+
+// Wide blocks where the tiles leave the chip short of work and a step lasts as long as its chains of tiles: up to one
+// wave of wide blocks, or two where body tiles, the longest chains, are among them.  Per step, 128 threads against 288
+// (the step before the packed tile in brackets): no body 64 x 64 29 us, 18 (23), 640 x 320 46, 45 (48), 768 x 384 49, 57
+// (60); cylinder 64 x 64 37, 29 (35), 256 x 128 47, 35 (43), 512 x 256 50, 40 (51), 640 x 320 58, 45 (59), 1024 x 512
+// 75, 90 (92).
+extern "C" int ibm__stage_wide(int nt, int nb, int sms) {
+  return nt <= WIDE_BLOCKS * sms || (nb > 0 && nt <= 2 * WIDE_BLOCKS * sms);
+}
+bool stage_wide(int nt, int nb) { return ibm__stage_wide(nt, nb, sm_count()) != 0; }
 
 int stage_tiles(const Consts &k) { return ((k.nx + TX - 1) / TX) * ((k.ny + TY - 1) / TY); }
 
@@ -275,9 +285,15 @@ void launch_stage_f32(const Consts &k, int stage, float *Mn, const float *In, fl
   std::memset(&tm, 0, sizeof tm);
   if (tmap) tm = *tmap;
   const int ut = tmap ? 1 : 0;
+  const bool wide = stage_wide(nt, nb);
 #define IBM_ARGS k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, ds, fuse_cfl, ncfl, tm, ut
 #define IBM_STAGE_PAIR(S)                                                      \
   do {                                                                         \
+    if (wide) {                                                                \
+      if (nb && with_body) k_stage_f32<S, true, WIDE_BLOCKS, WIDE><<<nb, WIDE, 0, sb>>>(IBM_ARGS); \
+      k_stage_f32<S, false, WIDE_BLOCKS, WIDE><<<nt, WIDE, 0, s>>>(IBM_ARGS);  \
+      break;                                                                   \
+    }                                                                          \
     if (nb && with_body) k_stage_f32<S, true, 0><<<nb, NTH, 0, sb>>>(IBM_ARGS); \
     if (plain_variant == 1)                                                    \
       k_stage_f32<S, false, 7><<<nt, NTH, 0, s>>>(IBM_ARGS);                   \
@@ -308,19 +324,23 @@ cudaError_t launch_stage_f32_one(const Consts &k, int stage, float *Mn, const fl
   const int ut = tmap ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)(nt + nb));
-  cfg.blockDim = dim3(NTH);
+  const bool wide = stage_wide(nt, nb);
+  cfg.blockDim = dim3(wide ? WIDE : NTH);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = pdl ? 1 : 0;
-#define IBM_ONE(S, MB)                                                                                        \
-  cudaLaunchKernelEx(&cfg, k_stage_f32_one<S, MB>, k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, nb, \
-                     ds, fuse_cfl, ncfl, tm, ut)
-#define IBM_ONE_V(S) (plain_variant == 1 ? IBM_ONE(S, 7) : plain_variant == 2 ? IBM_ONE(S, 6) : IBM_ONE(S, 8))
-#define IBM_VAR(S, T, Q)                                                                                       \
-  cudaLaunchKernelEx(&cfg, k_stage_f32_var<S, T, Q>, k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, nb, \
+#define IBM_ONE(S, ...)                                                                                       \
+  cudaLaunchKernelEx(&cfg, k_stage_f32_one<S, __VA_ARGS__>, k, c, Mn, In, Out, D, tag, sid, rs, tile_body,        \
+                     body_tiles, nb, ds, fuse_cfl, ncfl, tm, ut)
+#define IBM_ONE_V(S)                                                                                           \
+  (wide ? IBM_ONE(S, WIDE_BLOCKS, WIDE)                                                                        \
+        : plain_variant == 1 ? IBM_ONE(S, 7) : plain_variant == 2 ? IBM_ONE(S, 6) : IBM_ONE(S, 8))
+#define IBM_VAR(S, T, Q) (wide ? IBM_VAR_N(S, T, Q, WIDE) : IBM_VAR_N(S, T, Q, NTH))
+#define IBM_VAR_N(S, T, Q, N)                                                                                  \
+  cudaLaunchKernelEx(&cfg, k_stage_f32_var<S, T, Q, N>, k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, nb, \
                      ds, fuse_cfl, ncfl, tm, ut, rsq)
 #define IBM_VAR_S(S) \
   (k.tvd2 && k.quad ? IBM_VAR(S, true, true) : k.tvd2 ? IBM_VAR(S, true, false) : IBM_VAR(S, false, true))
@@ -328,6 +348,7 @@ cudaError_t launch_stage_f32_one(const Consts &k, int stage, float *Mn, const fl
                                    : (stage == 1 ? IBM_ONE_V(1) : stage == 2 ? IBM_ONE_V(2) : IBM_ONE_V(3));
 #undef IBM_VAR_S
 #undef IBM_VAR
+#undef IBM_VAR_N
 #undef IBM_ONE_V
 #undef IBM_ONE
   return e;

@@ -405,6 +405,8 @@ __host__ inline PertConsts pert_consts(const Consts &k) {
 // registers, six blocks); with_body = false launches the plain kernel only
 // (autotuning).
 constexpr int PLAIN_VARIANTS = 3;
+// Wide blocks (stage32.cuh) for the explicit stage of nt tiles and nb body-tile slots.
+bool stage_wide(int nt, int nb);
 void launch_stage_f32(const Consts &k, int stage, float *Mn, const float *In, float *Out, double *D,
                       const uint8_t *tag, const int *sid, const RStencil32 *rs, const uint8_t *tile_body,
                       const int *body_tiles, int body_cap, DevState *ds, bool fuse_cfl, cudaStream_t s,
@@ -438,7 +440,9 @@ struct StepSched {
   unsigned int pad;
   // followed by one completion count per tile
 };
-constexpr int STEP_VARIANTS = 2;  // register budget: 0 -> 72 registers (seven blocks per SM), 1 -> 80 (six)
+// variant of the persistent kernel by the grid's tiles: 1 wide blocks (up to two waves of them), 2 four blocks of 128
+// threads per SM (up to eight tiles per SM), 0 seven
+int step_f32_variant(const Consts &k);
 size_t step_sched_bytes(const Consts &k);
 // grid of the persistent kernel: resident blocks per SM x SMs, at most 3 x tiles
 int step_f32_grid(const Consts &k, int variant);

@@ -175,6 +175,13 @@ __device__ __forceinline__ void ldfss_pert2(const PertConsts &c, f2 drL, f2 unL,
 // the face storage (eight blocks of 27.5 KB per SM) it is 2.56 ms: issue slots 71% busy, FP32 pipe 57%, the rest the
 // phases' barriers.
 constexpr int NTH = 128;
+// A wide block is 288 threads on the same tile: one pair of cells, half a reconstruction item, one pair of faces (there
+// are 272) and one cell each, for a chain less than half as long, three blocks per SM at 72 registers.  It serves grids
+// of few tiles (ibm__stage_wide, ibm__dual_wide).
+constexpr int WIDE = 288, WIDE_BLOCKS = 3;
+// Blocks of 128 threads of the block-table kernels per SM: 16 requests 11.3 ms, with seven (72 registers) 11.6, with six
+// (80, hardly a spill) 11.4
+constexpr int BATCH_BLOCKS = 8;
 constexpr int TX = STAGE_TILE, TY = STAGE_TILE, HX = TX + 2 * NG, HY = TY + 2 * NG;
 // Shared memory is laid out for pairs: a thread reconstructs two adjacent rows (x direction) or columns (y direction)
 // and forms the fluxes of their two faces with packed arithmetic.  The face values of a direction are [variable][face
@@ -184,8 +191,7 @@ constexpr int TX = STAGE_TILE, TY = STAGE_TILE, HX = TX + 2 * NG, HY = TY + 2 * 
 // 8 row pairs x 2 halves x 2 variables fall in 32 banks.
 constexpr int FP = TX, NF1 = (TX + 1) * FP, NFD = 4 * NF1;  // one variable's, one direction's and side's face values
 constexpr int VP = 498;
-constexpr int CELLS = TX * TY / NTH, CROWS = NTH / TX;  // cells a thread updates, rows between them
-static_assert(CELLS == 2 && TX == TY && VP >= HY * HX && VP % 2 == 0 && HX % 2 == 0, "pairs are 8-byte aligned");
+static_assert(TX == TY && VP >= HY * HX && VP % 2 == 0 && HX % 2 == 0, "pairs are 8-byte aligned");
 constexpr int RB_MAX = 192;  // IB / ghost nodes a body tile's loaded region may hold
 
 // Shared memory of one tile.  face holds, in turn: the TMA box of the tile's
@@ -205,7 +211,7 @@ struct TileSmem {
   __device__ __forceinline__ int *rbe() { return rbm() + RB_MAX; }
   float wm[7];    // wall velocity and acceleration at the stage time; 1 if Eq. 7 applies (else 0); the rotation
                   // rate and its rate of change of a pitching body (else 0)
-  float lred[NTH / 32];  // per-warp maxima of the CFL reduction
+  float lred[WIDE / 32];  // per-warp maxima of the CFL reduction
   int nrb[2];     // listed IB and ghost nodes (body tiles)
 };
 static_assert(RB_MAX * (sizeof(RStencil32) + 2 * sizeof(int)) <= sizeof(float) * 4 * NFD, "node stencils fit the face storage");
@@ -283,6 +289,7 @@ __device__ __forceinline__ float cfl_lambda(const Consts &k, const PertConsts &c
 
 // block maximum of lam (all threads call), then the grid-wide maximum and
 // dt through the last-block pattern
+template <int NT>
 __device__ __forceinline__ void cfl_block_max(const Consts &k, float lam, float *red, DevState *ds,
                                               unsigned int nblocks, bool defer) {
   for (int off = 16; off > 0; off >>= 1) lam = fmaxf(lam, __shfl_xor_sync(0xffffffffu, lam, off));
@@ -290,7 +297,7 @@ __device__ __forceinline__ void cfl_block_max(const Consts &k, float lam, float 
   __syncthreads();
   if (threadIdx.x == 0) {
     float m = red[0];
-    for (int w = 1; w < NTH / 32; w++) m = fmaxf(m, red[w]);
+    for (int w = 1; w < NT / 32; w++) m = fmaxf(m, red[w]);
     atomicMax(&ds->lmax_bits, (unsigned long long)__double_as_longlong((double)m));
     finish_cfl(k, ds, nblocks, defer);
   }
@@ -430,7 +437,7 @@ static __device__ __noinline__ void rebuild_ib(const Consts &k, const PertConsts
 // TVD: the second-order TVD reconstruction in place of WENO5 (Sec. 2), compiled into its own kernels so that
 // the WENO5 kernels carry no branch for it.
 template <int STAGE, bool BODY, bool DUAL = false, bool TMA = false, bool PERSIST = false, bool TVD = false,
-          bool QUAD = false>
+          bool QUAD = false, int NT = NTH>
 __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c, float *Mn,
                                            const float *__restrict__ In, float *Out, double *D,
                                            const uint8_t *__restrict__ tag,
@@ -439,6 +446,8 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
                                            DevState *ds, bool fuse_cfl, unsigned int ncfl, int blk, TileSmem &sm,
                                            const DualPtrs &dp = DualPtrs{}, const CUtensorMap *tmap = nullptr,
                                            const RStencilQ *__restrict__ rsq = nullptr) {
+  static_assert(NT == NTH || NT == WIDE, "threads of a block");
+  constexpr int CROWS = NT / TX, CELLS = (TY + CROWS - 1) / CROWS;  // rows between a thread's cells, cells it updates
   static_assert(!TMA || 4 * HY * TMA_W <= RB_MAX * (int)sizeof(RStencil32) / 4, "TMA box ahead of the listed nodes");
   float *s_face = sm.face;
   unsigned long long &s_mbar = sm.mbar;
@@ -480,7 +489,8 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
 #pragma unroll
   for (int h = 0; h < CELLS; h++) {
     const int ci = i0 + tx, cj = j0 + ty0 + h * CROWS;
-    tags[h] = ci < k.nx && cj < k.ny ? tag[cj * k.nx + ci] : (uint8_t)SOLID;
+    const bool in = (NT == NTH || ty0 < TY) && ci < k.nx && cj < k.ny;  // (wide: threads beyond the tile's cells)
+    tags[h] = in ? tag[cj * k.nx + ci] : (uint8_t)SOLID;
     // stages 1 and 3 also keep the IB / ghost nodes of U^n current; stage 2 only needs the cells it advances
     work |= STAGE == 2 ? advanced(k, tags[h]) : tags[h] != SOLID;
   }
@@ -540,11 +550,11 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
     wm[6] = (float)al;
   }
   // body tiles: the listed nodes of the thread's cells, on their way while the copy is
-  int esid[(HX * HY / 2 + NTH - 1) / NTH][2];
+  int esid[(HX * HY / 2 + NT - 1) / NT][2];
   if (BODY && interior) {
 #pragma unroll
-    for (int r = 0; r < (HX * HY / 2 + NTH - 1) / NTH; r++) {
-      const int m = min((int)threadIdx.x + r * NTH, HX * HY / 2 - 1), b = m / (HX / 2), a = 2 * (m - b * (HX / 2));
+    for (int r = 0; r < (HX * HY / 2 + NT - 1) / NT; r++) {
+      const int m = min((int)threadIdx.x + r * NT, HX * HY / 2 - 1), b = m / (HX / 2), a = 2 * (m - b * (HX / 2));
       const int *ps = sid + (j0 - NG + b) * k.nx + i0 - NG + a;
       esid[r][0] = ps[0];
       esid[r][1] = ps[1];
@@ -586,10 +596,10 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
     }
   };
   if (interior) {  // no domain mapping: two cells at a time, from the tensor copy's box or from memory
-    constexpr int NC = (HX * HY / 2 + NTH - 1) / NTH;
+    constexpr int NC = (HX * HY / 2 + NT - 1) / NT;
 #pragma unroll
     for (int r = 0; r < NC; r++) {
-      const int m = threadIdx.x + r * NTH, b = m / (HX / 2), a = 2 * (m - b * (HX / 2));
+      const int m = threadIdx.x + r * NT, b = m / (HX / 2), a = 2 * (m - b * (HX / 2));
       if (m >= HX * HY / 2) break;
       f2 w[4], u, v, pp, Tp;
       if (TMA && tma) {
@@ -615,12 +625,12 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
     }
   } else {
     // every load of the thread's cells before the first use
-    constexpr int NC = (HX * HY + NTH - 1) / NTH;
+    constexpr int NC = (HX * HY + NT - 1) / NT;
     float w[NC][4];
     int e[NC];
 #pragma unroll
     for (int r = 0; r < NC; r++) {
-      const int m = threadIdx.x + r * NTH;
+      const int m = threadIdx.x + r * NT;
       int gi = i0 - NG + m % HX, gj = j0 - NG + m / HX;
       const bool in = m < HX * HY && halo_map(k, gi, gj);
       const float *p = In + cidx(k, gi, gj);
@@ -630,7 +640,7 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
     }
 #pragma unroll
     for (int r = 0; r < NC; r++) {
-      const int m = threadIdx.x + r * NTH;
+      const int m = threadIdx.x + r * NT;
       if (m >= HX * HY) break;
       float u, v, pp, Tp;
       pert_prim(c, w[r][0], w[r][1], w[r][2], w[r][3], u, v, pp, Tp);
@@ -648,7 +658,7 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
   if (PERSIST && TMA && tma && threadIdx.x == 0) sm.mbar_phase ^= 1u;
   if (BODY) {
     const int nib = min(s_nrb[0], RB_MAX), ngh = min(s_nrb[1], RB_MAX - nib);
-    for (int r = threadIdx.x; r < nib + ngh; r += NTH) {
+    for (int r = threadIdx.x; r < nib + ngh; r += NT) {
       const int slot = r < nib ? r : RB_MAX - 1 - (r - nib);
       s_rs[slot] = rs[s_rbe[slot]];
     }
@@ -659,7 +669,7 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
     // dependent global loads) overlap; the node's first lane sums the corners in stencil order
     for (int pass = k.ib_advance ? 1 : 0; pass < 2; pass++) {  // IB nodes (pass 0) unless advanced
       const int np = pass == 0 ? nib : ngh;
-      for (int t0 = 0; t0 < 4 * np; t0 += NTH) {  // block-uniform: every lane takes part in the shuffles
+      for (int t0 = 0; t0 < 4 * np; t0 += NT) {  // block-uniform: every lane takes part in the shuffles
         const int t = (t0 + (int)threadIdx.x) >> 2, cq = threadIdx.x & 3, r = pass == 0 ? t : RB_MAX - 1 - t;
         const bool listed_node = t < np;
         bool node = false;
@@ -762,18 +772,25 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
   // Every operation of the window is one packed instruction for both lines (40 and 4 reciprocals for 4 face states),
   // and the results are stored as pairs.
   static_assert(TX == 16 && TY == 16, "items: 2 directions x 4 variables x 2 halves x 8 line pairs");
-  static_assert(NTH == 128, "one item per thread");
-  {
-    const int lp = threadIdx.x & 7, half = threadIdx.x >> 3 & 1, v = threadIdx.x >> 4 & 3;
-    const bool xdir = threadIdx.x < 64;
+  // Wide blocks break each half in two (five and four centres), for a chain of half the length.
+  constexpr int WN = NT == NTH ? 9 : 5;
+  if (NT == NTH || threadIdx.x < 256) {
+    const int lp = threadIdx.x & 7, half = threadIdx.x >> 3 & 1, v = threadIdx.x >> 4 & 3, part = threadIdx.x >> 7;
+    const bool xdir = (threadIdx.x & 64) == 0;
     const int ls = xdir ? 1 : HX, ps = xdir ? HX : 1;  // strides along the line and between the pair's lines
-    const int p0 = 2 + 9 * half;
-    const float *lp0 = &sm.q[v][xdir ? (NG + 2 * lp) * HX : NG + 2 * lp] + (p0 - 2) * ls, *lp1 = lp0 + ps;
-    // left state of face pc - 2 (between cells pc and pc + 1), right state of face pc - 3
-    // at face_slot(p0 - 2 + i, 2 lp), formed from the slot's bits: p0 - 2 = 9 half is half mod 2
-    float *const of = s_face + (xdir ? 0 : 2 * NFD) + v * NF1 + (p0 - 2) * FP;
+    const int w0 = 9 * half + 5 * part;                // the item's first window, centred at local w0 + 2
+    const float *lp0 = &sm.q[v][xdir ? (NG + 2 * lp) * HX : NG + 2 * lp] + w0 * ls, *lp1 = lp0 + ps;
+    // window w gives the left state of face w (between local cells w + 2 and w + 3) and the right state of face w - 1,
+    // at face_slot(w, 2 lp), formed from the slot's bits: with two halves w0 is half mod 2
+    float *const of = s_face + (xdir ? 0 : 2 * NFD) + v * NF1 + w0 * FP;
     const int slot0 = 2 * lp ^ 8 * half, hp = 2 * half;
     auto store = [&](int i, f2 qL, f2 qR, float *&prev) {
+      if constexpr (NT == WIDE) {
+        const int w = w0 + i, slot = 2 * lp;
+        if (w <= TX) st2(of + i * FP + (slot ^ (w & 14)), qL);
+        if (w >= 1) st2(of + (i - 1) * FP + (slot ^ ((w - 1) & 14)) + NFD, qR);
+        return;
+      }
       float *const p = of + i * FP + (slot0 ^ (i & 1 ? (i & 14) + hp : i & 14));
       if (i < 8 || half == 0) st2(p, qL);
       if (i > 0) st2(prev + NFD, qR);
@@ -792,7 +809,8 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
         return m;
       };
 #pragma unroll
-      for (int i = 0; i < 9; i++) {
+      for (int i = 0; i < WN; i++) {
+        if (NT == WIDE && i == 4 && part == 1) break;  // the second part (whole warps) has four windows
         const f2 f3 = {lp0[(i + 3) * ls], lp1[(i + 3) * ls]};
         const f2 a = f2c - f1, b = f3 - f2c;
         // minmod(a, b) for the left state at the right face, minmod(-b, -a) = -minmod(a, b) for the right state
@@ -813,7 +831,8 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
       f2 am = fma2((13.f / 12.f) * dm, dm, eps), ac = fma2((13.f / 12.f) * dc, dc, eps);
       f2 xm = 0.5f * gm, x0 = 0.5f * g0, ym = (1.f / 6.f) * dm, yc = (1.f / 6.f) * dc;
 #pragma unroll
-      for (int i = 0; i < 9; i++) {
+      for (int i = 0; i < WN; i++) {
+        if (NT == WIDE && i == 4 && part == 1) break;  // the second part (whole warps) has four windows
         const f2 fe = {lp0[(i + 4) * ls], lp1[(i + 4) * ls]};
         const f2 g1 = fe - fd, dn = g1 - g0;
         const f2 an = fma2((13.f / 12.f) * dn, dn, eps), yp = (1.f / 6.f) * dn;
@@ -845,7 +864,7 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
 
   const float mu = c.mu, kap = c.kappa, idx = c.idx, idy = c.idy;
   // an item is the faces of two adjacent rows (x direction) or columns (y direction) at one place of the line
-  for (int m = threadIdx.x; m < 2 * (TX + 1) * (TX / 2); m += NTH) {
+  for (int m = threadIdx.x; m < 2 * (TX + 1) * (TX / 2); m += NT) {
     const bool xdir = m < (TX + 1) * (TX / 2);
     const int mm = xdir ? m : m - (TX + 1) * (TX / 2), f = mm >> 3, l = 2 * (mm & 7);
     float *fl = s_face + (xdir ? 0 : 2 * NFD) + sm.face_slot(f, l);  // left states, then the flux; right states NFD further
@@ -927,7 +946,7 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
       const float *x0 = s_face + sm.face_slot(tx, ty), *x1 = s_face + sm.face_slot(tx + 1, ty);
       const float *y0 = s_face + 2 * NFD + sm.face_slot(ty, tx), *y1 = s_face + 2 * NFD + sm.face_slot(ty + 1, tx);
       for (int v = 0; v < 4; v++)
-        L[v] = -((x1[v * NF1] - x0[v * NF1]) * idx + (y1[v * NF1] - y0[v * NF1]) * idy);
+        L[v] = -__fmaf_rn(x1[v * NF1] - x0[v * NF1], idx, __fmul_rn(y1[v * NF1] - y0[v * NF1], idy));
       if (DUAL) {
         dual_update_cell<STAGE>(k, c, id, P, L, dp, Out, ds->steps > 0);
       } else if (STAGE == 1) {
@@ -954,14 +973,15 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
     }
   }
   // one call site for the whole block (the reduction has a barrier)
-  if (STAGE == 3 && fuse_cfl) cfl_block_max(k, lam, lred, ds, ncfl, PERSIST);
+  if (STAGE == 3 && fuse_cfl) cfl_block_max<NT>(k, lam, lred, ds, ncfl, PERSIST);
 }
 
 // The block's copy of a table entry's case.  Indexed in the kernel's parameters, the constants and pointers were read
 // early and held across the tile in spilled registers; shared memory is read where a value is used.
+template <int NT>
 __device__ __forceinline__ void load_case(StageCase &dst, const StageCase &src) {
   static_assert(sizeof(StageCase) % 8 == 0, "copied in 8-byte words");
-  for (int i = threadIdx.x; i < (int)(sizeof(StageCase) / 8); i += NTH)
+  for (int i = threadIdx.x; i < (int)(sizeof(StageCase) / 8); i += NT)
     reinterpret_cast<unsigned long long *>(&dst)[i] = reinterpret_cast<const unsigned long long *>(&src)[i];
   __syncthreads();
 }

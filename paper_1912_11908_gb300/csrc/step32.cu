@@ -70,10 +70,14 @@ __device__ __forceinline__ void wait_neighbours(const Consts &k, const unsigned 
   __syncthreads();
 }
 
-// MINB: resident blocks per SM the register allocation must allow (7: 72
-// registers, 6: 80 registers).
-template <int MINB>
-__global__ void __launch_bounds__(NTH, MINB)
+// MINB: resident blocks per SM the register allocation must allow; NT threads
+// of a block.  A step of 128-thread blocks against wide ones and against four
+// of 128 threads per SM (the form before the packed tile in brackets), without
+// a body and around a cylinder: 512 x 256 62 us, 46 (57) and 87, 62 (74);
+// 768 x 384 67, 70, 66 (67) and 95, 73, 82 (83); 1024 x 512 94, 113, 109 (95)
+// and 110, 119, 111 (100).
+template <int MINB, int NT = NTH>
+__global__ void __launch_bounds__(NT, MINB)
     k_step_f32(Consts k, PertConsts c, float *M, float *F1, float *F2, double *D, const uint8_t *__restrict__ tag,
                const int *__restrict__ sid, const RStencil32 *__restrict__ rs, const uint8_t *__restrict__ tile_body,
                const int *__restrict__ body_tiles, int body_cap, DevState *ds, StepSched *sch, bool fuse_cfl,
@@ -118,10 +122,10 @@ __global__ void __launch_bounds__(NTH, MINB)
 #define IBM_ITEM(S, IN, OUT, TM)                                                                                    \
   do {                                                                                                              \
     if (body)                                                                                                       \
-      stage_tile<S, true, false, true, true>(k, c, M, IN, OUT, D, tag, sid, rs, tile_body, nullptr, ds, fuse_cfl,   \
+      stage_tile<S, true, false, true, true, false, false, NT>(k, c, M, IN, OUT, D, tag, sid, rs, tile_body, nullptr, ds, fuse_cfl,   \
                                              (unsigned int)nt, tile, sm, DualPtrs{}, use_tma ? &TM : nullptr);      \
     else                                                                                                            \
-      stage_tile<S, false, false, true, true>(k, c, M, IN, OUT, D, tag, sid, rs, tile_body, nullptr, ds, fuse_cfl,  \
+      stage_tile<S, false, false, true, true, false, false, NT>(k, c, M, IN, OUT, D, tag, sid, rs, tile_body, nullptr, ds, fuse_cfl,  \
                                               (unsigned int)nt, tile, sm, DualPtrs{}, use_tma ? &TM : nullptr);     \
   } while (0)
     if (st == 1) IBM_ITEM(1, M, F1, tm1);
@@ -157,11 +161,16 @@ __global__ void __launch_bounds__(NTH, MINB)
 
 size_t step_sched_bytes(const Consts &k) { return sizeof(StepSched) + sizeof(unsigned int) * (size_t)stage_tiles(k); }
 
+int step_f32_variant(const Consts &k) {
+  const int nt = stage_tiles(k), sms = sm_count();
+  return nt <= 2 * WIDE_BLOCKS * sms ? 1 : nt <= 8 * sms ? 2 : 0;
+}
+
 int step_f32_grid(const Consts &k, int variant) {
-  int dev = 0, sms = 0, per = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (variant == 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_step_f32<6>, NTH, 0);
+  const int sms = sm_count();
+  int per = 0;
+  if (variant == 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_step_f32<WIDE_BLOCKS, WIDE>, WIDE, 0);
+  else if (variant == 2) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_step_f32<4>, NTH, 0);
   else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_step_f32<7>, NTH, 0);
   long long g = (long long)per * sms;
   const long long items = 3LL * stage_tiles(k);
@@ -182,7 +191,7 @@ cudaError_t launch_step_f32(const Consts &k, float *M, float *F1, float *F2, dou
   // all blocks resident at once
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)grid);
-  cfg.blockDim = dim3(NTH);
+  cfg.blockDim = dim3(variant == 1 ? WIDE : NTH);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -191,7 +200,10 @@ cudaError_t launch_step_f32(const Consts &k, float *M, float *F1, float *F2, dou
   cfg.attrs = at;
   cfg.numAttrs = 1;
   if (variant == 1)
-    return cudaLaunchKernelEx(&cfg, k_step_f32<6>, k, c, M, F1, F2, D, tag, sid, rs, tile_body, body_tiles, body_cap,
+    return cudaLaunchKernelEx(&cfg, k_step_f32<WIDE_BLOCKS, WIDE>, k, c, M, F1, F2, D, tag, sid, rs, tile_body,
+                              body_tiles, body_cap, ds, sch, fuse_cfl, tm[0], tm[1], tm[2], ut, s_first, s_last);
+  if (variant == 2)
+    return cudaLaunchKernelEx(&cfg, k_step_f32<4>, k, c, M, F1, F2, D, tag, sid, rs, tile_body, body_tiles, body_cap,
                               ds, sch, fuse_cfl, tm[0], tm[1], tm[2], ut, s_first, s_last);
   return cudaLaunchKernelEx(&cfg, k_step_f32<7>, k, c, M, F1, F2, D, tag, sid, rs, tile_body, body_tiles, body_cap,
                             ds, sch, fuse_cfl, tm[0], tm[1], tm[2], ut, s_first, s_last);

@@ -35,3 +35,31 @@ def test_shape_is_the_least_work_of_the_fullest_sm(shape):
         cost = [-(-(-(-nx // tx) * -(-ny // ty)) // sms) * w for (tx, ty), w in zip(TILES, work)]
         assert cost[shape(nx, ny, sms)] == min(cost), (nx, ny, sms)
     assert shape(257, 131, 152) == 1 and shape(768, 384, 152) == 0 and shape(64, 64, 152) == 2
+
+
+@pytest.fixture(scope="module")
+def wide():
+    from paper_1912_11908_gb300 import _build, ibm as mod
+    _build.build()
+    f = mod.lib().ibm__stage_wide
+    f.argtypes = [ctypes.c_int] * 3
+    f.restype = ctypes.c_int
+    return f
+
+
+def test_wide_blocks_for_few_tiles(wide):
+    """One wave of wide blocks (three per SM) without body tiles, two with them."""
+    for sms in (1, 76, 148, 152):
+        for nt, nb, want in ((1, 0, 1), (3 * sms, 0, 1), (3 * sms + 1, 0, 0), (3 * sms + 1, 1, 1), (6 * sms, 9, 1),
+                             (6 * sms + 1, 9, 0)):
+            assert bool(wide(nt, nb, sms)) == bool(want), (nt, nb, sms)
+
+
+def test_wide_blocks_in_dual_time(wide):
+    """Up to sixteen tiles per SM for a case alone, six for a group."""
+    from paper_1912_11908_gb300 import ibm as mod
+    f = mod.lib().ibm__dual_wide
+    f.argtypes = [ctypes.c_int] * 3
+    f.restype = ctypes.c_int
+    for sms in (1, 152):
+        assert [f(16 * sms, 1, sms), f(16 * sms + 1, 1, sms), f(6 * sms, 2, sms), f(6 * sms + 1, 2, sms)] == [1, 0, 1, 0]
