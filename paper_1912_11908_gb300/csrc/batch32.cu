@@ -48,6 +48,23 @@ __global__ void __launch_bounds__(NT, NT == NTH ? BATCH_BLOCKS : WIDE_BLOCKS) k_
   }
 }
 
+// Blocks of the table's stage kernel resident per SM.
+extern "C" int ibm__batch_blocks_per_sm(int wide, int tvd, int quad) {
+  int per = 0;
+#define IBM_OCC(T, Q)                                                                                                 \
+  (wide ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_stage_f32_batch_one<1, T, Q, WIDE>, WIDE, 0)          \
+        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_stage_f32_batch_one<1, T, Q, NTH>, NTH, 0))
+  const cudaError_t e = tvd ? (quad ? IBM_OCC(true, true) : IBM_OCC(true, false))
+                            : (quad ? IBM_OCC(false, true) : IBM_OCC(false, false));
+#undef IBM_OCC
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess ? per : 0;
+}
+
+int batch_stage_blocks(const StageBatch &b) {
+  return ibm__batch_blocks_per_sm(stage_wide(b.plain_start[b.n], b.body_start[b.n]), b.cs[0].k.tvd2, b.cs[0].k.quad);
+}
+
 cudaError_t launch_stage_f32_batch_one(const StageBatch &b, int stage, int grid, bool pdl, cudaStream_t s) {
   const int total = b.body_start[b.n] + b.plain_start[b.n];
   if (total == 0) return cudaSuccess;

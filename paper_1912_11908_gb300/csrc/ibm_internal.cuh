@@ -527,6 +527,8 @@ void fill_stage_case(const Consts &k, float *M, float *F1, float *F2, double *D,
 // entries: one block per entry; fewer: persistent blocks striding over the
 // table); pdl: chained to the previous launch by programmatic dependent launch.
 cudaError_t launch_stage_f32_batch_one(const StageBatch &b, int stage, int grid, bool pdl, cudaStream_t s);
+// resident blocks per SM of that launch's kernel
+int batch_stage_blocks(const StageBatch &b);
 // Dual-time pseudo stage `stage` of every (dual-time, not TVD-2) case of the
 // table as one launch over the combined table, with the same grid and pdl
 // meanings: the one-launch form of a dual-time case alone (a table of one) and

@@ -349,12 +349,14 @@ static void autotune(ibm_server *s, Group *g) {
     return;
   }
   const int entries = g->batch->plain_start[g->batch->n] + g->batch->body_start[g->batch->n];
-  const int cands[3] = {0, 6 * s->nsms, 3 * s->nsms};
+  // one block per entry, or blocks striding over the table: as many as are resident, or half of them
+  const int resident = batch_stage_blocks(*g->batch) * s->nsms;
+  const int cands[3] = {0, resident, resident / 2};
   int best = 0;
   float best_ms = 1e30f;
   for (int ci = 0; ci < 3; ci++) {
     const int grid = cands[ci];
-    if (ci > 0 && grid >= entries) continue;
+    if (ci > 0 && (grid < 1 || grid >= entries)) continue;
     launch_stage_f32_batch_one(*g->batch, 1, grid, true, g->s);  // warm-up
     cudaEventRecord(g->t0, g->s);
     for (int rep = 0; rep < 3; rep++) launch_stage_f32_batch_one(*g->batch, 1, grid, true, g->s);

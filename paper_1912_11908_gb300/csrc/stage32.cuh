@@ -977,7 +977,10 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
 }
 
 // The block's copy of a table entry's case.  Indexed in the kernel's parameters, the constants and pointers were read
-// early and held across the tile in spilled registers; shared memory is read where a value is used.
+// early and held across the tile in spilled registers (12.2 ms for a burst of 16 requests, 11.9 from shared memory); the
+// compiler still reads some early.
+static_assert(sizeof(TileSmem) + sizeof(StageCase) + 1024 <= 228 * 1024 / BATCH_BLOCKS,
+              "the resident blocks that the launch bounds of the table kernels count on (1 KB of each block is reserved)");
 template <int NT>
 __device__ __forceinline__ void load_case(StageCase &dst, const StageCase &src) {
   static_assert(sizeof(StageCase) % 8 == 0, "copied in 8-byte words");

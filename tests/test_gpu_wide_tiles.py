@@ -38,3 +38,13 @@ def test_alone_and_in_a_group(ibm, scheme, interp, count):  # noqa: F811
         assert r["status"] == ibm.IBM_OK and r["steps_done"] == 20
         np.testing.assert_allclose(r["forces"], want, rtol=2e-5, atol=2e-5 * np.abs(want).max())
     s.close()
+
+
+def test_residency_of_the_table_kernels(ibm):  # noqa: F811
+    """Eight 128-thread blocks or three wide ones per SM, as their launch bounds and the group tuner count on."""
+    import ctypes
+    f = ibm.lib().ibm__batch_blocks_per_sm
+    f.argtypes = [ctypes.c_int] * 3
+    f.restype = ctypes.c_int
+    for wide, want in ((0, 8), (1, 3)):
+        assert [f(wide, t, q) for t in (0, 1) for q in (0, 1)] == [want] * 4
