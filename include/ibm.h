@@ -512,6 +512,16 @@ ibm_status ibm_persistent_grid(ibm_case *c, int blocks);
  * a second.  IBM_EINVAL for a NULL pointer, IBM_ECUDA if a CUDA call fails. */
 ibm_status ibm_check_float_conversions(uint64_t *checked, uint64_t *mismatched);
 
+/* Evaluates the FP64 arithmetic that the FP64 residuals and the dual-time
+ * update form on the integer pipes (Sec. 2), for checks against exact values:
+ * out[i] = op(a[i], b[i]) on the current device.  op: IBM_FP64_MUL a * b;
+ * IBM_FP64_HALF a / 2; IBM_FP64_RCP 1 / a; IBM_FP64_RSQRT 1 / sqrt(a);
+ * IBM_FP64_SQRT sqrt(a) (b is read by IBM_FP64_MUL only and may be NULL
+ * otherwise).  Host pointers; synchronous.  IBM_EINVAL for a NULL pointer or
+ * an unknown op, IBM_ENOMEM / IBM_ECUDA if a CUDA call fails. */
+enum { IBM_FP64_MUL = 0, IBM_FP64_HALF = 1, IBM_FP64_RCP = 2, IBM_FP64_RSQRT = 3, IBM_FP64_SQRT = 4 };
+ibm_status ibm_fp64_arithmetic(int op, const double *a, const double *b, double *out, size_t n);
+
 /* Replay each step from a CUDA graph captured on first use (default on);
  * enable = 0 launches every kernel directly. */
 ibm_status ibm_use_graphs(ibm_case *c, int enable);

@@ -1102,6 +1102,24 @@ extern "C" ibm_status ibm_check_float_conversions(uint64_t *checked, uint64_t *m
   return IBM_OK;
 }
 
+extern "C" ibm_status ibm_fp64_arithmetic(int op, const double *a, const double *b, double *out, size_t n) {
+  if (!a || !out || (op == IBM_FP64_MUL && !b)) return fail(IBM_EINVAL, "ibm_fp64_arithmetic: NULL argument");
+  if (op < IBM_FP64_MUL || op > IBM_FP64_SQRT) return fail(IBM_EINVAL, "ibm_fp64_arithmetic: unknown operation %d", op);
+  if (n == 0) return IBM_OK;
+  double *d = nullptr;
+  if (cudaMalloc(&d, 3 * n * sizeof(double)) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(IBM_ENOMEM, "ibm_fp64_arithmetic: device allocation failed");
+  }
+  cudaError_t e = cudaMemcpy(d, a, n * sizeof(double), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && op == IBM_FP64_MUL) e = cudaMemcpy(d + n, b, n * sizeof(double), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = launch_fp64_arithmetic(op, d, d + n, d + 2 * n, n);
+  if (e == cudaSuccess) e = cudaMemcpy(out, d + 2 * n, n * sizeof(double), cudaMemcpyDeviceToHost);
+  cudaFree(d);
+  if (e != cudaSuccess) return fail(IBM_ECUDA, "ibm_fp64_arithmetic: %s", cudaGetErrorString(e));
+  return IBM_OK;
+}
+
 extern "C" ibm_status ibm_use_graphs(ibm_case *c, int enable) {
   if (!c) return fail(IBM_EINVAL, "case is NULL");
   c->use_graphs = enable != 0;

@@ -560,4 +560,21 @@ void launch_stage_f64(const Consts &k, int stage, const double *Un, const double
   launch_tiles_f64<false>(k, stage, Un, In, Out, nullptr, nullptr, tag, ds, s);
 }
 
+__global__ void k_fp64_arithmetic(int op, const double *__restrict__ a, const double *__restrict__ b,
+                                  double *__restrict__ out, size_t n) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    const double x = a[i];
+    out[i] = op == IBM_FP64_MUL     ? mul64(x, b[i])
+             : op == IBM_FP64_HALF  ? half64(x)
+             : op == IBM_FP64_RCP   ? rcp64(x)
+             : op == IBM_FP64_RSQRT ? rsqrt64(x)
+                                    : sqrt64(x);
+  }
+}
+
+cudaError_t launch_fp64_arithmetic(int op, const double *a, const double *b, double *out, size_t n) {
+  k_fp64_arithmetic<<<(unsigned)std::min<size_t>((n + 255) / 256, 1024), 256>>>(op, a, b, out, n);
+  return cudaGetLastError();
+}
+
 }  // namespace ibm

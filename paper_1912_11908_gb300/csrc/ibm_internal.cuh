@@ -301,6 +301,8 @@ void launch_stage_f64(const Consts &k, int stage, const double *Un, const double
 void launch_dual_f64(const Consts &k, int stage, const double *A, const double *In, double *Out, const double *Wn,
                      const double *Wm, const uint8_t *tag, DevState *ds, cudaStream_t s);
 void launch_dual_end(const Consts &k, DevState *ds, cudaStream_t s);
+// out[i] = op(a[i], b[i]) in the arithmetic of fp64_math.cuh (device pointers; op: IBM_FP64_*)
+cudaError_t launch_fp64_arithmetic(int op, const double *a, const double *b, double *out, size_t n);
 
 // Compact FP32 form of an IB / ghost stencil for the FP32-bulk reconstruction
 // (built once per classification from the FP64 record).

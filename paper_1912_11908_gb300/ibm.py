@@ -92,7 +92,7 @@ EXPORTS = ["ibm_create_case", "ibm_classify", "ibm_step", "ibm_get_state", "ibm_
            "ibm_server_create", "ibm_server_submit", "ibm_server_progress", "ibm_server_poll",
            "ibm_server_destroy", "ibm_server_set_mode", "ibm_server_stats", "ibm_autotune", "ibm_use_tma",
            "ibm_use_persistent", "ibm_persistent_grid", "ibm_stage_launches",
-           "ibm_check_float_conversions", "ibm_fma_peak", "ibm_body3d_create", "ibm_body3d_classify",
+           "ibm_check_float_conversions", "ibm_fp64_arithmetic", "ibm_fma_peak", "ibm_body3d_create", "ibm_body3d_classify",
            "ibm_body3d_get", "ibm_body3d_destroy", "ibm_case3d_create", "ibm_case3d_step", "ibm_case3d_get",
            "ibm_case3d_set_state", "ibm_case3d_forces", "ibm_case3d_launch_count", "ibm_case3d_destroy"]
 REQ_PENDING, REQ_RUNNING, REQ_DONE, REQ_FAILED = range(4)
@@ -165,6 +165,8 @@ def load():
     L.ibm_stage_launches.restype = ip
     L.ibm_check_float_conversions.argtypes = [ctypes.POINTER(ctypes.c_uint64), ctypes.POINTER(ctypes.c_uint64)]
     L.ibm_check_float_conversions.restype = ip
+    L.ibm_fp64_arithmetic.argtypes = [ip, vp, vp, vp, sz]
+    L.ibm_fp64_arithmetic.restype = ip
     L.ibm_tag_nodes_noalloc.argtypes = [ctypes.POINTER(ibm_grid), vp, ip, vp, vp, ctypes.c_int32, vp, vp]
     L.ibm_tag_nodes_noalloc.restype = ip
     L.ibm_server_create.argtypes = [sz, ip, ip, ctypes.POINTER(vp)]
@@ -260,6 +262,21 @@ def check_float_conversions():
     n, bad = ctypes.c_uint64(0), ctypes.c_uint64(0)
     _check(lib().ibm_check_float_conversions(ctypes.byref(n), ctypes.byref(bad)))
     return int(n.value), int(bad.value)
+
+
+FP64_MUL, FP64_HALF, FP64_RCP, FP64_RSQRT, FP64_SQRT = range(5)
+
+
+def fp64_arithmetic(op, a, b=None):
+    """op(a, b) element by element in the FP64 residuals' integer-pipe arithmetic (ibm_fp64_arithmetic)."""
+    a = np.ascontiguousarray(a, np.float64)
+    b = None if b is None else np.ascontiguousarray(b, np.float64)
+    assert b is None or b.shape == a.shape
+    out = np.empty_like(a)
+    _check(lib().ibm_fp64_arithmetic(int(op), a.ctypes.data_as(ctypes.c_void_p),
+                                     None if b is None else b.ctypes.data_as(ctypes.c_void_p),
+                                     out.ctypes.data_as(ctypes.c_void_p), a.size))
+    return out
 
 
 def case_device_bytes(spec):
