@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cfloat>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -54,7 +55,8 @@ struct Mesh {
   const FaceExact *fx;// [ntri]
   const float4 *cl;   // [ncl][2] bounding box of a cluster's faces, widened by 1e-5 of the extent: lo, hi
   const float4 *fp;   // [FPLANES][ncl * CL] FP32 faces of the clusters: vertices, unit normal, the unit in-plane
-                      // normals of the edges (inward), face index (bits; -1: padding), 1 = never pruned
+                      // normals of the edges (inward), face index (bits; -1: padding), thickness and relative error
+                      // of a thin face (0: not thin)
   float ext;          // largest coordinate magnitude of the mesh (at least 1)
   double bb[6];       // axis-aligned bounding box: lo x, y, z, hi x, y, z
 };
@@ -525,8 +527,11 @@ __device__ __forceinline__ float warp_min(float x) {
 // exact evaluation finds, by the margin mg (far above the FP32 rounding of coordinates and operations).  Every term
 // is well conditioned whatever the face's shape: the distances to the three edge segments, the distance to the plane,
 // and the signed in-plane distances to the edge lines, which say whether the projection falls inside, outside, or
-// within the margin of an edge (then the plane's distance bounds from below only).  Faces whose barycentric system
-// is too flat for that to describe its FP64 solution are never pruned and prune nothing.
+// within the margin of an edge (then the plane's distance bounds from below only).
+// A thin face's barycentric system is too flat for that to describe its FP64 solution, off by up to `error` times the
+// farthest vertex' distance; but whatever the solution, the point it accepts lies in the face, whose points are within
+// the face's thickness of its longest edge and no farther away than the farthest vertex.  (Never pruned and pruning
+// nothing, the thin sides of a tube sent most nodes to the evaluation of all faces.)
 __device__ __forceinline__ void face_bounds(const Mesh &m, int c, int lane, const float P[3], float mg, float &lb,
                                             float &ub, int &f) {
   const int i = c * CL + lane, n = m.ncl * CL;
@@ -559,8 +564,12 @@ __device__ __forceinline__ void face_bounds(const Mesh &m, int c, int lane, cons
   ub = (tin >= mg ? dm : de) + mg;
   lb = (tin >= -mg ? dm : de) - mg;
   if (r[22] != 0.0f) {
-    lb = -INFINITY;
-    ub = INFINITY;
+    float v2 = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 3; k++) v2 = fmaxf(v2, fmaf(w[k][0], w[k][0], fmaf(w[k][1], w[k][1], w[k][2] * w[k][2])));
+    const float W = sqrtf(v2);
+    ub = fminf(W, fmaf(r[23], W, de)) + mg;
+    lb = r[22] < INFINITY ? de - r[22] - mg : -INFINITY;
   }
   if (f < 0) lb = ub = INFINITY;
 }
@@ -1063,9 +1072,19 @@ extern "C" ibm_status ibm_body3d_create(const double *verts, int nverts, const i
           }
         }
         for (int a = 0; a < 3; a++) r[9 + a] = (float)n[a];
-        // sin^2 of the angle at the first vertex below 1e-8: the FP64 barycentric solution may be off by more than
-        // the margin
-        r[22] = !(x.det >= 1e-8 * (x.a11 * x.a22)) ? 1.0f : 0.0f;
+        // sin^2 of the angle at the first vertex below 1e-8 (thin): the FP64 barycentric solution may be off by more
+        // than the margin.  With u = 2^-53, w the vertices' distances and the solution's s, t in [0, 1], each of its
+        // products carries at most 13 u |w| |e|^3 and det 24 u |e|^4: the point is off by less than 150 u max|w| / sin^2.
+        // Thickness: the height over the longest edge, |e1| |e2| sin / longest, rounding of det included; no bound
+        // (infinity) where that is not a number
+        const double aa = x.a11 * x.a22;
+        if (!(x.det >= 1e-8 * aa)) {
+          const double longest = std::max(x.ee[0], std::max(x.ee[1], x.ee[2]));
+          const double h = 1.01 * std::sqrt((std::max(x.det, 0.0) + 1e-14 * aa) / longest);
+          const double sin2 = x.det / aa - 1e-14;
+          r[22] = h > 0.0 ? std::max((float)h, FLT_MIN) : x.a11 == 0.0 || x.a22 == 0.0 ? FLT_MIN : INFINITY;
+          r[23] = sin2 > 0.0 ? (float)std::min(2e-14 / sin2, 1.0) : 1.0f;
+        }
       }
       std::memcpy(&r[21], &f, sizeof f);
       for (int p = 0; p < FPLANES; p++)
