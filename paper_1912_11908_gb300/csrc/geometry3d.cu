@@ -488,6 +488,27 @@ __device__ __forceinline__ double face_closest(const FaceExact &F, const double 
   return dot3(dq, dq);
 }
 
+// the closest so far of a lane's faces (f = 0x7fffffff: none)
+struct Nearest {
+  double d2, q[3];
+  int f, fk, fe, fv;
+};
+// face f taken into account, the lowest index among equal distances (a call: inlined into the search of the survivors, its
+// registers pushed the search's own into local memory)
+__device__ __noinline__ void take_face(const FaceExact &F, int f, const double P[3], Nearest &b) {
+  double q[3];
+  int fk, fe, fv;
+  const double d2 = face_closest(F, P, q, fk, fe, fv);
+  if (d2 < b.d2 || (d2 == b.d2 && f < b.f)) {
+    b.d2 = d2;
+    for (int d = 0; d < 3; d++) b.q[d] = q[d];
+    b.f = f;
+    b.fk = fk;
+    b.fe = fe;
+    b.fv = fv;
+  }
+}
+
 // the record of node n from the winning face's closest feature: its pseudo-normal (Sec. 4.2) is the face normal, the
 // angle-weighted vertex normal (Eq. 2) or the normalised sum of the two faces' normals at an edge (Eq. 3)
 __device__ __forceinline__ void write_record(const Mesh &m, int n, int f, int fk, int fe, int fv, const double q[3],
@@ -664,6 +685,7 @@ __global__ void __launch_bounds__(B3, 3) k3_closest(Lattice L, Mesh m, const int
         int f;
         face_bounds(m, c, lane, P, mg, lb, fu, f);
         ub = fminf(ub, warp_min(fu));
+        if (over) return;
         const bool ok = f >= 0 && lb <= ub;
         const unsigned bal = __ballot_sync(0xffffffffu, ok);
         const int more = __popc(bal);
@@ -680,17 +702,20 @@ __global__ void __launch_bounds__(B3, 3) k3_closest(Lattice L, Mesh m, const int
         cnt += more;
         __syncwarp();
       };
-      visit(c0);
-      for (int b = 0; b < m.ncl && !over; b += 32) {
-        const int c = b + lane;
-        float d = b == 0 ? kept0 : kept1, unused;
-        if (b >= 64 && c < m.ncl) d = box(c, unused);
-        for (unsigned todo = __ballot_sync(0xffffffffu, c < m.ncl && c != c0 && d <= ub); todo && !over;
-             todo &= todo - 1) {
-          const int src = __ffs(todo) - 1;
-          if (__shfl_sync(0xffffffffu, d, src) <= ub) visit(b + src);
+      // every cluster but `but` whose box is within the current upper bound
+      auto for_near = [&](int but, auto fn) {
+        for (int b = 0; b < m.ncl; b += 32) {
+          const int c = b + lane;
+          float d = b == 0 ? kept0 : kept1, unused;
+          if (b >= 64 && c < m.ncl) d = box(c, unused);
+          for (unsigned todo = __ballot_sync(0xffffffffu, c < m.ncl && c != but && d <= ub); todo; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1;
+            if (__shfl_sync(0xffffffffu, d, src) <= ub) fn(b + src);
+          }
         }
-      }
+      };
+      visit(c0);
+      for_near(c0, visit);
       int first = PAIRS;
       if (!over) {
         compact();
@@ -707,30 +732,39 @@ __global__ void __launch_bounds__(B3, 3) k3_closest(Lattice L, Mesh m, const int
         __syncwarp();
         continue;
       }
-      // more survivors than the batch has room for: the warp evaluates them itself (all faces if they were not kept)
+      // more survivors than the batch has room for: the warp evaluates them itself (found once more by their bounds if
+      // they were not kept -- all faces instead: 1.5 s for 64^3 nodes around 400,000 faces, most nodes having a hundred of
+      // them as near as the bounds can tell)
       if (!over && lane == 0)
         for (int i = first; i < PAIRS; i++) p_entry[i] = -1;  // the part of the claim inside the list stays empty
       double X[3];
       node_xyz(L, n, X, ijk);
-      double best = INFINITY, bq[3] = {0.0, 0.0, 0.0};
-      int bf = 0x7fffffff, bk = 0, be = 0, bv = 0;
-      const int nc = over ? m.ntri : cnt;
-      for (int i = lane; i < nc; i += 32) {
-        const int f = over ? i : s_face[warp][i];
-        double y[3];
-        int fk, fe, fv;
-        const double d2 = face_closest(m.fx[f], X, y, fk, fe, fv);
-        if (d2 < best || (d2 == best && f < bf)) {
-          best = d2;
-          bf = f;
-          bk = fk;
-          be = fe;
-          bv = fv;
-          for (int d = 0; d < 3; d++) bq[d] = y[d];
+      Nearest near_face = {INFINITY, {0.0, 0.0, 0.0}, 0x7fffffff, 0, 0, 0};
+      if (over) cnt = 0;
+      auto evaluate_kept = [&]() {
+        for (int i = lane; i < cnt; i += 32) {
+          const int f = s_face[warp][i];
+          take_face(m.fx[f], f, X, near_face);
         }
+        cnt = 0;
+        __syncwarp();
+      };
+      if (over) {
+        for_near(-1, [&](int c) {
+          float lb, fu;
+          int f;
+          face_bounds(m, c, lane, P, mg, lb, fu, f);
+          const bool ok = f >= 0 && lb <= ub;
+          const unsigned bal = __ballot_sync(0xffffffffu, ok);
+          if (cnt + __popc(bal) > KEEP) evaluate_kept();
+          if (ok) s_face[warp][cnt + __popc(bal & ((1u << lane) - 1u))] = f;
+          cnt += __popc(bal);
+          __syncwarp();
+        });
       }
-      double md = best;
-      int mf = bf;
+      evaluate_kept();
+      double md = near_face.d2;
+      int mf = near_face.f;
       for (int o = 16; o > 0; o >>= 1) {
         const double od = __shfl_xor_sync(0xffffffffu, md, o);
         const int of = __shfl_xor_sync(0xffffffffu, mf, o);
@@ -739,7 +773,8 @@ __global__ void __launch_bounds__(B3, 3) k3_closest(Lattice L, Mesh m, const int
           mf = of;
         }
       }
-      if (bf == mf && bf != 0x7fffffff) write_record(m, n, bf, bk, be, bv, bq, rec + e);
+      if (near_face.f == mf && mf != 0x7fffffff)
+        write_record(m, n, mf, near_face.fk, near_face.fe, near_face.fv, near_face.q, rec + e);
       __syncwarp();
     }
     __syncthreads();

@@ -91,3 +91,18 @@ def test_thin_faces_are_excluded(ibm):  # noqa: F811
     fat, thin = (_seconds(ibm, *_tube(5, length), n, lo, hi) for length in (2.0, 8.0))
     print("sides above and below the angle of a thin face: %.0f us, %.0f us" % (1e6 * fat, 1e6 * thin))
     assert thin <= 4.0 * fat, (fat, thin)
+
+
+def test_fine_meshes(ibm, orc):  # noqa: F811
+    """Far more faces than cells: nodes with more than the hundred survivors that a warp keeps, thin faces among them."""
+    verts, tris = W.uv_sphere(3, 4000, 0.35, (0.503, 0.498, 0.501))
+    _check(ibm, orc, verts, tris, (14, 13, 12), (0.0, 0.0, 0.0), (1.0, 1.0, 1.0))
+
+
+def test_fine_meshes_are_searched(ibm):  # noqa: F811
+    """200,000 faces in three rings against 200,000 of usual shape: 700 times as long when a node of more survivors than a
+    warp keeps evaluates every face, about 20 times as long when it evaluates the survivors."""
+    n, lo, hi = (40,) * 3, (-2.0,) * 3, (2.0,) * 3
+    plain, rings = (_seconds(ibm, *W.uv_sphere(a, b), n, lo, hi) for a, b in ((251, 400), (3, 50000)))
+    print("usual shape %.0f us, three rings %.0f us" % (1e6 * plain, 1e6 * rings))
+    assert rings <= 100.0 * plain, (plain, rings)
