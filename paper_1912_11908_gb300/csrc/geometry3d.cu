@@ -1048,7 +1048,7 @@ extern "C" ibm_status ibm_body3d_create(const double *verts, int nverts, const i
       bhi[a] = std::max(bhi[a], verts[3 * k + a]);
     }
   for (int a = 0; a < 3; a++) ext = std::max(ext, std::max(std::fabs(blo[a]), std::fabs(bhi[a])));
-  ext = std::max(ext, 1.0);
+  ext = std::max(ext, 1e-12);  // (FP32 squares of smaller distances would underflow)
   const double margin = 1e-5 * ext;
   std::vector<FaceExact> fx((size_t)ntris);
   std::vector<std::pair<uint32_t, int>> order((size_t)ntris);

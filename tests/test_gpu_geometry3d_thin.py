@@ -93,6 +93,20 @@ def test_thin_faces_are_excluded(ibm):  # noqa: F811
     assert thin <= 4.0 * fat, (fat, thin)
 
 
+@pytest.mark.parametrize("scale", [1e-3, 1e-5, 1e-9])
+def test_small_bodies(ibm, orc, scale):  # noqa: F811
+    verts, tris = W.uv_sphere(13, 18, 0.35 * scale, (0.503 * scale, 0.498 * scale, 0.501 * scale))
+    _check(ibm, orc, verts, tris, (26, 27, 33), (0.0,) * 3, (scale,) * 3)
+
+
+def test_small_bodies_are_searched_as_fast(ibm):  # noqa: F811
+    n = (160,) * 3
+    verts, tris = W.uv_sphere()
+    plain = _seconds(ibm, verts, tris, n, (-2.0,) * 3, (2.0,) * 3)
+    small = _seconds(ibm, verts * 1e-6, tris, n, (-2e-6,) * 3, (2e-6,) * 3)
+    assert small <= 4.0 * plain, (plain, small)
+
+
 def test_fine_meshes(ibm, orc):  # noqa: F811
     """Far more faces than cells: nodes with more than the hundred survivors that a warp keeps, thin faces among them."""
     verts, tris = W.uv_sphere(3, 4000, 0.35, (0.503, 0.498, 0.501))
