@@ -57,7 +57,7 @@ struct Mesh {
   const float4 *fp;   // [FPLANES][ncl * CL] FP32 faces of the clusters: vertices, unit normal, the unit in-plane
                       // normals of the edges (inward), face index (bits; -1: padding), thickness and relative error
                       // of a thin face (0: not thin)
-  float ext;          // largest coordinate magnitude of the mesh (at least 1)
+  float ext;          // largest coordinate magnitude of the mesh (at least 1e-12)
   double bb[6];       // axis-aligned bounding box: lo x, y, z, hi x, y, z
 };
 
