@@ -178,9 +178,8 @@ enum {
   IBM_STENCILS = 3,     /* ibm_stencil[#IB + #G1 + #G2 + #G3], IB first then G1, G2, G3, each in row-major order */
   IBM_TIME = 4,         /* double[2]: t, last dt */
   IBM_STEPS = 5,        /* int64_t: steps taken */
-  IBM_TUNING = 6,       /* int32_t[2] (host only): register-budget variants of the FP32-bulk stage kernel
-                           picked by the autotuner for stage 1 and for stages 2-3 (0..2; -1 before the first
-                           step, or FP64) */
+  IBM_TUNING = 6,       /* int32_t[2] (host only): register-budget variants of the FP32-bulk stage kernel for
+                           stage 1 and for stages 2-3 (0, the only one; -1 before the first step, or FP64) */
   IBM_STAGE_LAUNCH = 7, /* int32_t (host only): launch form of the FP32-bulk stages (0..2, see
                            ibm_stage_launches; the autotuner's pick unless set; -1 for FP64) */
   IBM_BODY = 8          /* double[6]: body displacement x, y and velocity u, v at the current time, and the
@@ -444,14 +443,13 @@ int64_t ibm_launch_count(const ibm_case *c);
 ibm_status ibm_profile_enable(ibm_case *c, int enable);
 ibm_status ibm_profile_read(ibm_case *c, double *ms, int64_t *launches, int n_groups);
 
-/* Autotuning (default on).  FP32-bulk explicit cases time the stage kernels
- * (plain tiles and the concurrent body tiles) under three register budgets of
- * the plain kernel (six, five and four resident blocks per SM), separately
- * for stage 1 and stage 2, on their first ibm_step -- about a hundred extra
- * launches and a few host waits -- and keep the fastest (stage 3 follows
- * stage 2); the choice is cached per device and grid size for the process.  enable = 0 uses the compiler's default budget.  Results do not
- * depend on the choice beyond FP32 rounding.  Only before the first step
- * (IBM_ESTATE afterwards). */
+/* Autotuning (default on).  FP32-bulk explicit cases whose launch form is not
+ * set (ibm_stage_launches) time stages 1 and 2 in forms 0 and 2 on their
+ * first ibm_step -- about 180 extra launches and 20 host waits -- and keep
+ * the form with the shorter step; the choice is cached per device and grid
+ * size for the process.  enable = 0 keeps form 2.  Results do not depend on
+ * the choice beyond FP32 rounding.  Only before the first step (IBM_ESTATE
+ * afterwards). */
 ibm_status ibm_autotune(ibm_case *c, int enable);
 
 /* FP32-bulk explicit stages: stage the loaded region (tile + 3-cell halo) of
@@ -473,8 +471,8 @@ ibm_status ibm_use_tma(ibm_case *c, int enable);
  *   2: as 1, each stage launched with programmatic dependent launch, so that
  *      its blocks are resident, waiting for the previous stage, while the
  *      previous stage's last blocks finish.
- * Unless this is called, the autotuner times forms 0 and 2 with their
- * register budgets on an explicit case's first step and keeps the faster
+ * Unless this is called, the autotuner times forms 0 and 2 on an explicit
+ * case's first step and keeps the faster
  * (IBM_STAGE_LAUNCH reports it; without autotuning, and for dual time, the
  * form is 2).  Modes 1 and 2 run the same
  * kernel and give bit-identical results; mode 0's kernels are compiled

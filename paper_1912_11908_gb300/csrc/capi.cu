@@ -45,8 +45,7 @@ struct ibm_case {
   CUtensorMap tmap[3];              // FP32-bulk: tensor maps of M, F1, F2 for the TMA tile staging
   bool have_tmap = false;           // tensor maps built
   bool use_tma = true;              // stage interior tiles with TMA (ibm_use_tma)
-  int plain_variant[2] = {-1, -1};  // FP32-bulk: register budget of the plain stage kernel for stage 1 and for
-                                    // stages 2-3 (-1: not tuned yet)
+  bool tuned = false;               // FP32-bulk: launch form picked
   unsigned int *sch_words = nullptr;  // FP32-bulk explicit: schedule of the persistent step kernel (StepSched)
   bool use_persist = false;           // one persistent launch per step (ibm_use_persistent)
   int stage_launch = 2;               // FP32-bulk explicit stages: 0 plain + body kernels on two streams, 1 one
@@ -753,12 +752,11 @@ static int enqueue_step(ibm_case *c) {
     // inside the stage kernel's tile load; the end of the step (t += dt) is
     // folded into stage 3
     prof_mark(c, 0, true);
-    const int pv = c->plain_variant[st == 1 ? 0 : 1] < 0 ? 0 : c->plain_variant[st == 1 ? 0 : 1];
     if (f64) launch_stage_f64(c->k, st, c->A, in64[st - 1], out64[st - 1], c->tag, c->ds, s);
     else if (c->stage_launch > 0) {
       // one launch for all tiles of the stage (body-tile slots first)
       launch_stage_f32_one(c->k, st, c->M, in32[st - 1], out32[st - 1], c->A, c->tag, c->sid, c->rst, c->tile_body,
-                           c->body_tiles, c->body_cap, c->ds, fuse_cfl, pv,
+                           c->body_tiles, c->body_cap, c->ds, fuse_cfl,
                            c->have_tmap && c->use_tma ? &c->tmap[st - 1] : nullptr, c->stage_launch == 2, s,
                            c->rsq);
     } else {
@@ -766,7 +764,7 @@ static int enqueue_step(ibm_case *c) {
       cudaEventRecord(c->ev_fork, s);
       cudaStreamWaitEvent(c->sb, c->ev_fork, 0);
       launch_stage_f32(c->k, st, c->M, in32[st - 1], out32[st - 1], c->A, c->tag, c->sid, c->rst, c->tile_body,
-                       c->body_tiles, c->body_cap, c->ds, fuse_cfl, s, c->sb, pv, true,
+                       c->body_tiles, c->body_cap, c->ds, fuse_cfl, s, c->sb,
                        c->have_tmap && c->use_tma ? &c->tmap[st - 1] : nullptr, c->rsq);
       cudaEventRecord(c->ev_join, c->sb);
       cudaStreamWaitEvent(s, c->ev_join, 0);
@@ -784,117 +782,83 @@ static int enqueue_step(ibm_case *c) {
   return nl;
 }
 
-// Autotuner of the FP32-bulk step: for each launch form (plain-tile and
-// body-tile kernels on two streams; one kernel per stage with programmatic
-// launch) and each register budget, time repeated launches of stage 1 and of
-// stage 2 as the step runs them, in interleaved rounds keeping each
-// candidate's best time; per form the best budget per stage group, then the
-// form with the shorter step (stage 3 takes stage 2's choice).  Picked once
-// per device, grid size and pinned form for the whole process.  Between steps stages
+// Autotuner of the FP32-bulk step: time repeated launches of stage 1 and of
+// stage 2 in either launch form (plain-tile and body-tile kernels on two
+// streams; one kernel per stage with programmatic launch) as the step runs
+// them, in interleaved rounds keeping each form's best times, and take the
+// form with the shorter step (stage 3 counted as stage 2).  Picked once per
+// device and grid size for the whole process.  Between steps stages
 // 1 and 2 leave the solution unchanged: they read the mirror of U^n (and the
 // stage-1 array) and write the stage arrays, the stage times, and U^n on IB /
 // ghost nodes with the values the step's own stage 1 writes again.
+// (Register budgets for seven and six blocks per SM were candidates beside
+// eight; on grids of 200 to 18,432 tiles none was faster by the margin that a
+// warm L2 asks for, and with caches flushed between steps they were slower.)
 static std::mutex g_tune_mu;
-struct Tuned {
-  int v1, v2, launch;
-};
-static std::map<std::tuple<int, int, int, int>, Tuned> g_tuned;
+static std::map<std::tuple<int, int, int>, int> g_tuned;
 
-static ibm_status tune_plain_variant(ibm_case *c) {
-  if (c->precision != IBM_PREC_FP32_BULK || c->plain_variant[0] >= 0) return IBM_OK;
-  if (!c->autotune || c->k.dual) {  // dual time has its own kernels
-    c->plain_variant[0] = c->plain_variant[1] = 0;
+static ibm_status tune_launch_form(ibm_case *c) {
+  if (c->precision != IBM_PREC_FP32_BULK || c->tuned) return IBM_OK;
+  if (!c->autotune || c->k.dual || c->launch_pinned) {  // dual time has its own kernels
+    c->tuned = true;
     return IBM_OK;
   }
-  // candidates: the register budgets of the launch form the caller pinned, or of both forms (two-stream plain and
-  // body kernels; one kernel per stage with programmatic launch)
-  const auto key = std::make_tuple(c->device, c->k.nx, c->k.ny, c->launch_pinned ? c->stage_launch : -1);
+  const auto key = std::make_tuple(c->device, c->k.nx, c->k.ny);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tuned.find(key);
     if (it != g_tuned.end()) {
-      c->plain_variant[0] = it->second.v1;
-      c->plain_variant[1] = it->second.v2;
-      c->stage_launch = it->second.launch;
+      c->tuned = true;
+      c->stage_launch = it->second;
       return IBM_OK;
     }
   }
-  // (wide blocks have one budget)
-  const int nvar = stage_wide(stage_tiles(c->k), c->body_cap) ? 1 : PLAIN_VARIANTS;
-  int forms[2] = {c->stage_launch, -1}, nforms = 1;
-  if (!c->launch_pinned) {
-    forms[0] = 2;
-    forms[1] = 0;
-    nforms = 2;
-  }
+  const int forms[2] = {2, 0};
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   CU(cudaEventCreate(&e0));
   CU(cudaEventCreate(&e1));
   const bool fuse = fused_cfl(c);
   cudaStream_t s = c->stream;
-  auto pair = [&](int stage, int v, int form) {
+  auto launch = [&](int stage, int form) {
     const CUtensorMap *tm = c->have_tmap && c->use_tma ? &c->tmap[stage - 1] : nullptr;
     if (form > 0) {
       launch_stage_f32_one(c->k, stage, c->M, stage == 1 ? c->M : c->F1, stage == 1 ? c->F1 : c->F2, c->A, c->tag,
-                           c->sid, c->rst, c->tile_body, c->body_tiles, c->body_cap, c->ds, fuse, v, tm, form == 2, s,
-                           c->rsq);
+                           c->sid, c->rst, c->tile_body, c->body_tiles, c->body_cap, c->ds, fuse, tm, true, s, c->rsq);
       return;
     }
     cudaEventRecord(c->ev_fork, s);
     cudaStreamWaitEvent(c->sb, c->ev_fork, 0);
     launch_stage_f32(c->k, stage, c->M, stage == 1 ? c->M : c->F1, stage == 1 ? c->F1 : c->F2, c->A, c->tag, c->sid,
-                     c->rst, c->tile_body, c->body_tiles, c->body_cap, c->ds, fuse, s, c->sb, v, true, tm, c->rsq);
+                     c->rst, c->tile_body, c->body_tiles, c->body_cap, c->ds, fuse, s, c->sb, tm, c->rsq);
     cudaEventRecord(c->ev_join, c->sb);
     cudaStreamWaitEvent(s, c->ev_join, 0);
   };
   constexpr int ROUNDS = 5, REPS = 8;
-  float best[2][2][PLAIN_VARIANTS];  // form, stage, variant
-  for (int f = 0; f < 2; f++)
-    for (int st = 0; st < 2; st++)
-      for (int v = 0; v < PLAIN_VARIANTS; v++) best[f][st][v] = 1e30f;
-  pair(1, 0, forms[0]);  // stage-1 array for the stage-2 timings
-  long long nl = 1 + (c->body_cap > 0 && forms[0] == 0);
+  float best[2][2] = {{1e30f, 1e30f}, {1e30f, 1e30f}};  // form, stage
+  launch(1, forms[0]);  // stage-1 array for the stage-2 timings
+  long long nl = 1;
   cudaError_t e = cudaSuccess;
   for (int round = 0; round < ROUNDS && e == cudaSuccess; round++)
-    for (int f = 0; f < nforms && e == cudaSuccess; f++)
-      for (int st = 0; st < 2 && e == cudaSuccess; st++)
-        for (int v = 0; v < nvar && e == cudaSuccess; v++) {
-          pair(st + 1, v, forms[f]);  // warm-up
-          cudaEventRecord(e0, s);
-          for (int rep = 0; rep < REPS; rep++) pair(st + 1, v, forms[f]);
-          cudaEventRecord(e1, s);
-          nl += (REPS + 1) * (1 + (c->body_cap > 0 && forms[f] == 0));
-          float ms = 0.f;
-          e = cudaEventSynchronize(e1);
-          if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-          if (e == cudaSuccess && ms < best[f][st][v]) best[f][st][v] = ms;
-        }
+    for (int f = 0; f < 2 && e == cudaSuccess; f++)
+      for (int st = 0; st < 2 && e == cudaSuccess; st++) {
+        launch(st + 1, forms[f]);  // warm-up
+        cudaEventRecord(e0, s);
+        for (int rep = 0; rep < REPS; rep++) launch(st + 1, forms[f]);
+        cudaEventRecord(e1, s);
+        nl += (REPS + 1) * (1 + (c->body_cap > 0 && forms[f] == 0));
+        float ms = 0.f;
+        e = cudaEventSynchronize(e1);
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+        if (e == cudaSuccess && ms < best[f][st]) best[f][st] = ms;
+      }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (e != cudaSuccess) return fail(IBM_ECUDA, "autotuning failed: %s", cudaGetErrorString(e));
-  // per form the best budget per stage group; the form with the shorter step (stage 3 runs stage 2's choice)
-  int pick[2][2];
-  float step_ms[2];
-  for (int f = 0; f < nforms; f++) {
-    for (int st = 0; st < 2; st++) {
-      // another budget replaces eight blocks per SM only when it is far faster here: these timings run from a warm
-      // L2, and with caches flushed between steps the resident blocks hide the loads (768 x 384 step: eight blocks
-      // 66 us, seven 75, the pick at a 4% margin 79; warm 72.5, 72.3 and 73.4; 3072 x 1536, four steps: 2.60 ms,
-      // seven blocks 2.67)
-      int b = 0;
-      for (int v = 1; v < PLAIN_VARIANTS; v++)
-        if (best[f][st][v] < (b == 0 ? 0.85f : 1.f) * best[f][st][b]) b = v;
-      pick[f][st] = b;
-    }
-    step_ms[f] = best[f][0][pick[f][0]] + 2.f * best[f][1][pick[f][1]];
-  }
-  const int fb = nforms == 2 && step_ms[1] < step_ms[0] ? 1 : 0;
-  c->stage_launch = forms[fb];
-  c->plain_variant[0] = pick[fb][0];
-  c->plain_variant[1] = pick[fb][1];
+  c->stage_launch = forms[best[1][0] + 2.f * best[1][1] < best[0][0] + 2.f * best[0][1] ? 1 : 0];
+  c->tuned = true;
   c->launches += nl;
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  g_tuned[key] = Tuned{c->plain_variant[0], c->plain_variant[1], c->stage_launch};
+  g_tuned[key] = c->stage_launch;
   return IBM_OK;
 }
 
@@ -936,8 +900,8 @@ extern "C" ibm_status ibm_step(ibm_case *c, int nsteps) {
     c->launches += nl;
     c->dt_valid = true;
   }
-  if (c->plain_variant[0] < 0 && !persistent_step(c)) {
-    ibm_status r = tune_plain_variant(c);
+  if (!c->tuned && !persistent_step(c)) {
+    ibm_status r = tune_launch_form(c);
     if (r != IBM_OK) return r;
   }
   if (c->use_graphs && !c->profiling) {
@@ -1040,7 +1004,7 @@ extern "C" ibm_status ibm_autotune(ibm_case *c, int enable) {
   if (!c) return fail(IBM_EINVAL, "case is NULL");
   if (c->graph) return fail(IBM_ESTATE, "ibm_autotune: the case has already stepped");
   c->autotune = enable != 0;
-  c->plain_variant[0] = c->plain_variant[1] = -1;
+  c->tuned = false;
   return IBM_OK;
 }
 
@@ -1074,7 +1038,7 @@ extern "C" ibm_status ibm_stage_launches(ibm_case *c, int mode) {
     cudaGraphExecDestroy(c->graph);
     c->graph = nullptr;
   }
-  if ((mode > 0) != (c->stage_launch > 0)) c->plain_variant[0] = c->plain_variant[1] = -1;  // other kernels: retune
+  if ((mode > 0) != (c->stage_launch > 0)) c->tuned = false;
   c->stage_launch = mode;
   c->launch_pinned = true;
   return IBM_OK;
@@ -1254,7 +1218,7 @@ extern "C" ibm_status ibm_get_state(ibm_case *c, int what, void *dst, size_t byt
     case IBM_TUNING: {
       if (bytes < 2 * sizeof(int32_t) || dst_on_device)
         return fail(IBM_EINVAL, "IBM_TUNING: host int32[2] destination");
-      const int32_t v[2] = {c->plain_variant[0], c->plain_variant[1]};
+      const int32_t t = c->tuned && c->precision == IBM_PREC_FP32_BULK ? 0 : -1, v[2] = {t, t};
       std::memcpy(dst, v, sizeof v);
       break;
     }

@@ -109,10 +109,9 @@ void launch_compact_stencils(const Consts &k, const ibm_stencil *st, RStencil32 
 }
 
 // A case stepped on its own: one block per tile (plain) or body-tile slot.
-// MINB: resident blocks per SM the register allocation must allow (8: 64 registers and the most that shared memory
-// holds; 7: 72; 6: 80) -- the autotuner picks one per grid size.
-template <int STAGE, bool BODY, int MINB, int NT = NTH>
-__global__ void __launch_bounds__(NT, MINB) k_stage_f32(Consts k, PertConsts c, float *Mn, const float *__restrict__ In,
+// Eight blocks per SM are 64 registers and the most that shared memory holds.
+template <int STAGE, bool BODY, int NT>
+__global__ void __launch_bounds__(NT, NT == WIDE ? WIDE_BLOCKS : BODY ? 0 : 8) k_stage_f32(Consts k, PertConsts c, float *Mn, const float *__restrict__ In,
                                                    float *Out, double *D, const uint8_t *__restrict__ tag,
                                                    const int *__restrict__ sid, const RStencil32 *__restrict__ rs,
                                                    const uint8_t *__restrict__ tile_body,
@@ -131,8 +130,8 @@ __global__ void __launch_bounds__(NT, MINB) k_stage_f32(Consts k, PertConsts c, 
 // block of this one has started; its blocks then wait at the top for this
 // grid to complete and its stores to become visible, so the next stage's
 // blocks are resident when the tail of this one ends.
-template <int STAGE, int MINB, int NT = NTH>
-__global__ void __launch_bounds__(NT, MINB)
+template <int STAGE, int NT>
+__global__ void __launch_bounds__(NT, NT == WIDE ? WIDE_BLOCKS : 8)
     k_stage_f32_one(Consts k, PertConsts c, float *Mn, const float *__restrict__ In, float *Out, double *D,
                     const uint8_t *__restrict__ tag, const int *__restrict__ sid, const RStencil32 *__restrict__ rs,
                     const uint8_t *__restrict__ tile_body, const int *__restrict__ body_tiles, int nb, DevState *ds,
@@ -154,7 +153,7 @@ __global__ void __launch_bounds__(NT, MINB)
 // The same stage with the TVD-2 reconstruction (Sec. 2) and / or the quadratic IB / ghost reconstruction
 // (Sec. 4.5, Sec. 5) compiled in: a case with either takes this kernel in every launch form (the two-stream
 // form runs it as one launch on the case stream), so that the default kernels carry neither.
-template <int STAGE, bool TVD, bool QUAD, int NT = NTH>
+template <int STAGE, bool TVD, bool QUAD, int NT>
 __global__ void __launch_bounds__(NT, NT == NTH ? 7 : WIDE_BLOCKS)
     k_stage_f32_var(Consts k, PertConsts c, float *Mn, const float *__restrict__ In, float *Out, double *D,
                     const uint8_t *__restrict__ tag, const int *__restrict__ sid, const RStencil32 *__restrict__ rs,
@@ -270,11 +269,11 @@ void launch_tile_lists(const Consts &k, const uint8_t *tag, uint8_t *tile_body, 
 void launch_stage_f32(const Consts &k, int stage, float *Mn, const float *In, float *Out, double *D,
                       const uint8_t *tag, const int *sid, const RStencil32 *rs, const uint8_t *tile_body,
                       const int *body_tiles, int body_cap, DevState *ds, bool fuse_cfl, cudaStream_t s,
-                      cudaStream_t sb, int plain_variant, bool with_body, const CUtensorMap *tmap,
+                      cudaStream_t sb, const CUtensorMap *tmap,
                       const RStencilQ *rsq) {
   if (k.tvd2 || k.quad) {  // the variant kernel holds plain and body tiles: one launch on the case stream
-    launch_stage_f32_one(k, stage, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, with_body ? body_cap : 0, ds,
-                         fuse_cfl, plain_variant, tmap, false, s, rsq);
+    launch_stage_f32_one(k, stage, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, body_cap, ds, fuse_cfl, tmap,
+                         false, s, rsq);
     return;
   }
   PertConsts c = pert_consts(k);
@@ -287,31 +286,27 @@ void launch_stage_f32(const Consts &k, int stage, float *Mn, const float *In, fl
   const int ut = tmap ? 1 : 0;
   const bool wide = stage_wide(nt, nb);
 #define IBM_ARGS k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, ds, fuse_cfl, ncfl, tm, ut
-#define IBM_STAGE_PAIR(S)                                                      \
+#define IBM_STAGE_PAIR_N(S, N)                                                \
   do {                                                                         \
-    if (wide) {                                                                \
-      if (nb && with_body) k_stage_f32<S, true, WIDE_BLOCKS, WIDE><<<nb, WIDE, 0, sb>>>(IBM_ARGS); \
-      k_stage_f32<S, false, WIDE_BLOCKS, WIDE><<<nt, WIDE, 0, s>>>(IBM_ARGS);  \
-      break;                                                                   \
-    }                                                                          \
-    if (nb && with_body) k_stage_f32<S, true, 0><<<nb, NTH, 0, sb>>>(IBM_ARGS); \
-    if (plain_variant == 1)                                                    \
-      k_stage_f32<S, false, 7><<<nt, NTH, 0, s>>>(IBM_ARGS);                   \
-    else if (plain_variant == 2)                                               \
-      k_stage_f32<S, false, 6><<<nt, NTH, 0, s>>>(IBM_ARGS);                   \
-    else                                                                       \
-      k_stage_f32<S, false, 8><<<nt, NTH, 0, s>>>(IBM_ARGS);                   \
+    if (nb) k_stage_f32<S, true, N><<<nb, N, 0, sb>>>(IBM_ARGS);               \
+    k_stage_f32<S, false, N><<<nt, N, 0, s>>>(IBM_ARGS);                       \
+  } while (0)
+#define IBM_STAGE_PAIR(S)               \
+  do {                                  \
+    if (wide) IBM_STAGE_PAIR_N(S, WIDE); \
+    else IBM_STAGE_PAIR_N(S, NTH);      \
   } while (0)
   if (stage == 1) IBM_STAGE_PAIR(1);
   else if (stage == 2) IBM_STAGE_PAIR(2);
   else IBM_STAGE_PAIR(3);
 #undef IBM_STAGE_PAIR
+#undef IBM_STAGE_PAIR_N
 #undef IBM_ARGS
 }
 
 cudaError_t launch_stage_f32_one(const Consts &k, int stage, float *Mn, const float *In, float *Out, double *D,
                                  const uint8_t *tag, const int *sid, const RStencil32 *rs, const uint8_t *tile_body,
-                                 const int *body_tiles, int body_cap, DevState *ds, bool fuse_cfl, int plain_variant,
+                                 const int *body_tiles, int body_cap, DevState *ds, bool fuse_cfl,
                                  const CUtensorMap *tmap, bool pdl, cudaStream_t s, const RStencilQ *rsq) {
   if (k.quad && !rsq) return cudaErrorInvalidValue;  // the quadratic kernels read the second probes
   const PertConsts c = pert_consts(k);
@@ -332,12 +327,10 @@ cudaError_t launch_stage_f32_one(const Consts &k, int stage, float *Mn, const fl
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = pdl ? 1 : 0;
-#define IBM_ONE(S, ...)                                                                                       \
-  cudaLaunchKernelEx(&cfg, k_stage_f32_one<S, __VA_ARGS__>, k, c, Mn, In, Out, D, tag, sid, rs, tile_body,        \
-                     body_tiles, nb, ds, fuse_cfl, ncfl, tm, ut)
-#define IBM_ONE_V(S)                                                                                           \
-  (wide ? IBM_ONE(S, WIDE_BLOCKS, WIDE)                                                                        \
-        : plain_variant == 1 ? IBM_ONE(S, 7) : plain_variant == 2 ? IBM_ONE(S, 6) : IBM_ONE(S, 8))
+#define IBM_ONE(S, N)                                                                                         \
+  cudaLaunchKernelEx(&cfg, k_stage_f32_one<S, N>, k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, nb,  \
+                     ds, fuse_cfl, ncfl, tm, ut)
+#define IBM_ONE_V(S) (wide ? IBM_ONE(S, WIDE) : IBM_ONE(S, NTH))
 #define IBM_VAR(S, T, Q) (wide ? IBM_VAR_N(S, T, Q, WIDE) : IBM_VAR_N(S, T, Q, NTH))
 #define IBM_VAR_N(S, T, Q, N)                                                                                  \
   cudaLaunchKernelEx(&cfg, k_stage_f32_var<S, T, Q, N>, k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, nb, \

@@ -401,25 +401,20 @@ __host__ inline PertConsts pert_consts(const Consts &k) {
 // Stage kernels of one case: the plain kernel (stream s) covers tiles without
 // IB / ghost nodes near them; the body kernel (stream sb, may run concurrently)
 // covers the listed body tiles and rebuilds IB and ghost nodes from rs / sid
-// while it loads a tile (no separate reconstruction launch).  plain_variant
-// selects the plain kernel's register budget, i.e. its resident blocks per SM
-// (0: 64 registers, eight blocks; 1: 72 registers, seven blocks; 2: 80
-// registers, six blocks); with_body = false launches the plain kernel only
-// (autotuning).
-constexpr int PLAIN_VARIANTS = 3;
+// while it loads a tile (no separate reconstruction launch).
 // Wide blocks (stage32.cuh) for the explicit stage of nt tiles and nb body-tile slots.
 bool stage_wide(int nt, int nb);
 void launch_stage_f32(const Consts &k, int stage, float *Mn, const float *In, float *Out, double *D,
                       const uint8_t *tag, const int *sid, const RStencil32 *rs, const uint8_t *tile_body,
                       const int *body_tiles, int body_cap, DevState *ds, bool fuse_cfl, cudaStream_t s,
-                      cudaStream_t sb, int plain_variant, bool with_body, const CUtensorMap *tmap,
+                      cudaStream_t sb, const CUtensorMap *tmap,
                       const RStencilQ *rsq = nullptr);
 // The same stage as one launch on stream s: body-tile slots first, then one
 // block per tile (no second stream); pdl: launch with programmatic dependent
 // launch, so that the launch overlaps the tail of the preceding stage kernel.
 cudaError_t launch_stage_f32_one(const Consts &k, int stage, float *Mn, const float *In, float *Out, double *D,
                                  const uint8_t *tag, const int *sid, const RStencil32 *rs, const uint8_t *tile_body,
-                                 const int *body_tiles, int body_cap, DevState *ds, bool fuse_cfl, int plain_variant,
+                                 const int *body_tiles, int body_cap, DevState *ds, bool fuse_cfl,
                                  const CUtensorMap *tmap, bool pdl, cudaStream_t s,
                                  const RStencilQ *rsq = nullptr);
 // Tensor maps of the FP32 stage inputs arrays[0..2] (pitch x rows x 4 planes)
