@@ -30,7 +30,7 @@ struct ibm_case {
   double *A = nullptr, *B = nullptr, *C = nullptr;  // FP64 conserved: state, stage arrays (FP64 mode)
   double *Wn = nullptr, *Wm = nullptr;               // dual time: states at time levels n and n-1
   double *G = nullptr;  // FP32-bulk dual time: the step's constant part of the BDF term (in place of W^{n-1})
-  double *Q0 = nullptr;                              // FP32-bulk dual time: (p', u, v, T') of the sub-iteration start
+  double *Q0 = nullptr;                              // FP32-bulk dual time: (p', u', v', T') of the sub-iteration start
   float *M = nullptr, *F1 = nullptr, *F2 = nullptr;  // FP32-bulk: perturbation mirror and stage arrays
   double *stage64 = nullptr;  // FP32-bulk: absolute-variable staging for ibm_get_state (allocated on first use)
   uint8_t *solid = nullptr, *tag = nullptr;

@@ -248,8 +248,9 @@ void launch_recon_f64(const Consts &k, double *U, const ibm_stencil *st, int cap
 // The kernel is bound by the FP64 pipe (fp64_math.cuh; 85% busy in ncu):
 // a window per state with IEEE divisions took about 2,000 FP64 instructions
 // per cell and stage, the shared windows and reciprocals about 540, with
-// products on the integer pipes 370.  768 x 384 wedge: 1.15 -> 0.39 -> 0.245
-// ms per stage, two steps 6.90 -> 3.07 -> 2.21 ms.
+// products on the integer pipes 370, with reciprocals and square roots there
+// too about 330.  768 x 384 wedge, two steps: 6.90 -> 3.07 -> 2.21 -> 1.56 ms
+// (the last with the reconstruction on a cluster).
 // ---------------------------------------------------------------------------
 struct F64Consts {
   double ih[2], g1, ig1, iR;

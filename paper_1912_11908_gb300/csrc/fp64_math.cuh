@@ -3,9 +3,9 @@
 // here is written to issue few of them: plain products, reciprocals and square roots on the integer pipes (the
 // arguments are densities, pressures, speeds and smoothness weights in the normal range); one reciprocal shared where
 // several quotients stand side by side; signs and magnitudes against 1 tested on the integer bits.  With reciprocals and
-// square roots corrected on the FP64 pipe instead: 768 x 384 FP64 wedge, two steps, 1.71 ms (1.53 here); 257 x 131 FP64
-// dual time 5.80 (5.13, also with the update's products off the pipe); 96 x 48 x 48 FP64 sphere 2.94 (2.73); FP32-bulk
-// dual time 2048 x 1024 27.8 (25.5).
+// square roots corrected on the FP64 pipe instead: 768 x 384 FP64 wedge, two steps, 1.71 ms (1.56 here); 257 x 131 FP64
+// dual time 5.80 (5.25, also with the update's products off the pipe); 96 x 48 x 48 FP64 sphere 2.94 (2.76); FP32-bulk
+// dual time 2048 x 1024 27.8 (25.6).
 #pragma once
 
 namespace ibm {
