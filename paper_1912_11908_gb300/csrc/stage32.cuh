@@ -282,7 +282,7 @@ __device__ __forceinline__ bool tma_wait(unsigned long long *mbar, unsigned pari
 __device__ __forceinline__ float cfl_lambda(const Consts &k, const PertConsts &c, const float m[4]) {
   float u, v, pp, Tp;
   pert_prim(c, m[0], m[1], m[2], m[3], u, v, pp, Tp);
-  const float r = 1.f + m[0];
+  const float r = __fadd_rn(1.f, m[0]);  // as pert_prim has it: one reciprocal
   const float cs = sqrtf(c.gamma * (c.R + pp) / r);
   return (fabsf(u) + cs) * c.idx + (fabsf(v) + cs) * c.idy + c.vis / r;
 }
@@ -638,19 +638,24 @@ __device__ __forceinline__ void stage_tile(const Consts &k, const PertConsts &c,
 #pragma unroll
       for (int q = 0; q < 4; q++) w[r][q] = in ? ld_stage<PERSIST>(p + q * P) : 0.f;  // free stream: zero perturbation
     }
+    static_assert(NC % 2 == 0, "converted two at a time");
 #pragma unroll
-    for (int r = 0; r < NC; r++) {
-      const int m = threadIdx.x + r * NT;
-      if (m >= HX * HY) break;
-      float u, v, pp, Tp;
-      pert_prim(c, w[r][0], w[r][1], w[r][2], w[r][3], u, v, pp, Tp);
-      float *o = &sm.q[0][m];
-      o[0] = w[r][0];
-      o[VP] = u;
-      o[2 * VP] = v;
-      o[3 * VP] = pp;
-      o[4 * VP] = Tp;
-      if (BODY) list_node(m, e[r]);
+    for (int r = 0; r < NC; r += 2) {
+      f2 u, v, pp, Tp;
+      pert_prim2(c, f2{w[r][0], w[r + 1][0]}, f2{w[r][1], w[r + 1][1]}, f2{w[r][2], w[r + 1][2]},
+                 f2{w[r][3], w[r + 1][3]}, u, v, pp, Tp);
+#pragma unroll
+      for (int s = 0; s < 2; s++) {
+        const int m = threadIdx.x + (r + s) * NT;
+        if (m >= HX * HY) break;
+        float *o = &sm.q[0][m];
+        o[0] = w[r + s][0];
+        o[VP] = s ? u.y : u.x;
+        o[2 * VP] = s ? v.y : v.x;
+        o[3 * VP] = s ? pp.y : pp.x;
+        o[4 * VP] = s ? Tp.y : Tp.x;
+        if (BODY) list_node(m, e[r + s]);
+      }
     }
   }
   __syncthreads();
