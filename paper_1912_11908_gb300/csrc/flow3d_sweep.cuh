@@ -11,7 +11,7 @@
 // One thread per face with both windows of every face, and flux arrays in memory, took 1.5x the instructions and 35
 // array passes per stage; a thread marching along y or z with the windows sliding through registers took fewest
 // instructions but waits on memory with too few warps (192 x 96 x 96, FP32-bulk, per sweep: 65 us by faces, 129 us
-// marching, 52 here).  FP32-bulk is bound by issue slots (63-79% busy) and, in the x sweep, by the update's operands;
+// marching, 52 here).  FP32-bulk is bound by issue slots (74-80% busy) and, in the x sweep, by the update's operands;
 // FP64 by the FP64 pipe.  A step: FP32-bulk 192 x 96 x 96 0.95 -> 0.75 ms, FP64 96 x 48 x 48 3.92 -> 1.46 ms (1.38 with
 // the reciprocals on the integer pipes).
 #pragma once
