@@ -529,8 +529,8 @@ int batch_stage_blocks(const StageBatch &b);
 // Dual-time pseudo stage `stage` of every (dual-time, not TVD-2) case of the
 // table as one launch over the combined table, with the same grid and pdl
 // meanings: the one-launch form of a dual-time case alone (a table of one) and
-// of a group of them.
-cudaError_t launch_dual_f32_batch_one(const StageBatch &b, int stage, int grid, bool pdl, cudaStream_t s);
+// of a group of them.  others: tiles of the cases that run beside the table's (the block width's rule).
+cudaError_t launch_dual_f32_batch_one(const StageBatch &b, int stage, int grid, bool pdl, cudaStream_t s, int others = 0);
 
 // ---- batching support (capi.cu), used by the request loop (serve.cu) ----
 // FP32-bulk cases (explicit RK3 with any motion and either reconstruction,

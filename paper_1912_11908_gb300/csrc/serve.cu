@@ -246,6 +246,15 @@ static void retire(ibm_server *s, Active *a, ibm_status st) {
   delete a;
 }
 
+// stage tiles of the running cases that are not in group g
+static int tiles_beside(const ibm_server *s, const Group *g) {
+  const auto along = [](int cells) { return (cells + STAGE_TILE - 1) / STAGE_TILE; };
+  long long n = 0;
+  for (const Active *a : s->active)
+    if (a->group != g) n += (long long)along(a->req->grid.nx) * along(a->req->grid.ny);
+  return (int)std::min(n, 1LL << 30);
+}
+
 // the group's table: member descriptors and tile offsets (kernel parameters of the stage launches)
 static void build_table(Group *g) {
   const int n = (int)g->members.size();
@@ -280,9 +289,10 @@ static ibm_status capture_group(ibm_server *s, Group *g) {
   // one launch per stage over the combined table, stages chained by programmatic launch
   const bool nonempty = b.plain_start[b.n] + b.body_start[b.n] > 0;
   if (g->subiters > 0) {
+    const int others = tiles_beside(s, g);
     for (int it = 0; it < g->subiters; it++)
       for (int st = 1; st <= 3; st++) {
-        launch_dual_f32_batch_one(b, st, g->plain_grid, true, g->s);
+        launch_dual_f32_batch_one(b, st, g->plain_grid, true, g->s, others);
         nk += nonempty;
       }
   } else {
