@@ -48,6 +48,12 @@ __global__ void __launch_bounds__(NT, NT == NTH ? BATCH_BLOCKS : WIDE_BLOCKS) k_
   }
 }
 
+static bool table_wide(const StageBatch &b) {
+  bool rebuild = false;
+  for (int q = 0; q < b.n; q++) rebuild |= b.cs[q].nb > 0 && !b.cs[q].k.ib_advance;
+  return stage_wide(b.plain_start[b.n], b.body_start[b.n], rebuild);
+}
+
 // Blocks of the table's stage kernel resident per SM.
 extern "C" int ibm__batch_blocks_per_sm(int wide, int tvd, int quad) {
   int per = 0;
@@ -62,7 +68,7 @@ extern "C" int ibm__batch_blocks_per_sm(int wide, int tvd, int quad) {
 }
 
 int batch_stage_blocks(const StageBatch &b) {
-  return ibm__batch_blocks_per_sm(stage_wide(b.plain_start[b.n], b.body_start[b.n]), b.cs[0].k.tvd2, b.cs[0].k.quad);
+  return ibm__batch_blocks_per_sm(table_wide(b), b.cs[0].k.tvd2, b.cs[0].k.quad);
 }
 
 cudaError_t launch_stage_f32_batch_one(const StageBatch &b, int stage, int grid, bool pdl, cudaStream_t s) {
@@ -70,7 +76,7 @@ cudaError_t launch_stage_f32_batch_one(const StageBatch &b, int stage, int grid,
   if (total == 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)(grid > 0 && grid < total ? grid : total));
-  const bool wide = stage_wide(b.plain_start[b.n], b.body_start[b.n]);
+  const bool wide = table_wide(b);
   cfg.blockDim = dim3(wide ? WIDE : NTH);
   cfg.stream = s;
   cudaLaunchAttribute at[1];

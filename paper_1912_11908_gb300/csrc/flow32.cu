@@ -177,14 +177,16 @@ __global__ void __launch_bounds__(NT, NT == NTH ? 7 : WIDE_BLOCKS)
 }
 
 // Wide blocks where the tiles leave the chip short of work and a step lasts as long as its chains of tiles: up to one
-// wave of wide blocks, or two where body tiles, the longest chains, are among them.  Per step, 128 threads against 288
-// (the step before the packed tile in brackets): no body 64 x 64 29 us, 18 (23), 640 x 320 46, 45 (48), 768 x 384 49, 57
-// (60); cylinder 64 x 64 37, 29 (35), 256 x 128 47, 35 (43), 512 x 256 50, 40 (51), 640 x 320 58, 45 (59), 1024 x 512
-// 75, 90 (92).
-extern "C" int ibm__stage_wide(int nt, int nb, int sms) {
-  return nt <= WIDE_BLOCKS * sms || (nb > 0 && nt <= 2 * WIDE_BLOCKS * sms);
+// wave of wide blocks; two where body tiles, the longest chains, are among them; and where these rebuild IB nodes, up
+// to the one wave that 128-thread blocks would make (eight per SM).  Per step, 128 threads against 288 (the step before
+// the packed tile in brackets): no body 64 x 64 29 us, 18 (23), 640 x 320 46, 45 (48), 768 x 384 49, 57 (60); cylinder
+// 64 x 64 37, 29 (35), 256 x 128 47, 35 (43), 512 x 256 50, 40 (51), 640 x 352 59, 46 (59), 512 x 512 60, 55 (59),
+// 736 x 384 68, 59 (66), 1024 x 512 75, 90 (92); with IB nodes advanced 512 x 288 44, 39 (42), 640 x 352 48, 45 (49),
+// 640 x 384 48, 53 (55), 768 x 384 49, 57 (60).
+extern "C" int ibm__stage_wide(int nt, int nb, int rebuild, int sms) {
+  return nt <= (nb <= 0 ? WIDE_BLOCKS : rebuild ? 8 : 2 * WIDE_BLOCKS) * sms;
 }
-bool stage_wide(int nt, int nb) { return ibm__stage_wide(nt, nb, sm_count()) != 0; }
+bool stage_wide(int nt, int nb, bool rebuild) { return ibm__stage_wide(nt, nb, rebuild, sm_count()) != 0; }
 
 int stage_tiles(const Consts &k) { return ((k.nx + TX - 1) / TX) * ((k.ny + TY - 1) / TY); }
 
@@ -284,7 +286,7 @@ void launch_stage_f32(const Consts &k, int stage, float *Mn, const float *In, fl
   std::memset(&tm, 0, sizeof tm);
   if (tmap) tm = *tmap;
   const int ut = tmap ? 1 : 0;
-  const bool wide = stage_wide(nt, nb);
+  const bool wide = stage_wide(nt, nb, !k.ib_advance);
 #define IBM_ARGS k, c, Mn, In, Out, D, tag, sid, rs, tile_body, body_tiles, ds, fuse_cfl, ncfl, tm, ut
 #define IBM_STAGE_PAIR_N(S, N)                                                \
   do {                                                                         \
@@ -319,7 +321,7 @@ cudaError_t launch_stage_f32_one(const Consts &k, int stage, float *Mn, const fl
   const int ut = tmap ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)(nt + nb));
-  const bool wide = stage_wide(nt, nb);
+  const bool wide = stage_wide(nt, nb, !k.ib_advance);
   cfg.blockDim = dim3(wide ? WIDE : NTH);
   cfg.stream = s;
   cudaLaunchAttribute at[1];

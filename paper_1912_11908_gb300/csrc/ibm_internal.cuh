@@ -402,8 +402,8 @@ __host__ inline PertConsts pert_consts(const Consts &k) {
 // IB / ghost nodes near them; the body kernel (stream sb, may run concurrently)
 // covers the listed body tiles and rebuilds IB and ghost nodes from rs / sid
 // while it loads a tile (no separate reconstruction launch).
-// Wide blocks (stage32.cuh) for the explicit stage of nt tiles and nb body-tile slots.
-bool stage_wide(int nt, int nb);
+// Wide blocks (stage32.cuh) for the explicit stage of nt tiles and nb body-tile slots, rebuild: IB nodes among them.
+bool stage_wide(int nt, int nb, bool rebuild);
 void launch_stage_f32(const Consts &k, int stage, float *Mn, const float *In, float *Out, double *D,
                       const uint8_t *tag, const int *sid, const RStencil32 *rs, const uint8_t *tile_body,
                       const int *body_tiles, int body_cap, DevState *ds, bool fuse_cfl, cudaStream_t s,

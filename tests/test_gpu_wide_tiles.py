@@ -10,7 +10,7 @@ from test_gpu_pairs32 import _run
 
 pytestmark = pytest.mark.gpu
 
-GRIDS = [(1009, 249), (497, 507)]  # 1,024 tiles each, all four sides ragged
+GRIDS = [(1009, 249), (497, 507), (1009, 331), (661, 507)]  # 1,024 tiles each, then 1,344: all four sides ragged
 
 
 @pytest.mark.parametrize("nx,ny", GRIDS)

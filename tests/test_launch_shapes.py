@@ -42,17 +42,19 @@ def wide():
     from paper_1912_11908_gb300 import _build, ibm as mod
     _build.build()
     f = mod.lib().ibm__stage_wide
-    f.argtypes = [ctypes.c_int] * 3
+    f.argtypes = [ctypes.c_int] * 4
     f.restype = ctypes.c_int
     return f
 
 
 def test_wide_blocks_for_few_tiles(wide):
-    """One wave of wide blocks (three per SM) without body tiles, two with them."""
+    """One wave of wide blocks (three per SM) without body tiles, two with them, one of 128-thread blocks (eight per
+    SM) where IB nodes are rebuilt in them."""
     for sms in (1, 76, 148, 152):
-        for nt, nb, want in ((1, 0, 1), (3 * sms, 0, 1), (3 * sms + 1, 0, 0), (3 * sms + 1, 1, 1), (6 * sms, 9, 1),
-                             (6 * sms + 1, 9, 0)):
-            assert bool(wide(nt, nb, sms)) == bool(want), (nt, nb, sms)
+        for nt, nb, rebuild, want in ((1, 0, 1, 1), (3 * sms, 0, 1, 1), (3 * sms + 1, 0, 1, 0), (3 * sms + 1, 1, 0, 1),
+                                      (6 * sms, 9, 0, 1), (6 * sms + 1, 9, 0, 0), (8 * sms, 9, 1, 1),
+                                      (8 * sms + 1, 9, 1, 0)):
+            assert bool(wide(nt, nb, rebuild, sms)) == bool(want), (nt, nb, rebuild, sms)
 
 
 def test_wide_blocks_in_dual_time(wide):
