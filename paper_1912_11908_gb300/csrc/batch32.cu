@@ -18,8 +18,10 @@ namespace ibm {
 // complete).
 // TVD / QUAD: the TVD-2 reconstruction and / or the quadratic IB / ghost reconstruction compiled in (a group
 // holds cases of one variant)
-template <int STAGE, bool TVD, bool QUAD, int NT>
-__global__ void __launch_bounds__(NT, NT == NTH ? BATCH_BLOCKS : WIDE_BLOCKS) k_stage_f32_batch_one(const __grid_constant__ StageBatch b) {
+// BLOCKS of NT threads per SM: BATCH_BLOCKS, BATCH_FEW (80 registers and 68 to 308 bytes of spills where 64 registers
+// leave 152 to 384: a case's constants come from memory, not as operands from the parameters) or WIDE_BLOCKS
+template <int STAGE, bool TVD, bool QUAD, int NT, int BLOCKS>
+__global__ void __launch_bounds__(NT, BLOCKS) k_stage_f32_batch_one(const __grid_constant__ StageBatch b) {
   __shared__ TileSmem sm;
   __shared__ StageCase sc;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -54,21 +56,36 @@ static bool table_wide(const StageBatch &b) {
   return stage_wide(b.plain_start[b.n], b.body_start[b.n], rebuild);
 }
 
-// Blocks of the table's stage kernel resident per SM.
-extern "C" int ibm__batch_blocks_per_sm(int wide, int tvd, int quad) {
+// Blocks of 128 threads per SM of a table of nt plain tiles.  Where the table is a wave or two, the spills lengthen
+// every tile's chain and the eighth block is not needed; more tiles use the room.  Per step, eight blocks against six
+// (the step before the packed tile in brackets): 640 x 512 alone 78 us, 68 (66), three of 384 x 384 88, 79 (81),
+// 1024 x 512 96, 93 (91), moving 169, 160 (160), three of 512 x 512 136, 135 (130); 2048 x 1024 295, 307 (314).
+extern "C" int ibm__batch_blocks(int nt, int sms) { return nt <= 20LL * sms ? BATCH_FEW : BATCH_BLOCKS; }
+
+// Form of a table's launch: 0 BATCH_BLOCKS, 1 wide blocks, 2 BATCH_FEW.
+static int table_form(const StageBatch &b) {
+  return table_wide(b) ? 1 : ibm__batch_blocks(b.plain_start[b.n], sm_count()) == BATCH_FEW ? 2 : 0;
+}
+
+// Blocks of that form's stage kernel resident per SM.
+extern "C" int ibm__batch_blocks_per_sm(int form, int tvd, int quad) {
   int per = 0;
-#define IBM_OCC(T, Q)                                                                                                 \
-  (wide ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_stage_f32_batch_one<1, T, Q, WIDE>, WIDE, 0)          \
-        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_stage_f32_batch_one<1, T, Q, NTH>, NTH, 0))
+#define IBM_OCC_N(T, Q, N, B) \
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_stage_f32_batch_one<1, T, Q, N, B>, N, 0)
+#define IBM_OCC(T, Q)                                 \
+  (form == 1   ? IBM_OCC_N(T, Q, WIDE, WIDE_BLOCKS)   \
+   : form == 2 ? IBM_OCC_N(T, Q, NTH, BATCH_FEW)      \
+               : IBM_OCC_N(T, Q, NTH, BATCH_BLOCKS))
   const cudaError_t e = tvd ? (quad ? IBM_OCC(true, true) : IBM_OCC(true, false))
                             : (quad ? IBM_OCC(false, true) : IBM_OCC(false, false));
 #undef IBM_OCC
+#undef IBM_OCC_N
   if (e != cudaSuccess) cudaGetLastError();
   return e == cudaSuccess ? per : 0;
 }
 
 int batch_stage_blocks(const StageBatch &b) {
-  return ibm__batch_blocks_per_sm(table_wide(b), b.cs[0].k.tvd2, b.cs[0].k.quad);
+  return ibm__batch_blocks_per_sm(table_form(b), b.cs[0].k.tvd2, b.cs[0].k.quad);
 }
 
 cudaError_t launch_stage_f32_batch_one(const StageBatch &b, int stage, int grid, bool pdl, cudaStream_t s) {
@@ -76,8 +93,8 @@ cudaError_t launch_stage_f32_batch_one(const StageBatch &b, int stage, int grid,
   if (total == 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)(grid > 0 && grid < total ? grid : total));
-  const bool wide = table_wide(b);
-  cfg.blockDim = dim3(wide ? WIDE : NTH);
+  const int form = table_form(b);
+  cfg.blockDim = dim3(form == 1 ? WIDE : NTH);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -88,15 +105,18 @@ cudaError_t launch_stage_f32_batch_one(const StageBatch &b, int stage, int grid,
   if (quad)
     for (int q = 0; q < b.n; q++)
       if (!b.cs[q].rsq) return cudaErrorInvalidValue;  // the quadratic kernels read the second probes
-#define IBM_BATCH(S, T, Q)                                                  \
-  (wide ? cudaLaunchKernelEx(&cfg, k_stage_f32_batch_one<S, T, Q, WIDE>, b) \
-        : cudaLaunchKernelEx(&cfg, k_stage_f32_batch_one<S, T, Q, NTH>, b))
+#define IBM_BATCH_N(S, T, Q, N, B) cudaLaunchKernelEx(&cfg, k_stage_f32_batch_one<S, T, Q, N, B>, b)
+#define IBM_BATCH(S, T, Q)                              \
+  (form == 1   ? IBM_BATCH_N(S, T, Q, WIDE, WIDE_BLOCKS) \
+   : form == 2 ? IBM_BATCH_N(S, T, Q, NTH, BATCH_FEW)    \
+               : IBM_BATCH_N(S, T, Q, NTH, BATCH_BLOCKS))
 #define IBM_BATCH_S(S)                                                                                          \
   (tvd ? (quad ? IBM_BATCH(S, true, true) : IBM_BATCH(S, true, false))                                          \
        : (quad ? IBM_BATCH(S, false, true) : IBM_BATCH(S, false, false)))
   const cudaError_t e = stage == 1 ? IBM_BATCH_S(1) : stage == 2 ? IBM_BATCH_S(2) : IBM_BATCH_S(3);
 #undef IBM_BATCH_S
 #undef IBM_BATCH
+#undef IBM_BATCH_N
   return e;
 }
 

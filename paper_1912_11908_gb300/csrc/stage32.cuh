@@ -180,8 +180,8 @@ constexpr int NTH = 128;
 // of few tiles (ibm__stage_wide, ibm__dual_wide).
 constexpr int WIDE = 288, WIDE_BLOCKS = 3;
 // Blocks of 128 threads of the block-table kernels per SM: 16 requests 11.3 ms, with seven (72 registers) 11.6, with six
-// (80, hardly a spill) 11.4
-constexpr int BATCH_BLOCKS = 8;
+// (80) 11.4; explicit tables of few tiles take six (ibm__batch_blocks)
+constexpr int BATCH_BLOCKS = 8, BATCH_FEW = 6;
 constexpr int TX = STAGE_TILE, TY = STAGE_TILE, HX = TX + 2 * NG, HY = TY + 2 * NG;
 // Shared memory is laid out for pairs: a thread reconstructs two adjacent rows (x direction) or columns (y direction)
 // and forms the fluxes of their two faces with packed arithmetic.  The face values of a direction are [variable][face

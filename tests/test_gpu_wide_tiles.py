@@ -48,3 +48,31 @@ def test_residency_of_the_table_kernels(ibm):  # noqa: F811
     f.restype = ctypes.c_int
     for wide, want in ((0, 8), (1, 3)):
         assert [f(wide, t, q) for t in (0, 1) for q in (0, 1)] == [want] * 4
+
+
+def test_residency_for_few_tiles(ibm):  # noqa: F811
+    """Six 128-thread blocks per SM of the form that groups of a wave or two take."""
+    import ctypes
+    f = ibm.lib().ibm__batch_blocks_per_sm
+    f.argtypes = [ctypes.c_int] * 3
+    f.restype = ctypes.c_int
+    assert [f(2, t, q) for t in (0, 1) for q in (0, 1)] == [6] * 4
+
+
+@pytest.mark.parametrize("scheme", [W.SCHEME_WENO5, W.SCHEME_TVD2])
+@pytest.mark.parametrize("interp", [W.INTERP_LINEAR, W.INTERP_QUADRATIC])
+@pytest.mark.parametrize("count", [1, 3])
+def test_groups_of_many_tiles(ibm, scheme, interp, count):  # noqa: F811
+    """1,344 tiles (six blocks per SM), three times as many (eight), a case alone: equal up to FP32 rounding."""
+    spec = W.cylinder_m02_re40(1009, 331, precision=W.PREC_FP32_BULK, scheme=scheme, ib_interp=interp)
+    c = ibm.Case(spec)
+    c.step(20)
+    want = c.forces()
+    s = ibm.Server(max_active=32, steps_per_chunk=10)
+    ids = [s.submit(spec, 20) for _ in range(count)]
+    s.drain()
+    for i in ids:
+        r = s.poll(i)
+        assert r["status"] == ibm.IBM_OK and r["steps_done"] == 20
+        np.testing.assert_allclose(r["forces"], want, rtol=2e-5, atol=2e-5 * np.abs(want).max())
+    s.close()

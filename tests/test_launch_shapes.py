@@ -77,3 +77,13 @@ def test_dual_time_groups_beside_other_cases(wide):
         assert [f(4 * sms, 2, 20 * sms, sms), f(4 * sms, 2, 20 * sms + 1, sms), f(7 * sms, 2, 0, sms)] == [1, 0, 0]
         assert [f(16 * sms, 1, 0, sms), f(16 * sms, 1, 8 * sms, sms), f(16 * sms, 1, 9 * sms, sms)] == [1, 1, 0]
         assert f(1, 1, 1 << 30, sms) == 0
+
+
+def test_blocks_of_a_group(wide):
+    """Six 128-thread blocks per SM for explicit groups of up to 20 tiles per SM, eight for larger ones."""
+    from paper_1912_11908_gb300 import ibm as mod
+    f = mod.lib().ibm__batch_blocks
+    f.argtypes = [ctypes.c_int] * 2
+    f.restype = ctypes.c_int
+    for sms in (1, 152):
+        assert [f(1, sms), f(20 * sms, sms), f(20 * sms + 1, sms), f(2 ** 31 - 1, sms)] == [6, 6, 8, 8]
