@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(NT, BLOCKS) k_stage_f32_batch_one(const __grid
 static bool table_wide(const StageBatch &b) {
   bool rebuild = false;
   for (int q = 0; q < b.n; q++) rebuild |= b.cs[q].nb > 0 && !b.cs[q].k.ib_advance;
-  return stage_wide(b.plain_start[b.n], b.body_start[b.n], rebuild);
+  return stage_wide(b.plain_start[b.n], b.body_start[b.n], rebuild, b.cs[0].k.beside);
 }
 
 // Blocks of 128 threads per SM of a table of nt plain tiles.  Where the table is a wave or two, the spills lengthen
@@ -64,7 +64,9 @@ extern "C" int ibm__batch_blocks(int nt, int sms) { return nt <= 20LL * sms ? BA
 
 // Form of a table's launch: 0 BATCH_BLOCKS, 1 wide blocks, 2 BATCH_FEW.
 static int table_form(const StageBatch &b) {
-  return table_wide(b) ? 1 : ibm__batch_blocks(b.plain_start[b.n], sm_count()) == BATCH_FEW ? 2 : 0;
+  const int nt = b.plain_start[b.n];
+  if (table_wide(b)) return 1;
+  return ibm__batch_blocks(nt, sm_count()) == BATCH_FEW && !crowded(nt, b.cs[0].k.beside) ? 2 : 0;
 }
 
 // Blocks of that form's stage kernel resident per SM.

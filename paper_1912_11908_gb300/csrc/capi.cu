@@ -982,6 +982,8 @@ int case_enqueue_poststage(ibm_case *c) {
   return 0;
 }
 
+void case_set_beside(ibm_case *c, int tiles) { c->k.beside = tiles; }
+
 void case_stage_desc(const ibm_case *c, StageCase *out) {
   fill_stage_case(c->k, c->M, c->F1, c->F2, c->A, c->tag, c->sid, c->rst, c->tile_body, c->body_tiles, c->body_cap,
                   c->ds, fused_cfl(c), out);

@@ -15,15 +15,9 @@ namespace ibm {
 // GPU with each other: 16 requests 11.3 ms with wide blocks up to six tiles per SM, 11.5 up to 16; two to eight requests
 // 4 to 18% less than without.
 extern "C" int ibm__dual_wide(int nt, int cases, int sms) { return nt <= (cases > 1 ? 6 : 16) * sms; }
-// Beside `others` tiles of cases that run at the same time, 24 per SM and more in all, the GPU is full either way, and
-// the next pseudo stage's wide blocks, resident and waiting, hold room that the others could use: 16 requests of 48
-// tiles per SM 9.7 ms with them, 9.2 without (9.15 before there were wide blocks); seven to ten requests of up to 20
-// tiles per SM 9 to 26% less with them.
-extern "C" int ibm__dual_wide_beside(int nt, int cases, int others, int sms) {
-  return ibm__dual_wide(nt, cases, sms) && (others <= 0 || nt + (long long)others <= 24LL * sms);
-}
-static bool dual_wide(int nt, int cases = 1, int others = 0) {
-  return ibm__dual_wide_beside(nt, cases, others, sm_count()) != 0;
+// (A burst of 16 requests of 48 tiles per SM took 9.7 ms with wide blocks beside many tiles, 9.2 without.)
+static bool dual_wide(int nt, int beside, int cases = 1) {
+  return ibm__dual_wide(nt, cases, sm_count()) && !crowded(nt, beside);
 }
 
 // Dual-time pseudo stage of one case (FP32 residual, FP64 point-implicit
@@ -82,7 +76,7 @@ cudaError_t launch_dual_f32_var(const Consts &k, int stage, const float *In32, f
   dp.Q0 = Q0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)(nt + nb));
-  const bool wide = dual_wide(nt);
+  const bool wide = dual_wide(nt, k.beside);
   cfg.blockDim = dim3(wide ? WIDE : NTH);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -145,12 +139,12 @@ __global__ void __launch_bounds__(NT, NT == NTH ? BATCH_BLOCKS : WIDE_BLOCKS) k_
   }
 }
 
-cudaError_t launch_dual_f32_batch_one(const StageBatch &b, int stage, int grid, bool pdl, cudaStream_t s, int others) {
+cudaError_t launch_dual_f32_batch_one(const StageBatch &b, int stage, int grid, bool pdl, cudaStream_t s) {
   const int total = b.body_start[b.n] + b.plain_start[b.n];
   if (total == 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)(grid > 0 && grid < total ? grid : total));
-  const bool wide = dual_wide(b.plain_start[b.n], b.n, others);
+  const bool wide = dual_wide(b.plain_start[b.n], b.cs[0].k.beside, b.n);
   cfg.blockDim = dim3(wide ? WIDE : NTH);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -211,7 +205,7 @@ void launch_dual_f32(const Consts &k, int stage, const float *In32, float *Out32
     if (wide) IBM_DUAL_PAIR_N(S, WIDE); \
     else IBM_DUAL_PAIR_N(S, NTH);   \
   } while (0)
-  const bool wide = dual_wide(nt);
+  const bool wide = dual_wide(nt, k.beside);
   if (stage == 1) IBM_DUAL_PAIR(1);
   else if (stage == 2) IBM_DUAL_PAIR(2);
   else IBM_DUAL_PAIR(3);

@@ -78,6 +78,7 @@ struct Consts {
   int dual;         // dual time stepping (preconditioned pseudo time, BDF2 physical time)
   int ib_advance;   // IB nodes advanced by the flux update; the ghost layers alone impose the wall
   int subiters;     // dual time: sub-iterations per physical step
+  int beside;       // stage tiles of other cases that run at the same time (set by the request loop; launch rules only)
   double dt_phys;   // dual time: physical step
   double cfl_tau;   // dual time: pseudo-time CFL number
   double iR, ig1;   // 1/R and 1/(gamma - 1)
@@ -402,8 +403,10 @@ __host__ inline PertConsts pert_consts(const Consts &k) {
 // IB / ghost nodes near them; the body kernel (stream sb, may run concurrently)
 // covers the listed body tiles and rebuilds IB and ghost nodes from rs / sid
 // while it loads a tile (no separate reconstruction launch).
+// Do nt tiles and `beside` tiles of other cases fill the GPU whatever the block width?
+bool crowded(int nt, int beside);
 // Wide blocks (stage32.cuh) for the explicit stage of nt tiles and nb body-tile slots, rebuild: IB nodes among them.
-bool stage_wide(int nt, int nb, bool rebuild);
+bool stage_wide(int nt, int nb, bool rebuild, int beside);
 void launch_stage_f32(const Consts &k, int stage, float *Mn, const float *In, float *Out, double *D,
                       const uint8_t *tag, const int *sid, const RStencil32 *rs, const uint8_t *tile_body,
                       const int *body_tiles, int body_cap, DevState *ds, bool fuse_cfl, cudaStream_t s,
@@ -529,8 +532,8 @@ int batch_stage_blocks(const StageBatch &b);
 // Dual-time pseudo stage `stage` of every (dual-time, not TVD-2) case of the
 // table as one launch over the combined table, with the same grid and pdl
 // meanings: the one-launch form of a dual-time case alone (a table of one) and
-// of a group of them.  others: tiles of the cases that run beside the table's (the block width's rule).
-cudaError_t launch_dual_f32_batch_one(const StageBatch &b, int stage, int grid, bool pdl, cudaStream_t s, int others = 0);
+// of a group of them.
+cudaError_t launch_dual_f32_batch_one(const StageBatch &b, int stage, int grid, bool pdl, cudaStream_t s);
 
 // ---- batching support (capi.cu), used by the request loop (serve.cu) ----
 // FP32-bulk cases (explicit RK3 with any motion and either reconstruction,
@@ -558,6 +561,8 @@ int case_enqueue_prestage(ibm_case *c);
 // enqueued.  Graph-capturable.
 int case_enqueue_poststage(ibm_case *c);
 void case_stage_desc(const ibm_case *c, StageCase *out);
+// tiles of other cases beside the case's (before its first step)
+void case_set_beside(ibm_case *c, int tiles);
 cudaStream_t case_stream(const ibm_case *c);
 void case_add_launches(ibm_case *c, long long n);
 

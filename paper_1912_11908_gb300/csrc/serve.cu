@@ -246,27 +246,31 @@ static void retire(ibm_server *s, Active *a, ibm_status st) {
   delete a;
 }
 
-// stage tiles of the running cases that are not in group g
-static int tiles_beside(const ibm_server *s, const Group *g) {
+// stage tiles of the running cases beside group g, or beside a case on its own stream
+static int tiles_beside(const ibm_server *s, const Group *g, const Active *own) {
   const auto along = [](int cells) { return (cells + STAGE_TILE - 1) / STAGE_TILE; };
   long long n = 0;
   for (const Active *a : s->active)
-    if (a->group != g) n += (long long)along(a->req->grid.nx) * along(a->req->grid.ny);
+    if (a != own && (!g || a->group != g)) n += (long long)along(a->req->grid.nx) * along(a->req->grid.ny);
   return (int)std::min(n, 1LL << 30);
 }
 
 // the group's table: member descriptors and tile offsets (kernel parameters of the stage launches)
-static void build_table(Group *g) {
+static void build_table(const ibm_server *s, Group *g) {
   const int n = (int)g->members.size();
   StageCase cs[MAX_BATCH];
-  for (int q = 0; q < n; q++) case_stage_desc(g->members[q]->c, &cs[q]);
+  const int beside = tiles_beside(s, g, nullptr);
+  for (int q = 0; q < n; q++) {
+    case_stage_desc(g->members[q]->c, &cs[q]);
+    cs[q].k.beside = beside;
+  }
   build_stage_batch(cs, n, g->batch);
 }
 
 // Capture one step of the group: pre-stage work of each member on its own
 // stream, then the three batched stages (one launch each over the combined table).
 static ibm_status capture_group(ibm_server *s, Group *g) {
-  build_table(g);
+  build_table(s, g);
   const StageBatch &b = *g->batch;
   cudaGraph_t graph = nullptr;
   if (cudaStreamBeginCapture(g->s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
@@ -289,10 +293,9 @@ static ibm_status capture_group(ibm_server *s, Group *g) {
   // one launch per stage over the combined table, stages chained by programmatic launch
   const bool nonempty = b.plain_start[b.n] + b.body_start[b.n] > 0;
   if (g->subiters > 0) {
-    const int others = tiles_beside(s, g);
     for (int it = 0; it < g->subiters; it++)
       for (int st = 1; st <= 3; st++) {
-        launch_dual_f32_batch_one(b, st, g->plain_grid, true, g->s, others);
+        launch_dual_f32_batch_one(b, st, g->plain_grid, true, g->s);
         nk += nonempty;
       }
   } else {
@@ -481,6 +484,7 @@ extern "C" ibm_status ibm_server_progress(ibm_server *s, int *n_active, int *n_p
     if (a->group || a->launched >= a->req->nsteps) continue;
     if (cudaEventQuery(a->done) == cudaErrorNotReady) continue;
     const int n = std::min(a->req->nsteps - a->launched, s->chunk);
+    if (a->launched == 0) case_set_beside(a->c, tiles_beside(s, nullptr, a));
     ibm_status st = ibm_step(a->c, n);
     if (st != IBM_OK) {
       a->launched = a->req->nsteps;  // retired (as failed) on the next pass
@@ -501,7 +505,7 @@ extern "C" ibm_status ibm_server_progress(ibm_server *s, int *n_active, int *n_p
     if (g->dirty) {
       const auto h0 = std::chrono::steady_clock::now();
       if (s->mode & IBM_SERVE_AUTOTUNE) {
-        build_table(g);
+        build_table(s, g);
         autotune(s, g);
       }
       st = capture_group(s, g);

@@ -67,16 +67,15 @@ def test_wide_blocks_in_dual_time(wide):
         assert [f(16 * sms, 1, sms), f(16 * sms + 1, 1, sms), f(6 * sms, 2, sms), f(6 * sms + 1, 2, sms)] == [1, 0, 1, 0]
 
 
-def test_dual_time_groups_beside_other_cases(wide):
-    """Wide blocks only while the group and the cases beside it hold up to 24 tiles per SM."""
+def test_beside_other_cases(wide):
+    """Crowded from 24 tiles per SM on, a case's or group's own and those beside it; never alone."""
     from paper_1912_11908_gb300 import ibm as mod
-    f = mod.lib().ibm__dual_wide_beside
-    f.argtypes = [ctypes.c_int] * 4
+    f = mod.lib().ibm__crowded
+    f.argtypes = [ctypes.c_int] * 3
     f.restype = ctypes.c_int
     for sms in (1, 152):
-        assert [f(4 * sms, 2, 20 * sms, sms), f(4 * sms, 2, 20 * sms + 1, sms), f(7 * sms, 2, 0, sms)] == [1, 0, 0]
-        assert [f(16 * sms, 1, 0, sms), f(16 * sms, 1, 8 * sms, sms), f(16 * sms, 1, 9 * sms, sms)] == [1, 1, 0]
-        assert f(1, 1, 1 << 30, sms) == 0
+        assert [f(4 * sms, 20 * sms, sms), f(4 * sms, 20 * sms + 1, sms), f(100 * sms, 0, sms)] == [0, 1, 0]
+        assert f(1, 1 << 30, sms) == 1
 
 
 def test_blocks_of_a_group(wide):
